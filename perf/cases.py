@@ -104,8 +104,8 @@ def _features(kind, rows, cols, g):
     return x
 
 
-def prepare(case, seed):
-    widths, l, nS, op = _widths(case), case["l"], case["nS"], case["op"]
+def _inputs(case, seed):
+    widths, l, nS = _widths(case), case["l"], case["nS"]
     g = torch.Generator(device=DEVICE)
     g.manual_seed(seed)
     X = _features(case["x"], l, widths[0], g)
@@ -121,7 +121,12 @@ def prepare(case, seed):
     theta = torch.cat(parts)
     idx = torch.randperm(l, device=DEVICE, generator=g)[:nS].to(torch.int32)
     v = torch.randn(theta.numel(), device=DEVICE, generator=g)
+    return X, Y, theta, idx, v
 
+
+def prepare(case, seed):
+    widths, l, op = _widths(case), case["l"], case["op"]
+    X, Y, theta, idx, v = _inputs(case, seed)
     ctx = gn.GnContext(widths, float(l), X, Y, gn.GN_TF32 if case["prec"] == "tf32" else gn.GN_FP32_ACCURATE)
     if case.get("split"):
         ctx.set_split([int(s) for s in case["split"].split("-")])
@@ -163,6 +168,173 @@ def run(s):
     s["direction"].zero_()
     rep = ctx.newton_iter(s["theta_new"], s["idx"], s["direction"], s["params"])
     return {"theta": s["theta_new"], "direction": s["direction"], "f_before": rep["f_before"], "f_after": rep["f_after"]}
+
+
+class _Exact:
+    """The same mathematics in 64 bits: explicit layers, rows taken `ROWS` at a time."""
+    ROWS = 16384
+
+    def __init__(self, case, seed):
+        X, Y, theta, idx, v = _inputs(case, seed)
+        self.widths, self.l, self.X, self.Y, self.S = _widths(case), case["l"], X, Y, idx.long()
+        self.theta, self.v, self.C = theta.double(), v.double(), float(case["l"])
+        self.L = len(self.widths) - 1
+        self.masks = self._masks([int(s) for s in case["split"].split("-")]) if case.get("split") else None
+
+    def layers(self, vec):
+        """[(W^m as n_m x n_{m-1}, b^m)] views of a vector laid out like theta."""
+        out, at = [], 0
+        for a, b in zip(self.widths[:-1], self.widths[1:]):
+            out.append((vec[at:at + a * b].view(b, a), vec[at + a * b:at + (a + 1) * b]))
+            at += (a + 1) * b
+        return out
+
+    def _masks(self, split):
+        """One vector of booleans per partition: group a of layer m - 1 to group b of layer m, biases with a = 0."""
+        group = [torch.zeros(w, dtype=torch.long, device=DEVICE) for w in self.widths]
+        for w, s, gr in zip(self.widths, split, group):
+            for k in range(s):
+                gr[k * w // s:(k + 1) * w // s] = k
+        masks = []
+        for m in range(1, self.L + 1):
+            for a in range(split[m - 1]):
+                for b in range(split[m]):
+                    mask = torch.zeros_like(self.theta, dtype=torch.bool)
+                    W, bias = self.layers(mask)[m - 1]
+                    W.copy_((group[m] == b)[:, None] & (group[m - 1] == a)[None, :])
+                    bias.copy_((group[m] == b) & (a == 0))
+                    masks.append(mask)
+        return masks
+
+    def forward(self, theta, x):
+        z = [x.double()]
+        for m, (W, b) in enumerate(self.layers(theta), 1):
+            s = torch.addmm(b, z[-1], W.T)
+            z.append(torch.sigmoid(s) if m < self.L else s)
+        return z
+
+    def backward(self, z, delta, out, scale, lowest=1):
+        """out += scale J^T delta for the layers from `lowest` up."""
+        W, O = self.layers(self.theta_now), self.layers(out)
+        for m in range(self.L, lowest - 1, -1):
+            O[m - 1][0].addmm_(delta.T, z[m - 1], alpha=scale)
+            O[m - 1][1].add_(delta.sum(0), alpha=scale)
+            if m > lowest:
+                delta = (delta @ W[m - 1][0]) * z[m - 1] * (1 - z[m - 1])
+
+    def fun(self, theta, grad=None):
+        self.theta_now, loss = theta, 0.0
+        for r in range(0, self.l, self.ROWS):
+            z = self.forward(theta, self.X[r:r + self.ROWS])
+            d = z[-1] - self.Y[r:r + self.ROWS]
+            loss += float((d * d).sum())
+            if grad is not None:
+                self.backward(z, 2 * d, grad, 1.0 / self.l)
+        if grad is not None:
+            grad.add_(theta, alpha=1.0 / self.C)
+        return float(theta @ theta) / (2 * self.C) + loss / self.l
+
+    def grad(self):
+        g = torch.zeros_like(self.theta)
+        f = self.fun(self.theta, g)
+        return g, f
+
+    def Gv(self, v, blocks=False):
+        """G^S v, or, `blocks`, the part of it that stays inside each block (layer, or partition of the split)."""
+        self.theta_now, out = self.theta, v / self.C
+        W, n = self.layers(self.theta), self.S.numel()
+        if not blocks:
+            parts = [None]
+        elif self.masks is None:
+            parts = list(range(1, self.L + 1))
+        else:
+            parts = self.masks
+        for r in range(0, n, self.ROWS):
+            z = self.forward(self.theta, self.X[self.S[r:r + self.ROWS]])
+            for part in parts:
+                mask = part if torch.is_tensor(part) else None
+                V = self.layers(v if mask is None else v * mask)
+                only = range(1, self.L + 1) if not isinstance(part, int) else [part]
+                rz = torch.zeros_like(z[0])
+                for m in range(1, self.L + 1):
+                    rs = rz @ W[m - 1][0].T
+                    if m in only:
+                        rs += torch.addmm(V[m - 1][1], z[m - 1], V[m - 1][0].T)
+                    rz = rs * z[m] * (1 - z[m]) if m < self.L else rs
+                if part is None:
+                    self.backward(z, 2 * rz, out, 1.0 / n)
+                    continue
+                add = torch.zeros_like(out)
+                if isinstance(part, int):
+                    self.backward(z, 2 * rz, add, 1.0 / n, part)
+                    for m, (A, b) in enumerate(self.layers(add), 1):
+                        if m != part:
+                            A.zero_(), b.zero_()
+                else:
+                    self.backward(z, 2 * rz, add, 1.0 / n)
+                    add *= mask
+                out += add
+        return out
+
+    def cg(self, g, steps, blocks, tol=0.0):
+        """At most `steps` steps of conjugate gradient from zero; one independent solve per layer with `blocks`."""
+        ends = [0]
+        for a, b in zip(self.widths[:-1], self.widths[1:]):
+            ends.append(ends[-1] + (a + 1) * b)
+        spans = [slice(a, b) for a, b in zip(ends[:-1], ends[1:])] if blocks else [slice(0, ends[-1])]
+        d, r = torch.zeros_like(g), -g
+        p, rho = r.clone(), [float(r[s] @ r[s]) for s in spans]
+        norms, goal = [math.sqrt(sum(rho))], [tol * math.sqrt(k) for k in rho]
+        for _ in range(steps):
+            if all(math.sqrt(k) <= t for k, t in zip(rho, goal)):
+                break
+            q = self.Gv(p, blocks) + LAMBDA * p
+            for k, s in enumerate(spans):
+                pq = float(p[s] @ q[s])
+                if math.sqrt(rho[k]) <= goal[k]:
+                    continue                # this solve has met its test
+                alpha = rho[k] / pq
+                d[s] += alpha * p[s]
+                r[s] -= alpha * q[s]
+                new = float(r[s] @ r[s])
+                p[s] = r[s] + new / rho[k] * p[s]
+                rho[k] = new
+            norms.append(math.sqrt(sum(rho)))
+        return d, norms
+
+    def newton(self, steps):
+        eta, max_backtrack = 1e-4, 30       # what NewtonParams sets where a caller does not
+        g, f0 = self.grad()
+        d, _ = self.cg(g, steps, True)      # (the previous direction is zero: the two-variable system reduces to d)
+        alpha, slope, f1 = 1.0, float(g @ d), 0.0
+        for k in range(max_backtrack + 1):
+            f1 = self.fun(self.theta + alpha * d)
+            if f1 <= f0 + eta * alpha * slope or k == max_backtrack:
+                break
+            alpha /= 2
+        return {"theta": self.theta + alpha * d, "direction": d, "f_before": f0, "f_after": f1}
+
+
+def exact(case, seed):
+    op = case["op"]
+    if case.get("split"):
+        s = [int(k) for k in case["split"].split("-")]
+        if sum(a * b for a, b in zip(s[:-1], s[1:])) * _macs(_widths(case))["gv"] * 2.0 * case["nS"] > 1.5e14:
+            return None                     # (one pass per partition)
+    e = _Exact(case, seed)
+    if op in ("gv", "first"):
+        return e.Gv(e.v)
+    if op == "block":
+        return e.Gv(e.v, True)
+    if op == "cg":
+        d, norms = e.cg(e.grad()[0], case["steps"], bool(case.get("blockdiag")), case["tol"])
+        return {"d": d, "steps": None, "residuals": np.asarray(norms)}
+    if op == "grad":
+        g, f = e.grad()
+        return {"g": g, "f": f}
+    if op == "fun":
+        return e.fun(e.theta)
+    return e.newton(case["steps"])
 
 
 def _macs(widths):
