@@ -37,10 +37,7 @@ FP32_LANES_PER_SM, SMS = 128, 148
 # that workload; for every other workload `traffic` is None and the small-case figure is quoted beside it.
 TRAFFIC = {("tf32", "mnist2000_5"): {"bytes_per_launch": 145.1e6, "kernel": "gemm_tf32_2cta_kernel",
                                      "launch": "forward R pass of a hidden layer, 3000 x 2000 x (2000 + 2000); 128 MB algorithmic",
-                                     "source": "profiles/gemm_tf32_2cta_mnist2000_5_ncu.md"},
-           ("fp32", "mnist2000_5"): {"bytes_per_launch": 144.4e6, "kernel": "gemm_tf32x3_kernel",
-                                     "launch": "3000 x 2000 x 2000-class contraction on hi / lo parts",
-                                     "source": "profiles/gemm_tf32x3_mnist2000_5_ncu.md"}}
+                                     "source": "profiles/gemm_tf32_2cta_mnist2000_5_ncu.md"}}
 
 
 def peaks():
@@ -451,10 +448,10 @@ def run_ours(args):
         roof = {"bound": "tensor", "unit": "TFLOP/s", "peak": peak,
                 "peak_note": f"TF32 = 1/2 of the {pk['src']} sustained bf16 cuBLAS rate ({pk['bf16_sustained']} TFLOP/s)"}
     elif args.mode == "fp32":
-        peak = pk["bf16_sustained"] / 6.0
+        peak = pk["bf16_sustained"] / 3.0
         roof = {"bound": "tensor", "unit": "TFLOP/s", "peak": peak,
-                "peak_note": f"FP32-accurate on the tensor cores takes 3 TF32 products per term: 1/3 of the TF32 peak, "
-                             f"itself 1/2 of the {pk['src']} sustained bf16 cuBLAS rate ({pk['bf16_sustained']} TFLOP/s)"}
+                "peak_note": f"FP32-accurate on the tensor cores takes 3 FP16 products per term: 1/3 of the {pk['src']} "
+                             f"sustained bf16 cuBLAS rate ({pk['bf16_sustained']} TFLOP/s)"}
     else:
         peak = SMS * FP32_LANES_PER_SM * 2 * pk["sm_max_mhz"] * 1e6 / 1e12
         roof = {"bound": "alu", "unit": "TFLOP/s", "peak": peak,
@@ -462,7 +459,7 @@ def run_ours(args):
     main = {"tf32": "tensor", "fp32": "tensor_x3", "fp32_fma": "ffma"}[args.mode]
     kern = prof[main]
     achieved = kern["flop"] / (kern["ms"] * 1e-3) / 1e12 if kern["ms"] > 0 else None
-    roof.update({"kernel": {"tensor": "gemm_tf32_2cta_kernel", "tensor_x3": "gemm_tf32x3_kernel",
+    roof.update({"kernel": {"tensor": "gemm_tf32_2cta_kernel", "tensor_x3": "gemm_f16x3_kernel",
                             "ffma": "gemm_ffma_kernel"}[main],
                  "achieved": achieved, "frac": achieved / peak if achieved else None,
                  "traffic": (TRAFFIC.get((args.mode, args.workload)) or {}).get("bytes_per_launch"),

@@ -64,10 +64,12 @@ typedef enum {
 } gn_status;
 
 typedef enum {
-  GN_TF32 = 0,         /* contractions on the tensor cores with TF32 operands, FP32 accumulate   */
+  GN_TF32 = 0,         /* contractions on the tensor cores with TF32 operands, FP32 accumulate;  */
+                       /* to FP32 accuracy where TMA cannot address the operands (rows that are */
+                       /* no multiple of four floats)                                           */
   GN_FP32_ACCURATE = 1 /* results at FP32 accuracy: error-compensated tensor-core contractions  */
-                       /* (3 x TF32 on hi / lo operand parts) where the shape allows, the FP32  */
-                       /* FMA GEMM elsewhere; see gn_set_accurate_method                        */
+                       /* (3 products of two-part FP16 operands) or the FP32 FMA GEMM; see      */
+                       /* gn_set_accurate_method                                                */
 } gn_precision;
 
 /*
@@ -130,17 +132,18 @@ gn_status gn_set_blockdiag_method(gn_ctx* ctx, int method);
 /*
  * gn_set_accurate_method - how GN_FP32_ACCURATE contexts compute the dense contractions (the paper does not fix a
  * floating-point width; the acceptance bound of this mode is 1e-5 relative L2 against float64).
- *   0  choose (default): the tensor cores in error-compensated form wherever the shape suits the CTA-pair kernel
- *      (more than 128 rows and at least 128 columns of output), the FP32 FMA GEMM elsewhere;
+ *   0  choose (default): the tensor cores in error-compensated form wherever that is the faster one, the FP32 FMA
+ *      GEMM (small problems) elsewhere;
  *   1  the FP32 FMA GEMM for everything;
  *   2  same as 0.
- * Error-compensated form: every operand X is split into X = Xhi + Xlo, both exactly representable in TF32
- * (|X - Xhi - Xlo| <= 2^-22 |X|); the product is Alo Bhi + Ahi Blo + Ahi Bhi accumulated in FP32, with the sum over k
- * cut into chunks of 128 terms that are added in FP32 round-to-nearest outside the tensor core (its own accumulator
- * truncates).  Splits of theta and of the stored activations are kept until set_theta / set_subsample; they
- * double the memory those take.  If the kernel cannot be launched on this device or a split buffer cannot be
- * allocated, the contraction runs on the FP32 FMA GEMM instead.  No effect on GN_TF32 contexts.  GN_EINVAL for
- * another value.
+ * Error-compensated form: every operand X is split into two FP16 matrices, X 2^e = Xhi + Xlo, with the power of two
+ * that takes the largest |X| to [2^14, 2^15), so |X - (Xhi + Xlo) 2^-e| <= 2^-23 |x| down to 2^-18 of the largest element
+ * and <= 2^-40 of the largest element below that; the product is Alo Bhi + Ahi Blo + Ahi Bhi accumulated in FP32, with
+ * the sum over k cut into chunks of at most 128 terms that are added in FP32 round-to-nearest outside the tensor core
+ * (its own accumulator truncates).  Splits of theta and of the stored activations are kept until set_theta /
+ * set_subsample; they take as much memory as those.  If the kernel cannot be launched on this device or a split buffer
+ * cannot be allocated, the contraction runs on the FP32 FMA GEMM instead.  On GN_TF32 contexts the form serves, whatever
+ * this setting, the contractions whose operands TMA cannot address.  GN_EINVAL for another value.
  */
 gn_status gn_set_accurate_method(gn_ctx* ctx, int method);
 
@@ -349,7 +352,8 @@ gn_status gn_profile_read(gn_ctx* ctx, double* gemm_ms, double* gemm_flop, int64
  * followed by at least 128 readable bytes, which lets it fetch them with one TMA box per stage;
  * 4 and 5 = as 3 with one CTA per 128-row tile, respectively a CTA pair per 256-row tile, forced;
  * 6 = as 5 but whole tiles only, i.e. without the stream-K split of tiles between CTA pairs;
- * 7 = the error-compensated tensor-core form of GN_FP32_ACCURATE contexts, see gn_set_accurate_method).  a_kmajor: A is [M][K]
+ * 7 = the error-compensated tensor-core form, see gn_set_accurate_method, for results of more than 128 rows and at
+ * least 128 columns; 8 = the same for any shape).  a_kmajor: A is [M][K]
  * (else [K][M]); b_kmajor: B is [N][K] (else [K][N]); all row-major with the given leading
  * dimensions.  GN_EINVAL if the chosen kernel cannot take the operands (alignment, shape).
  */
@@ -379,8 +383,9 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* ctx, int kind, int M, int N, int K, con
  * device is touched by it; option 3: the bias column sums and the n_L-row weight block of a layer on a side stream
  * next to the layer's large contractions (value 0 = everything on the context's stream); option 4: consecutive
  * layers of a pass as one launch whose tiles wait for the tiles they read (value 0 = one launch per layer, 1 = the
- * stored forward pass, the default, 2 = also the forward R pass of a product).  Option 5 (GN_FP32_ACCURATE contexts): the error-compensated kernel also writes the hi / lo parts
- * of a result that a later contraction takes as an operand (value 0 = a separate pass splits it).  Option 6: fixed-length
+ * stored forward pass, the default, 2 = also the forward R pass of a product).  Option 5: the
+ * error-compensated kernel also records the largest magnitude of a result that a later contraction takes as an operand
+ * (value 0 = a separate pass finds it).  Option 6: fixed-length
  * CG solves of small problems replay one captured step as a CUDA graph (value 0 = plain launches).  Option 7: the
  * weight blocks of the stored-factor block product as two chained parts of the subsample's rows (value 0 = one
  * contraction per block; the two forms differ in the order of two partial sums, i.e. by rounding).  Option 8: the

@@ -227,7 +227,7 @@ class GnContext:
         self._check(self._lib.gn_set_blockdiag_method(self._h, int(method)))
 
     def set_accurate_method(self, method):
-        """0 choose, 1 FP32 FMA GEMM only, 2 error-compensated tensor-core form where the shape allows."""
+        """0 choose, 1 FP32 FMA GEMM only, 2 as 0."""
         self._check(self._lib.gn_set_accurate_method(self._h, int(method)))
 
     def set_split(self, split):

@@ -23,18 +23,14 @@
 //              advances 1024 B.
 // Every wait on an mbarrier is bounded: after about two seconds the waiting role records an error
 // code in global memory and the CTA drains and exits (tensor memory is always released).
-#include <cuda.h>
-
-#include <utility>
-
 #include "gn_kernels.h"
+#include "tc_common.cuh"
 
 namespace gn {
 namespace {
 
 constexpr int BM = 128, BK = 32, BN_MAX = 256;
 constexpr int A_STAGE_BYTES = BM * BK * 4;  // 16 KB
-constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 
 struct Tf32Params {
   int M, N;
@@ -47,9 +43,6 @@ struct Tf32Params {
   float alpha;
   const float* cin; long long ld_cin; float beta;
   int vec_epi;          // D, bias, dsig, cin all 16-byte aligned with leading dimensions % 4 == 0
-  // error-compensated kernel only: also write the two-term TF32 split of every stored value (hi = value rounded to
-  // TF32, lo = value - hi rounded to TF32) to these matrices, for the contraction that takes D as an operand next
-  float* Dhi; float* Dlo; long long ld_parts;
   int bn;               // tile width: multiple of 32, 32 <= bn <= 256
   int tiles_n, tiles;
   int* err;
@@ -86,82 +79,6 @@ struct GroupParams {
 };
 struct GroupMaps { CUtensorMap m[MAX_GROUP][4]; };   // per problem: A0, B0, A1, B1
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long globaltimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Programmatic dependent launch.  The kernels below are launched with the stream-serialisation attribute, so
-// their CTAs may become resident, set up their barriers and allocate tensor memory while the kernel before
-// them in the stream is still draining; nothing of global memory is touched before grid_dep_wait() returns,
-// which is when that kernel has completed and its writes are visible.  grid_dep_launch() lets the kernel
-// after this one do the same.  Without the attribute both are no-ops.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-__device__ __forceinline__ float round_tf32(float x) {
-  uint32_t u;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
-  return __uint_as_float(u);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-
-// Potentially blocking form: the thread may be suspended until the phase completes or about `ns` nanoseconds
-// have passed, instead of re-issuing the test in a loop (a spinning warp takes issue slots and load/store-unit
-// queue entries from the working warps of its scheduler).
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity, uint32_t ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(ns) : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// layout: 2 = 128-byte swizzle (16-byte atoms), 1 = 128-byte swizzle with 32-byte atoms
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint32_t layout) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of this architecture
-  d |= (uint64_t)layout << 61;
-  return d;
-}
-
 __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -169,72 +86,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Accumulator read in the 16 x 256-bit fragment shape: one instruction covers 16 tensor-memory lanes (rows) and
-// 32 columns; thread t of the warp receives, in register 4j + 2e + i (j = 0..3, e = 0..1, i = 0..1), the element
-// of row (t / 4) + 8 e and column 8 j + 2 (t mod 4) + i.  Four neighbouring threads hold 32 contiguous bytes of a
-// row, so a warp-wide 8-byte access to global memory touches 8 rows x one full 32-byte sector each, where the
-// 32 x 32-bit shape (lane = row) makes every access touch 32 rows x half a sector: half the requests per byte
-// on the load/store unit, which is what the epilogue is bound by.  The caller waits (tmem_ld_wait) before use.
-__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Bounded wait that also gives up at once when another role of this CTA has already failed.
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
-  if (mbar_test_wait(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity, 100000u)) {     // wakes at the latest every ~0.1 ms to look at the clock
-    if (*abort_flag) return false;
-    if (globaltimer() - t0 > WAIT_LIMIT_NS) {
-      atomicCAS(err, 0, code);
-      *abort_flag = 1;
-      return false;
-    }
-  }
-  return true;
-}
-
 // Persistent kernel: CTA b works on tiles b, b + gridDim.x, ...  Tile = 128 rows x p.bn columns
 // (p.bn a multiple of 32, at most 256).  Two accumulators of 256 tensor-memory columns alternate so
 // that the epilogue of one tile overlaps the MMAs of the next.
@@ -456,38 +307,6 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
 // order, and runs the epilogue on it - all of this on the epilogue warps while the MMA issuer is already
 // working on the pair's first whole tile in the other accumulator.  The order of every sum is fixed, so
 // results are deterministic.
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
-  return r;
-}
-// Cluster-wide barrier.  Warps may arrive here after divergent role code, so they reconverge first
-// and the non-aligned forms are used.
-__device__ __forceinline__ void cluster_sync_all() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ void tma2_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar_cluster_addr) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr)
-      : "memory");
-}
-__device__ __forceinline__ void tma2_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar_cluster_addr) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster_addr)
-      : "memory");
-}
 __device__ __forceinline__ void mma2_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -495,13 +314,6 @@ __device__ __forceinline__ void mma2_tf32(uint32_t tmem_d, uint64_t adesc, uint6
       "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
-// commit of the pair's MMAs, arriving on the barrier at this offset in both CTAs
-__device__ __forceinline__ void mma2_commit_both(uint64_t* bar) {
-  const uint16_t mask = 3;
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"(mask) : "memory");
-}
-
 struct Work { int prob, tile, kb0, kb1, sliced; };
 
 // idx-th piece of work of CTA pair `pair` (see Tf32Params and GroupParams); false when the pair has no more.
@@ -950,295 +762,6 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
   }
 }
 
-// ------------------------------------------------------------------------------------------------
-// Error-compensated variant (FP32-accurate results from the TF32 tensor cores).
-// Every operand X arrives as two matrices X = Xhi + Xlo, both exactly representable in TF32.  A logical
-// product A B is computed as Alo Bhi + Ahi Blo + Ahi Bhi: a ring slot holds the hi and lo tiles of both
-// operands for one k-block (64 KB per CTA) and every K = 8 step issues the three products, small terms
-// first, so each operand byte is fetched once for three MMAs.  The tensor core adds into its FP32
-// accumulator with truncation (measured: a relative bias of about 1e-9 per unit of K in a plain TF32
-// accumulation), so the K range is cut into chunks of xp.chunk_kb k-blocks; each chunk is accumulated in
-// tensor memory on its own (the two 256-column accumulators alternate per chunk) and the epilogue warps add
-// the chunks into a running sum held in registers, in FP32 with round-to-nearest.  That needs 128 registers per epilogue thread for the sums
-// alone, so the block has three warpgroups and moves registers between them:
-//   warps 0..3   (56 registers)   0 = TMA producer, 1 = MMA issuer, 2 = tensor-memory allocation, 3 idle
-//   warps 4..11  (224 registers)  epilogue, two warps per 32-lane quadrant of tensor memory
-// Whole tiles only, in wave order (no K slices).  Same pair protocol as the kernel above.
-constexpr int MAX_PAIRS = 2;                          // logical operand pairs accumulated into one tile
-constexpr int X3_THREADS = 384;
-constexpr int X3_STAGES = 3;
-constexpr int X3_STAGE_BYTES = 2 * STAGE2_BYTES;      // 64 KB: A hi, A lo, B-half hi, B-half lo
-constexpr int X3_REGS_LOW = 56, X3_REGS_HIGH = 224;   // 128 * 56 + 256 * 224 = 384 * 168
-
-struct MapSet { CUtensorMap a_hi[MAX_PAIRS], a_lo[MAX_PAIRS], b_hi[MAX_PAIRS], b_lo[MAX_PAIRS]; };
-
-struct X3Params {
-  int n_pairs;
-  int kblocks[MAX_PAIRS];
-  int chunk_kb;
-};
-
-// One whole, 16-byte-aligned chunk of 32 finished sums of a row (lane = row) through the epilogue options and out,
-// with the options fixed at compile time as in epilogue_full_chunk: 0 = alpha * sum (+ bias), 1 = sigmoid,
-// 2 = times the sigmoid derivative of zrow, 3 = plus beta * crow, 4 = any combination, tested per element.  In modes
-// 2 and 3 the 128 bytes of the operand are requested before the first of them is used (the running sums of the
-// other chunks leave room for that one buffer); in mode 4 the loads stay beside their use, two steps at a time.
-template <int MODE>
-__device__ __forceinline__ void x3_store_chunk(const Tf32Params& p, const float* run, const float* zrow, const float* crow,
-                                               float* drow, int nb, float* hrow, float* lrow) {
-  const bool use_sigm = MODE == 4 ? p.sigmoid != 0 : MODE == 1;
-  const bool use_dsig = MODE == 4 ? zrow != nullptr : MODE == 2;
-  const bool use_cin = MODE == 4 ? crow != nullptr : MODE == 3;
-  float4 op[8];
-  if (MODE == 2 || MODE == 3) {
-    const float4* src = reinterpret_cast<const float4*>(MODE == 2 ? zrow : crow);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) op[q] = __ldg(src + q);
-  }
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    float4 bz = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (p.bias) bz = __ldg(reinterpret_cast<const float4*>(p.bias + nb) + q);
-    float4 o = make_float4(0.f, 0.f, 0.f, 0.f), o2 = o;
-    if (MODE == 2 || MODE == 3) o = op[q];
-    if (MODE == 4 && use_dsig) o = __ldg(reinterpret_cast<const float4*>(zrow) + q);
-    if (MODE == 4 && use_cin) o2 = __ldg(reinterpret_cast<const float4*>(crow) + q);
-    float x[4] = {run[4 * q] + bz.x, run[4 * q + 1] + bz.y, run[4 * q + 2] + bz.z, run[4 * q + 3] + bz.w};
-    const float z[4] = {o.x, o.y, o.z, o.w};
-    const float cv[4] = {MODE == 4 ? o2.x : o.x, MODE == 4 ? o2.y : o.y, MODE == 4 ? o2.z : o.z, MODE == 4 ? o2.w : o.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (use_sigm) x[e] = 1.f / (1.f + expf(-x[e]));
-      if (use_dsig) x[e] *= z[e] * (1.f - z[e]);
-      x[e] *= p.alpha;
-      if (use_cin) x[e] = fmaf(p.beta, cv[e], x[e]);
-    }
-    reinterpret_cast<float4*>(drow)[q] = make_float4(x[0], x[1], x[2], x[3]);
-    if (hrow) {
-      float h[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) { h[e] = round_tf32(x[e]); x[e] = round_tf32(x[e] - h[e]); }
-      reinterpret_cast<float4*>(hrow)[q] = make_float4(h[0], h[1], h[2], h[3]);
-      reinterpret_cast<float4*>(lrow)[q] = make_float4(x[0], x[1], x[2], x[3]);
-    }
-    // the running sums leave few registers: keep the loads of at most two steps in flight
-    if (MODE == 4 && (q & 1)) asm volatile("" ::: "memory");
-  }
-}
-
-template <int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(X3_THREADS, 1)
-gemm_tf32x3_kernel(const __grid_constant__ MapSet maps, const Tf32Params p, const X3Params xp) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * X3_STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* acc_full = empty + STAGES;   // [2]
-  uint64_t* acc_empty = acc_full + 2;    // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
-  const int pair = blockIdx.x >> 1;
-  int total_kb = 0;
-  for (int i = 0; i < xp.n_pairs; ++i) total_kb += xp.kblocks[i];
-  const int n_chunks_k = (total_kb + xp.chunk_kb - 1) / xp.chunk_kb;
-  const int bn = p.bn, hb = p.bn >> 1;
-  const uint32_t pair_tx = 4u * (A_STAGE_BYTES + (uint32_t)hb * BK * 4);   // two CTAs x (hi + lo) x (A + B half)
-  // tiles of this pair: pair, pair + P, ... (whole waves), then one of the `rem` left over
-  const int my_tiles = p.waves + (pair < p.rem ? 1 : 0);
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 16); }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 2) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  cluster_sync_all();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  grid_dep_wait();
-  grid_dep_launch();
-
-  if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(X3_REGS_LOW));
-    if (warp == 0) {
-      // ---------------------------------------------------------------- producer (both CTAs)
-      int it = 0;
-      bool ok = true;
-      for (int ti = 0; ti < my_tiles && ok; ++ti) {
-        const int t = ti * p.P + pair;
-        const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM;
-        const int n0 = (t % p.tiles_n) * bn + (int)rank * hb;
-        int pr = 0, kk = 0;                       // operand pair and k-block inside it
-        for (int kb = 0; kb < total_kb; ++kb, ++it, ++kk) {
-          while (kk >= xp.kblocks[pr]) { kk = 0; ++pr; }
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          int good = 1;
-          if (lane == 0) good = wait_or_abort(&empty[s], ph ^ 1, abort_flag, p.err, 1) ? 1 : 0;
-          good = __shfl_sync(0xffffffffu, good, 0);
-          if (!good) { ok = false; break; }
-          if (rank == 0 && lane == 0) mbar_expect_tx(&full[s], pair_tx);
-          __syncwarp();
-          const uint32_t full_leader = map_to_cta(smem_u32(&full[s]), 0);
-          const int k0 = kk * BK;
-          uint8_t* sa = smem + s * X3_STAGE_BYTES;            // A hi | A lo | B hi | B lo
-          uint8_t* sb = sa + 2 * A_STAGE_BYTES;
-          if (!p.a_mn) {
-            if (lane == 0) tma2_load_2d(sa, &maps.a_hi[pr], k0, m0, full_leader);
-            if (lane == 1) tma2_load_2d(sa + A_STAGE_BYTES, &maps.a_lo[pr], k0, m0, full_leader);
-          } else {
-            if (lane == 0) tma2_load_3d(sa, &maps.a_hi[pr], 0, k0, m0 / 32, full_leader);
-            if (lane == 1) tma2_load_3d(sa + A_STAGE_BYTES, &maps.a_lo[pr], 0, k0, m0 / 32, full_leader);
-          }
-          if (!p.b_mn) {
-            if (lane == 8) tma2_load_2d(sb, &maps.b_hi[pr], k0, n0, full_leader);
-            if (lane == 9) tma2_load_2d(sb + B2_STAGE_MAX, &maps.b_lo[pr], k0, n0, full_leader);
-          } else {
-            if (lane == 8) tma2_load_3d(sb, &maps.b_hi[pr], 0, k0, n0 / 32, full_leader);
-            if (lane == 9) tma2_load_3d(sb + B2_STAGE_MAX, &maps.b_lo[pr], 0, k0, n0 / 32, full_leader);
-          }
-        }
-      }
-    } else if (warp == 1 && rank == 0 && lane == 0) {
-      // ---------------------------------------------------------------- MMA issuer (leader CTA only)
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(p.a_mn ? 1 : 0) << 15) |
-                             ((uint32_t)(p.b_mn ? 1 : 0) << 16) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-      const uint32_t a_lbo = p.a_mn ? BK * 128 : 16, b_lbo = p.b_mn ? BK * 128 : 16;
-      const uint32_t a_step = p.a_mn ? 1024 : 32, b_step = p.b_mn ? 1024 : 32;
-      const uint32_t a_sbo = p.a_mn ? 512 : 1024, b_sbo = p.b_mn ? 512 : 1024;
-      const uint32_t a_lay = p.a_mn ? 1 : 2, b_lay = p.b_mn ? 1 : 2;
-      int it = 0, ci = 0;                          // ring position, running chunk count (accumulator phase)
-      bool ok = true;
-      for (int ti = 0; ti < my_tiles && ok; ++ti) {
-        for (int ch = 0; ch < n_chunks_k && ok; ++ch, ++ci) {
-          const int kb0 = ch * xp.chunk_kb, kb1 = min(total_kb, kb0 + xp.chunk_kb);
-          const int buf = ci & 1;
-          const uint32_t aph = (ci >> 1) & 1;
-          ok = wait_or_abort(&acc_empty[buf], aph ^ 1, abort_flag, p.err, 4);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN_MAX);
-          for (int kb = kb0; kb < kb1; ++kb, ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (it / STAGES) & 1;
-            ok = wait_or_abort(&full[s], ph, abort_flag, p.err, 2);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t sa = smem_u32(smem + s * X3_STAGE_BYTES);
-            const uint32_t sb = sa + 2 * A_STAGE_BYTES;
-#pragma unroll
-            for (int k = 0; k < BK / 8; ++k) {
-              const uint64_t ah = make_desc(sa + k * a_step, a_lbo, a_sbo, a_lay);
-              const uint64_t al = make_desc(sa + A_STAGE_BYTES + k * a_step, a_lbo, a_sbo, a_lay);
-              const uint64_t bh = make_desc(sb + k * b_step, b_lbo, b_sbo, b_lay);
-              const uint64_t bl = make_desc(sb + B2_STAGE_MAX + k * b_step, b_lbo, b_sbo, b_lay);
-              mma2_tf32(tmem_d, al, bh, idesc, (kb > kb0 || k != 0) ? 1u : 0u);   // small terms first
-              mma2_tf32(tmem_d, ah, bl, idesc, 1u);
-              mma2_tf32(tmem_d, ah, bh, idesc, 1u);
-            }
-            mma2_commit_both(&empty[s]);
-          }
-          if (ok) mma2_commit_both(&acc_full[buf]);
-        }
-      }
-    }
-  } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(X3_REGS_HIGH));
-    // ------------------------------------------------------------------ epilogue (warps 4..11, both CTAs)
-    const int quad = warp & 3;
-    const int half = (warp - 4) >> 2;
-    const int row = quad * 32 + lane;
-    int ci = 0;
-    bool alive = true;
-    for (int ti = 0; ti < my_tiles && alive; ++ti) {
-      const int t = ti * p.P + pair;
-      const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (t % p.tiles_n) * bn;
-      const int n_cc = min(bn / 32, (p.N - n0 + 31) / 32);       // column chunks of this tile that exist
-      float run[4][32];                                          // this warp's chunks: half, half + 2, half + 4, half + 6
-      for (int ch = 0; ch < n_chunks_k; ++ch, ++ci) {
-        const int buf = ci & 1;
-        const uint32_t aph = (ci >> 1) & 1;
-        int good = 1;
-        if (lane == 0) good = wait_or_abort(&acc_full[buf], aph, abort_flag, p.err, 3) ? 1 : 0;
-        good = __shfl_sync(0xffffffffu, good, 0);
-        if (!good) { alive = false; break; }
-        tc_fence_after();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = half + 2 * j;
-          if (c < n_cc) {                                        // warp-uniform
-            float v[32];
-            tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN_MAX + c * 32), v);
-            // (a select, not a branch: two code paths over the 128 sums would double their registers)
-#pragma unroll
-            for (int i = 0; i < 32; ++i) run[j][i] = (ch == 0 ? 0.f : run[j][i]) + v[i];
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&acc_empty[buf]), 0));
-      }
-      if (!alive) break;
-      const int m = m0 + row;
-      if (m >= p.M) continue;
-      const float* zrow = p.dsig ? p.dsig + (long long)((m / p.dsig_div) % p.dsig_rows) * p.ld_dsig : nullptr;
-      const float* crow = p.cin ? p.cin + (long long)m * p.ld_cin : nullptr;
-      float* drow = p.D + (long long)m * p.ldd;
-      const int n_opt = (p.sigmoid ? 1 : 0) + (p.dsig ? 1 : 0) + (p.cin ? 1 : 0);
-      const int xmode = n_opt == 0 ? 0 : n_opt > 1 ? 4 : p.sigmoid ? 1 : p.dsig ? 2 : 3;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = half + 2 * j;
-        if (c >= n_cc) continue;
-        const int nb = n0 + c * 32;
-        if (p.vec_epi && nb + 32 <= p.N) {
-          float* const hrow = p.Dhi ? p.Dhi + (long long)m * p.ld_parts + nb : nullptr;
-          float* const lrow = p.Dhi ? p.Dlo + (long long)m * p.ld_parts + nb : nullptr;
-          switch (xmode) {
-            case 0: x3_store_chunk<0>(p, run[j], zrow ? zrow + nb : nullptr, crow ? crow + nb : nullptr, drow + nb, nb, hrow, lrow); break;
-            case 1: x3_store_chunk<1>(p, run[j], zrow ? zrow + nb : nullptr, crow ? crow + nb : nullptr, drow + nb, nb, hrow, lrow); break;
-            case 2: x3_store_chunk<2>(p, run[j], zrow ? zrow + nb : nullptr, crow ? crow + nb : nullptr, drow + nb, nb, hrow, lrow); break;
-            case 3: x3_store_chunk<3>(p, run[j], zrow ? zrow + nb : nullptr, crow ? crow + nb : nullptr, drow + nb, nb, hrow, lrow); break;
-            default: x3_store_chunk<4>(p, run[j], zrow ? zrow + nb : nullptr, crow ? crow + nb : nullptr, drow + nb, nb, hrow, lrow); break;
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int n = nb + i;
-            if (n < p.N) {
-              float x = run[j][i] + (p.bias ? __ldg(p.bias + n) : 0.f);
-              if (p.sigmoid) x = 1.f / (1.f + expf(-x));
-              if (zrow) { const float z = __ldg(zrow + n); x *= z * (1.f - z); }
-              x *= p.alpha;
-              if (crow) x = fmaf(p.beta, __ldg(crow + n), x);
-              drow[n] = x;
-              if (p.Dhi) {
-                const float h = round_tf32(x);
-                p.Dhi[(long long)m * p.ld_parts + n] = h;
-                p.Dlo[(long long)m * p.ld_parts + n] = round_tf32(x - h);
-              }
-            }
-          }
-        }
-      }
-    }
-  }
-  tc_fence_before();
-  cluster_sync_all();
-  if (warp == 2) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
-  }
-}
-
 // One CTA waits on an mbarrier that nothing ever arrives on, with the same bounded-wait code the GEMM
 // roles use but a caller-chosen limit; it must record its code and return.  Exercises the path from a
 // timed-out device wait to GN_ETIMEOUT on the host without hanging anything.
@@ -1255,26 +778,6 @@ __global__ void timeout_probe_kernel(int* err, unsigned long long limit_ns) {
 }
 
 // ---- host side ---------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-    else
-      cudaGetLastError();
-  }
-  return fn;
-}
-
 // 2-D map over a row-major [rows][cols] float matrix with leading dimension ld; box = (box_c, box_r).
 bool make_map(CUtensorMap* m, const float* base, long long rows, long long cols, long long ld, int box_c, int box_r,
               CUtensorMapSwizzle swz) {
@@ -1307,20 +810,8 @@ bool make_map_mn3d(CUtensorMap* m, const float* base, long long K, long long MN,
   return r == CUDA_SUCCESS;
 }
 
-inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
-
 constexpr int kStages = 4;
 constexpr int kSmemBytes = kStages * (A_STAGE_BYTES + BN_MAX * BK * 4) + 1024 + 256;
-
-int num_sms() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-  }
-  return n;
-}
 
 // Tile width against wave quantisation: every CTA runs ceil(tiles / SMs) tiles.  Measured tile times
 // on B200 fit (320 + bn) units: the operand pipeline is latency-bound, so a narrower tile is only
@@ -1380,22 +871,6 @@ int64_t gemm_tf32_workspace_floats() { return (int64_t)(num_sms() / 2) * 2 * BM 
 int gemm_tf32_workspace_flags() { return num_sms() / 2; }
 
 namespace {
-
-// Launch with the programmatic stream-serialisation attribute (see grid_dep_wait above).
-template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3((unsigned)block, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
 
 // Tensor maps and kernel parameters of one problem for a given tile width (two_cta: 256 x bn tiles of a CTA pair).
 bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUtensorMap* maps, Tf32Params& p) {
@@ -1692,89 +1167,6 @@ double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K,
   double ms = 0.0;
   if (plan_group_impl(n, M, N, K, num_sms() / 2, keep_order, nullptr, nullptr, nullptr, nullptr, &ms) < 0) return -1.0;
   return ms;
-}
-
-// ---- error-compensated form ---------------------------------------------------------------------
-// 4 k-blocks = 128 terms (384 products) per accumulation in tensor memory: the truncation bias of one chunk stays
-// below 1e-6 relative (measured), and the running sums outside are round-to-nearest.
-constexpr int kChunkKb = 4;
-constexpr int kSmemBytes3 = X3_STAGES * X3_STAGE_BYTES + 1024 + 256;
-
-// The register split of the kernel (128 x 56 + 256 x 224) must not exceed what the block is launched with, and
-// the kernel needs its dynamic shared memory granted: checked once.
-bool gemm_tf32x3_usable() {
-  static int usable = -1;
-  if (usable < 0) {
-    cudaFuncAttributes fa;
-    usable = encode_fn() != nullptr &&
-             cudaFuncGetAttributes(&fa, gemm_tf32x3_kernel<X3_STAGES>) == cudaSuccess &&
-             fa.numRegs * X3_THREADS >= 128 * X3_REGS_LOW + 256 * X3_REGS_HIGH &&
-             cudaFuncSetAttribute(gemm_tf32x3_kernel<X3_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes3) == cudaSuccess;
-    cudaGetLastError();
-  }
-  return usable != 0;
-}
-
-bool gemm_tf32x3_eligible(const GemmArgs& g) {
-  // the operands' own alignment does not matter: the kernel reads their hi / lo copies
-  return g.M > BM && g.N >= 128 && gemm_tf32x3_usable();
-}
-
-int launch_gemm_tf32x3(const GemmArgs& g, int* err_flag, cudaStream_t st) {
-  const bool usable = gemm_tf32x3_usable();
-  if (!usable || !g.A1lo || !g.B1lo || (g.A2 && (!g.A2lo || !g.B2lo))) return -1;
-  // this kernel is bound by its MMAs, not by the operand feed: a tile's time is nearly proportional to its width
-  // (measured: 96 + bn units against the TF32 kernel's 320 + bn), so narrower tiles win more often
-  const int bn = choose_bn2(g.M, g.N, false, 96);
-  const int b_rows = bn / 2;
-  const float* Ah[2] = {g.A1, g.A2}; const float* Al[2] = {g.A1lo, g.A2lo};
-  const float* Bh[2] = {g.B1, g.B2}; const float* Bl[2] = {g.B1lo, g.B2lo};
-  const int Ks[2] = {g.K1, g.A2 ? g.K2 : 0};
-  const long long lda[2] = {g.lda1, g.lda2}, ldb[2] = {g.ldb1, g.ldb2};
-  MapSet maps;
-  const CUtensorMapSwizzle kmaj = CU_TENSOR_MAP_SWIZZLE_128B;
-  for (int s = 0; s < MAX_PAIRS; ++s) {
-    const int src = Ah[s] ? s : 0;      // unused second pair: repeat the first (never dereferenced)
-    bool ok = true;
-    const float* as[2] = {Ah[src], Al[src]}; CUtensorMap* am[2] = {&maps.a_hi[s], &maps.a_lo[s]};
-    const float* bs[2] = {Bh[src], Bl[src]}; CUtensorMap* bm[2] = {&maps.b_hi[s], &maps.b_lo[s]};
-    for (int h = 0; h < 2 && ok; ++h) {
-      if (g.a_kmajor) ok = make_map(am[h], as[h], g.M, Ks[src], lda[src], BK, BM, kmaj);
-      else            ok = make_map_mn3d(am[h], as[h], Ks[src], g.M, lda[src], BM / 32);
-      if (g.b_kmajor) ok = ok && make_map(bm[h], bs[h], g.N, Ks[src], ldb[src], BK, b_rows, kmaj);
-      else            ok = ok && make_map_mn3d(bm[h], bs[h], Ks[src], g.N, ldb[src], b_rows / 32);
-    }
-    if (!ok) return -1;
-  }
-  Tf32Params p{};
-  X3Params xp{};
-  p.M = g.M; p.N = g.N;
-  xp.n_pairs = g.A2 ? 2 : 1;
-  for (int s = 0; s < xp.n_pairs; ++s) xp.kblocks[s] = (Ks[s] + BK - 1) / BK;
-  xp.chunk_kb = kChunkKb;
-  p.a_mn = g.a_kmajor ? 0 : 1; p.b_mn = g.b_kmajor ? 0 : 1;
-  p.a_3d = p.a_mn; p.b_3d = p.b_mn;
-  p.D = g.D; p.ldd = g.ldd;
-  p.bias = g.bias; p.sigmoid = g.sigmoid;
-  p.dsig = g.dsig; p.ld_dsig = g.ld_dsig; p.dsig_rows = g.dsig_rows > 0 ? g.dsig_rows : 1; p.dsig_div = g.dsig_div > 0 ? g.dsig_div : 1;
-  p.alpha = g.alpha;
-  p.cin = g.cin; p.ld_cin = g.ld_cin; p.beta = g.beta;
-  p.vec_epi = aligned16(g.D) && (g.ldd % 4 == 0) && (!g.bias || aligned16(g.bias)) &&
-              (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
-              (!g.cin || (aligned16(g.cin) && g.ld_cin % 4 == 0));
-  p.Dhi = g.Dhi; p.Dlo = g.Dlo; p.ld_parts = g.ld_parts;
-  if (p.Dhi && !(aligned16(g.Dhi) && aligned16(g.Dlo) && g.ld_parts % 4 == 0)) return -1;
-  p.bn = bn;
-  p.tiles_n = (g.N + bn - 1) / bn;
-  p.err = err_flag;
-  p.tiles = ((g.M + 2 * BM - 1) / (2 * BM)) * p.tiles_n;
-  const int pairs = num_sms() / 2;
-  p.P = p.tiles < pairs ? p.tiles : pairs;
-  p.waves = p.tiles / p.P;
-  p.rem = p.tiles - p.waves * p.P;
-  p.slices = 1;
-  launch_pdl(gemm_tf32x3_kernel<X3_STAGES>, 2 * p.P, X3_THREADS, kSmemBytes3, st, maps, p, xp);
-  return 1;
 }
 
 }  // namespace gn

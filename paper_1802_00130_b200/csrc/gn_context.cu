@@ -91,27 +91,35 @@ struct gn_ctx {
   bool fly_enabled = true;                 // last hidden layer's factor formed on the fly in the stored-factor product
   int back_chain = 2;                      // hidden layers of a backward pass as one chained launch: 0 never, 1 always, 2 where it pays
   int* chain_ctr = nullptr; int64_t chain_ctr_cap = 0;   // finished-tile counters of such a launch
-  // FP32-accurate mode on the tensor cores (3 x TF32): hi / lo parts of the operands
-  int acc_method = 0;        // 0 choose (tensor cores where the shape allows), 1 FP32 FMA only, 2 as 0
-  bool x3_usable = true;     // cleared if the error-compensated kernel could not be launched
+  // FP32-accurate contractions on the tensor cores (gemm_f16x3.cu): two FP16 parts of every operand
+  int acc_method = 0;        // 0 choose (tensor cores where they are faster), 1 FP32 FMA only, 2 as 0
+  bool x3_usable = true;     // cleared if the tensor-core kernel could not be launched
   uint64_t theta_epoch = 1, sub_epoch = 1;   // bumped whenever theta / the stored activations are rewritten
-  struct SplitBuf { float* hi = nullptr; float* lo = nullptr; int64_t cap = 0; };
-  struct SplitEntry {        // split of a matrix that lives in theta or in the stored Z_m, kept until those change
-    const float* src; int64_t rows; int cols; int64_t ld; int kind; uint64_t epoch; SplitBuf buf;
-  };
+  // [hi part: cap elements][lo part: cap elements][bit pattern of the largest magnitude]
+  struct SplitBuf { uint16_t* p = nullptr; int64_t cap = 0; unsigned* bits() const { return reinterpret_cast<unsigned*>(p + 2 * cap); } };
+  // Parts kept until the matrix changes: of matrices inside theta (kind 1) and the stored Z_m (kind 2), and, for the
+  // length of one launch sequence, inside the product's v (kind 3) and the row batch's X and Z_m (kind 4).  The key is
+  // the matrix's place in those, never an address of the caller's.  Whole layers' matrices have their place in one
+  // allocation per kind (arena), anything else (a sub-block of a split structure) a buffer of its own.
+  struct SplitEntry { int kind; int64_t key; int64_t rows; int cols; int64_t ld; uint64_t epoch; SplitBuf buf; bool in_arena; };
   std::vector<SplitEntry> split_cache;
-  struct SplitSlot {         // split of any other operand: one slot per operand role, overwritten by the next use
+  uint16_t* arena[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; int64_t arena_rows[5] = {0, 0, 0, 0, 0};
+  const float* cur_v = nullptr;                            // the vector of the product in progress
+  const float* cur_x = nullptr; int64_t cur_x_count = 0;   // the rows of X of the batch in progress
+  struct SplitSlot {         // parts of any other operand: one slot per operand role, overwritten by the next use
     const float* src = nullptr; int64_t rows = 0; int cols = 0; int64_t ld = 0; SplitBuf buf;
     uint64_t seq = 0;        // contraction (gemm_seq) that wrote these parts
   };
   SplitSlot split_slot[4];
-  // hi / lo parts written by the epilogue of the error-compensated kernel for a result that a later contraction of
-  // the SAME launch sequence takes as an operand (R z^m, delta s^m, and their row-batch twins): keyed by the result's
-  // address, valid only while parts_epoch stands (every launch sequence that may rewrite those buffers bumps it)
-  struct PartsEntry { const float* src = nullptr; int64_t rows = 0; int cols = 0; int64_t ld = 0; uint64_t epoch = 0; SplitBuf buf; };
-  std::vector<PartsEntry> parts;
+  unsigned* split_part = nullptr;                          // scratch of the splitting pass, then kMaxRecords maxima
+  SplitOperand h_ops[4]; unsigned* h_amax_out = nullptr;   // of the contraction being launched
+  // max|D| accumulated by the contraction that produced D, for the splitting pass of a later contraction of the SAME
+  // launch sequence (R z^m, delta s^m, Z_m): valid only while parts_epoch stands (every launch sequence that may
+  // rewrite those buffers bumps it).  dirty: the word has not been cleared by a consumer yet.
+  struct AmaxEntry { const float* src = nullptr; int64_t rows = 0; int cols = 0; int64_t ld = 0; uint64_t epoch = 0; unsigned* acc = nullptr; bool dirty = false; };
+  std::vector<AmaxEntry> amax;
   uint64_t parts_epoch = 1;
-  bool parts_enabled = false;  // (measured 7 % slower than a separate splitting pass: off unless asked for)
+  bool amax_enabled = true;
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
   double* partial = nullptr; int64_t partial_cap = 0;
   double* dscal = nullptr;   // device: [0] loss, [1] theta^T theta, [2] cg sum rho, [3] cg active
@@ -256,6 +264,13 @@ struct SideJoin {
   ~SideJoin() { side_join(c); c->side_region = false; }
 };
 
+// The vector of a product in progress (its layers' parts are kept for the length of the product).
+struct CurrentVector {
+  gn_ctx* c;
+  CurrentVector(gn_ctx* ctx, const float* v) : c(ctx) { c->cur_v = v; }
+  ~CurrentVector() { c->cur_v = nullptr; }
+};
+
 // Before a workspace that side-stream kernels may still read is released.
 void quiesce(gn_ctx* c) {
   cudaStreamSynchronize(c->st);
@@ -306,8 +321,8 @@ void run_gemm_kind(gn_ctx* c, const GemmArgs& g, int kind, cudaStream_t st = nul
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "cuTensorMapEncodeTiled failed"; }
     else c->launches += r;
   } else if (kind == 3) {
-    const int r = launch_gemm_tf32x3(g, c->err_flag + 1, st);
-    if (r < 0) { c->sticky = GN_ECUDA; c->err = "the error-compensated tensor-core kernel could not be launched"; c->x3_usable = false; }
+    const int r = launch_gemm_f16x3(g, c->h_ops, c->sk_ws, c->h_amax_out, c->err_flag + 1, st);
+    if (r < 0) { c->sticky = GN_ECUDA; c->err = "the FP32-accurate tensor-core kernel could not be launched"; c->x3_usable = false; }
     else c->launches += r;
   } else if (kind == 2) {
     c->launches += launch_gemm_thin(g, c->thin_scratch, st);
@@ -328,129 +343,238 @@ gn_status ensure_sk_workspace(gn_ctx* c) {
   return c->sk_ws ? GN_OK : GN_ENOMEM;
 }
 
-inline int64_t round4(int64_t x) { return (x + 3) & ~(int64_t)3; }
+inline int64_t round8(int64_t x) { return (x + 7) & ~(int64_t)7; }
 
 bool split_buf_reserve(gn_ctx* c, gn_ctx::SplitBuf& b, int64_t need) {
   if (need <= b.cap) return true;
-  cudaStreamSynchronize(c->st);   // an earlier contraction may still be reading the old buffers
-  dev_free(c, b.hi, b.cap); dev_free(c, b.lo, b.cap);
+  cudaStreamSynchronize(c->st);   // an earlier contraction may still be reading the old buffer
+  dev_free(c, b.p);
   b.cap = 0;
-  if (dev_alloc(c, &b.hi, need) != GN_OK) return false;
-  if (dev_alloc(c, &b.lo, need) != GN_OK) { dev_free(c, b.hi, need); return false; }
+  if (dev_alloc(c, &b.p, 2 * need + 8) != GN_OK) return false;
   b.cap = need;
   return true;
 }
 
-// The results whose parts the epilogue writes live in the subsample and row-batch workspaces: when those move,
-// the parts kept for their old addresses go.
-void drop_parts(gn_ctx* c) {
-  for (auto& e : c->parts) { dev_free(c, e.buf.hi); dev_free(c, e.buf.lo); }
-  c->parts.clear();
+// The matrices whose maxima are recorded live in the subsample and row-batch workspaces: when those move, the records
+// kept for their old addresses go.
+constexpr size_t kMaxRecords = 256;
+void drop_amax(gn_ctx* c) { c->amax.clear(); }
+
+gn_status ensure_split_scratch(gn_ctx* c) {
+  if (c->split_part) return GN_OK;
+  return dev_alloc(c, &c->split_part, kSplitBlocks + (int64_t)kMaxRecords);
 }
 
-// hi / lo parts of the stored matrix [rows][cols] (leading dimension ld) that serves as an operand.  Matrices
-// inside theta or inside the stored activations Z_m are split once per set_theta / set_subsample; anything
-// else goes through the slot of its operand role (0 = A1, 1 = B1, 2 = A2, 3 = B2) and is split again on every
+// The parts of kind `kind` go (their workspace is about to move or to change size).
+void drop_kept_parts(gn_ctx* c, int kind) {
+  for (size_t i = 0; i < c->split_cache.size();) {
+    if (c->split_cache[i].kind == kind) {
+      if (!c->split_cache[i].in_arena) dev_free(c, c->split_cache[i].buf.p);
+      c->split_cache.erase(c->split_cache.begin() + (long)i);
+    } else {
+      ++i;
+    }
+  }
+  dev_free(c, c->arena[kind]);
+  c->arena_rows[kind] = 0;
+}
+
+// Buffer of the kept parts of a whole layer's matrix inside the kind's arena: kinds 1 and 3 hold every W^m-shaped
+// matrix, kinds 2 and 4 the operands z^0 .. z^{L-1} of the subsample and of the row batch at their workspaces' capacity.
+// False if the matrix has no place there.
+bool arena_buffer(gn_ctx* c, int kind, int64_t key, int64_t rows, int cols, int64_t ld, gn_ctx::SplitBuf* out) {
+  const bool vec = kind == 1 || kind == 3;
+  const int64_t cap_rows = kind == 2 ? c->capS : kind == 4 ? c->capB : 0;
+  int64_t total = 0, at = -1, size = 0;
+  for (int m = 0; m < c->L; ++m) {
+    const int64_t n = vec ? (int64_t)c->w[m + 1] * round8(c->w[m]) : cap_rows * round8(c->w[m]);
+    const int64_t k = vec ? c->w_off[m + 1] : (int64_t)m << 48;
+    if (key == k && cols == c->w[m] && ld == c->w[m] && rows <= (vec ? c->w[m + 1] : cap_rows)) { at = total; size = n; }
+    total += 2 * n + 8;
+  }
+  if (at < 0) return false;
+  if (!c->arena[kind]) {
+    if (dev_alloc(c, &c->arena[kind], total) != GN_OK) return false;
+    c->arena_rows[kind] = cap_rows;
+  } else if (c->arena_rows[kind] != cap_rows) {
+    return false;
+  }
+  out->p = c->arena[kind] + at; out->cap = size;
+  return true;
+}
+
+// Place of `src` in a matrix set whose parts are kept (SplitEntry::kind), or 0.
+int split_kind(const gn_ctx* c, const float* src, int64_t* key, uint64_t* epoch) {
+  if (src >= c->theta && src < c->theta + c->n) { *key = src - c->theta; *epoch = c->theta_epoch; return 1; }
+  for (int m = 0; m <= c->L; ++m)
+    if (c->Z[m] && src >= c->Z[m] && src < c->Z[m] + c->capS * c->w[m]) {
+      *key = ((int64_t)m << 48) + (src - c->Z[m]); *epoch = c->sub_epoch;
+      return 2;
+    }
+  *epoch = c->parts_epoch;
+  if (c->cur_v && src >= c->cur_v && src < c->cur_v + c->n) { *key = src - c->cur_v; return 3; }
+  if (c->cur_x && src >= c->cur_x && src < c->cur_x + c->cur_x_count) { *key = src - c->cur_x; return 4; }
+  for (int m = 1; m <= c->L; ++m)
+    if (c->Zb[m] && src >= c->Zb[m] && src < c->Zb[m] + c->capB * c->w[m]) { *key = ((int64_t)m << 48) + (src - c->Zb[m]); return 4; }
+  return 0;
+}
+
+// The two FP16 parts of the stored matrix [rows][cols] (leading dimension ld) that serves as an operand: in `out`, with
+// the splitting job they still need, if any, appended to `jobs`.  Matrices of the kept kinds are split once per epoch;
+// anything else goes through the slot of its operand role (0 = A1, 1 = B1, 2 = A2, 3 = B2) and is split again on every
 // use unless the caller vouches (reuse) that the contraction just before this one read this very operand,
 // unchanged.  The caller's word is checked: the parts are taken over only if that previous contraction is
 // the one that wrote the slot (it may have gone to another kernel and left the slot alone).
-constexpr int64_t kMaxTransientSplitFloats = 1500LL * 1000 * 1000;   // 6 GB per part
+constexpr int64_t kMaxTransientSplitFloats = 1500LL * 1000 * 1000;   // 6 GB for both parts
 
 bool split_operand(gn_ctx* c, const float* src, int64_t rows, int cols, int64_t ld, int role, bool reuse,
-                   const float** hi, const float** lo, int64_t* ld_out) {
-  const int64_t ldo = round4(cols);
-  *ld_out = ldo;
-  int kind = 0;
+                   SplitOperand* out, std::vector<SplitJob>& jobs) {
+  const int64_t ldo = round8(cols);
+  if (rows * ldo > kMaxTransientSplitFloats) return false;
+  int64_t key = 0;
   uint64_t epoch = 0;
-  if (src >= c->theta && src < c->theta + c->n) { kind = 1; epoch = c->theta_epoch; }
-  else {
-    for (int m = 0; m <= c->L && kind == 0; ++m)
-      if (c->Z[m] && src >= c->Z[m] && src < c->Z[m] + c->capS * c->w[m]) { kind = 2; epoch = c->sub_epoch; }
-  }
+  const int kind = split_kind(c, src, &key, &epoch);
+  gn_ctx::SplitBuf* buf = nullptr;
+  bool fresh = false;
   if (kind != 0) {
-    // one entry per start address: a matrix that comes back with another shape (a subsample of another
-    // size in the same buffers) replaces the old parts instead of adding to them
+    // one entry per place: a matrix that comes back with another shape (a subsample of another size in the same
+    // buffers) replaces the old parts instead of adding to them
     gn_ctx::SplitEntry* e = nullptr;
     for (auto& x : c->split_cache)
-      if (x.src == src && x.kind == kind) { e = &x; break; }
+      if (x.kind == kind && x.key == key) { e = &x; break; }
     if (!e) {
       if (c->split_cache.size() >= 4096) return false;
       gn_ctx::SplitEntry x{};
-      x.src = src; x.kind = kind; x.epoch = 0;
+      x.kind = kind; x.key = key;
+      x.in_arena = arena_buffer(c, kind, key, rows, cols, ld, &x.buf);
       c->split_cache.push_back(x);
       e = &c->split_cache.back();
     }
-    if (e->epoch != epoch || e->rows != rows || e->cols != cols || e->ld != ld) {
+    fresh = e->epoch == epoch && e->rows == rows && e->cols == cols && e->ld == ld;
+    if (!fresh) {
       e->epoch = 0;
-      if (!split_buf_reserve(c, e->buf, rows * ldo)) return false;
-      c->launches += launch_split_tf32(src, rows, cols, ld, e->buf.hi, e->buf.lo, ldo, c->st);
+      if (rows * ldo > e->buf.cap) {
+        if (e->in_arena) { e->buf = gn_ctx::SplitBuf{}; e->in_arena = false; }
+        if (!split_buf_reserve(c, e->buf, rows * ldo)) return false;
+      }
       e->rows = rows; e->cols = cols; e->ld = ld; e->epoch = epoch;
     }
-    *hi = e->buf.hi; *lo = e->buf.lo;
-    return true;
-  }
-  for (auto& e : c->parts)
-    if (e.src == src && e.epoch == c->parts_epoch && e.rows == rows && e.cols == cols && e.ld == ld && e.buf.hi) {
-      *hi = e.buf.hi; *lo = e.buf.lo;      // written by the epilogue that produced this operand
-      return true;
-    }
-  if (rows * ldo > kMaxTransientSplitFloats) return false;
-  gn_ctx::SplitSlot& sl = c->split_slot[role];
-  const bool same = reuse && sl.seq != 0 && sl.seq + 1 == c->gemm_seq && sl.src == src && sl.rows == rows &&
-                    sl.cols == cols && sl.ld == ld && sl.buf.hi;
-  if (!same) {
-    sl.src = nullptr; sl.seq = 0;
-    if (!split_buf_reserve(c, sl.buf, rows * ldo)) return false;
-    c->launches += launch_split_tf32(src, rows, cols, ld, sl.buf.hi, sl.buf.lo, ldo, c->st);
-    sl.src = src; sl.rows = rows; sl.cols = cols; sl.ld = ld;
-  }
-  sl.seq = c->gemm_seq;
-  *hi = sl.buf.hi; *lo = sl.buf.lo;
-  return true;
-}
-
-// FP32-accurate contraction on the tensor cores: every operand as hi + lo TF32 parts, three products per
-// operand pair, accumulation in chunks (gemm_tf32.cu).  False if the problem has to go to the FP32 FMA GEMM.
-bool run_gemm_x3(gn_ctx* c, const GemmArgs& g) {
-  if (!c->x3_usable || !gemm_tf32x3_eligible(g)) return false;
-  GemmArgs h = g;
-  const float *hi = nullptr, *lo = nullptr;
-  int64_t ldo = 0;
-  // stored matrices: A is [M][K] (K-major) or [K][M]; B is [N][K] (K-major) or [K][N]
-  if (!split_operand(c, g.A1, g.a_kmajor ? g.M : g.K1, g.a_kmajor ? g.K1 : g.M, g.lda1, 0, g.a1_split_fresh, &hi, &lo, &ldo)) return false;
-  h.A1 = hi; h.A1lo = lo; h.lda1 = ldo;
-  if (!split_operand(c, g.B1, g.b_kmajor ? g.N : g.K1, g.b_kmajor ? g.K1 : g.N, g.ldb1, 1, false, &hi, &lo, &ldo)) return false;
-  h.B1 = hi; h.B1lo = lo; h.ldb1 = ldo;
-  if (g.A2) {
-    if (!split_operand(c, g.A2, g.a_kmajor ? g.M : g.K2, g.a_kmajor ? g.K2 : g.M, g.lda2, 2, false, &hi, &lo, &ldo)) return false;
-    h.A2 = hi; h.A2lo = lo; h.lda2 = ldo;
-    if (!split_operand(c, g.B2, g.b_kmajor ? g.N : g.K2, g.b_kmajor ? g.K2 : g.N, g.ldb2, 3, false, &hi, &lo, &ldo)) return false;
-    h.B2 = hi; h.B2lo = lo; h.ldb2 = ldo;
-  }
-  h.mn_padded = true;     // the parts live in context allocations, which carry slack after their last row
-  gn_ctx::PartsEntry* pe = nullptr;
-  if (g.emit_parts && c->parts_enabled && (int64_t)g.M * round4(g.N) <= kMaxTransientSplitFloats) {
-    // the result is an operand later in this launch sequence: have the epilogue write its hi / lo parts as well
-    for (auto& e : c->parts)
-      if (e.src == g.D) { pe = &e; break; }
-    if (!pe && c->parts.size() < 1024) { c->parts.emplace_back(); pe = &c->parts.back(); pe->src = g.D; }
-    if (pe) {
-      pe->epoch = 0;
-      if (split_buf_reserve(c, pe->buf, (int64_t)g.M * round4(g.N))) {
-        h.Dhi = pe->buf.hi; h.Dlo = pe->buf.lo; h.ld_parts = round4(g.N);
-      } else {
-        pe = nullptr;
+    buf = &e->buf;
+  } else {
+    gn_ctx::SplitSlot& sl = c->split_slot[role];
+    fresh = reuse && sl.seq != 0 && sl.seq + 1 == c->gemm_seq && sl.src == src && sl.rows == rows && sl.cols == cols &&
+            sl.ld == ld && sl.buf.p;
+    if (!fresh) {
+      sl.src = nullptr; sl.seq = 0;
+      int64_t want = rows * ldo;
+      if (want > sl.buf.cap) {       // (grow at once to what this role will meet in the current workspaces)
+        int64_t widest = 0;
+        for (int m = 1; m < c->L; ++m) widest = std::max<int64_t>(widest, round8(c->w[m]));
+        if (role == 0) want = std::max(want, std::max(c->nS, c->capB) * widest);
+        if (!split_buf_reserve(c, sl.buf, want)) return false;
       }
+      sl.src = src; sl.rows = rows; sl.cols = cols; sl.ld = ld;
     }
+    sl.seq = c->gemm_seq;
+    buf = &sl.buf;
   }
-  run_gemm_kind(c, h, 3);
-  if (pe && c->x3_usable) { pe->rows = g.M; pe->cols = g.N; pe->ld = g.ldd; pe->epoch = c->parts_epoch; }
+  out->hi = buf->p; out->lo = buf->p + buf->cap; out->ld = ldo; out->amax = buf->bits(); out->reset = nullptr;
+  if (!fresh) {
+    SplitJob j{};
+    j.src = src; j.rows = rows; j.cols = cols; j.ld = ld;
+    j.hi = buf->p; j.lo = buf->p + buf->cap; j.ld_out = ldo; j.bits = buf->bits();
+    for (auto& e : c->amax)
+      if (e.src == src && e.dirty && e.epoch == c->parts_epoch && e.rows == rows && e.cols == cols && e.ld == ld) {
+        j.acc = e.acc;                       // recorded by the contraction that produced this operand
+        out->reset = e.acc;
+        e.dirty = false;
+      }
+    jobs.push_back(j);
+  }
   return true;
 }
 
-// Kernel choice: streaming kernels for the n_L-wide shapes (both precisions: they are exact FP32),
-// the tensor-core kernel in TF32 mode when TMA can address the operands and, in its error-compensated
-// form, in FP32-accurate mode when the shape suits the CTA-pair kernel; else the FP32 FMA GEMM.
+void run_splits(gn_ctx* c, const std::vector<SplitJob>& jobs) {
+  for (size_t i = 0; i < jobs.size(); i += kSplitSegs) {
+    const int r = launch_split_f16(jobs.data() + i, (int)std::min<size_t>(kSplitSegs, jobs.size() - i), c->split_part, c->st);
+    if (r < 0) { c->sticky = GN_ECUDA; c->err = "an operand could not be split"; return; }
+    c->launches += r;
+  }
+}
+
+// Stored matrices: A is [M][K] (K-major) or [K][M]; B is [N][K] (K-major) or [K][N].
+struct OperandView { const float* p; int64_t rows; int cols; int64_t ld; };
+OperandView operand_view(const GemmArgs& g, int role) {
+  const int K = role < 2 ? g.K1 : g.K2;
+  if (role % 2 == 0) {
+    const float* p = role == 0 ? g.A1 : g.A2;
+    const int64_t ld = role == 0 ? g.lda1 : g.lda2;
+    return g.a_kmajor ? OperandView{p, g.M, K, ld} : OperandView{p, K, g.M, ld};
+  }
+  const float* p = role == 1 ? g.B1 : g.B2;
+  const int64_t ld = role == 1 ? g.ldb1 : g.ldb2;
+  return g.b_kmajor ? OperandView{p, g.N, K, ld} : OperandView{p, K, g.N, ld};
+}
+
+// FP32-accurate contraction on the FP16 tensor cores.  False if it has to go to the FP32 FMA GEMM.  Chunks of 128
+// terms (about 4e-7 of the result) on FP32-accurate contexts at the shapes of whole CTA-pair tiles, of 64 terms
+// (about 2e-7, below what a chain of K FP32 additions leaves) where the alternative is the FMA GEMM.
+bool run_gemm_f16x3(gn_ctx* c, const GemmArgs& args) {
+  GemmArgs g = args;
+  g.chunk_kb = c->prec == GN_FP32_ACCURATE && g.M > 128 && g.N >= 128 ? 2 : 1;
+  if (!c->x3_usable || !gemm_f16x3_usable() || g.K1 < 1 || (g.A2 && g.K2 < 1)) return false;
+  if (ensure_split_scratch(c) != GN_OK) return false;
+  if (!c->sk_enabled || (gemm_f16x3_workspace_floats(g) > 0 && ensure_sk_workspace(c) != GN_OK)) g.whole_tiles = true;
+  // (the record of the result's maximum first: what follows takes records away, and must not be undone)
+  gn_ctx::AmaxEntry* ae = nullptr;
+  if (g.emit_amax && c->amax_enabled) {
+    for (auto& e : c->amax)
+      if (e.src == g.D) { ae = &e; break; }
+    if (!ae && c->amax.size() < kMaxRecords) {
+      gn_ctx::AmaxEntry e;
+      e.acc = c->split_part + kSplitBlocks + c->amax.size();
+      e.src = g.D; e.dirty = true;
+      c->amax.push_back(e);
+      ae = &c->amax.back();
+    }
+  }
+  std::vector<SplitJob> jobs;
+  SplitOperand ops[4];
+  for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
+    const OperandView v = operand_view(g, role);
+    if (!split_operand(c, v.p, v.rows, v.cols, v.ld, role, role == 0 && g.a1_split_fresh, &ops[role], jobs)) {
+      run_splits(c, jobs);                       // (what has been recorded as split must be)
+      for (auto& e : c->amax) { e.epoch = 0; e.dirty = true; }
+      return false;
+    }
+  }
+  run_splits(c, jobs);
+  if (ae) {
+    if (ae->dirty) cudaMemsetAsync(ae->acc, 0, sizeof(unsigned), c->st);   // (new, or nobody read the last record)
+    ae->rows = g.M; ae->cols = g.N; ae->ld = g.ldd; ae->epoch = c->parts_epoch; ae->dirty = true;
+  }
+  for (int k = 0; k < 4; ++k) c->h_ops[k] = ops[k];
+  c->h_amax_out = ae ? ae->acc : nullptr;
+  run_gemm_kind(c, g, 3);
+  return true;
+}
+
+// Whether the tensor-core form is the faster way to FP32 accuracy.  The FP32 FMA GEMM walks K alone in 128 x 128
+// tiles, about 0.1 us per unit of K and round of tiles; the tensor-core form pays for splitting its operands
+// (two launches, about 5 us, and their bytes) before it starts.
+bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
+  if (!c->x3_usable || !gemm_f16x3_usable()) return false;
+  if (c->prec == GN_FP32_ACCURATE && c->acc_method == 1) return false;
+  const double K = (double)g.K1 + (g.A2 ? g.K2 : 0);
+  const double blocks = ((g.M + 127) / 128) * (double)((g.N + 127) / 128);
+  const double rounds = blocks <= 148.0 ? 1.0 : blocks / 148.0;
+  const double fma_us = 3.0 + rounds * K * 0.1;
+  return gemm_f16x3_estimate_us(g) + 8.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5 < fma_us;
+}
+
+// Kernel choice: streaming kernels for the n_L-wide shapes (both precisions: they are exact FP32), the TF32
+// tensor-core kernel in TF32 mode when TMA can address the operands; everything else is computed to FP32 accuracy, by
+// the FP16 tensor-core kernel or the FP32 FMA GEMM, whichever is the faster at that size.
 void run_gemm(gn_ctx* c, const GemmArgs& g, cudaStream_t st = nullptr) {
   ++c->gemm_seq;
   const ThinKind thin = gemm_thin_kind(g);
@@ -473,8 +597,29 @@ void run_gemm(gn_ctx* c, const GemmArgs& g, cudaStream_t st = nullptr) {
     run_gemm_kind(c, g, 2, st);
     return;
   }
-  if (c->prec == GN_FP32_ACCURATE && c->acc_method != 1 && run_gemm_x3(c, g)) return;
-  run_gemm_kind(c, g, (c->prec == GN_TF32 && gemm_tf32_eligible(g)) ? 0 : 1, st);
+  if (c->prec == GN_TF32 && gemm_tf32_eligible(g)) { run_gemm_kind(c, g, 0, st); return; }
+  if (!st && wants_f16x3(c, g) && run_gemm_f16x3(c, g)) return;
+  run_gemm_kind(c, g, 1, st);
+}
+
+// The parts of the operands in `roles` (bit per role) of several contractions that will go to the FP32-accurate
+// tensor-core kernel, in one splitting launch instead of one per contraction.  Kept kinds only.
+void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
+  std::vector<SplitJob> jobs;
+  for (int i = 0; i < n; ++i) {
+    const GemmArgs& g = gs[i];
+    const bool tf32 = c->prec == GN_TF32 && gemm_tf32_eligible(g);
+    if (tf32 || gemm_thin_kind(g) != THIN_NONE || !wants_f16x3(c, g)) continue;
+    if (ensure_split_scratch(c) != GN_OK) return;
+    for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
+      const OperandView v = operand_view(g, role);
+      int64_t key = 0;
+      uint64_t epoch = 0;
+      SplitOperand op;
+      if ((roles >> role & 1) && split_kind(c, v.p, &key, &epoch) != 0) split_operand(c, v.p, v.rows, v.cols, v.ld, role, false, &op, jobs);
+    }
+  }
+  run_splits(c, jobs);
 }
 
 // Independent contractions issued together (any order is allowed).  In TF32 mode those that suit the CTA-pair
@@ -519,6 +664,7 @@ void run_gemm_group(gn_ctx* c, const GemmArgs* gs, int n) {
     }
     flush();
   }
+  presplit(c, gs, n, 0xf);
   for (int i = 0; i < n; ++i)
     if (i >= 16 || !taken[i]) run_gemm(c, gs[i]);
 }
@@ -614,7 +760,7 @@ const float* Wm(const gn_ctx* c, const float* vec, int m) { return vec + c->w_of
 const float* bm(const gn_ctx* c, const float* vec, int m) { return vec + c->b_off[m]; }
 
 // Eq. (xtoz): Zout[m] = sigma(Zout[m-1] W^m + 1 b^mT), m = 1..L, over `rows` rows; Zout[0] = Z0.
-void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout, bool emit_parts = false) {
+void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout, bool emit_amax = false) {
   std::vector<GemmArgs> gs((size_t)c->L);
   std::vector<int> dep((size_t)c->L), dep_all((size_t)c->L, 0);
   for (int m = 1; m <= c->L; ++m) {
@@ -626,9 +772,10 @@ void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>&
     g.D = Zout[m]; g.ldd = c->w[m];
     g.bias = bm(c, c->theta, m);
     g.sigmoid = m < c->L;
-    g.emit_parts = emit_parts && m < c->L;   // Z_m is an operand of layer m + 1 and of its weight block
+    g.emit_amax = emit_amax && m < c->L;   // Z_m is an operand of layer m + 1 and of its weight block
     dep[(size_t)m - 1] = m - 2;          // layer m reads the rows layer m - 1 writes
   }
+  presplit(c, gs.data(), c->L, 0x2);       // theta's weights
   run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), c->L);
 }
 
@@ -678,7 +825,7 @@ GemmArgs backward_data_args(const gn_ctx* c, int m, const float* ds, int64_t row
   g.dsig = Zprev; g.ld_dsig = c->w[m - 1]; g.dsig_rows = (int)z_rows;
   g.D = dst; g.ldd = c->w[m - 1];
   g.mn_padded = true;     // B is the context's own (padded) copy of theta
-  g.emit_parts = ds_just_used;   // in the full product and the gradient, delta s^{m-1} feeds the two contractions of layer m - 1
+  g.emit_amax = ds_just_used;   // in the full product and the gradient, delta s^{m-1} feeds the two contractions of layer m - 1
   return g;
 }
 
@@ -756,6 +903,7 @@ gn_status backward_hidden_layers(gn_ctx* c, int m_top, const float* ds_top, cons
 gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("G v");
   SideJoin side_guard(c);
+  CurrentVector current(c, v);
   ++c->parts_epoch;
   const int L = c->L;
   const int64_t nS = c->nS;
@@ -775,9 +923,10 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
       if (m < L) { g.dsig = c->Z[m]; g.ld_dsig = c->w[m]; g.dsig_rows = (int)nS; }
       else g.alpha = 2.f;                                   // B = 2I
       g.D = c->RZ[m]; g.ldd = c->w[m];
-      g.emit_parts = m < L;              // R z^m is an operand of layer m + 1
+      g.emit_amax = m < L;              // R z^m is an operand of layer m + 1
       dep[(size_t)m - 1] = m - 2;        // R z^{m-1} of the layer below
     }
+    presplit(c, gs.data(), L, 0xf);
     run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), L, 2);
   }
   const float inv = (float)(1.0 / (double)nS);
@@ -797,7 +946,7 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
 gn_status ensure_stacked(gn_ctx* c) {
   if (c->stacked) return GN_OK;
   quiesce(c);
-  drop_parts(c);
+  drop_amax(c);
   for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m]); dev_free(c, c->DS[m]); }
   c->stacked = true;
   for (int m = 1; m <= c->L; ++m) {
@@ -806,6 +955,7 @@ gn_status ensure_stacked(gn_ctx* c) {
     if (st != GN_OK) {
       // leave a consistent, empty state: the next set_subsample allocates afresh
       for (int k = 1; k <= c->L; ++k) { dev_free(c, c->RZ[k]); dev_free(c, c->DS[k]); }
+      drop_kept_parts(c, 2);
       for (int k = 0; k <= c->L; ++k) dev_free(c, c->Z[k]);
       dev_free(c, c->idx);
       c->capS = 0; c->have_sub = false; c->factors_valid = false;
@@ -818,6 +968,7 @@ gn_status ensure_stacked(gn_ctx* c) {
 gn_status product_blockdiag(gn_ctx* c, const float* v, float* out, float coef) {
   GN_TRY(ensure_stacked(c));
   SideJoin side_guard(c);
+  CurrentVector current(c, v);
   ++c->parts_epoch;
   const int L = c->L;
   const int64_t nS = c->nS;
@@ -895,6 +1046,7 @@ gn_status ensure_factors(gn_ctx* c) {
 
 gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float coef) {
   SideJoin side_guard(c);
+  CurrentVector current(c, v);
   ++c->parts_epoch;
   GN_TRY(ensure_factors(c));
   const int L = c->L, nL = c->w[L];
@@ -937,7 +1089,9 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   // More and shorter tiles fill the rounds better, and a short second part fills them best (the long tiles go
   // first, the short ones level the loads): the cut is the one of 1/2, 5/8, 3/4 of the rows for which the host's
   // work list comes out shortest.  The order of the two partial sums is fixed.
-  const bool halves = c->prec == GN_TF32 && c->chain_level >= 1 && c->split_k_enabled && nS >= 4096 && L - 1 >= 1 && L - 1 <= kGroup;
+  bool tf32_operands = true;                                  // (the FP32-accurate kernel cuts K by itself)
+  for (int m = 0; m < L; ++m) tf32_operands = tf32_operands && c->w[m] % 4 == 0;
+  const bool halves = c->prec == GN_TF32 && c->chain_level >= 1 && c->split_k_enabled && nS >= 4096 && L - 1 >= 1 && L - 1 <= kGroup && tf32_operands;
   if (halves) {
     GemmArgs gs[2 * kGroup];
     int dep[2 * kGroup], dep_all[2 * kGroup];
@@ -989,6 +1143,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
 // Q_a[:, T_b] = D[:, :, T_b]^T 2 D[:, :, T_b] U_a[:, T_b]; then out_W[T_a, :] = Z_{m-1}[:, T_a]^T Q_a / |S|.
 // At the output layer D = I, so Q_a = 2 U_a.
 gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
+  CurrentVector current(c, v);
   ++c->parts_epoch;
   const int L = c->L, nL = c->w[L];
   const int64_t nS = c->nS;
@@ -1075,7 +1230,8 @@ gn_status ensure_batch(gn_ctx* c) {
   const int64_t rows = c->batch_rows < c->l ? c->batch_rows : c->l;
   if (rows <= c->capB) return GN_OK;
   quiesce(c);
-  drop_parts(c);
+  drop_amax(c);
+  drop_kept_parts(c, 4);
   for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
   c->capB = 0;
   for (int m = 1; m <= c->L; ++m) {
@@ -1097,10 +1253,12 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
   GN_TRY(ensure_partials(c, per_batch * nb + (c->n + kCgChunk - 1) / kCgChunk + 16));
   const float inv_l = (float)(1.0 / (double)c->l);
   const float inv_C = (float)(1.0 / c->C);
+  struct CurrentBatch { gn_ctx* c; ~CurrentBatch() { c->cur_x = nullptr; c->cur_x_count = 0; } } current{c};
   for (int64_t b = 0; b < nb; ++b) {
     const int64_t r0 = b * Rb;
     const int64_t rows = (c->l - r0 < Rb) ? c->l - r0 : Rb;
     const float* X0 = c->dX + r0 * c->w[0];
+    c->cur_x = X0; c->cur_x_count = rows * c->w[0];
     ++c->parts_epoch;           // the batch buffers are rewritten
     forward_pass(c, X0, rows, c->Zb, true);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
@@ -1118,9 +1276,9 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
       std::vector<const float*> zprev((size_t)L);
       for (int m = 1; m <= L; ++m) zprev[(size_t)m - 1] = m == 1 ? X0 : c->Zb[m - 1];
       // layer 1 reads the caller's X, which has no slack after its last row: in the last batch all but the final
-      // 32 rows use the padded fast path, the rest is added by a second, unpadded contraction
+      // 32 rows use the TF32 kernel's padded fast path, the rest is added by a second, unpadded contraction
       const bool last = r0 + rows == c->l;
-      const bool tail = last && rows > 64;
+      const bool tail = last && rows > 64 && c->prec == GN_TF32 && c->w[0] % 4 == 0 && c->w[1] % 4 == 0;
       const int64_t head = tail ? rows - 32 : rows;
       if (L > 1) {
         GN_TRY(layer_backward(c, L, c->Db[L], rows, c->Db[L], rows, c->Zb[L - 1], rows, inv_l, cin0, beta0, d_grad, c->Db[L - 1]));
@@ -1330,7 +1488,8 @@ gn_status gn_set_batch_rows(gn_ctx* c, int64_t rows) {
   if ((rows < c->l ? rows : c->l) != c->capB && c->capB > 0) {
     // shrink or grow on next use: drop the old workspace now so memory stays bounded
     quiesce(c);
-    drop_parts(c);
+    drop_amax(c);
+    drop_kept_parts(c, 4);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
     c->capB = 0;
   }
@@ -1348,7 +1507,7 @@ gn_status gn_set_blockdiag_method(gn_ctx* c, int method) {
 
 gn_status gn_set_accurate_method(gn_ctx* c, int method) {
   if (!c) return GN_EINVAL;
-  if (method < 0 || method > 2) return fail(c, GN_EINVAL, "method must be 0 (choose), 1 (FP32 FMA) or 2 (3 x TF32 where the shape allows)");
+  if (method < 0 || method > 2) return fail(c, GN_EINVAL, "method must be 0 (choose), 1 (FP32 FMA) or 2 (as 0)");
   c->acc_method = method;
   return GN_OK;
 }
@@ -1422,17 +1581,8 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   ++c->parts_epoch;
   if (nS > c->capS) {
     GN_TRY(sync(c, "set_subsample"));
-    // the stored activations move: the hi / lo parts kept for matrices inside the old buffers go with them
-    for (size_t i = 0; i < c->split_cache.size();) {
-      if (c->split_cache[i].kind == 2) {
-        dev_free(c, c->split_cache[i].buf.hi, c->split_cache[i].buf.cap);
-        dev_free(c, c->split_cache[i].buf.lo, c->split_cache[i].buf.cap);
-        c->split_cache.erase(c->split_cache.begin() + (long)i);
-      } else {
-        ++i;
-      }
-    }
-    drop_parts(c);
+    drop_kept_parts(c, 2);      // the stored activations move: their parts are made anew
+    drop_amax(c);
     dev_free(c, c->idx, c->capS);
     for (int m = 0; m <= c->L; ++m) dev_free(c, c->Z[m], c->capS * c->w[m]);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m], m * c->capS * c->w[m]); dev_free(c, c->DS[m], m * c->capS * c->w[m]); }
@@ -1451,7 +1601,7 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   GN_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->st));
   c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
   GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
-  forward_pass(c, c->Z[0], nS, c->Z);
+  forward_pass(c, c->Z[0], nS, c->Z, true);
   GN_TRY(check_launch(c, "set_subsample"));
   GN_TRY(sync(c, "set_subsample"));
   if (*c->h_err) return fail(c, GN_EINVAL, "a subsample index lies outside [0, l)");
@@ -1696,7 +1846,7 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* c, int kind, int M, int N, int K, const
                                  int sigmoid, const float* d_dsig, int64_t ld_dsig, float alpha, const float* d_cin,
                                  int64_t ld_cin, float beta) {
   if (!c) return GN_EINVAL;
-  if (!dA || !dB || !dD || M < 1 || N < 1 || K < 1 || kind < 0 || kind > 7) return fail(c, GN_EINVAL, "bad GEMM arguments");
+  if (!dA || !dB || !dD || M < 1 || N < 1 || K < 1 || kind < 0 || kind > 8) return fail(c, GN_EINVAL, "bad GEMM arguments");
   if ((d_dsig && ld_dsig < N) || (d_cin && ld_cin < N)) return fail(c, GN_EINVAL, "leading dimension of an epilogue operand below N");
   GemmArgs g;
   g.M = M; g.N = N; g.K1 = K;
@@ -1715,9 +1865,9 @@ static gn_status debug_gemm_impl(gn_ctx* c, int kind, GemmArgs g) {
   // 4 = one CTA per tile forced, 5 = CTA pair per tile forced, 6 = as 5 without splitting tiles
   // between pairs (all with padded operands)
   ++c->parts_epoch;
-  if (kind == 7) {          // error-compensated tensor-core form (3 x TF32, chunked accumulation)
+  if (kind == 7 || kind == 8) {   // FP32-accurate tensor-core form: 7 = shapes that fill a CTA-pair tile only, 8 = any
     ++c->gemm_seq;
-    if (!run_gemm_x3(c, g)) return fail(c, GN_EINVAL, "the error-compensated tensor-core form does not take this problem");
+    if ((kind == 7 && (g.M <= 128 || g.N < 128)) || !run_gemm_f16x3(c, g)) return fail(c, GN_EINVAL, "the FP32-accurate tensor-core form does not take this problem");
     GN_TRY(check_launch(c, "debug_gemm"));
     return sync(c, "debug_gemm");
   }
@@ -1812,7 +1962,7 @@ gn_status gn_debug_option(gn_ctx* c, int option, int value) {
   if (option == 8) { c->back_chain = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }
   if (option == 9) { c->fly_enabled = value != 0; return GN_OK; }
   if (option == 6) { c->graph_enabled = value != 0; return GN_OK; }
-  if (option == 5) { c->parts_enabled = value != 0; return GN_OK; }
+  if (option == 5) { c->amax_enabled = value != 0; return GN_OK; }
   if (option == 4) { c->chain_level = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }
   if (option == 0) c->group_enabled = value != 0;
   else if (option == 1) c->sk_enabled = value != 0 && c->sk_enabled;

@@ -22,16 +22,10 @@ struct GemmArgs {
   int M = 0, N = 0;
   const float* A1 = nullptr; const float* B1 = nullptr; int K1 = 0; int64_t lda1 = 0, ldb1 = 0;
   const float* A2 = nullptr; const float* B2 = nullptr; int K2 = 0; int64_t lda2 = 0, ldb2 = 0;
-  // Error-compensated form of the tensor-core kernel (3 x TF32): when A1lo is set, every operand X is given as
-  // X = Xhi + Xlo with both parts exactly representable in TF32 (A1, B1, A2, B2 hold the hi parts; same
-  // layouts and leading dimensions for the lo parts), and acc = sum Alo Bhi + Ahi Blo + Ahi Bhi.
-  const float* A1lo = nullptr; const float* B1lo = nullptr; const float* A2lo = nullptr; const float* B2lo = nullptr;
   bool a1_split_fresh = false;   // caller's word that A1 is, unchanged, the A1 of the previous contraction
-  // Error-compensated form: the result will itself be an operand of a later contraction (emit_parts, set by the
-  // caller), and where the hi / lo parts of every stored value go (Dhi, Dlo with leading dimension ld_parts,
-  // filled in by the host logic that owns the buffers).
-  bool emit_parts = false;
-  float* Dhi = nullptr; float* Dlo = nullptr; int64_t ld_parts = 0;
+  int chunk_kb = 1;              // FP32-accurate tensor-core form: 64-term k-blocks per accumulation in tensor memory
+  bool whole_tiles = false;      // ... without K slices (no workspace)
+  bool emit_amax = false;        // the result is an operand of a later contraction of this launch sequence
   bool a_kmajor = true, b_kmajor = true;
   bool mn_padded = false;  // every MN-major operand is followed by >= 128 readable bytes
   int two_cta = -1;        // tensor-core kernel: -1 choose, 0 one CTA per tile, 1 CTA pair per 256-row tile
@@ -56,11 +50,6 @@ int launch_gemm_ffma(const GemmArgs& g, cudaStream_t st);
 // first launch; every launch that completes leaves them zero again (after a launch that gave up on a
 // bounded wait they must be cleared by the caller).
 bool gemm_tf32_eligible(const GemmArgs& g);
-// Error-compensated form (GemmArgs::A1lo ...): whether it takes a problem (the shape must suit the CTA-pair
-// kernel; the hi / lo parts must be 16-byte aligned with leading dimensions that are multiples of 4 and be
-// followed by >= 128 readable bytes), and its launch.  Returns launches made, or -1 if it cannot run.
-bool gemm_tf32x3_eligible(const GemmArgs& g);
-int launch_gemm_tf32x3(const GemmArgs& g, int* err_flag, cudaStream_t st);
 int64_t gemm_tf32_workspace_floats();
 int gemm_tf32_workspace_flags();
 int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_flags, cudaStream_t st);
@@ -83,6 +72,29 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
 int gemm_tf32_plan_group(int n, const int* M, const int* N, const int* K, int pairs, int keep_order, int* counts,
                          int* waves, int* order_out, int* tiles_out);
 double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K, int keep_order);
+
+// FP32-accurate contraction on the FP16 tensor cores (gemm_f16x3.cu): any shape and alignment, because it reads
+// split copies of its operands.
+//   SplitOperand  the two FP16 parts of a stored matrix X (X 2^e = hi + lo; leading dimension a multiple of 8, 16-byte
+//                 aligned) and the device word with the bit pattern of max|X| that e follows from; `reset`, if set, is a
+//                 word the contraction clears (see SplitJob::acc).
+//   SplitJob      one matrix to be split.  acc: a device word into which the contraction that produced the matrix has
+//                 accumulated max|X| (amax_out below), or nullptr to have it found in a pass of its own.
+// ops: A1, B1, A2, B2.  ws: gemm_f16x3_workspace_floats(g) floats (K slices; never more than
+// gemm_tf32_workspace_floats()).  amax_out: if set, atomically raised to the bit pattern of the largest finite |D|.
+// Both return launches made, or -1 if the launch failed.
+struct SplitOperand { const void* hi = nullptr; const void* lo = nullptr; int64_t ld = 0; const unsigned* amax = nullptr; unsigned* reset = nullptr; };
+struct SplitJob {
+  const float* src; int64_t rows; int cols; int64_t ld;
+  void* hi; void* lo; int64_t ld_out; unsigned* bits; unsigned* acc;
+};
+constexpr int kSplitSegs = 8;
+constexpr int kSplitBlocks = 148 * 8;   // blocks of a splitting launch at most; `part` holds that many words
+bool gemm_f16x3_usable();
+double gemm_f16x3_estimate_us(const GemmArgs& g);
+int64_t gemm_f16x3_workspace_floats(const GemmArgs& g);
+int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, unsigned* amax_out, int* err_flag, cudaStream_t st);
+int launch_split_f16(const SplitJob* jobs, int n, unsigned* part, cudaStream_t st);
 
 // Streaming FP32 kernels for contractions with one dimension <= 16 (the n_L-wide output layer).
 // gemm_thin_kind says which of them (if any) takes a problem; THIN_M needs a scratch buffer of
@@ -118,11 +130,6 @@ int launch_sum_partials(const double* partial, int count, double* out, bool accu
 
 // out[i] = a x[i] + b y[i]; out may be x or y.
 int launch_axpby(int64_t n, float a, const float* x, float b, const float* y, float* out, cudaStream_t st);
-
-// Two-term TF32 split of a [rows][cols] matrix with leading dimension ld into hi and lo (leading dimension
-// ld_out): hi = x rounded to TF32, lo = (x - hi) rounded to TF32, so x = hi + lo up to 2^-22 |x|.
-int launch_split_tf32(const float* src, int64_t rows, int cols, int64_t ld, float* hi, float* lo, int64_t ld_out,
-                      cudaStream_t st);
 
 // Stored Jacobian factors (d z^L / d s^m per sample, Section 3.3.1).  D is [rows * nL][n] with row i * nL + u.
 // factor_last: D[(i, u)][t] = WL[u * n + t] * z (1 - z), z = Zprev[i * n + t]   (layer L-1 from the linear output layer)
