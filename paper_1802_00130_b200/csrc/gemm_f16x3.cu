@@ -48,7 +48,7 @@ struct HEpilogue {
   const float* dsig; long long ld_dsig; int dsig_rows, dsig_div, dsig_direct;
   float alpha;
   const float* cin; long long ld_cin; float beta;
-  int vec;                                   // D, bias, dsig, cin all 16-byte aligned with leading dimensions % 4 == 0
+  int vec;                                   // N % 4 == 0; D, bias, dsig, cin 16-byte aligned, leading dimensions % 4 == 0
   unsigned* amax_out;                        // |D| maximum (bit pattern) is accumulated here when set
 };
 
@@ -96,7 +96,7 @@ __device__ __forceinline__ long long dsig_row(const HEpilogue& e, int m) {
 
 __device__ __forceinline__ float finish(const HEpilogue& e, float x, float bz, float z, float c) {
   x += bz;
-  if (e.sigmoid) x = 1.f / (1.f + expf(-x));
+  if (e.sigmoid) x = sigmoid_from(expf(-x));
   if (e.dsig) x *= z * (1.f - z);
   x *= e.alpha;
   if (e.cin) x = fmaf(e.beta, c, x);
@@ -107,71 +107,90 @@ __device__ __forceinline__ float finish(const HEpilogue& e, float x, float bz, f
 // bits, so that a column of groups, a row of groups and a row of single elements are all free of bank conflicts.
 __device__ __forceinline__ int stg_at(int r, int q) { return r * 32 + ((q ^ (r & 7)) << 2); }
 
-// One 32 x 32 chunk of finished sums from a warp's staging tile through the epilogue options and out.  VEC: lane l takes
-// columns 4 (l % 8) .. + 3 of rows l / 8, l / 8 + 4, ..., one 16-byte access per four values and four whole rows per
-// instruction; otherwise lane = column, one row per instruction.  Few warps run this beside the main loop, so its own
-// instruction stream is what bounds it: MODE fixes the options at compile time (0 = alpha * x (+ bias), 1 = sigmoid,
-// 2 = times the sigmoid derivative of dsig, 3 = plus beta * cin, 4 = any combination), and the operand of modes 2 and 3
-// is requested a few rows before its use (more in flight would spill beside the 128 running sums).  Against one path
-// for all options with one 4-byte access per value: 12000 x 2000 x 2000 from 285 to 245 us.
+// A warp's share of a finished tile through the epilogue options and out: `n_mine` chunks of 32 rows x 32 columns, 64
+// columns apart from column nb0 on, read back from tensor memory at `ta` (lane = row) and turned through the warp's
+// staging tile so that accesses to global memory are whole rows of 128 bytes whatever the alignment of the matrices.
+// VEC (16-byte aligned rows, N a multiple of 4): lane l takes columns 4 (l % 8) .. + 3 of rows l / 8, l / 8 + 4, ...;
+// otherwise lane = column, one row per access.  MODE fixes the options at compile time: 0 = alpha * x (+ bias), 1 =
+// sigmoid, 2 = times the sigmoid derivative of dsig, 3 = plus beta * cin, 4 = any combination.  Eight warps with
+// nothing to hide latency behind: what bounds this is the operand's round trips, so the operand of modes 2 and 3 is
+// requested for a whole chunk before the first use.  That takes registers the 128 running sums would not leave, hence
+// their detour through the tensor memory they came from, and the kernel is compiled per form so that no form's
+// registers are another's spills.  (Requested 2 to 4 rows at a time beside the sums, all forms in one kernel: 12000 x
+// 2000 x 2000 with dsig 319 us, now 236; 4001 x 1201 x 617 with unaligned rows 83, now 58.)
 template <int MODE, bool VEC>
-__device__ __forceinline__ void store_chunk(const HEpilogue& e, const float* stg, int m0, int rows, int nb, int lane, unsigned& mag) {
-  constexpr int W = VEC ? 4 : 1, STEP = VEC ? 4 : 1, IT = 32 / STEP, GRP = MODE == 4 ? 1 : VEC ? 2 : 4;
+__device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint32_t ta, int n_mine, int m0, int rows, int nb0, int lane, unsigned& mag) {
+  constexpr int W = VEC ? 4 : 1, STEP = VEC ? 4 : 1, IT = 32 / STEP;
+  constexpr bool ONE_OP = MODE == 2 || MODE == 3;
   const int col = VEC ? (lane & 7) * 4 : lane, r_first = VEC ? lane >> 3 : 0;
-  const int n = nb + col;
-  if (!VEC && n >= e.N) return;
   const bool use_sigm = MODE == 4 ? e.sigmoid != 0 : MODE == 1;
   const bool use_dsig = MODE == 4 ? e.dsig != nullptr : MODE == 2;
   const bool use_cin = MODE == 4 ? e.cin != nullptr : MODE == 3;
-  float bz[W];
+  float op[ONE_OP ? IT : 1][W];
+#pragma unroll 1
+  for (int j = 0; j < n_mine; ++j) {
+    const int n = nb0 + 64 * j + col;
+    if (ONE_OP && n < e.N) {
+      const float* src = MODE == 2 ? e.dsig + n : e.cin + (long long)(m0 + r_first) * e.ld_cin + n;
+      if (MODE == 2 && e.dsig_direct) src += (long long)(m0 + r_first) * e.ld_dsig;
+      const long long step = STEP * (MODE == 2 ? e.ld_dsig : e.ld_cin);
 #pragma unroll
-  for (int q = 0; q < W; ++q) bz[q] = 0.f;
-  if (e.bias) {
-    if (VEC) *reinterpret_cast<float4*>(bz) = __ldg(reinterpret_cast<const float4*>(e.bias + n));
-    else bz[0] = __ldg(e.bias + n);
-  }
-#pragma unroll MODE == 4 ? 1 : IT / GRP
-  for (int g = 0; g < IT; g += GRP) {
-    float op[GRP][W];
-    if (MODE == 2 || MODE == 3) {
-#pragma unroll
-      for (int i = 0; i < GRP; ++i) {
-        const int r = r_first + (g + i) * STEP;
-        const float* src = MODE == 2 ? e.dsig + dsig_row(e, m0 + r) * e.ld_dsig + n : e.cin + (long long)(m0 + r) * e.ld_cin + n;
+      for (int i = 0; i < IT; ++i) {
+        const int r = r_first + i * STEP;
+        const float* q = MODE == 2 && !e.dsig_direct ? src + dsig_row(e, m0 + r) * e.ld_dsig : src;
         if (r < rows) {
-          if (VEC) *reinterpret_cast<float4*>(op[i]) = __ldg(reinterpret_cast<const float4*>(src));
-          else op[i][0] = __ldg(src);
+          if (VEC) *reinterpret_cast<float4*>(op[ONE_OP ? i : 0]) = __ldg(reinterpret_cast<const float4*>(q));
+          else op[ONE_OP ? i : 0][0] = __ldg(q);
         }
+        if (MODE == 3 || e.dsig_direct) src += step;
       }
     }
+    {
+      float v[32];
+      tmem_ld32(ta + (uint32_t)(64 * j), v);
+      __syncwarp();
 #pragma unroll
-    for (int i = 0; i < GRP; ++i) {
-      const int r = r_first + (g + i) * STEP;
-      if (r >= rows) continue;
-      float x[W], z[W], c[W];
-      if (VEC) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(stg + stg_at(r, lane & 7));
-      else x[0] = stg[stg_at(r, lane >> 2) + (lane & 3)];
-      if (MODE == 4 && use_dsig) {
-        const float* src = e.dsig + dsig_row(e, m0 + r) * e.ld_dsig + n;
-        if (VEC) *reinterpret_cast<float4*>(z) = __ldg(reinterpret_cast<const float4*>(src)); else z[0] = __ldg(src);
-      }
-      if (MODE == 4 && use_cin) {
-        const float* src = e.cin + (long long)(m0 + r) * e.ld_cin + n;
-        if (VEC) *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(src)); else c[0] = __ldg(src);
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(stg + stg_at(lane, i >> 2)) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      __syncwarp();
+    }
+    if (n < e.N) {
+      float bz[W];
+#pragma unroll
+      for (int q = 0; q < W; ++q) bz[q] = 0.f;
+      if (e.bias) {
+        if (VEC) *reinterpret_cast<float4*>(bz) = __ldg(reinterpret_cast<const float4*>(e.bias + n));
+        else bz[0] = __ldg(e.bias + n);
       }
 #pragma unroll
-      for (int q = 0; q < W; ++q) {
-        float t = x[q] + bz[q];
-        if (use_sigm) t = 1.f / (1.f + expf(-t));
-        if (use_dsig) { const float zz = MODE == 4 ? z[q] : op[i][q]; t *= zz * (1.f - zz); }
-        t *= e.alpha;
-        if (use_cin) t = fmaf(e.beta, MODE == 4 ? c[q] : op[i][q], t);
-        x[q] = t;
-        if (e.amax_out) mag = max(mag, finite_magnitude(t));
+      for (int i = 0; i < IT; ++i) {
+        const int r = r_first + i * STEP;
+        if (r >= rows) continue;
+        float x[W], z[W], c[W];
+        if (VEC) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(stg + stg_at(r, lane & 7));
+        else x[0] = stg[stg_at(r, lane >> 2) + (lane & 3)];
+        if (MODE == 4 && use_dsig) {
+          const float* src = e.dsig + dsig_row(e, m0 + r) * e.ld_dsig + n;
+          if (VEC) *reinterpret_cast<float4*>(z) = __ldg(reinterpret_cast<const float4*>(src)); else z[0] = __ldg(src);
+        }
+        if (MODE == 4 && use_cin) {
+          const float* src = e.cin + (long long)(m0 + r) * e.ld_cin + n;
+          if (VEC) *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(src)); else c[0] = __ldg(src);
+        }
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+          float t = x[q] + bz[q];
+          if (use_sigm) t = sigmoid_from(expf(-t));
+          if (use_dsig) { const float zz = MODE == 4 ? z[q] : op[ONE_OP ? i : 0][q]; t *= zz * (1.f - zz); }
+          t *= e.alpha;
+          if (use_cin) t = fmaf(e.beta, MODE == 4 ? c[q] : op[ONE_OP ? i : 0][q], t);
+          x[q] = t;
+          if (e.amax_out) mag = max(mag, finite_magnitude(t));
+        }
+        float* d = e.D + (long long)(m0 + r) * e.ldd + n;
+        if (VEC) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(x);
+        else d[0] = x[0];
       }
-      float* d = e.D + (long long)(m0 + r) * e.ldd + n;
-      if (VEC) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(x);
-      else d[0] = x[0];
     }
   }
 }
@@ -200,6 +219,7 @@ __device__ __forceinline__ Item item_at(const HParams& p, int i, int n_chunks) {
   return Item{p.whole + k - sl * p.rem, (int)((long long)n_chunks * sl / p.slices), (int)((long long)n_chunks * (sl + 1) / p.slices), k};
 }
 
+template <int MODE, bool VEC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(H_THREADS, 1)
 gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -382,55 +402,48 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
             }
           }
         }
+        if (ch + 1 == w.c1) break;                               // (the last buffer takes the finished sums first)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
       }
       if (!alive) break;
-      if (m0 >= e.M) continue;                                   // warp-uniform
-      const int rows = min(32, e.M - m0);
-      // Each 32 x 32 chunk is turned through shared memory so that accesses to global memory are whole rows of 128
-      // bytes, whatever the alignment of the matrices.
-      const int n_opt = (e.sigmoid ? 1 : 0) + (e.dsig ? 1 : 0) + (e.cin ? 1 : 0);
-      const int mode = n_opt == 0 ? 0 : n_opt > 1 ? 4 : e.sigmoid ? 1 : e.dsig ? 2 : 3;
-#pragma unroll 1
-      for (int j = 0; j < 4; ++j) {
-        const int c = half + 2 * j;
-        if (c >= n_cc) break;
-        __syncwarp();
+      const int buf = ci & 1;
+      ++ci;
+      const uint32_t ta = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * H_BN_MAX + half * 32);
+      const int n_mine = (n_cc - half + 1) / 2;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (k == j) {                                          // (register arrays need indices known at compile time)
+      for (int j = 0; j < 4; ++j)
+        if (j < n_mine) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) run[j][i] = run[j][i] * u0 * u1;
+          tmem_st32(ta + (uint32_t)(j * 64), run[j]);
+        }
+      tmem_st_wait();
+      if (m0 < e.M) {                                            // warp-uniform
+        const int rows = min(32, e.M - m0), nb0 = n0 + half * 32;
+        if (w.slot >= 0) {                                       // (the workspace holds whole tiles)
+          float* o = p.ws + ((long long)w.slot * (2 * H_BM) + (int)rank * H_BM + quad * 32 + (lane >> 3)) * bn + half * 32 + (lane & 7) * 4;
+#pragma unroll 1
+          for (int j = 0; j < n_mine; ++j) {
+            float v[32];
+            tmem_ld32(ta + (uint32_t)(64 * j), v);
+            __syncwarp();
 #pragma unroll
             for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(stg + stg_at(lane, i >> 2)) =
-                  make_float4(run[k][i] * u0 * u1, run[k][i + 1] * u0 * u1, run[k][i + 2] * u0 * u1, run[k][i + 3] * u0 * u1);
-          }
-        __syncwarp();
-        const int nb = n0 + c * 32;
-        if (w.slot >= 0) {                                       // (the workspace holds whole tiles)
-          float* o = p.ws + ((long long)w.slot * (2 * H_BM) + (int)rank * H_BM + quad * 32 + (lane >> 3)) * bn + c * 32 + (lane & 7) * 4;
+              *reinterpret_cast<float4*>(stg + stg_at(lane, i >> 2)) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            __syncwarp();
 #pragma unroll
-          for (int r = 0; r < 32; r += 4)
-            __stcg(reinterpret_cast<float4*>(o + r * bn), *reinterpret_cast<const float4*>(stg + stg_at(r + (lane >> 3), lane & 7)));
-        } else if (e.vec && nb + 32 <= e.N) {                    // warp-uniform
-          switch (mode) {
-            case 0: store_chunk<0, true>(e, stg, m0, rows, nb, lane, mag); break;
-            case 1: store_chunk<1, true>(e, stg, m0, rows, nb, lane, mag); break;
-            case 2: store_chunk<2, true>(e, stg, m0, rows, nb, lane, mag); break;
-            case 3: store_chunk<3, true>(e, stg, m0, rows, nb, lane, mag); break;
-            default: store_chunk<4, true>(e, stg, m0, rows, nb, lane, mag); break;
+            for (int r = 0; r < 32; r += 4)
+              __stcg(reinterpret_cast<float4*>(o + r * bn + 64 * j), *reinterpret_cast<const float4*>(stg + stg_at(r + (lane >> 3), lane & 7)));
           }
         } else {
-          switch (mode) {
-            case 0: store_chunk<0, false>(e, stg, m0, rows, nb, lane, mag); break;
-            case 1: store_chunk<1, false>(e, stg, m0, rows, nb, lane, mag); break;
-            case 2: store_chunk<2, false>(e, stg, m0, rows, nb, lane, mag); break;
-            case 3: store_chunk<3, false>(e, stg, m0, rows, nb, lane, mag); break;
-            default: store_chunk<4, false>(e, stg, m0, rows, nb, lane, mag); break;
-          }
+          store_tile<MODE, VEC>(e, stg, ta, n_mine, m0, rows, nb0, lane, mag);
         }
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
     }
     if (e.amax_out) {
       mag = __reduce_max_sync(0xffffffffu, mag);
@@ -609,7 +622,7 @@ HPlan plan_f16x3(const GemmArgs& g) {
   for (int bn : widths) {
     if (bn > 32 && bn / 2 >= g.N) continue;                // a narrower tile covers N
     const long long tiles = tiles_m * ((g.N + bn - 1) / bn);
-    const double t_kb = 0.9 * (96 + bn) / 352.0, t_item = 2.0 + 4.0 * bn / 256.0;
+    const double t_kb = 0.9 * (96 + bn) / 352.0, t_item = 3.0 + 5.0 * bn / 256.0;
     const long long rounds = tiles / pairs, rem = tiles - rounds * pairs;
     const double t_whole = rounds * (kb * t_kb + t_item);
     const double t = t_whole + (rem ? kb * t_kb + t_item : 0.0);
@@ -630,7 +643,7 @@ HEpilogue make_epilogue(const GemmArgs& g, unsigned* amax_out) {
   e.dsig = g.dsig; e.ld_dsig = g.ld_dsig; e.dsig_rows = g.dsig_rows > 0 ? g.dsig_rows : 1; e.dsig_div = g.dsig_div > 0 ? g.dsig_div : 1;
   e.dsig_direct = e.dsig_div == 1 && e.dsig_rows >= g.M;
   e.alpha = g.alpha; e.cin = g.cin; e.ld_cin = g.ld_cin; e.beta = g.beta;
-  e.vec = aligned16(g.D) && g.ldd % 4 == 0 && (!g.bias || aligned16(g.bias)) && (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
+  e.vec = g.N % 4 == 0 && aligned16(g.D) && g.ldd % 4 == 0 && (!g.bias || aligned16(g.bias)) && (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
           (!g.cin || (aligned16(g.cin) && g.ld_cin % 4 == 0));
   e.amax_out = amax_out;
   return e;
@@ -638,14 +651,25 @@ HEpilogue make_epilogue(const GemmArgs& g, unsigned* amax_out) {
 
 }  // namespace
 
+namespace {
+typedef void (*HKernel)(const HMaps, const HParams);
+// [2 * mode + vec], see store_tile
+HKernel const kKernels[10] = {
+    gemm_f16x3_kernel<0, false>, gemm_f16x3_kernel<0, true>, gemm_f16x3_kernel<1, false>, gemm_f16x3_kernel<1, true>,
+    gemm_f16x3_kernel<2, false>, gemm_f16x3_kernel<2, true>, gemm_f16x3_kernel<3, false>, gemm_f16x3_kernel<3, true>,
+    gemm_f16x3_kernel<4, false>, gemm_f16x3_kernel<4, true>};
+}  // namespace
+
 // The register split of the kernel (128 x 56 + 256 x 224) must not exceed what the block is launched with, and the
 // kernel needs its dynamic shared memory granted: checked once.
 bool gemm_f16x3_usable() {
   static const bool usable = [] {
-    cudaFuncAttributes fa;
-    const bool ok = encode_fn() != nullptr && cudaFuncGetAttributes(&fa, gemm_f16x3_kernel) == cudaSuccess &&
-                    fa.numRegs * H_THREADS >= 128 * H_REGS_LOW + 256 * H_REGS_HIGH &&
-                    cudaFuncSetAttribute(gemm_f16x3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, H_SMEM_BYTES) == cudaSuccess;
+    bool ok = encode_fn() != nullptr;
+    for (HKernel k : kKernels) {
+      cudaFuncAttributes fa;
+      ok = ok && cudaFuncGetAttributes(&fa, k) == cudaSuccess && fa.numRegs * H_THREADS >= 128 * H_REGS_LOW + 256 * H_REGS_HIGH &&
+           cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, H_SMEM_BYTES) == cudaSuccess;
+    }
     cudaGetLastError();
     return ok;
   }();
@@ -698,7 +722,10 @@ int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, uns
   p.P = p.items < pairs ? p.items : pairs;
   p.ws = ws;
   p.err = err_flag;
-  if (launch_pdl(gemm_f16x3_kernel, 2 * p.P, H_THREADS, H_SMEM_BYTES, st, maps, p) != cudaSuccess) return -1;
+  // (left-over tiles' slices store raw sums: with no whole tile in the list every form of the kernel is the same)
+  const int n_opt = (p.e.sigmoid ? 1 : 0) + (p.e.dsig ? 1 : 0) + (p.e.cin ? 1 : 0);
+  const int mode = p.whole == 0 || n_opt == 0 ? 0 : n_opt > 1 ? 4 : p.e.sigmoid ? 1 : p.e.dsig ? 2 : 3;
+  if (launch_pdl(kKernels[2 * mode + (p.e.vec ? 1 : 0)], 2 * p.P, H_THREADS, H_SMEM_BYTES, st, maps, p) != cudaSuccess) return -1;
   if (p.rem == 0) return 1;
   const int gx = p.rem * (p.bn / 32);
   int gy = (148 * 8 + gx - 1) / gx;

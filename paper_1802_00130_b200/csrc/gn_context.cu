@@ -560,16 +560,21 @@ bool run_gemm_f16x3(gn_ctx* c, const GemmArgs& args) {
 }
 
 // Whether the tensor-core form is the faster way to FP32 accuracy.  The FP32 FMA GEMM walks K alone in 128 x 128
-// tiles, about 0.1 us per unit of K and round of tiles; the tensor-core form pays for splitting its operands
-// (two launches, about 5 us, and their bytes) before it starts.
+// tiles: about 10 us plus 0.12 us per unit of K and round of tiles (17 us at K = 37, 53 at 333).  The tensor-core form
+// pays for splitting its operands before it starts (two launches, about 8 us, and their bytes) and about 6 us of ramp.
 bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
   if (!c->x3_usable || !gemm_f16x3_usable()) return false;
   if (c->prec == GN_FP32_ACCURATE && c->acc_method == 1) return false;
   const double K = (double)g.K1 + (g.A2 ? g.K2 : 0);
   const double blocks = ((g.M + 127) / 128) * (double)((g.N + 127) / 128);
   const double rounds = blocks <= 148.0 ? 1.0 : blocks / 148.0;
-  const double fma_us = 3.0 + rounds * K * 0.1;
-  return gemm_f16x3_estimate_us(g) + 8.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5 < fma_us;
+  const double fma_us = 10.0 + rounds * K * 0.12;
+  return gemm_f16x3_estimate_us(g) + 14.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5 < fma_us;
+}
+
+// Whether run_gemm will send a contraction to that form.
+bool goes_f16x3(const gn_ctx* c, const GemmArgs& g) {
+  return gemm_thin_kind(g) == THIN_NONE && !(c->prec == GN_TF32 && gemm_tf32_eligible(g)) && wants_f16x3(c, g);
 }
 
 // Kernel choice: streaming kernels for the n_L-wide shapes (both precisions: they are exact FP32), the TF32
@@ -608,8 +613,7 @@ void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
   std::vector<SplitJob> jobs;
   for (int i = 0; i < n; ++i) {
     const GemmArgs& g = gs[i];
-    const bool tf32 = c->prec == GN_TF32 && gemm_tf32_eligible(g);
-    if (tf32 || gemm_thin_kind(g) != THIN_NONE || !wants_f16x3(c, g)) continue;
+    if (!goes_f16x3(c, g)) continue;
     if (ensure_split_scratch(c) != GN_OK) return;
     for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
       const OperandView v = operand_view(g, role);
@@ -760,7 +764,7 @@ const float* Wm(const gn_ctx* c, const float* vec, int m) { return vec + c->w_of
 const float* bm(const gn_ctx* c, const float* vec, int m) { return vec + c->b_off[m]; }
 
 // Eq. (xtoz): Zout[m] = sigma(Zout[m-1] W^m + 1 b^mT), m = 1..L, over `rows` rows; Zout[0] = Z0.
-void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout, bool emit_amax = false) {
+void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout) {
   std::vector<GemmArgs> gs((size_t)c->L);
   std::vector<int> dep((size_t)c->L), dep_all((size_t)c->L, 0);
   for (int m = 1; m <= c->L; ++m) {
@@ -772,9 +776,9 @@ void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>&
     g.D = Zout[m]; g.ldd = c->w[m];
     g.bias = bm(c, c->theta, m);
     g.sigmoid = m < c->L;
-    g.emit_amax = emit_amax && m < c->L;   // Z_m is an operand of layer m + 1 and of its weight block
     dep[(size_t)m - 1] = m - 2;          // layer m reads the rows layer m - 1 writes
   }
+  for (int m = 1; m < c->L; ++m) gs[(size_t)m - 1].emit_amax = goes_f16x3(c, gs[(size_t)m]);   // Z_m feeds layer m + 1
   presplit(c, gs.data(), c->L, 0x2);       // theta's weights
   run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), c->L);
 }
@@ -923,9 +927,9 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
       if (m < L) { g.dsig = c->Z[m]; g.ld_dsig = c->w[m]; g.dsig_rows = (int)nS; }
       else g.alpha = 2.f;                                   // B = 2I
       g.D = c->RZ[m]; g.ldd = c->w[m];
-      g.emit_amax = m < L;              // R z^m is an operand of layer m + 1
       dep[(size_t)m - 1] = m - 2;        // R z^{m-1} of the layer below
     }
+    for (int m = 1; m < L; ++m) gs[(size_t)m - 1].emit_amax = goes_f16x3(c, gs[(size_t)m]);   // R z^m feeds layer m + 1
     presplit(c, gs.data(), L, 0xf);
     run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), L, 2);
   }
@@ -1260,7 +1264,7 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
     const float* X0 = c->dX + r0 * c->w[0];
     c->cur_x = X0; c->cur_x_count = rows * c->w[0];
     ++c->parts_epoch;           // the batch buffers are rewritten
-    forward_pass(c, X0, rows, c->Zb, true);
+    forward_pass(c, X0, rows, c->Zb);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
                                      c->partial + b * per_batch, c->st);
     {
@@ -1601,7 +1605,7 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   GN_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->st));
   c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
   GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
-  forward_pass(c, c->Z[0], nS, c->Z, true);
+  forward_pass(c, c->Z[0], nS, c->Z);
   GN_TRY(check_launch(c, "set_subsample"));
   GN_TRY(sync(c, "set_subsample"));
   if (*c->h_err) return fail(c, GN_EINVAL, "a subsample index lies outside [0, l)");
