@@ -947,10 +947,18 @@ int choose_slices(int tiles, int total_kb, int pairs) {
 
 int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_flags, cudaStream_t st) {
   set_kernel_attributes();
-  const bool two_cta = g.two_cta >= 0 ? g.two_cta != 0 : suits_pair_kernel(g);
-  bool stream_k = two_cta && sk_ws && sk_flags;
   const int pairs = num_sms() / 2;
   const int total_kb_all = (g.K1 + BK - 1) / BK + (g.A2 ? (g.K2 + BK - 1) / BK : 0);
+  bool two_cta = g.two_cta >= 0 ? g.two_cta != 0 : suits_pair_kernel(g);
+  if (!two_cta && g.two_cta < 0 && sk_ws && sk_flags && g.M <= BM && g.N >= 128) {
+    // Up to 128 rows leave half of a pair's tile empty, but the pair kernel can cut a long K (the weight block of an
+    // output layer wider than the streaming kernels take) where the one-CTA kernel walks it alone on a few SMs, at about
+    // 0.5 us per k-block: 100 x 4096 x 32768 took 566 us there.  A slice costs 0.45 us per k-block and 16 us on top.
+    const int tiles = (g.N + 255) / 256;
+    const int sl = choose_slices(tiles, total_kb_all, pairs);
+    two_cta = sl >= 2 && tiles <= pairs && 0.45 * total_kb_all / sl + 16.0 < 0.5 * total_kb_all;
+  }
+  bool stream_k = two_cta && sk_ws && sk_flags;
   int bn = two_cta ? choose_bn2(g.M, g.N, stream_k) : choose_bn(g.M, g.N);
   if (stream_k) {
     // the width chosen for an even split of the work only stands if the left-over tiles will in fact be cut
