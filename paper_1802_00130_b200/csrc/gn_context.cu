@@ -121,6 +121,8 @@ struct gn_ctx {
   uint64_t parts_epoch = 1;
   bool amax_enabled = true;
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
+  float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
+  bool small_enabled = true;
   double* partial = nullptr; int64_t partial_cap = 0;
   double* dscal = nullptr;   // device: [0] loss, [1] theta^T theta, [2] cg sum rho, [3] cg active
   double* hscal = nullptr;   // pinned mirror
@@ -757,6 +759,39 @@ gn_status ensure_colsum(gn_ctx* c, int64_t rows, int cols) {
   return GN_OK;
 }
 
+// Whole passes of a small network in one launch (small_net.cu): the description for `rows` rows, and whether the pass
+// is to go that way.
+enum SmallKind { kSmallGv = 0, kSmallBlock = 1, kSmallGrad = 2, kSmallFun = 3, kSmallForward = 4 };
+bool small_pass(const gn_ctx* c, SmallKind kind, int64_t rows, SmallNet* a) {
+  if (!c->small_enabled || c->L > kSmallLayers || c->n > 60000) return false;
+  *a = SmallNet{};
+  a->L = c->L; a->n = (int)c->n; a->rows = rows;
+  for (int m = 0; m <= c->L; ++m) a->w[m] = c->w[m];
+  for (int m = 1; m <= c->L; ++m) { a->w_off[m] = (int)c->w_off[m]; a->b_off[m] = (int)c->b_off[m]; }
+  a->theta = c->theta;
+  return small_net_fits(*a, kind);
+}
+
+gn_status run_small_pass(gn_ctx* c, SmallKind kind, SmallNet& a, float alpha, const float* cin, float beta, float* out, double* loss_out) {
+  if (kind != kSmallForward) {
+    const int64_t blocks = small_net_blocks(a.rows);
+    const int64_t need = (blocks * 2 + 3) / 4 * 4 + blocks * a.n;            // the losses (doubles), then the sums
+    if (need > c->small_cap) {
+      quiesce(c);
+      dev_free(c, c->small_scratch);
+      c->small_cap = 0;
+      GN_TRY(dev_alloc(c, &c->small_scratch, need));
+      c->small_cap = need;
+    }
+    a.loss = reinterpret_cast<double*>(c->small_scratch);
+    a.scratch = c->small_scratch + (blocks * 2 + 3) / 4 * 4;
+  }
+  const int r = launch_small_net(a, kind, alpha, cin, beta, out, loss_out, c->st);
+  if (r < 0) return fail(c, GN_ECUDA, "the small network's pass could not be launched");
+  c->launches += r;
+  return GN_OK;
+}
+
 // First neuron of group g when a layer of n neurons is cut into `groups` contiguous groups.
 int group_lo(int n, int groups, int g) { return (int)(((long long)g * n) / groups); }
 
@@ -906,6 +941,13 @@ gn_status backward_hidden_layers(gn_ctx* c, int m_top, const float* ds_top, cons
 // out = coef v + (1/|S|) J^T (2 J v) over the stored subsample (Eq. sampled-Gauss).
 gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("G v");
+  SmallNet small;
+  if (small_pass(c, kSmallGv, c->nS, &small)) {
+    small.v = v;
+    for (int m = 0; m < c->L; ++m) small.z[m] = c->Z[m];
+    GN_TRY(run_small_pass(c, kSmallGv, small, (float)(1.0 / (double)c->nS), v, coef, out, nullptr));
+    return check_launch(c, "G v");
+  }
   SideJoin side_guard(c);
   CurrentVector current(c, v);
   ++c->parts_epoch;
@@ -1222,6 +1264,13 @@ constexpr int kFactorBreakEven = 8;
 gn_status product_blockdiag_any(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("block-diagonal G v");
   if (c->has_split) return product_split(c, v, out, coef);
+  SmallNet small;
+  if (c->bd_method != 2 && small_pass(c, kSmallBlock, c->nS, &small)) {
+    small.v = v;
+    for (int m = 0; m < c->L; ++m) small.z[m] = c->Z[m];
+    GN_TRY(run_small_pass(c, kSmallBlock, small, (float)(1.0 / (double)c->nS), v, coef, out, nullptr));
+    return check_launch(c, "block-diagonal G v");
+  }
   bool stored = c->bd_method == 2;
   if (c->bd_method == 0 && stored_factors_applicable(c))
     stored = c->factors_valid || c->bd_expect >= kFactorBreakEven || c->bd_count + 1 >= kFactorBreakEven;
@@ -1246,9 +1295,24 @@ gn_status ensure_batch(gn_ctx* c) {
   return GN_OK;
 }
 
+// f from the summed loss and theta^T theta on the device.
+gn_status read_loss(gn_ctx* c, double* f_host) {
+  GN_CUDA(c, cudaMemcpyAsync(c->hscal, c->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+  GN_TRY(check_launch(c, "f / grad"));
+  GN_TRY(sync(c, "f / grad"));
+  *f_host = c->hscal[1] / (2.0 * c->C) + c->hscal[0] / (double)c->l;
+  return GN_OK;
+}
+
 // f and (optionally) the gradient over all rows in row batches (Section 6.1 in its one-GPU form).
 gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
   GN_PHASE("f / gradient");
+  SmallNet small;
+  if (small_pass(c, d_grad ? kSmallGrad : kSmallFun, c->l, &small)) {
+    small.z[0] = c->dX; small.Y = c->dY; small.theta_sq = c->dscal + 1;
+    GN_TRY(run_small_pass(c, d_grad ? kSmallGrad : kSmallFun, small, (float)(1.0 / (double)c->l), c->theta, (float)(1.0 / c->C), d_grad, c->dscal));
+    return f_host ? read_loss(c, f_host) : check_launch(c, "grad");
+  }
   GN_TRY(ensure_batch(c));
   const int L = c->L;
   const int64_t Rb = c->capB;
@@ -1300,11 +1364,7 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
     double* tp = c->partial + per_batch * nb;
     c->launches += launch_cg_dot(c->theta, c->theta, c->chunks[0], c->n_chunks[0], tp, nullptr, 0, nullptr, c->st);
     c->launches += launch_sum_partials(tp, c->n_chunks[0], c->dscal + 1, false, c->st);
-    GN_CUDA(c, cudaMemcpyAsync(c->hscal, c->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
-    GN_TRY(check_launch(c, "f / grad"));
-    GN_TRY(sync(c, "f / grad"));
-    *f_host = c->hscal[1] / (2.0 * c->C) + c->hscal[0] / (double)c->l;
-    return GN_OK;
+    return read_loss(c, f_host);
   }
   return check_launch(c, "grad");
 }
@@ -1603,9 +1663,17 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   c->nS = nS;
   GN_CUDA(c, cudaMemcpyAsync(c->idx, idx, nS * sizeof(int32_t), kind, c->st));
   GN_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->st));
-  c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
-  GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
-  forward_pass(c, c->Z[0], nS, c->Z);
+  SmallNet small;
+  if (small_pass(c, kSmallForward, nS, &small)) {
+    small.z[0] = c->dX; small.idx = c->idx; small.x_rows = c->l; small.err_flag = c->err_flag;
+    for (int m = 0; m <= c->L; ++m) small.z_out[m] = c->Z[m];
+    GN_TRY(run_small_pass(c, kSmallForward, small, 0.f, nullptr, 0.f, nullptr, nullptr));
+    GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+  } else {
+    c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
+    GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+    forward_pass(c, c->Z[0], nS, c->Z);
+  }
   GN_TRY(check_launch(c, "set_subsample"));
   GN_TRY(sync(c, "set_subsample"));
   if (*c->h_err) return fail(c, GN_EINVAL, "a subsample index lies outside [0, l)");
@@ -1964,6 +2032,7 @@ gn_status gn_debug_option(gn_ctx* c, int option, int value) {
   if (option == 3) { quiesce(c); c->side_enabled = value != 0; return GN_OK; }
   if (option == 7) { c->split_k_enabled = value != 0; return GN_OK; }
   if (option == 8) { c->back_chain = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }
+  if (option == 10) { c->small_enabled = value != 0; return GN_OK; }
   if (option == 9) { c->fly_enabled = value != 0; return GN_OK; }
   if (option == 6) { c->graph_enabled = value != 0; return GN_OK; }
   if (option == 5) { c->amax_enabled = value != 0; return GN_OK; }

@@ -96,6 +96,27 @@ int64_t gemm_f16x3_workspace_floats(const GemmArgs& g);
 int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, unsigned* amax_out, int* err_flag, cudaStream_t st);
 int launch_split_f16(const SplitJob* jobs, int n, unsigned* part, cudaStream_t st);
 
+// Whole passes of a small network (small_net.cu).  kind 0: G^S v, 1: block-diagonal G^S v, 2: loss and gradient, 3: loss,
+// 4: row gather and stored forward pass.  The blocks' sums go to scratch (small_net_blocks(rows) * n floats) and their losses to
+// loss (one double per block); launch_small_net then writes out = alpha * sum + beta * cin and *loss_out.  theta_sq (kinds 2, 3)
+// receives theta^T theta.  Returns launches made, or -1 if a launch failed.
+constexpr int kSmallLayers = 8;
+constexpr double kSmallUs = 40.0;       // estimated time up to which a pass goes this way (see small_net_fits)
+struct SmallNet {
+  int L, n;
+  int w[kSmallLayers + 1], w_off[kSmallLayers + 1], b_off[kSmallLayers + 1];
+  int64_t rows;
+  const float* theta; const float* v;
+  const float* z[kSmallLayers];         // z^0 .. z^{L-1} of the subsample (kinds 0, 1), or z[0] = X (2, 3, 4)
+  float* z_out[kSmallLayers + 1];       // kind 4: where the gathered rows and z^1 .. z^L go
+  const int32_t* idx; int64_t x_rows; int* err_flag;   // kind 4
+  const float* Y;
+  float* scratch; double* loss; double* theta_sq;
+};
+int64_t small_net_blocks(int64_t rows);
+bool small_net_fits(const SmallNet& a, int kind);
+int launch_small_net(const SmallNet& a, int kind, float alpha, const float* cin, float beta, float* out, double* loss_out, cudaStream_t st);
+
 // Streaming FP32 kernels for contractions with one dimension <= 16 (the n_L-wide output layer).
 // gemm_thin_kind says which of them (if any) takes a problem; THIN_M needs a scratch buffer of
 // gemm_thin_scratch_floats(g) floats.  launch_gemm_thin returns the launches made (0 = not taken).
