@@ -6,6 +6,7 @@
 // 128 x 128 x 16 tiles, 256 threads, 8 x 8 accumulators per thread, double-buffered shared memory
 // with the next tile's global loads in flight during the current tile's arithmetic.
 #include "gn_kernels.h"
+#include "tc_common.cuh"
 
 namespace gn {
 namespace {
@@ -43,6 +44,8 @@ __device__ __forceinline__ float4 load4(const float* __restrict__ base, long lon
 
 template <bool A_KMAJOR, bool B_KMAJOR>
 __global__ void __launch_bounds__(NT, 2) gemm_ffma_kernel(const FfmaParams p) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ __align__(16) float As[2][BK][BM + PAD];
   __shared__ __align__(16) float Bs[2][BK][BN + PAD];
 
@@ -65,8 +68,8 @@ __global__ void __launch_bounds__(NT, 2) gemm_ffma_kernel(const FfmaParams p) {
   auto fetch = [&](int kt) {
     const int s = kt < nk0 ? 0 : 1;
     const int k0 = (s == 0 ? kt : kt - nk0) * BK;
-    const float* A = p.A[s];
-    const float* B = p.B[s];
+    const float* A = dep(p.A[s]);
+    const float* B = dep(p.B[s]);
     const int K = p.K[s];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -171,7 +174,6 @@ __global__ void __launch_bounds__(NT, 2) gemm_ffma_kernel(const FfmaParams p) {
   }
 }
 
-inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
 
@@ -194,10 +196,10 @@ int launch_gemm_ffma(const GemmArgs& g, cudaStream_t st) {
               (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
               (!g.cin || (aligned16(g.cin) && g.ld_cin % 4 == 0));
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-  if (g.a_kmajor && g.b_kmajor)        gemm_ffma_kernel<true, true><<<grid, NT, 0, st>>>(p);
-  else if (g.a_kmajor && !g.b_kmajor)  gemm_ffma_kernel<true, false><<<grid, NT, 0, st>>>(p);
-  else if (!g.a_kmajor && g.b_kmajor)  gemm_ffma_kernel<false, true><<<grid, NT, 0, st>>>(p);
-  else                                 gemm_ffma_kernel<false, false><<<grid, NT, 0, st>>>(p);
+  if (g.a_kmajor && g.b_kmajor)        launch_pdl_grid(gemm_ffma_kernel<true, true>, dim3(grid), NT, 0, st, p);
+  else if (g.a_kmajor && !g.b_kmajor)  launch_pdl_grid(gemm_ffma_kernel<true, false>, dim3(grid), NT, 0, st, p);
+  else if (!g.a_kmajor && g.b_kmajor)  launch_pdl_grid(gemm_ffma_kernel<false, true>, dim3(grid), NT, 0, st, p);
+  else                                 launch_pdl_grid(gemm_ffma_kernel<false, false>, dim3(grid), NT, 0, st, p);
   return 1;
 }
 

@@ -10,11 +10,11 @@
 
 #include "../../include/gn.h"
 #include "gn_kernels.h"
+#include "tc_common.cuh"
 
 namespace gn {
 namespace {
 
-inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 struct Epi {
   float* D; long long ldd;
@@ -59,6 +59,8 @@ struct ThinNParams {
 
 template <int NMAX>
 __global__ void __launch_bounds__(128, 3) gemm_thin_n_kernel(const ThinNParams p) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int lane = threadIdx.x & 31;
   const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int m0 = warp * TR;
@@ -70,8 +72,8 @@ __global__ void __launch_bounds__(128, 3) gemm_thin_n_kernel(const ThinNParams p
     for (int n = 0; n < NMAX; ++n) acc[r][n] = 0.f;
 
   for (int s = 0; s < 2; ++s) {
-    const float* __restrict__ A = p.A[s];
-    const float* __restrict__ B = p.B[s];
+    const float* __restrict__ A = dep(p.A[s]);
+    const float* __restrict__ B = dep(p.B[s]);
     if (!A) continue;
     const int K = p.K[s];
     const float* arow[TR];
@@ -134,12 +136,16 @@ struct ThinMParams {
 
 template <int MMAX>
 __global__ void __launch_bounds__(256) gemm_thin_m_partial_kernel(const ThinMParams p) {
+  grid_dep_wait();
+  grid_dep_launch();
   // 256 threads = 2 row-halves x 128 column threads: half h takes rows h, h + 2, ... of the chunk, so
   // that twice as many 16-byte loads of B are in flight; the halves are added at the end.
   __shared__ __align__(16) float As[TM_ROWS][MMAX];    // (MMAX is a multiple of 4: a row is read back as 16-byte groups)
   __shared__ float4 Hs[MMAX][128];
   const int ct = threadIdx.x & 127, half = threadIdx.x >> 7;
   const int n = (blockIdx.x * 128 + ct) * 4;
+  const float* const pA = dep(p.A);
+  const float* const pB = dep(p.B);
   const long long r_begin = (long long)blockIdx.y * p.chunk_rows;
   const long long r_end = min(p.rows, r_begin + p.chunk_rows);
   float4 acc[MMAX];
@@ -150,13 +156,13 @@ __global__ void __launch_bounds__(256) gemm_thin_m_partial_kernel(const ThinMPar
     __syncthreads();
     for (int i = threadIdx.x; i < cnt * MMAX; i += 256) {
       const int r = i / MMAX, m = i % MMAX;
-      As[r][m] = m < p.M ? __ldg(p.A + (rb + r) * p.lda + m) : 0.f;
+      As[r][m] = m < p.M ? __ldg(pA + (rb + r) * p.lda + m) : 0.f;
     }
     __syncthreads();
     if (n < p.N) {
 #pragma unroll 8
       for (int r = half; r < cnt; r += 2) {
-        const float4 b = __ldg(reinterpret_cast<const float4*>(p.B + (rb + r) * p.ldb + n));
+        const float4 b = __ldg(reinterpret_cast<const float4*>(pB + (rb + r) * p.ldb + n));
 #pragma unroll
         for (int m4 = 0; m4 < MMAX / 4; ++m4) {
           const float4 a4 = *reinterpret_cast<const float4*>(&As[r][4 * m4]);   // one shared-memory read per four rows of A
@@ -191,7 +197,10 @@ __global__ void __launch_bounds__(256) gemm_thin_m_partial_kernel(const ThinMPar
 // and the eight warp sums are added in warp order: a fixed order, and eight short chains instead of one long one.
 __global__ void __launch_bounds__(256) gemm_thin_m_final_kernel(const float* __restrict__ scratch, int chunks, int M, int N,
                                                                 const Epi e) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ float sh[8][33];
+  scratch = dep(scratch);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long total = (long long)M * N;
   const long long i = (long long)blockIdx.x * 32 + lane;
@@ -222,6 +231,8 @@ struct ThinKParams {
 
 template <int KMAX>
 __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p) {
+  grid_dep_wait();
+  grid_dep_launch();
   // Rows are taken 64 at a time: their A values are staged in shared memory, then groups of 8 rows
   // first issue all their reads of the sigma' operand and only then compute and store, so
   // that 8 independent 16-byte loads per thread are in flight (a store between two loads would
@@ -230,10 +241,12 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
   __shared__ __align__(16) float As[RB][KMAX];         // (KMAX is a multiple of 4: a row is read back as 16-byte groups)
   const int n = (blockIdx.x * 128 + threadIdx.x) * 4;
   const bool n_ok = n < p.N;
+  const float* const pA = dep(p.A);
+  const float* const pB = dep(p.B);
   float4 b[KMAX];
 #pragma unroll
   for (int k = 0; k < KMAX; ++k)
-    b[k] = (n_ok && k < p.K) ? __ldg(reinterpret_cast<const float4*>(p.B + (long long)k * p.ldb + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    b[k] = (n_ok && k < p.K) ? __ldg(reinterpret_cast<const float4*>(pB + (long long)k * p.ldb + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
   float4 bz = make_float4(0.f, 0.f, 0.f, 0.f);
   if (p.e.bias && n_ok) bz = __ldg(reinterpret_cast<const float4*>(p.e.bias + n));
   const int m_begin = blockIdx.y * p.rows_per_block;
@@ -243,7 +256,7 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
     __syncthreads();
     for (int i = threadIdx.x; i < cnt * KMAX; i += 128) {
       const int r = i / KMAX, k = i % KMAX;
-      As[r][k] = k < p.K ? __ldg(p.A + (long long)(mb + r) * p.lda + k) : 0.f;
+      As[r][k] = k < p.K ? __ldg(pA + (long long)(mb + r) * p.lda + k) : 0.f;
     }
     __syncthreads();
     if (!n_ok) continue;
@@ -337,10 +350,10 @@ int launch_gemm_thin(const GemmArgs& g, float* scratch, cudaStream_t st) {
     p.e = make_epi(g);
     const int warps = (g.M + TR - 1) / TR;
     const int grid = (warps + 3) / 4;
-    if (g.N <= 4) gemm_thin_n_kernel<4><<<grid, 128, 0, st>>>(p);
-    else if (g.N <= 8) gemm_thin_n_kernel<8><<<grid, 128, 0, st>>>(p);
-    else if (g.N <= 12) gemm_thin_n_kernel<12><<<grid, 128, 0, st>>>(p);
-    else gemm_thin_n_kernel<16><<<grid, 128, 0, st>>>(p);
+    if (g.N <= 4) launch_pdl_grid(gemm_thin_n_kernel<4>, dim3(grid), 128, 0, st, p);
+    else if (g.N <= 8) launch_pdl_grid(gemm_thin_n_kernel<8>, dim3(grid), 128, 0, st, p);
+    else if (g.N <= 12) launch_pdl_grid(gemm_thin_n_kernel<12>, dim3(grid), 128, 0, st, p);
+    else launch_pdl_grid(gemm_thin_n_kernel<16>, dim3(grid), 128, 0, st, p);
     return 1;
   }
   if (kind == THIN_M) {
@@ -351,12 +364,12 @@ int launch_gemm_thin(const GemmArgs& g, float* scratch, cudaStream_t st) {
     const int used = (int)((g.K1 + p.chunk_rows - 1) / p.chunk_rows);
     p.A = g.A1; p.lda = g.lda1; p.B = g.B1; p.ldb = g.ldb1; p.scratch = scratch;
     dim3 grid((g.N + 511) / 512, used);
-    if (g.M <= 4) gemm_thin_m_partial_kernel<4><<<grid, 256, 0, st>>>(p);
-    else if (g.M <= 8) gemm_thin_m_partial_kernel<8><<<grid, 256, 0, st>>>(p);
-    else if (g.M <= 12) gemm_thin_m_partial_kernel<12><<<grid, 256, 0, st>>>(p);
-    else gemm_thin_m_partial_kernel<16><<<grid, 256, 0, st>>>(p);
+    if (g.M <= 4) launch_pdl_grid(gemm_thin_m_partial_kernel<4>, dim3(grid), 256, 0, st, p);
+    else if (g.M <= 8) launch_pdl_grid(gemm_thin_m_partial_kernel<8>, dim3(grid), 256, 0, st, p);
+    else if (g.M <= 12) launch_pdl_grid(gemm_thin_m_partial_kernel<12>, dim3(grid), 256, 0, st, p);
+    else launch_pdl_grid(gemm_thin_m_partial_kernel<16>, dim3(grid), 256, 0, st, p);
     const long long total = (long long)g.M * g.N;
-    gemm_thin_m_final_kernel<<<(unsigned)((total + 31) / 32), 256, 0, st>>>(scratch, used, g.M, g.N, make_epi(g));
+    launch_pdl_grid(gemm_thin_m_final_kernel, dim3((unsigned)((total + 31) / 32)), 256, 0, st, scratch, used, g.M, g.N, make_epi(g));
     return 2;
   }
   if (kind == THIN_K) {
@@ -368,10 +381,10 @@ int launch_gemm_thin(const GemmArgs& g, float* scratch, cudaStream_t st) {
     if (row_blocks > g.M) row_blocks = g.M;
     p.rows_per_block = (g.M + row_blocks - 1) / row_blocks;
     dim3 grid(col_tiles, (g.M + p.rows_per_block - 1) / p.rows_per_block);
-    if (g.K1 <= 4) gemm_thin_k_kernel<4><<<grid, 128, 0, st>>>(p);
-    else if (g.K1 <= 8) gemm_thin_k_kernel<8><<<grid, 128, 0, st>>>(p);
-    else if (g.K1 <= 12) gemm_thin_k_kernel<12><<<grid, 128, 0, st>>>(p);
-    else gemm_thin_k_kernel<16><<<grid, 128, 0, st>>>(p);
+    if (g.K1 <= 4) launch_pdl_grid(gemm_thin_k_kernel<4>, dim3(grid), 128, 0, st, p);
+    else if (g.K1 <= 8) launch_pdl_grid(gemm_thin_k_kernel<8>, dim3(grid), 128, 0, st, p);
+    else if (g.K1 <= 12) launch_pdl_grid(gemm_thin_k_kernel<12>, dim3(grid), 128, 0, st, p);
+    else launch_pdl_grid(gemm_thin_k_kernel<16>, dim3(grid), 128, 0, st, p);
     return 1;
   }
   return 0;

@@ -27,6 +27,12 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 // after this one do the same.  Without the attribute both are no-ops.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A pointer as it is after the wait: the compiler must not move a read-only load through it above the wait.
+template <class T>
+__device__ __forceinline__ T* dep(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));

@@ -6,6 +6,7 @@
 #include <initializer_list>
 
 #include "gn_kernels.h"
+#include "tc_common.cuh"
 
 namespace gn {
 namespace {
@@ -42,6 +43,9 @@ __device__ __forceinline__ double block_sum_256(double v) {
 __global__ void __launch_bounds__(256) gather_rows_kernel(const float* __restrict__ src, long long src_rows, int cols,
                                                           const int32_t* __restrict__ idx, long long n_idx,
                                                           float* __restrict__ dst, int* err_flag, int vec) {
+  grid_dep_wait();
+  grid_dep_launch();
+  src = dep(src); idx = dep(idx); dst = dep(dst); err_flag = dep(err_flag);
   const int lane = threadIdx.x & 31;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_idx; r += warps) {
@@ -66,6 +70,9 @@ constexpr int CS_ROWS = 256;  // rows per block
 // Scalar version (any alignment): grid (ceil(cols/32), ceil(rows/CS_ROWS)); 8 warps stride rows.
 __global__ void __launch_bounds__(256) colsum_partial_kernel(const float* __restrict__ A, long long rows, int cols,
                                                              long long lda, float* __restrict__ scratch) {
+  grid_dep_wait();
+  grid_dep_launch();
+  A = dep(A); scratch = dep(scratch);
   __shared__ float sh[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
@@ -89,6 +96,9 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const float* __rest
 // beside a CTA of the tensor-core kernel (320 threads x 168 registers): the sums run on a side stream under it.
 __global__ void __launch_bounds__(256, 6) colsum_partial_vec_kernel(const float* __restrict__ A, long long rows, int cols,
                                                                  long long lda, float* __restrict__ scratch) {
+  grid_dep_wait();
+  grid_dep_launch();
+  A = dep(A); scratch = dep(scratch);
   __shared__ float4 sh[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = (blockIdx.x * 32 + lane) * 4;
@@ -127,6 +137,9 @@ __global__ void __launch_bounds__(256, 6) colsum_partial_vec_kernel(const float*
 __global__ void __launch_bounds__(256) colsum_final_kernel(const float* __restrict__ scratch, int n_parts, int cols,
                                                            float alpha, const float* __restrict__ cin, float beta,
                                                            float* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
+  scratch = dep(scratch); cin = dep(cin); out = dep(out);
   __shared__ double sh[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
@@ -151,6 +164,9 @@ constexpr int LOSS_PER_BLOCK = 256 * 8;
 __global__ void __launch_bounds__(256) loss_delta_kernel(const float* __restrict__ Z, const float* __restrict__ Y,
                                                          long long count, float* __restrict__ delta,
                                                          double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
+  Z = dep(Z); Y = dep(Y); delta = dep(delta); partial = dep(partial);
   const long long base = (long long)blockIdx.x * LOSS_PER_BLOCK;
   float s = 0.f;
 #pragma unroll
@@ -168,6 +184,9 @@ __global__ void __launch_bounds__(256) loss_delta_kernel(const float* __restrict
 
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partial, int count,
                                                            double* out, int accumulate) {
+  grid_dep_wait();
+  grid_dep_launch();
+  partial = dep(partial); out = dep(out);
   double s = 0.0;
   for (int i = threadIdx.x; i < count; i += 256) s += partial[i];
   const double t = block_sum_256(s);
@@ -177,6 +196,9 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 // ---------------------------------------------------------------------------------- out = a x + b y
 __global__ void __launch_bounds__(256) axpby_kernel(long long n, float a, const float* x, float b, const float* y,
                                                     float* out) {
+  grid_dep_wait();
+  grid_dep_launch();
+  x = dep(x); y = dep(y); out = dep(out);
   // out may be x or y (same index read and written by the same thread)
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
     out[i] = fmaf(a, x[i], b * y[i]);
@@ -186,6 +208,9 @@ __global__ void __launch_bounds__(256) axpby_kernel(long long n, float a, const 
 // D[(i, u)][t] = WL[u][t] * z (1 - z): one block per sample row i, threads over t (16-byte accesses when n % 4 == 0).
 __global__ void __launch_bounds__(256) factor_last_kernel(const float* __restrict__ WL, const float* __restrict__ Zprev,
                                                           int nL, int n, float* __restrict__ D) {
+  grid_dep_wait();
+  grid_dep_launch();
+  WL = dep(WL); Zprev = dep(Zprev); D = dep(D);
   const long long i = blockIdx.x;
   const float* z = Zprev + i * n;
   float* d = D + i * nL * n;
@@ -205,6 +230,9 @@ template <int NLMAX>
 __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restrict__ D, const float* __restrict__ U,
                                                            int nL, int n, int groups, int streams, long long stream_stride,
                                                            float* __restrict__ Q) {
+  grid_dep_wait();
+  grid_dep_launch();
+  D = dep(D); U = dep(U); Q = dep(Q);
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
@@ -355,6 +383,9 @@ __global__ void __launch_bounds__(256) cg_init_kernel(const float* __restrict__ 
                                                       float* __restrict__ r, float* __restrict__ p,
                                                       const CgChunk* __restrict__ chunks, double* __restrict__ partial,
                                                       CgSeg* seg, int n_seg, double tol, CgControl* ctl, int vec_ok) {
+  grid_dep_wait();
+  grid_dep_launch();
+  g = dep(g); d = dep(d); r = dep(r); p = dep(p); chunks = dep(chunks); partial = dep(partial); seg = dep(seg); ctl = dep(ctl);
   const CgChunk ch = chunks[blockIdx.x];
   float s = 0.f;
   int t0;
@@ -380,6 +411,9 @@ __global__ void __launch_bounds__(256) cg_init_kernel(const float* __restrict__ 
 __global__ void __launch_bounds__(256) cg_dot_kernel(const float* __restrict__ x, const float* __restrict__ y,
                                                      const CgChunk* __restrict__ chunks, double* __restrict__ partial,
                                                      CgSeg* seg, int n_seg, CgControl* ctl, int vec_ok) {
+  grid_dep_wait();
+  grid_dep_launch();
+  x = dep(x); y = dep(y); chunks = dep(chunks); partial = dep(partial); seg = dep(seg); ctl = dep(ctl);
   const CgChunk ch = chunks[blockIdx.x];
   float s = 0.f;
   int t0;
@@ -406,6 +440,9 @@ __global__ void __launch_bounds__(256) cg_update_kernel(const float* __restrict_
                                                         const CgChunk* __restrict__ chunks, CgSeg* seg, int n_seg,
                                                         double tol, double* __restrict__ partial, CgControl* ctl,
                                                         int vec_ok) {
+  grid_dep_wait();
+  grid_dep_launch();
+  p = dep(p); q = dep(q); d = dep(d); r = dep(r); chunks = dep(chunks); seg = dep(seg); partial = dep(partial); ctl = dep(ctl);
   const CgChunk ch = chunks[blockIdx.x];
   const float alpha = seg[ch.seg].alpha;
   const bool live = seg[ch.seg].active != 0;
@@ -441,6 +478,9 @@ __global__ void __launch_bounds__(256) cg_update_kernel(const float* __restrict_
 __global__ void __launch_bounds__(256) cg_direction_kernel(const float* __restrict__ r, float* __restrict__ p,
                                                            const CgChunk* __restrict__ chunks,
                                                            const CgSeg* __restrict__ seg, int vec_ok) {
+  grid_dep_wait();
+  grid_dep_launch();
+  r = dep(r); p = dep(p); chunks = dep(chunks); seg = dep(seg);
   const CgChunk ch = chunks[blockIdx.x];
   if (seg[ch.seg].beta == 0.f && seg[ch.seg].active == 0 && seg[ch.seg].alpha == 0.f) return;  // frozen before this step
   const float beta = seg[ch.seg].beta;
@@ -466,7 +506,7 @@ int launch_gather_rows(const float* src, int64_t src_rows, int cols, const int32
                   ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
   const long long blocks = (n_idx + 7) / 8;
   const int grid = (int)(blocks < 148LL * 16 ? blocks : 148LL * 16);
-  gather_rows_kernel<<<grid, 256, 0, st>>>(src, src_rows, cols, idx, n_idx, dst, err_flag, vec);
+  launch_pdl_grid(gather_rows_kernel, dim3(grid), 256, 0, st, src, src_rows, cols, idx, n_idx, dst, err_flag, vec);
   return 1;
 }
 
@@ -481,12 +521,12 @@ int launch_colsum(const float* A, int64_t rows, int cols, int64_t lda, float alp
                    ((reinterpret_cast<uintptr_t>(scratch) & 15) == 0);
   if (vec) {
     dim3 grid((cols + 127) / 128, parts);
-    colsum_partial_vec_kernel<<<grid, 256, 0, st>>>(A, rows, cols, lda, scratch);
+    launch_pdl_grid(colsum_partial_vec_kernel, dim3(grid), 256, 0, st, A, rows, cols, lda, scratch);
   } else {
     dim3 grid((cols + 31) / 32, parts);
-    colsum_partial_kernel<<<grid, 256, 0, st>>>(A, rows, cols, lda, scratch);
+    launch_pdl_grid(colsum_partial_kernel, dim3(grid), 256, 0, st, A, rows, cols, lda, scratch);
   }
-  colsum_final_kernel<<<(cols + 31) / 32, 256, 0, st>>>(scratch, parts, cols, alpha, cin, beta, out);
+  launch_pdl_grid(colsum_final_kernel, dim3((cols + 31) / 32), 256, 0, st, scratch, parts, cols, alpha, cin, beta, out);
   return 2;
 }
 
@@ -494,12 +534,12 @@ int loss_num_partials(int64_t count) { return (int)((count + LOSS_PER_BLOCK - 1)
 
 int launch_loss_delta(const float* Z, const float* Y, int64_t count, float* delta, double* partial,
                       cudaStream_t st) {
-  loss_delta_kernel<<<loss_num_partials(count), 256, 0, st>>>(Z, Y, count, delta, partial);
+  launch_pdl_grid(loss_delta_kernel, dim3(loss_num_partials(count)), 256, 0, st, Z, Y, count, delta, partial);
   return 1;
 }
 
 int launch_sum_partials(const double* partial, int count, double* out, bool accumulate, cudaStream_t st) {
-  sum_partials_kernel<<<1, 256, 0, st>>>(partial, count, out, accumulate ? 1 : 0);
+  launch_pdl_grid(sum_partials_kernel, dim3(1), 256, 0, st, partial, count, out, accumulate ? 1 : 0);
   return 1;
 }
 
@@ -514,6 +554,9 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
                                                                int nL, int n, int groups, int streams,
                                                                long long stream_stride, float* __restrict__ Q,
                                                                const float* __restrict__ WL, const float* __restrict__ Zprev) {
+  grid_dep_wait();
+  grid_dep_launch();
+  D = dep(D); U = dep(U); Q = dep(Q); WL = dep(WL); Zprev = dep(Zprev);
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
@@ -588,7 +631,7 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
 }
 
 int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL, int n, float* D, cudaStream_t st) {
-  factor_last_kernel<<<(unsigned)rows, 256, 0, st>>>(WL, Zprev, nL, n, D);
+  launch_pdl_grid(factor_last_kernel, dim3((unsigned)rows), 256, 0, st, WL, Zprev, nL, n, D);
   return 1;
 }
 
@@ -604,17 +647,17 @@ int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, in
   }
   const dim3 grid((unsigned)rows, (unsigned)groups);
   const long long ss = stream_stride;
-#define GN_FA_REG(NL, STR) { factor_apply_reg_kernel<NL, STR, false><<<grid, 256, 0, st>>>(D, U, nL, n, groups, streams, ss, Q, nullptr, nullptr); return 1; }
+#define GN_FA_REG(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, nullptr, nullptr); return 1; }
   if (vec && widest <= 1024 && nL <= 4)  GN_FA_REG(4, 1)
   if (vec && widest <= 1024 && nL <= 10) GN_FA_REG(10, 1)
   if (vec && widest <= 2048 && nL <= 4)  GN_FA_REG(4, 2)
   if (vec && widest <= 2048 && nL <= 10) GN_FA_REG(10, 2)
   if (vec && widest <= 1024 && nL <= 16) GN_FA_REG(16, 1)
 #undef GN_FA_REG
-  if (nL <= 4) factor_apply_kernel<4><<<grid, 256, 0, st>>>(D, U, nL, n, groups, streams, ss, Q);
-  else if (nL <= 10) factor_apply_kernel<10><<<grid, 256, 0, st>>>(D, U, nL, n, groups, streams, ss, Q);
-  else if (nL <= 16) factor_apply_kernel<16><<<grid, 256, 0, st>>>(D, U, nL, n, groups, streams, ss, Q);
-  else factor_apply_kernel<32><<<grid, 256, 0, st>>>(D, U, nL, n, groups, streams, ss, Q);
+  if (nL <= 4) launch_pdl_grid(factor_apply_kernel<4>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
+  else if (nL <= 10) launch_pdl_grid(factor_apply_kernel<10>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
+  else if (nL <= 16) launch_pdl_grid(factor_apply_kernel<16>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
+  else launch_pdl_grid(factor_apply_kernel<32>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
   return 1;
 }
 
@@ -626,7 +669,7 @@ int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U
                    ((reinterpret_cast<uintptr_t>(U) & 15) == 0) && ((reinterpret_cast<uintptr_t>(Q) & 15) == 0);
   if (!vec) return 0;
   const dim3 grid((unsigned)rows, 1);
-#define GN_FA_FLY(NL, STR) { factor_apply_reg_kernel<NL, STR, true><<<grid, 256, 0, st>>>(nullptr, U, nL, n, 1, 1, 0, Q, WL, Zprev); return 1; }
+#define GN_FA_FLY(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR, true>, dim3(grid), 256, 0, st, nullptr, U, nL, n, 1, 1, 0, Q, WL, Zprev); return 1; }
   if (n <= 1024 && nL <= 4)  GN_FA_FLY(4, 1)
   if (n <= 1024 && nL <= 10) GN_FA_FLY(10, 1)
   if (n <= 2048 && nL <= 4)  GN_FA_FLY(4, 2)
@@ -639,7 +682,7 @@ int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U
 int launch_axpby(int64_t n, float a, const float* x, float b, const float* y, float* out, cudaStream_t st) {
   long long blocks = (n + 255) / 256;
   if (blocks > 148LL * 16) blocks = 148LL * 16;
-  axpby_kernel<<<(unsigned)blocks, 256, 0, st>>>(n, a, x, b, y, out);
+  launch_pdl_grid(axpby_kernel, dim3((unsigned)blocks), 256, 0, st, n, a, x, b, y, out);
   return 1;
 }
 
@@ -653,22 +696,22 @@ inline int all_aligned16(std::initializer_list<const void*> ps) {
 
 int launch_cg_init(const float* g, float* d, float* r, float* p, const CgChunk* chunks, int n_chunks,
                    double* partial, CgSeg* seg, int n_seg, double tol, CgControl* ctl, cudaStream_t st) {
-  cg_init_kernel<<<n_chunks, 256, 0, st>>>(g, d, r, p, chunks, partial, seg, n_seg, tol, ctl, all_aligned16({g, d, r, p}));
+  launch_pdl_grid(cg_init_kernel, dim3(n_chunks), 256, 0, st, g, d, r, p, chunks, partial, seg, n_seg, tol, ctl, all_aligned16({g, d, r, p}));
   return 1;
 }
 int launch_cg_dot(const float* p, const float* q, const CgChunk* chunks, int n_chunks, double* partial,
                   CgSeg* seg, int n_seg, CgControl* ctl, cudaStream_t st) {
-  cg_dot_kernel<<<n_chunks, 256, 0, st>>>(p, q, chunks, partial, seg, n_seg, ctl, all_aligned16({p, q}));
+  launch_pdl_grid(cg_dot_kernel, dim3(n_chunks), 256, 0, st, p, q, chunks, partial, seg, n_seg, ctl, all_aligned16({p, q}));
   return 1;
 }
 int launch_cg_update(const float* p, const float* q, float* d, float* r, const CgChunk* chunks,
                      int n_chunks, CgSeg* seg, int n_seg, double tol, double* partial, CgControl* ctl, cudaStream_t st) {
-  cg_update_kernel<<<n_chunks, 256, 0, st>>>(p, q, d, r, chunks, seg, n_seg, tol, partial, ctl, all_aligned16({p, q, d, r}));
+  launch_pdl_grid(cg_update_kernel, dim3(n_chunks), 256, 0, st, p, q, d, r, chunks, seg, n_seg, tol, partial, ctl, all_aligned16({p, q, d, r}));
   return 1;
 }
 int launch_cg_direction(const float* r, float* p, const CgChunk* chunks, int n_chunks, const CgSeg* seg,
                         cudaStream_t st) {
-  cg_direction_kernel<<<n_chunks, 256, 0, st>>>(r, p, chunks, seg, all_aligned16({r, p}));
+  launch_pdl_grid(cg_direction_kernel, dim3(n_chunks), 256, 0, st, r, p, chunks, seg, all_aligned16({r, p}));
   return 1;
 }
 
