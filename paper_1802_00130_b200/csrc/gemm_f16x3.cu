@@ -105,7 +105,28 @@ __device__ __forceinline__ float finish(const HEpilogue& e, float x, float bz, f
 
 // Place of columns 4 q .. 4 q + 3 of row r in a staging tile: the 16-byte groups of a row are permuted by the row's low
 // bits, so that a column of groups, a row of groups and a row of single elements are all free of bank conflicts.
-__device__ __forceinline__ int stg_at(int r, int q) { return r * 32 + ((q ^ (r & 7)) << 2); }
+__device__ __forceinline__ uint32_t stg_at(uint32_t stg, int r, int q) { return stg + (uint32_t)(r * 128 + ((q ^ (r & 7)) << 4)); }
+// (through shared-space addresses: behind a generic pointer the compiler must keep every read of the tile behind the
+// global store before it, one latency per row)
+__device__ __forceinline__ void stg_put(uint32_t a, float x, float y, float z, float w) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+template <int W>
+__device__ __forceinline__ void stg_get(uint32_t a, float* v) {
+  if (W == 4)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[W > 1 ? 1 : 0]), "=f"(v[W > 2 ? 2 : 0]), "=f"(v[W > 3 ? 3 : 0]) : "r"(a));
+  else
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(a));
+}
+
+// W floats, read where the call stands.
+template <int W>
+__device__ __forceinline__ void load_now(const float* p, float* v) {
+  if (W == 4)
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[W > 1 ? 1 : 0]), "=f"(v[W > 2 ? 2 : 0]), "=f"(v[W > 3 ? 3 : 0]) : "l"(p));
+  else
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v[0]) : "l"(p));
+}
 
 // A warp's share of a finished tile through the epilogue options and out: `n_mine` chunks of 32 rows x 32 columns, 64
 // columns apart from column nb0 on, read back from tensor memory at `ta` (lane = row) and turned through the warp's
@@ -119,7 +140,7 @@ __device__ __forceinline__ int stg_at(int r, int q) { return r * 32 + ((q ^ (r &
 // registers are another's spills.  (Requested 2 to 4 rows at a time beside the sums, all forms in one kernel: 12000 x
 // 2000 x 2000 with dsig 319 us, now 236; 4001 x 1201 x 617 with unaligned rows 83, now 58.)
 template <int MODE, bool VEC>
-__device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint32_t ta, int n_mine, int m0, int rows, int nb0, int lane, unsigned& mag) {
+__device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uint32_t ta, int n_mine, int m0, int rows, int nb0, int lane, unsigned& mag) {
   constexpr int W = VEC ? 4 : 1, STEP = VEC ? 4 : 1, IT = 32 / STEP;
   constexpr bool ONE_OP = MODE == 2 || MODE == 3;
   const int col = VEC ? (lane & 7) * 4 : lane, r_first = VEC ? lane >> 3 : 0;
@@ -130,19 +151,16 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint3
 #pragma unroll 1
   for (int j = 0; j < n_mine; ++j) {
     const int n = nb0 + 64 * j + col;
-    if (ONE_OP && n < e.N) {
-      const float* src = MODE == 2 ? e.dsig + n : e.cin + (long long)(m0 + r_first) * e.ld_cin + n;
-      if (MODE == 2 && e.dsig_direct) src += (long long)(m0 + r_first) * e.ld_dsig;
-      const long long step = STEP * (MODE == 2 ? e.ld_dsig : e.ld_cin);
+    if (ONE_OP) {
+      // rows and columns past the end read the last ones: with a condition around it the compiler moves each load down
+      // to its use, one round trip per row
+      const int nc = min(n, e.N - W);
+      const float* const src = MODE == 2 ? e.dsig + nc : e.cin + nc;
+      const long long ld = MODE == 2 ? e.ld_dsig : e.ld_cin;
 #pragma unroll
       for (int i = 0; i < IT; ++i) {
-        const int r = r_first + i * STEP;
-        const float* q = MODE == 2 && !e.dsig_direct ? src + dsig_row(e, m0 + r) * e.ld_dsig : src;
-        if (r < rows) {
-          if (VEC) *reinterpret_cast<float4*>(op[ONE_OP ? i : 0]) = __ldg(reinterpret_cast<const float4*>(q));
-          else op[ONE_OP ? i : 0][0] = __ldg(q);
-        }
-        if (MODE == 3 || e.dsig_direct) src += step;
+        const int m = m0 + min(r_first + i * STEP, rows - 1);
+        load_now<W>(src + (MODE == 2 ? dsig_row(e, m) : (long long)m) * ld, op[ONE_OP ? i : 0]);
       }
     }
     {
@@ -151,9 +169,12 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint3
       __syncwarp();
 #pragma unroll
       for (int i = 0; i < 32; i += 4)
-        *reinterpret_cast<float4*>(stg + stg_at(lane, i >> 2)) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        stg_put(stg_at(stg, lane, i >> 2), v[i], v[i + 1], v[i + 2], v[i + 3]);
       __syncwarp();
     }
+    float xs[IT][W];                           // the whole chunk out of the staging tile before the first store
+#pragma unroll
+    for (int i = 0; i < IT; ++i) stg_get<W>(stg_at(stg, r_first + i * STEP, VEC ? lane & 7 : lane >> 2) + (VEC ? 0u : (lane & 3) * 4u), xs[i]);
     if (n < e.N) {
       float bz[W];
 #pragma unroll
@@ -167,8 +188,6 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint3
         const int r = r_first + i * STEP;
         if (r >= rows) continue;
         float x[W], z[W], c[W];
-        if (VEC) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(stg + stg_at(r, lane & 7));
-        else x[0] = stg[stg_at(r, lane >> 2) + (lane & 3)];
         if (MODE == 4 && use_dsig) {
           const float* src = e.dsig + dsig_row(e, m0 + r) * e.ld_dsig + n;
           if (VEC) *reinterpret_cast<float4*>(z) = __ldg(reinterpret_cast<const float4*>(src)); else z[0] = __ldg(src);
@@ -179,7 +198,7 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, float* stg, uint3
         }
 #pragma unroll
         for (int q = 0; q < W; ++q) {
-          float t = x[q] + bz[q];
+          float t = xs[i][q] + bz[q];
           if (use_sigm) t = sigmoid_from(expf(-t));
           if (use_dsig) { const float zz = MODE == 4 ? z[q] : op[ONE_OP ? i : 0][q]; t *= zz * (1.f - zz); }
           t *= e.alpha;
@@ -224,7 +243,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(H_THREADS, 1)
 gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  float* staging = reinterpret_cast<float*>(smem + H_STAGES * H_STAGE_BYTES);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + H_STAGES * H_STAGE_BYTES + H_STG_BYTES);
   uint64_t* empty = full + H_STAGES;
   uint64_t* acc_full = empty + H_STAGES;   // [2]
@@ -356,7 +374,7 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
     // ------------------------------------------------------------------ epilogue (warps 4..11, both CTAs)
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
-    float* const stg = staging + (warp - 4) * (32 * 32);
+    const uint32_t stg = smem_u32(smem + H_STAGES * H_STAGE_BYTES) + (uint32_t)(warp - 4) * 4096u;
     // what undoes the operands' scales: pair i's products are true values times 2^-E_i; sums are kept relative to
     // the largest E (the other pair's factor is a power of two below one), which is undone once per tile
     const int E0 = -(scale_exponent(__ldcg(p.amax[0])) + scale_exponent(__ldcg(p.amax[1])));
@@ -431,11 +449,14 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(stg + stg_at(lane, i >> 2)) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+              stg_put(stg_at(stg, lane, i >> 2), v[i], v[i + 1], v[i + 2], v[i + 3]);
             __syncwarp();
+            float x[8][4];
 #pragma unroll
-            for (int r = 0; r < 32; r += 4)
-              __stcg(reinterpret_cast<float4*>(o + r * bn + 64 * j), *reinterpret_cast<const float4*>(stg + stg_at(r + (lane >> 3), lane & 7)));
+            for (int r = 0; r < 8; ++r) stg_get<4>(stg_at(stg, 4 * r + (lane >> 3), lane & 7), x[r]);
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+              __stcg(reinterpret_cast<float4*>(o + 4 * r * bn + 64 * j), make_float4(x[r][0], x[r][1], x[r][2], x[r][3]));
           }
         } else {
           store_tile<MODE, VEC>(e, stg, ta, n_mine, m0, rows, nb0, lane, mag);

@@ -124,14 +124,17 @@ struct gn_ctx {
   float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
   bool small_enabled = true;
   double* partial = nullptr; int64_t partial_cap = 0;
-  double* dscal = nullptr;   // device: [0] loss, [1] theta^T theta, [2] cg sum rho, [3] cg active
-  double* hscal = nullptr;   // pinned mirror
-  int* err_flag = nullptr;   // [0] gather index error, [1] tensor-core pipeline timeout code
-  int* h_err = nullptr;      // pinned mirror of err_flag
+  // What the host reads at a synchronisation, in one device block with one pinned mirror, so that sync() brings all of
+  // it in one copy: scalars ([0] loss, [1] theta^T theta, [4..8] Newton's products), the solver's state, and the error
+  // words ([0] gather index error, [1] tensor-core pipeline timeout code).
+  struct Status { double scal[16]; CgControl ctl; int err[2]; };
+  Status* status = nullptr; Status* h_status = nullptr;
+  double* dscal = nullptr; double* hscal = nullptr;      // (into status and h_status, as the pointers below)
+  int* err_flag = nullptr; int* h_err = nullptr;
   gn_status sticky = GN_OK;  // a launch-time failure that must surface at the next check
   // CG
   float* cg_r = nullptr; float* cg_p = nullptr; float* cg_q = nullptr;
-  CgControl* cg_ctl = nullptr; CgControl* h_ctl = nullptr;   // device-resident solver state and its pinned mirror
+  CgControl* cg_ctl = nullptr; CgControl* h_ctl = nullptr;   // device-resident solver state and its mirror
   double* cg_hist = nullptr; int cg_hist_cap = 0;            // squared residual norms, one per step
   // One CG step (product + the three vector kernels) as a CUDA graph, for problems small enough that issuing the
   // step's ~20 launches from the host takes as long as running them: captured from the second step of a
@@ -279,9 +282,9 @@ void quiesce(gn_ctx* c) {
   if (c->st2) cudaStreamSynchronize(c->st2);
 }
 
-// Synchronise the stream; also fetch the tensor-core pipeline's timeout word.
+// Synchronise the stream; also fetch the status block and look at the tensor-core pipeline's timeout word.
 gn_status sync(gn_ctx* c, const char* where) {
-  cudaError_t e = cudaMemcpyAsync(c->h_err + 1, c->err_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  cudaError_t e = cudaMemcpyAsync(c->h_status, c->status, sizeof(gn_ctx::Status), cudaMemcpyDeviceToHost, c->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return cuda_fail(c, e, where);
   if (c->h_err[1] != 0) {
@@ -1189,6 +1192,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
 // Q_a[:, T_b] = D[:, :, T_b]^T 2 D[:, :, T_b] U_a[:, T_b]; then out_W[T_a, :] = Z_{m-1}[:, T_a]^T Q_a / |S|.
 // At the output layer D = I, so Q_a = 2 U_a.
 gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
+  SideJoin side_guard(c);
   CurrentVector current(c, v);
   ++c->parts_epoch;
   const int L = c->L, nL = c->w[L];
@@ -1231,9 +1235,13 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     batch.clear();
     const float* Q = c->SU;
     if (m < L) {
+      side_join(c);                                         // (the layer below's bias sums read what this overwrites)
       c->launches += launch_factor_apply(c->DF[m], c->SU, nS, nL, nm, sb, sa, stride, c->SQ, c->st);
       Q = c->SQ;
     }
+    // the bias sums on the side stream, beside this layer's weight blocks and the next layer's first contractions
+    GN_TRY(ensure_colsum(c, nS, nm));
+    c->launches += launch_colsum(Q, nS, nm, nm, inv, v + c->b_off[m], coef, out + c->b_off[m], c->colsum_scratch, side_fork(c));
     for (int a = 0; a < sa; ++a) {
       const int t0 = group_lo(np, sa, a), t1 = group_lo(np, sa, a + 1);
       GemmArgs g;
@@ -1249,8 +1257,6 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     }
     for (size_t b0 = 0; b0 < batch.size(); b0 += 16) run_gemm_group(c, batch.data() + b0, (int)std::min<size_t>(16, batch.size() - b0));
     batch.clear();
-    GN_TRY(ensure_colsum(c, nS, nm));
-    c->launches += launch_colsum(Q, nS, nm, nm, inv, v + c->b_off[m], coef, out + c->b_off[m], c->colsum_scratch, c->st);
   }
   return check_launch(c, "partition-wise G v");
 }
@@ -1297,7 +1303,6 @@ gn_status ensure_batch(gn_ctx* c) {
 
 // f from the summed loss and theta^T theta on the device.
 gn_status read_loss(gn_ctx* c, double* f_host) {
-  GN_CUDA(c, cudaMemcpyAsync(c->hscal, c->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   GN_TRY(check_launch(c, "f / grad"));
   GN_TRY(sync(c, "f / grad"));
   *f_host = c->hscal[1] / (2.0 * c->C) + c->hscal[0] / (double)c->l;
@@ -1501,18 +1506,16 @@ gn_status gn_create(gn_ctx** out, int L, const int32_t* widths, double C, int64_
     if ((s = dev_alloc(c, &c->cg_r, c->n)) != GN_OK) break;
     if ((s = dev_alloc(c, &c->cg_p, c->n)) != GN_OK) break;
     if ((s = dev_alloc(c, &c->cg_q, c->n)) != GN_OK) break;
-    if ((s = dev_alloc(c, &c->dscal, 16)) != GN_OK) break;
-    if ((s = dev_alloc(c, &c->cg_ctl, 1)) != GN_OK) break;
-    if (cudaMemset(c->cg_ctl, 0, sizeof(CgControl)) != cudaSuccess) { s = GN_ECUDA; break; }
-    if (cudaMallocHost(&c->h_ctl, sizeof(CgControl)) != cudaSuccess) { s = GN_ENOMEM; break; }
-    if ((s = dev_alloc(c, &c->err_flag, 2)) != GN_OK) break;
-    if (cudaMemset(c->err_flag, 0, 2 * sizeof(int)) != cudaSuccess) { s = GN_ECUDA; break; }
-    if (cudaMallocHost(&c->hscal, 16 * sizeof(double)) != cudaSuccess) { s = GN_ENOMEM; break; }
+    if ((s = dev_alloc(c, &c->status, 1)) != GN_OK) break;
+    if (cudaMemset(c->status, 0, sizeof(gn_ctx::Status)) != cudaSuccess) { s = GN_ECUDA; break; }
+    if (cudaMallocHost(&c->h_status, sizeof(gn_ctx::Status)) != cudaSuccess) { s = GN_ENOMEM; break; }
+    std::memset(c->h_status, 0, sizeof(gn_ctx::Status));
+    c->dscal = c->status->scal; c->hscal = c->h_status->scal;
+    c->cg_ctl = &c->status->ctl; c->h_ctl = &c->h_status->ctl;
+    c->err_flag = c->status->err; c->h_err = c->h_status->err;
     if (cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) { s = GN_ECUDA; break; }
-    if (cudaMallocHost(&c->h_err, 2 * sizeof(int)) != cudaSuccess) { s = GN_ENOMEM; break; }
-    c->h_err[0] = c->h_err[1] = 0;
     if ((s = build_chunks(c, false)) != GN_OK) break;
   } while (0);
   if (s != GN_OK) { gn_destroy(c); return s; }
@@ -1531,9 +1534,7 @@ gn_status gn_destroy(gn_ctx* c) {
   for (auto& o : c->owned)
     if (o.p) cudaFree(o.p);
   for (auto& p : c->ev) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
-  if (c->hscal) cudaFreeHost(c->hscal);
-  if (c->h_ctl) cudaFreeHost(c->h_ctl);
-  if (c->h_err) cudaFreeHost(c->h_err);
+  if (c->h_status) cudaFreeHost(c->h_status);
   cudaGetLastError();
   delete c;
   return GN_OK;
@@ -1668,10 +1669,8 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
     small.z[0] = c->dX; small.idx = c->idx; small.x_rows = c->l; small.err_flag = c->err_flag;
     for (int m = 0; m <= c->L; ++m) small.z_out[m] = c->Z[m];
     GN_TRY(run_small_pass(c, kSmallForward, small, 0.f, nullptr, 0.f, nullptr, nullptr));
-    GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
   } else {
     c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
-    GN_CUDA(c, cudaMemcpyAsync(c->h_err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     forward_pass(c, c->Z[0], nS, c->Z);
   }
   GN_TRY(check_launch(c, "set_subsample"));
@@ -1779,7 +1778,6 @@ gn_status gn_cg_solve(gn_ctx* c, const float* d_g, double lambda, int blockdiag,
   GN_TRY(check_launch(c, "cg init"));
   double active = 1.0;
   if (watch) {
-    GN_CUDA(c, cudaMemcpyAsync(c->h_ctl, c->cg_ctl, sizeof(CgControl), cudaMemcpyDeviceToHost, c->st));
     GN_TRY(sync(c, "cg init"));
     active = c->h_ctl->out[1];
   }
@@ -1846,15 +1844,13 @@ gn_status gn_cg_solve(gn_ctx* c, const float* d_g, double lambda, int blockdiag,
     if (d_iterates)
       GN_CUDA(c, cudaMemcpyAsync(d_iterates + (int64_t)it * c->n, d_d, c->n * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
     if (watch) {
-      GN_CUDA(c, cudaMemcpyAsync(c->h_ctl, c->cg_ctl, sizeof(CgControl), cudaMemcpyDeviceToHost, c->st));
       GN_TRY(sync(c, "cg step"));
       active = c->h_ctl->out[1];
     }
     ++it;
   }
-  // one read of the state at the end: steps in which a segment was still active, and the residual history
-  GN_CUDA(c, cudaMemcpyAsync(c->h_ctl, c->cg_ctl, sizeof(CgControl), cudaMemcpyDeviceToHost, c->st));
-  GN_TRY(sync(c, "cg solve"));
+  // the state at the end: steps in which a segment was still active, and the residual history
+  if (!watch) GN_TRY(sync(c, "cg solve"));     // (a watched solve has just read it)
   const int steps = watch ? it : c->h_ctl->steps;
   if (iters_host) *iters_host = steps;
   if (resnorm_host) {
@@ -1992,7 +1988,6 @@ gn_status gn_newton_iter(gn_ctx* c, float* d_theta, const int32_t* d_idx, int64_
   dot_to_slot(c, d_dir, Gx, 6);      // c  = dbar^T G dbar
   dot_to_slot(c, g, d, 7);           // g^T d
   dot_to_slot(c, g, d_dir, 8);       // g^T dbar
-  GN_CUDA(c, cudaMemcpyAsync(c->hscal + 4, c->dscal + 4, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   GN_TRY(check_launch(c, "newton: direction combination"));
   GN_TRY(sync(c, "newton: direction combination"));
   const double a = c->hscal[4], b = c->hscal[5], cc = c->hscal[6], gd = c->hscal[7], gdb = c->hscal[8];

@@ -694,24 +694,35 @@ inline int all_aligned16(std::initializer_list<const void*> ps) {
 }
 }  // namespace
 
+// The solver's vector kernels start early (programmatic dependent launch) only while all their blocks fit on the GPU
+// at once: blocks that wait in front of thousands of others cost more than the launch gap they hide (3072-1000-1000-10,
+// 1000 blocks: 1.5 % of a solve; 28-300-300-1, 24 blocks: 2 % the other way).
+namespace {
+template <class... KArgs, class... Args>
+void launch_cg(void (*kernel)(KArgs...), int blocks, cudaStream_t st, Args&&... args) {
+  if (blocks <= 148 * 4) launch_pdl_grid(kernel, dim3(blocks), 256, 0, st, std::forward<Args>(args)...);
+  else kernel<<<blocks, 256, 0, st>>>(std::forward<Args>(args)...);
+}
+}  // namespace
+
 int launch_cg_init(const float* g, float* d, float* r, float* p, const CgChunk* chunks, int n_chunks,
                    double* partial, CgSeg* seg, int n_seg, double tol, CgControl* ctl, cudaStream_t st) {
-  launch_pdl_grid(cg_init_kernel, dim3(n_chunks), 256, 0, st, g, d, r, p, chunks, partial, seg, n_seg, tol, ctl, all_aligned16({g, d, r, p}));
+  launch_cg(cg_init_kernel, n_chunks, st, g, d, r, p, chunks, partial, seg, n_seg, tol, ctl, all_aligned16({g, d, r, p}));
   return 1;
 }
 int launch_cg_dot(const float* p, const float* q, const CgChunk* chunks, int n_chunks, double* partial,
                   CgSeg* seg, int n_seg, CgControl* ctl, cudaStream_t st) {
-  launch_pdl_grid(cg_dot_kernel, dim3(n_chunks), 256, 0, st, p, q, chunks, partial, seg, n_seg, ctl, all_aligned16({p, q}));
+  launch_cg(cg_dot_kernel, n_chunks, st, p, q, chunks, partial, seg, n_seg, ctl, all_aligned16({p, q}));
   return 1;
 }
 int launch_cg_update(const float* p, const float* q, float* d, float* r, const CgChunk* chunks,
                      int n_chunks, CgSeg* seg, int n_seg, double tol, double* partial, CgControl* ctl, cudaStream_t st) {
-  launch_pdl_grid(cg_update_kernel, dim3(n_chunks), 256, 0, st, p, q, d, r, chunks, seg, n_seg, tol, partial, ctl, all_aligned16({p, q, d, r}));
+  launch_cg(cg_update_kernel, n_chunks, st, p, q, d, r, chunks, seg, n_seg, tol, partial, ctl, all_aligned16({p, q, d, r}));
   return 1;
 }
 int launch_cg_direction(const float* r, float* p, const CgChunk* chunks, int n_chunks, const CgSeg* seg,
                         cudaStream_t st) {
-  launch_pdl_grid(cg_direction_kernel, dim3(n_chunks), 256, 0, st, r, p, chunks, seg, all_aligned16({r, p}));
+  launch_cg(cg_direction_kernel, n_chunks, st, r, p, chunks, seg, all_aligned16({r, p}));
   return 1;
 }
 
