@@ -185,16 +185,11 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uin
       }
 #pragma unroll
       for (int i = 0; i < IT; ++i) {
-        const int r = r_first + i * STEP;
-        if (r >= rows) continue;
-        float x[W], z[W], c[W];
-        if (MODE == 4 && use_dsig) {
-          const float* src = e.dsig + dsig_row(e, m0 + r) * e.ld_dsig + n;
-          if (VEC) *reinterpret_cast<float4*>(z) = __ldg(reinterpret_cast<const float4*>(src)); else z[0] = __ldg(src);
-        }
-        if (MODE == 4 && use_cin) {
-          const float* src = e.cin + (long long)(m0 + r) * e.ld_cin + n;
-          if (VEC) *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(src)); else c[0] = __ldg(src);
+        float z[W], c[W];
+        if (MODE == 4) {                       // (rows past the end read the last one)
+          const int m = m0 + min(r_first + i * STEP, rows - 1);
+          if (use_dsig) load_now<W>(e.dsig + dsig_row(e, m) * e.ld_dsig + n, z);
+          if (use_cin) load_now<W>(e.cin + (long long)m * e.ld_cin + n, c);
         }
 #pragma unroll
         for (int q = 0; q < W; ++q) {
@@ -203,12 +198,33 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uin
           if (use_dsig) { const float zz = MODE == 4 ? z[q] : op[ONE_OP ? i : 0][q]; t *= zz * (1.f - zz); }
           t *= e.alpha;
           if (use_cin) t = fmaf(e.beta, MODE == 4 ? c[q] : op[ONE_OP ? i : 0][q], t);
-          x[q] = t;
-          if (e.amax_out) mag = max(mag, finite_magnitude(t));
+          xs[i][q] = t;
         }
-        float* d = e.D + (long long)(m0 + r) * e.ldd + n;
-        if (VEC) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(x);
-        else d[0] = x[0];
+      }
+      // (the record and the stores in loops of their own, whole chunks without a test per row: with rows that are no
+      // multiple of four floats every element is a store of its own, and what surrounds it counts)
+      if (e.amax_out) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i)
+#pragma unroll
+          for (int q = 0; q < W; ++q)
+            if (r_first + i * STEP < rows) mag = max(mag, finite_magnitude(xs[i][q]));
+      }
+      float* d = e.D + (long long)(m0 + r_first) * e.ldd + n;
+      const long long step = STEP * e.ldd;
+      if (rows == 32) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i, d += step) {
+          if (VEC) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(xs[i]);
+          else d[0] = xs[i][0];
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < IT; ++i, d += step)
+          if (r_first + i * STEP < rows) {
+            if (VEC) *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(xs[i]);
+            else d[0] = xs[i][0];
+          }
       }
     }
   }
