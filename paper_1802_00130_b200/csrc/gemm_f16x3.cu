@@ -698,19 +698,18 @@ HKernel const kKernels[10] = {
 }  // namespace
 
 // The register split of the kernel (128 x 56 + 256 x 224) must not exceed what the block is launched with, and the
-// kernel needs its dynamic shared memory granted: checked once.
+// kernel needs its dynamic shared memory granted: checked once per device.
 bool gemm_f16x3_usable() {
-  static const bool usable = [] {
+  static std::atomic<signed char> state[64];
+  return once_per_device(state, [] {
     bool ok = encode_fn() != nullptr;
     for (HKernel k : kKernels) {
       cudaFuncAttributes fa;
       ok = ok && cudaFuncGetAttributes(&fa, k) == cudaSuccess && fa.numRegs * H_THREADS >= 128 * H_REGS_LOW + 256 * H_REGS_HIGH &&
            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, H_SMEM_BYTES) == cudaSuccess;
     }
-    cudaGetLastError();
     return ok;
-  }();
-  return usable;
+  });
 }
 
 double gemm_f16x3_estimate_us(const GemmArgs& g) { return plan_f16x3(g).us; }

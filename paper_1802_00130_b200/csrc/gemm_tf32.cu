@@ -914,12 +914,11 @@ bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUten
 }
 
 void set_kernel_attributes() {
-  static bool done = false;
-  if (!done) {
-    cudaFuncSetAttribute(gemm_tf32_kernel<kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2);
-    done = true;
-  }
+  static std::atomic<signed char> state[64];
+  once_per_device(state, [] {
+    return cudaFuncSetAttribute(gemm_tf32_kernel<kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess;
+  });
 }
 
 inline bool suits_pair_kernel(const GemmArgs& g) { return g.M > BM && g.N >= 128; }

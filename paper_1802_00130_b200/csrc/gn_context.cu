@@ -120,6 +120,7 @@ struct gn_ctx {
   std::vector<AmaxEntry> amax;
   uint64_t parts_epoch = 1;
   bool amax_enabled = true;
+  bool own_capture = false, foreign_capture = false;       // the solver's step / the caller is capturing the stream
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
   float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
   bool small_enabled = true;
@@ -455,14 +456,16 @@ bool split_operand(gn_ctx* c, const float* src, int64_t rows, int cols, int64_t 
       c->split_cache.push_back(x);
       e = &c->split_cache.back();
     }
-    fresh = e->epoch == epoch && e->rows == rows && e->cols == cols && e->ld == ld;
+    // (a caller that captures its calls replays them after theta or the subsample have changed: a graph of the caller's
+    // splits everything it reads, and records nothing as split that has not run)
+    fresh = !c->foreign_capture && e->epoch == epoch && e->rows == rows && e->cols == cols && e->ld == ld;
     if (!fresh) {
       e->epoch = 0;
       if (rows * ldo > e->buf.cap) {
         if (e->in_arena) { e->buf = gn_ctx::SplitBuf{}; e->in_arena = false; }
         if (!split_buf_reserve(c, e->buf, rows * ldo)) return false;
       }
-      e->rows = rows; e->cols = cols; e->ld = ld; e->epoch = epoch;
+      e->rows = rows; e->cols = cols; e->ld = ld; e->epoch = c->foreign_capture ? 0 : epoch;
     }
     buf = &e->buf;
   } else {
@@ -528,6 +531,8 @@ bool run_gemm_f16x3(gn_ctx* c, const GemmArgs& args) {
   GemmArgs g = args;
   g.chunk_kb = c->prec == GN_FP32_ACCURATE && g.M > 128 && g.N >= 128 ? 2 : 1;
   if (!c->x3_usable || !gemm_f16x3_usable() || g.K1 < 1 || (g.A2 && g.K2 < 1)) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  c->foreign_capture = !c->own_capture && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
   if (ensure_split_scratch(c) != GN_OK) return false;
   if (!c->sk_enabled || (gemm_f16x3_workspace_floats(g) > 0 && ensure_sk_workspace(c) != GN_OK)) g.whole_tiles = true;
   // (the record of the result's maximum first: what follows takes records away, and must not be undone)
@@ -615,6 +620,9 @@ void run_gemm(gn_ctx* c, const GemmArgs& g, cudaStream_t st = nullptr) {
 // The parts of the operands in `roles` (bit per role) of several contractions that will go to the FP32-accurate
 // tensor-core kernel, in one splitting launch instead of one per contraction.  Kept kinds only.
 void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (!c->own_capture && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) return;
+  c->foreign_capture = false;
   std::vector<SplitJob> jobs;
   for (int i = 0; i < n; ++i) {
     const GemmArgs& g = gs[i];
@@ -1811,7 +1819,9 @@ gn_status gn_cg_solve(gn_ctx* c, const float* d_g, double lambda, int blockdiag,
         cudaGraph_t graph = nullptr;
         gn_status st = GN_OK;
         if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+          c->own_capture = true;
           st = one_step();
+          c->own_capture = false;
           const cudaError_t e = cudaStreamEndCapture(c->st, &graph);
           if (st == GN_OK && e == cudaSuccess && graph && gen == c->alloc_gen &&
               cudaGraphInstantiate(&cgg.exec, graph, 0) == cudaSuccess) {

@@ -332,13 +332,12 @@ typedef void (*SmallKernel)(const SmallNet);
 SmallKernel const kSmall[5] = {small_net_kernel<0>, small_net_kernel<1>, small_net_kernel<2>, small_net_kernel<3>, small_net_kernel<4>};
 
 bool small_usable() {
-  static const bool usable = [] {
+  static std::atomic<signed char> state[64];
+  return once_per_device(state, [] {
     bool ok = true;
     for (SmallKernel k : kSmall) ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SN_SMEM_MAX) == cudaSuccess;
-    cudaGetLastError();
     return ok;
-  }();
-  return usable;
+  });
 }
 
 }  // namespace

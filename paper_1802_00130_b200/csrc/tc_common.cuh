@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 namespace gn {
@@ -237,6 +238,21 @@ __device__ __forceinline__ float sigmoid_from(float e) {
 }
 
 // ---- host side ---------------------------------------------------------------------------------
+// A check or set-up that holds per device (function attributes do), made once on each: `make` runs with the device
+// current and says whether it worked.
+template <class F>
+bool once_per_device(std::atomic<signed char> (&state)[64], F make) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return false; }
+  signed char s = state[dev].load(std::memory_order_acquire);
+  if (s == 0) {
+    s = make() ? 1 : -1;
+    cudaGetLastError();
+    state[dev].store(s, std::memory_order_release);
+  }
+  return s > 0;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -107,3 +107,41 @@ def test_products_and_gradient_of_ragged_networks(widths, mode):
     assert rel(c.grad(), orc.grad(th, w, C, p["X"], p["Y"])) <= tol
     assert rel(c.Gv_blockdiag(dev(p["v"])), orc.Gv_blockdiag(th, w, C, XS, p["v"])) <= tol
     c.close()
+
+
+@pytest.mark.parametrize("mode", ["fp32", "tf32"])
+def test_a_captured_product_follows_theta_and_the_subsample(mode):
+    """A caller's own graph of a product, replayed after theta and the subsample have changed: the parts of theta and of
+    the stored activations that the context keeps must be made inside the graph, not taken from before it."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    from oracle import gn_oracle as orc
+    p = wl.make_custom((301, 403, 205, 5), 1500, 900, 15.0, seed=3)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    X, Y, v = dev(p["X"]), dev(p["Y"]), dev(p["v"])
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    ctx = gn.GnContext(p["widths"], p["C"], X, Y, gn.GN_TF32 if mode == "tf32" else gn.GN_FP32_ACCURATE, stream=stream)
+    out = torch.empty_like(v)
+    ctx.set_theta(dev(p["theta"]))
+    ctx.set_subsample(dev(p["idx"]))
+    ctx.Gv(v, out=out)                        # every workspace exists
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.Gv(v, out=out)
+    rel = lambda a, b: np.linalg.norm(a.cpu().numpy() - b) / np.linalg.norm(b)
+    plain = torch.empty_like(v)
+    for k in range(3):
+        th = (p["theta"] * (1.0 + 0.5 * k)).astype(np.float32)
+        idx = np.roll(np.arange(1500, dtype=np.int32), 37 * k)[:900].copy()
+        ctx.set_theta(dev(th))
+        ctx.set_subsample(dev(idx))
+        graph.replay()
+        torch.cuda.synchronize()
+        ref = orc.Gv(th, p["widths"], p["C"], p["X"][idx], p["v"])
+        assert rel(out, ref) <= 1e-5
+        ctx.Gv(v, out=plain)                  # and a plain call after it
+        torch.cuda.synchronize()
+        assert rel(plain, ref) <= 1e-5
+    ctx.close()
