@@ -582,9 +582,23 @@ bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
   return gemm_f16x3_estimate_us(g) + 14.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5 < fma_us;
 }
 
+// Whether a contraction of a TF32 context goes to the TF32 kernels.  Outside the CTA-pair kernel's shapes the one-CTA
+// kernel walks K alone, about 0.5 us per 32 terms and round of tiles: for a small result with a long K (the weight
+// blocks of narrow layers over many rows) the FP32-accurate form, which cuts K over all SMs, is the faster one although
+// it has operands to split (64 x 64 x 60000: about 900 us against 40).
+bool tf32_takes(const gn_ctx* c, const GemmArgs& g) {
+  if (c->prec != GN_TF32 || !gemm_tf32_eligible(g)) return false;
+  if (g.two_cta >= 0 || g.N >= 128 || !c->x3_usable || !gemm_f16x3_usable()) return true;
+  const double K = (double)g.K1 + (g.A2 ? g.K2 : 0);
+  const int64_t tiles = (g.M + 127) / 128;
+  const double one_us = 6.0 + (double)((tiles + 147) / 148) * K * (0.5 / 32.0);
+  return one_us <= gemm_f16x3_estimate_us(g) + 14.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5;
+}
+
 // Whether run_gemm will send a contraction to that form.
 bool goes_f16x3(const gn_ctx* c, const GemmArgs& g) {
-  return gemm_thin_kind(g) == THIN_NONE && !(c->prec == GN_TF32 && gemm_tf32_eligible(g)) && wants_f16x3(c, g);
+  if (gemm_thin_kind(g) != THIN_NONE || tf32_takes(c, g)) return false;
+  return wants_f16x3(c, g) || (c->prec == GN_TF32 && gemm_tf32_eligible(g));
 }
 
 // Kernel choice: streaming kernels for the n_L-wide shapes (both precisions: they are exact FP32), the TF32
@@ -612,9 +626,10 @@ void run_gemm(gn_ctx* c, const GemmArgs& g, cudaStream_t st = nullptr) {
     run_gemm_kind(c, g, 2, st);
     return;
   }
-  if (c->prec == GN_TF32 && gemm_tf32_eligible(g)) { run_gemm_kind(c, g, 0, st); return; }
-  if (!st && wants_f16x3(c, g) && run_gemm_f16x3(c, g)) return;
-  run_gemm_kind(c, g, 1, st);
+  const bool tf32 = c->prec == GN_TF32 && gemm_tf32_eligible(g);
+  if (tf32 && (st || tf32_takes(c, g))) { run_gemm_kind(c, g, 0, st); return; }
+  if (!st && (tf32 || wants_f16x3(c, g)) && run_gemm_f16x3(c, g)) return;
+  run_gemm_kind(c, g, tf32 ? 0 : 1, st);
 }
 
 // The parts of the operands in `roles` (bit per role) of several contractions that will go to the FP32-accurate

@@ -101,7 +101,8 @@ int launch_split_f16(const SplitJob* jobs, int n, unsigned* part, cudaStream_t s
 // loss (one double per block); launch_small_net then writes out = alpha * sum + beta * cin and *loss_out.  theta_sq (kinds 2, 3)
 // receives theta^T theta.  Returns launches made, or -1 if a launch failed.
 constexpr int kSmallLayers = 8;
-constexpr double kSmallUs = 40.0;       // estimated time up to which a pass goes this way (see small_net_fits)
+constexpr double kSmallUs = 42.0;       // estimated time up to which a pass goes this way (see small_net_fits) ...
+constexpr double kSmallUsPerElement = 20e-6;   // ... and what is added to it per row and neuron
 struct SmallNet {
   int L, n;
   int w[kSmallLayers + 1], w_off[kSmallLayers + 1], b_off[kSmallLayers + 1];

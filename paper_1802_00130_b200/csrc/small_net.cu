@@ -345,7 +345,10 @@ bool small_usable() {
 int64_t small_net_blocks(int64_t rows) { return (rows + SN_ROWS - 1) / SN_ROWS; }
 
 // The pass fits if its weights and 32 rows of activations do (227 KB), the blocks' sums take at most 32 MB, and the
-// estimated time stays below what the chain of kernels needs just to be launched.
+// estimated time stays below what the chain of kernels needs to be launched and to move the rows' activations.  Measured
+// (product, this way / the chain): 37-53-19-7 with 5000 rows 32 / 135 us, 60000 rows 159 / 318; 64-64-64-10 with 5000 rows
+// 69 / 101, 20000 rows 170 / 159; 100-100-10 with 1000 rows 41 / 52, 5000 rows 80 / 60; 784-16-10 with 1000 rows 38 / 59, 5000
+// rows 74 / 72.
 bool small_net_fits(const SmallNet& a, int kind) {
   if (a.L < 1 || a.L > kSmallLayers || !small_usable()) return false;
   const size_t smem = sn_smem_floats(a, kind) * sizeof(float);
@@ -361,7 +364,9 @@ bool small_net_fits(const SmallNet& a, int kind) {
   if (per_sm < 1) per_sm = 1;
   const double rounds = (double)((blocks + 148 * per_sm - 1) / (148 * per_sm));
   const double block_us = 3.0 + smem / 1.0e5 + 32.0 * macs * per_sm / 60.0e3;
-  return rounds * block_us <= kSmallUs;
+  double width = 0.0;
+  for (int m = 1; m <= a.L; ++m) width += a.w[m];
+  return rounds * block_us <= kSmallUs + kSmallUsPerElement * width * (double)a.rows;
 }
 
 int launch_small_net(const SmallNet& a, int kind, float alpha, const float* cin, float beta, float* out, double* loss_out, cudaStream_t st) {
