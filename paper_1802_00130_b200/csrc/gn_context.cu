@@ -124,6 +124,7 @@ struct gn_ctx {
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
   float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
   bool small_enabled = true;
+  int small_tf32 = -1;         // a TF32 context's passes are all small ones (-1: not looked at yet)
   double* partial = nullptr; int64_t partial_cap = 0;
   // What the host reads at a synchronisation, in one device block with one pinned mirror, so that sync() brings all of
   // it in one copy: scalars ([0] loss, [1] theta^T theta, [4..8] Newton's products), the solver's state, and the error
@@ -788,14 +789,27 @@ gn_status ensure_colsum(gn_ctx* c, int64_t rows, int cols) {
 // Whole passes of a small network in one launch (small_net.cu): the description for `rows` rows, and whether the pass
 // is to go that way.
 enum SmallKind { kSmallGv = 0, kSmallBlock = 1, kSmallGrad = 2, kSmallFun = 3, kSmallForward = 4 };
-bool small_pass(const gn_ctx* c, SmallKind kind, int64_t rows, SmallNet* a) {
+bool small_pass(gn_ctx* c, SmallKind kind, int64_t rows, SmallNet* a) {
   if (!c->small_enabled || c->L > kSmallLayers || c->n > 60000) return false;
   *a = SmallNet{};
   a->L = c->L; a->n = (int)c->n; a->rows = rows;
   for (int m = 0; m <= c->L; ++m) a->w[m] = c->w[m];
   for (int m = 1; m <= c->L; ++m) { a->w_off[m] = (int)c->w_off[m]; a->b_off[m] = (int)c->b_off[m]; }
   a->theta = c->theta;
-  return small_net_fits(*a, kind);
+  if (c->prec != GN_TF32) return small_net_fits(*a, kind);
+  // On a TF32 context all passes go this way or none: the gradient and the products of one solve have to round the
+  // same operator.  An exact gradient beside TF32 products (or the other way round) leaves an error in the first residual
+  // that is not along the gradient, and conjugate gradient amplifies it (96-100-50-200-1: iterates off by 1.4e-3 instead
+  // of 1e-4 although every single result was the more accurate one).
+  if (c->has_split || c->bd_method == 2) return false;
+  if (c->small_tf32 < 0) {
+    SmallNet all = *a;
+    all.rows = c->l;
+    c->small_tf32 = 1;
+    for (int k = kSmallGv; k <= kSmallForward; ++k)
+      if (!small_net_fits(all, k)) c->small_tf32 = 0;
+  }
+  return c->small_tf32 && (rows <= c->l || small_net_fits(*a, kind));
 }
 
 gn_status run_small_pass(gn_ctx* c, SmallKind kind, SmallNet& a, float alpha, const float* cin, float beta, float* out, double* loss_out) {

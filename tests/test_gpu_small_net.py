@@ -64,3 +64,20 @@ def test_an_index_out_of_range_is_still_refused():
     ctx.set_subsample(dev(p["idx"]))
     ctx.Gv(dev(p["v"]))
     ctx.close()
+
+
+@pytest.mark.parametrize("widths,nS,l", [((96, 100, 50, 200, 1), 554, 5540), ((60, 40, 20, 1), 2000, 100000), ((37, 53, 19, 7), 300, 900)])
+def test_tf32_solves_round_one_operator(widths, nS, l):
+    """Two steps of conjugate gradient on a TF32 context where only some of the passes would fit into one launch: the
+    first residual is a thousandth of the gradient, so a gradient and products that round differently show in the second
+    iterate.  Bound: the products' 1e-4, times the few times by which the second step amplifies a consistent rounding."""
+    import paper_1802_00130_b200 as gn
+    p = wl.make_custom(widths, l, nS, float(l), seed=5, x="sparse80")
+    ctx = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32)
+    ctx.set_theta(dev(p["theta"]))
+    ctx.set_subsample(dev(p["idx"]))
+    d, _, _ = ctx.cg_solve(ctx.grad(), 1.0, max_iter=2, tol=0.0)
+    th, w, C, XS = p["theta"], p["widths"], p["C"], p["X"][p["idx"]]
+    ref = orc.cg_solve(th, w, C, XS, orc.grad(th, w, C, p["X"], p["Y"]), 1.0, False, 2, 0.0)[0]
+    assert np.linalg.norm(d.cpu().numpy() - ref) <= 6e-4 * np.linalg.norm(ref)
+    ctx.close()
