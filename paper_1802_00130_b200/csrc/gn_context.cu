@@ -143,7 +143,7 @@ struct gn_ctx {
   // fixed-length solve and replayed for the rest; kept across solves while nothing it has baked in changes.
   struct CgGraph {
     cudaGraphExec_t exec = nullptr;
-    uint64_t alloc_gen = 0; int64_t nS = 0; float coef = 0.f; const float* d = nullptr; int stored = 0, method = 0, n_seg = 0;
+    uint64_t alloc_gen = 0, dispatch_gen = 0; int64_t nS = 0; float coef = 0.f; const float* d = nullptr; int stored = 0, method = 0, n_seg = 0;
     int64_t launches = 0;
   };
   CgGraph cg_graph[2];
@@ -151,6 +151,10 @@ struct gn_ctx {
   int64_t graph_replays = 0;
   bool own_stream = false;     // no stream was given: the context made one (stream capture cannot use the legacy default stream)
   uint64_t alloc_gen = 1;      // bumped by every device allocation and release of the context
+  // bumped by whatever sends contractions another way.  A captured step relies on the directly run first step of its
+  // solve for what that step leaves behind (split parts of theta and of the activations): it may only be replayed after a
+  // first step that went the same way
+  uint64_t dispatch_gen = 1;
   float* tmp_a = nullptr; float* tmp_b = nullptr;  // staging for *_host calls
   float* nt[4] = {nullptr, nullptr, nullptr, nullptr};  // Newton iteration: g, d, G d / G dbar, trial theta
   CgChunk* chunks[2] = {nullptr, nullptr}; int n_chunks[2] = {0, 0};
@@ -329,7 +333,7 @@ void run_gemm_kind(gn_ctx* c, const GemmArgs& g, int kind, cudaStream_t st = nul
     else c->launches += r;
   } else if (kind == 3) {
     const int r = launch_gemm_f16x3(g, c->h_ops, c->sk_ws, c->h_amax_out, c->err_flag + 1, st);
-    if (r < 0) { c->sticky = GN_ECUDA; c->err = "the FP32-accurate tensor-core kernel could not be launched"; c->x3_usable = false; }
+    if (r < 0) { c->sticky = GN_ECUDA; c->err = "the FP32-accurate tensor-core kernel could not be launched"; c->x3_usable = false; ++c->dispatch_gen; }
     else c->launches += r;
   } else if (kind == 2) {
     c->launches += launch_gemm_thin(g, c->thin_scratch, st);
@@ -344,7 +348,7 @@ gn_status ensure_sk_workspace(gn_ctx* c) {
     if (dev_alloc(c, &c->sk_ws, gemm_tf32_workspace_floats()) != GN_OK ||
         dev_alloc(c, &c->sk_flags, (int64_t)gemm_tf32_workspace_flags()) != GN_OK ||
         cudaMemsetAsync(c->sk_flags, 0, sizeof(int) * gemm_tf32_workspace_flags(), c->st) != cudaSuccess) {
-      c->sk_ws = nullptr; c->sk_flags = nullptr; c->sk_enabled = false;
+      c->sk_ws = nullptr; c->sk_flags = nullptr; c->sk_enabled = false; ++c->dispatch_gen;
     }
   }
   return c->sk_ws ? GN_OK : GN_ENOMEM;
@@ -1610,6 +1614,7 @@ gn_status gn_set_blockdiag_method(gn_ctx* c, int method) {
 gn_status gn_set_accurate_method(gn_ctx* c, int method) {
   if (!c) return GN_EINVAL;
   if (method < 0 || method > 2) return fail(c, GN_EINVAL, "method must be 0 (choose), 1 (FP32 FMA) or 2 (as 0)");
+  if (c->acc_method != method) ++c->dispatch_gen;
   c->acc_method = method;
   return GN_OK;
 }
@@ -1839,7 +1844,7 @@ gn_status gn_cg_solve(gn_ctx* c, const float* d_g, double lambda, int blockdiag,
     if (rule44 && it >= c->cg_min && (double)n_seg - active >= c->cg_share * (double)n_seg) break;
     if (use_graph && it >= 1) {
       // (the first step ran as plain launches: every workspace it needs exists and the stored factors are built)
-      const bool fits = cgg.exec && cgg.alloc_gen == c->alloc_gen && cgg.nS == c->nS && cgg.coef == coef && cgg.d == d_d &&
+      const bool fits = cgg.exec && cgg.alloc_gen == c->alloc_gen && cgg.dispatch_gen == c->dispatch_gen && cgg.nS == c->nS && cgg.coef == coef && cgg.d == d_d &&
                         cgg.stored == (c->factors_valid ? 1 : 0) && cgg.method == c->bd_method && cgg.n_seg == n_seg;
       if (!fits) {
         if (cgg.exec) { cudaGraphExecDestroy(cgg.exec); cgg.exec = nullptr; }
@@ -1854,7 +1859,7 @@ gn_status gn_cg_solve(gn_ctx* c, const float* d_g, double lambda, int blockdiag,
           const cudaError_t e = cudaStreamEndCapture(c->st, &graph);
           if (st == GN_OK && e == cudaSuccess && graph && gen == c->alloc_gen &&
               cudaGraphInstantiate(&cgg.exec, graph, 0) == cudaSuccess) {
-            cgg.alloc_gen = gen; cgg.nS = c->nS; cgg.coef = coef; cgg.d = d_d; cgg.stored = c->factors_valid ? 1 : 0;
+            cgg.alloc_gen = gen; cgg.dispatch_gen = c->dispatch_gen; cgg.nS = c->nS; cgg.coef = coef; cgg.d = d_d; cgg.stored = c->factors_valid ? 1 : 0;
             cgg.method = c->bd_method; cgg.n_seg = n_seg; cgg.launches = c->launches - before;
           } else {
             cgg.exec = nullptr;
@@ -2063,6 +2068,7 @@ gn_status gn_newton_iter(gn_ctx* c, float* d_theta, const int32_t* d_idx, int64_
 gn_status gn_debug_option(gn_ctx* c, int option, int value) {
   if (!c) return GN_EINVAL;
   if (option == 2) { if (value < 0) return fail(c, GN_EINVAL, "count must be >= 0"); c->fail_alloc_in = value; return GN_OK; }
+  if (option >= 0 && option <= 10) ++c->dispatch_gen;
   if (option == 3) { quiesce(c); c->side_enabled = value != 0; return GN_OK; }
   if (option == 7) { c->split_k_enabled = value != 0; return GN_OK; }
   if (option == 8) { c->back_chain = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }

@@ -145,3 +145,31 @@ def test_a_captured_product_follows_theta_and_the_subsample(mode):
         torch.cuda.synchronize()
         assert rel(plain, ref) <= 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("first,second", [(0, 1), (1, 0)])
+@pytest.mark.parametrize("blockdiag", [False, True])
+def test_a_kept_solver_step_follows_the_accurate_method(blockdiag, first, second):
+    """A fixed-length solve replays a captured step and keeps it for later solves.  After theta, the subsample and the way
+    FP32-accurate contractions are computed have changed, the step of before must not run on the parts it was captured with."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    from oracle import gn_oracle as orc
+    p = wl.make_custom((301, 403, 205, 5), 1500, 900, 15.0, seed=3)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    ctx = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]))
+    d = torch.empty(p["theta"].size, device="cuda")
+    for k, method in enumerate((first, second, first)):
+        th = (p["theta"] * (1.0 + 0.5 * k)).astype(np.float32)
+        idx = np.roll(np.arange(1500, dtype=np.int32), 37 * k)[:900].copy()
+        ctx.set_accurate_method(method)
+        ctx.set_theta(dev(th))
+        ctx.set_subsample(dev(idx))
+        g = orc.grad(th, p["widths"], p["C"], p["X"], p["Y"])
+        replays = ctx.graph_replays
+        ctx.cg_solve(dev(g.astype(np.float32)), 1.0, blockdiag=blockdiag, max_iter=5, tol=0.0, out=d)
+        assert ctx.graph_replays - replays == 4
+        ref = orc.cg_solve(th, p["widths"], p["C"], p["X"][idx], g, 1.0, blockdiag, 5, 0.0)[0]
+        # products within 1e-6, multiplied a few times by the five steps (systems of condition below 100)
+        assert np.linalg.norm(d.cpu().numpy() - ref) <= 1e-4 * np.linalg.norm(ref)
+    ctx.close()
