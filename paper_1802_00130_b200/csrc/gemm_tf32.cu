@@ -949,11 +949,13 @@ int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_fla
   const int pairs = num_sms() / 2;
   const int total_kb_all = (g.K1 + BK - 1) / BK + (g.A2 ? (g.K2 + BK - 1) / BK : 0);
   bool two_cta = g.two_cta >= 0 ? g.two_cta != 0 : suits_pair_kernel(g);
-  if (!two_cta && g.two_cta < 0 && sk_ws && sk_flags && g.M <= BM && g.N >= 128) {
-    // Up to 128 rows leave half of a pair's tile empty, but the pair kernel can cut a long K (the weight block of an
-    // output layer wider than the streaming kernels take) where the one-CTA kernel walks it alone on a few SMs, at about
-    // 0.5 us per k-block: 100 x 4096 x 32768 took 566 us there.  A slice costs 0.45 us per k-block and 16 us on top.
-    const int tiles = (g.N + 255) / 256;
+  if (!two_cta && g.two_cta < 0 && sk_ws && sk_flags) {
+    // A result of at most 128 rows or fewer than 128 columns leaves part of a pair's tile empty, but the pair kernel can
+    // cut a long K (the weight block of a narrow layer, or of an output layer wider than the streaming kernels take) where
+    // the one-CTA kernel walks it alone on a few SMs, at about 0.5 us per k-block: 100 x 4096 x 32768 took 566 us there,
+    // 64 x 64 x 60000 about 900.  A slice costs 0.45 us per k-block and 16 us on top.
+    const int bn2 = choose_bn2(g.M, g.N, true);
+    const int tiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + bn2 - 1) / bn2);
     const int sl = choose_slices(tiles, total_kb_all, pairs);
     two_cta = sl >= 2 && tiles <= pairs && 0.45 * total_kb_all / sl + 16.0 < 0.5 * total_kb_all;
   }

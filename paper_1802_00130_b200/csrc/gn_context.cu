@@ -587,23 +587,15 @@ bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
   return gemm_f16x3_estimate_us(g) + 14.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5 < fma_us;
 }
 
-// Whether a contraction of a TF32 context goes to the TF32 kernels.  Outside the CTA-pair kernel's shapes the one-CTA
-// kernel walks K alone, about 0.5 us per 32 terms and round of tiles: for a small result with a long K (the weight
-// blocks of narrow layers over many rows) the FP32-accurate form, which cuts K over all SMs, is the faster one although
-// it has operands to split (64 x 64 x 60000: about 900 us against 40).
-bool tf32_takes(const gn_ctx* c, const GemmArgs& g) {
-  if (c->prec != GN_TF32 || !gemm_tf32_eligible(g)) return false;
-  if (g.two_cta >= 0 || g.N >= 128 || !c->x3_usable || !gemm_f16x3_usable()) return true;
-  const double K = (double)g.K1 + (g.A2 ? g.K2 : 0);
-  const int64_t tiles = (g.M + 127) / 128;
-  const double one_us = 6.0 + (double)((tiles + 147) / 148) * K * (0.5 / 32.0);
-  return one_us <= gemm_f16x3_estimate_us(g) + 14.0 + (g.M + (double)g.N) * K * 8.0 / 4.0e6 * 0.5;
-}
+// Whether a contraction goes to the TF32 kernels: on a TF32 context every one whose operands TMA can address, whatever its
+// sizes.  The gradient (K or M up to a row batch) and the products (|S|) of one solve have to round the same operator: with
+// the weight blocks of narrow layers in FP32 accuracy from some K on (an earlier rule, 96-100-50-200-1, |S| = 554,
+// l = 5540) the first residual holds an error that is not along the gradient, and conjugate gradient amplifies it.
+bool on_tf32(const gn_ctx* c, const GemmArgs& g) { return c->prec == GN_TF32 && gemm_tf32_eligible(g); }
 
 // Whether run_gemm will send a contraction to that form.
 bool goes_f16x3(const gn_ctx* c, const GemmArgs& g) {
-  if (gemm_thin_kind(g) != THIN_NONE || tf32_takes(c, g)) return false;
-  return wants_f16x3(c, g) || (c->prec == GN_TF32 && gemm_tf32_eligible(g));
+  return gemm_thin_kind(g) == THIN_NONE && !on_tf32(c, g) && wants_f16x3(c, g);
 }
 
 // Kernel choice: streaming kernels for the n_L-wide shapes (both precisions: they are exact FP32), the TF32
@@ -631,10 +623,9 @@ void run_gemm(gn_ctx* c, const GemmArgs& g, cudaStream_t st = nullptr) {
     run_gemm_kind(c, g, 2, st);
     return;
   }
-  const bool tf32 = c->prec == GN_TF32 && gemm_tf32_eligible(g);
-  if (tf32 && (st || tf32_takes(c, g))) { run_gemm_kind(c, g, 0, st); return; }
-  if (!st && (tf32 || wants_f16x3(c, g)) && run_gemm_f16x3(c, g)) return;
-  run_gemm_kind(c, g, tf32 ? 0 : 1, st);
+  if (on_tf32(c, g)) { run_gemm_kind(c, g, 0, st); return; }
+  if (!st && wants_f16x3(c, g) && run_gemm_f16x3(c, g)) return;
+  run_gemm_kind(c, g, 1, st);
 }
 
 // The parts of the operands in `roles` (bit per role) of several contractions that will go to the FP32-accurate

@@ -94,3 +94,49 @@ def test_error_compensated_form_at_long_k_with_one_signed_terms(ctx):
     D = D.cpu().numpy().astype(np.float64)
     assert np.linalg.norm(D - ref) / np.linalg.norm(ref) <= 2e-6
     assert abs(np.mean(D - ref)) / np.mean(ref) <= 1.5e-6
+
+
+# results of few columns or few rows whose K the CTA-pair kernel cuts: one column chunk, a ragged one, the last width before
+# whole 128-column tiles; rows below, at and past a CTA's and a pair's tile
+NARROW = [(M, N, K, True, True) for M, N, K in ((64, 64, 60000), (300, 20, 4000), (129, 31, 9000), (257, 127, 3004), (1, 1, 5000))] + \
+    [(M, N, K, a_k, False) for a_k in (True, False)
+     for M, N, K in ((64, 64, 60000), (300, 20, 4001), (132, 36, 9000), (260, 124, 3004), (4, 300, 6000), (4, 4, 5000)) if not (a_k and K % 4)]
+
+
+@pytest.mark.parametrize("M,N,K,a_k,b_k", NARROW)
+def test_narrow_results_with_a_long_k_in_tf32(ctx, M, N, K, a_k, b_k):
+    import torch
+    A, B, ref = operands(M, N, K, a_k, b_k, seed=M + 7 * N + 13 * K)
+    bufs = []
+    for a in (A, B):                 # readable slack after the last row, as the library's own workspaces have
+        buf = torch.zeros(a.size + 64, dtype=torch.float32, device="cuda")
+        bufs.append(buf[: a.size].view(a.shape).copy_(torch.from_numpy(a)))
+    dA, dB = bufs
+    for kind in (0, 3):
+        D = ctx.debug_gemm(kind, dA, dB, a_kmajor=a_k, b_kmajor=b_k).cpu().numpy().astype(np.float64)
+        # operands of 11 significant bits, truncated: 2^-11 per product on average, averaging out over K
+        assert np.linalg.norm(D - ref) <= 1e-3 * np.linalg.norm(ref)
+        assert np.max(np.abs(D - ref)) <= 5e-2 * np.sqrt(K)
+
+
+@pytest.mark.parametrize("widths", [(96, 100, 52, 200, 4), (60, 40, 20, 20), (784, 64, 10), (300, 120, 80, 40)])
+def test_tf32_contexts_round_alike_at_every_number_of_rows(widths):
+    """The gradient (thousands of rows at a time) and the products (|S| rows) of a TF32 context are the same operator: no
+    contraction whose operands TMA can address turns to another precision at some number of rows."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    for nS, l in ((300, 600), (5000, 60000)):
+        p = wl.make_custom(widths, l, nS, float(l), seed=2)
+        c = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32)
+        c.debug_option(10, 0)
+        c.profile(True)
+        c.set_theta(dev(p["theta"]))
+        c.set_subsample(dev(p["idx"]))
+        c.grad()
+        c.Gv(dev(p["v"]))
+        c.Gv_blockdiag(dev(p["v"]))
+        kinds = c.profile_read()
+        assert kinds["tensor_x3"]["launches"] == 0 and kinds["ffma"]["launches"] == 0
+        assert kinds["tensor"]["launches"] + kinds["tensor_1cta"]["launches"] > 0
+        c.close()

@@ -66,7 +66,8 @@ def test_an_index_out_of_range_is_still_refused():
     ctx.close()
 
 
-@pytest.mark.parametrize("widths,nS,l", [((96, 100, 50, 200, 1), 554, 5540), ((60, 40, 20, 1), 2000, 100000), ((37, 53, 19, 7), 300, 900)])
+@pytest.mark.parametrize("widths,nS,l", [((96, 100, 50, 200, 1), 554, 5540), ((60, 40, 20, 1), 2000, 100000), ((37, 53, 19, 7), 300, 900),
+                                         ((300, 120, 80, 40), 700, 40000)])
 def test_tf32_solves_round_one_operator(widths, nS, l):
     """Two steps of conjugate gradient on a TF32 context where only some of the passes would fit into one launch: the
     first residual is a thousandth of the gradient, so a gradient and products that round differently show in the second
