@@ -136,10 +136,13 @@ gn_status gn_set_blockdiag_method(gn_ctx* ctx, int method);
  *      GEMM (small problems) elsewhere;
  *   1  the FP32 FMA GEMM for everything;
  *   2  same as 0.
- * Error-compensated form: every operand X is split into two FP16 matrices, X 2^e = Xhi + Xlo, with the power of two
- * that takes the largest |X| to [2^14, 2^15), so |X - (Xhi + Xlo) 2^-e| <= 2^-23 |x| down to 2^-18 of the largest element
- * and <= 2^-40 of the largest element below that; the product is Alo Bhi + Ahi Blo + Ahi Bhi accumulated in FP32, with
- * the sum over k cut into chunks of at most 128 terms that are added in FP32 round-to-nearest outside the tensor core
+ * Error-compensated form: every operand X is split into two FP16 matrices, cell by cell of 128 x 128 elements,
+ * X 2^e = Xhi + Xlo, with the power of two that takes the largest |X| of the cell to [2^14, 2^15), so
+ * |X - (Xhi + Xlo) 2^-e| <= 2^-23 |x| down to 2^-16 of the cell's largest element and <= 2^-39 of that below; a cell with a row or
+ * a column that lies wholly below 2^-20 of its largest element, or with an infinity or NaN, is not split: what meets it is
+ * summed with FP32 FMAs instead (slower, see gemm_f16x3.cu), so the range of an operand costs time and not precision, and
+ * infinities and NaN pass through a sum as in any FP32 arithmetic.  The product is Alo Bhi + Ahi Blo + Ahi Bhi accumulated in
+ * FP32, with the sum over k cut into chunks of at most 128 terms that are added in FP32 round-to-nearest outside the tensor core
  * (its own accumulator truncates).  Splits of theta and of the stored activations are kept until set_theta /
  * set_subsample; they take as much memory as those.  If the kernel cannot be launched on this device or a split buffer
  * cannot be allocated, the contraction runs on the FP32 FMA GEMM instead.  On GN_TF32 contexts the form serves, whatever
@@ -384,8 +387,7 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* ctx, int kind, int M, int N, int K, con
  * next to the layer's large contractions (value 0 = everything on the context's stream); option 4: consecutive
  * layers of a pass as one launch whose tiles wait for the tiles they read (value 0 = one launch per layer, 1 = the
  * stored forward pass, the default, 2 = also the forward R pass of a product).  Option 5: the
- * error-compensated kernel also records the largest magnitude of a result that a later contraction takes as an operand
- * (value 0 = a separate pass finds it).  Option 6: fixed-length
+ * operands of an error-compensated contraction are split by one launch (value 0 = one launch each).  Option 6: fixed-length
  * CG solves of small problems replay one captured step as a CUDA graph (value 0 = plain launches).  Option 7: the
  * weight blocks of the stored-factor block product as two chained parts of the subsample's rows (value 0 = one
  * contraction per block; the two forms differ in the order of two partial sums, i.e. by rounding).  Option 8: the

@@ -1,14 +1,23 @@
 // FP32-accurate contractions on the FP16 tensor cores (sm_100a).
 //
-// Every operand X arrives as two FP16 matrices, X 2^e = hi + lo with hi = rn16(X 2^e), lo = rn16(X 2^e - hi), where the
-// power of two 2^e takes the largest element of X to [2^14, 2^15).  hi and lo carry 11 significant bits each, so
-// |X - (hi + lo) 2^-e| <= 2^-23 |x| for elements down to 2^-18 of the largest one and <= 2^-40 max|X| below that.  A
-// logical product A B is Alo Bhi + Ahi Blo + Ahi Bhi (the dropped Alo Blo is below 2^-22 |a b|).
+// Every operand X arrives as two FP16 matrices, cut into cells of 128 x 128 elements with an exponent e each:
+// X 2^e = hi + lo, hi = rn16(X 2^e), lo = rn16(X 2^e - hi), where 2^e takes the largest element of the cell to [2^14, 2^15).
+// hi and lo carry 11 significant bits each, so |X - (hi + lo) 2^-e| <= 2^-23 |x| for elements down to 2^-16 of the cell's
+// largest, and <= 2^-39 of that below.  A logical product A B is Alo Bhi + Ahi Blo + Ahi Bhi (the dropped Alo Blo is below
+// 2^-22 |a b|).
+//
+// A cell is as long as a chunk of K (below) at most and as wide as a CTA's rows, so the exponents cost the main loop nothing:
+// what a chunk adds to the running sums is multiplied by a power of two anyway, which now belongs to the chunk's cells.
+// A cell with a row or a column that lies wholly below 2^-20 of its largest element, or with an infinity or NaN, is marked by
+// the splitting pass instead, and the epilogue warps compute the chunks that meet it as FP32 FMAs from the operands
+// themselves (fma_chunk): the range of a matrix costs time, not precision.  Why 2^-20: at that limit the elements of the row
+// or column are off by 5e-7 of its largest (root mean square), which is what an FP32 sum of some thousand terms leaves; and
+// the deltas of a scalar output, an outer product, have a row below 2^-18 in one of seventy products over 2000 rows.
 //
 // Why FP16 and not TF32 parts: the two formats have the same 11-bit significand, but kind::f16 runs at twice the rate
 // of kind::tf32 and its parts are half the bytes, so the three products cost 1.5 TF32 products instead of 3 and the
 // parts together are no larger than the FP32 operand.  What TF32 parts have and FP16 parts lack is exponent range;
-// the scale per operand puts the range where the operand is.
+// the exponent per cell puts the range where the cell is.
 //
 // The tensor core adds into its FP32 accumulator with truncation, a bias that grows with the number of additions, so
 // the K range is cut into chunks of 64 or 128 terms; each chunk is accumulated in tensor memory on its own (two
@@ -49,7 +58,6 @@ struct HEpilogue {
   float alpha;
   const float* cin; long long ld_cin; float beta;
   int vec;                                   // N % 4 == 0; D, bias, dsig, cin 16-byte aligned, leading dimensions % 4 == 0
-  unsigned* amax_out;                        // |D| maximum (bit pattern) is accumulated here when set
 };
 
 struct HParams {
@@ -57,9 +65,12 @@ struct HParams {
   int n_pairs;                               // logical operand pairs accumulated into one tile (1 or 2)
   int kblocks[2];
   int a_mn, b_mn;
-  const unsigned* amax[4];                   // bit pattern of max|X| of A1, B1, A2, B2
-  unsigned* reset[4];                        // accumulators of fused maxima to be cleared for their next use
-  int chunk_kb;                              // k-blocks per accumulation in tensor memory
+  // of A1, B1, A2, B2: the cells' exponents (kMarked: see the top), row by row of the stored matrix, and the matrix itself
+  const int8_t* cells[4]; int cells_ld[4];
+  const float* src[4]; long long ld_src[4];
+  int K[2];
+  int chunk_log;                             // log2 of the k-blocks per accumulation in tensor memory (0 or 1)
+  int chunks0;                               // chunks of the first operand pair
   // work list: items 0 .. whole - 1 are whole tiles, then slice sl of left-over tile j (tile whole + j) is item
   // whole + sl * rem + j; pair q takes items q, q + P, ...
   int bn, tiles_n, whole, rem, slices, items, P;
@@ -69,17 +80,16 @@ struct HParams {
 
 struct HMaps { CUtensorMap m[8]; };          // per pair: A hi, A lo, B hi, B lo
 
-// Exponent e of the scale 2^e for an operand whose largest magnitude has this bit pattern.
+constexpr int CELL = 128;                    // = H_BM = the longest chunk of K
+constexpr int kMarked = 127;
+constexpr unsigned FAR_LOG = 20;             // see the top
+// Exponent e of the scale 2^e for a cell whose largest magnitude has this bit pattern: -113 .. 126, 0 for a cell of zeros.
 __device__ __forceinline__ int scale_exponent(unsigned amax_bits) {
-  const int p = (int)(amax_bits >> 23) - 127;             // (zero and denormals: -127)
-  return min(14 - p, 126);
+  const int p = (int)(amax_bits >> 23) - 127;             // (denormals: -127)
+  return amax_bits ? min(14 - p, 126) : 0;
 }
-__device__ __forceinline__ float exp2_int(int e) {        // 2^e, 0 below the normal range
-  return e < -126 ? 0.f : __uint_as_float((unsigned)(min(e, 127) + 127) << 23);
-}
-__device__ __forceinline__ unsigned finite_magnitude(float x) {
-  const unsigned b = __float_as_uint(x) & 0x7fffffffu;
-  return b < 0x7f800000u ? b : 0u;                        // infinities and NaN do not set the scale
+__device__ __forceinline__ float exp2_int(int e) {        // 2^e, -149 <= e <= 127
+  return __uint_as_float(e < -126 ? 1u << (e + 149) : (unsigned)(e + 127) << 23);
 }
 
 __device__ __forceinline__ void mma2_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
@@ -140,7 +150,7 @@ __device__ __forceinline__ void load_now(const float* p, float* v) {
 // registers are another's spills.  (Requested 2 to 4 rows at a time beside the sums, all forms in one kernel: 12000 x
 // 2000 x 2000 with dsig 319 us, now 236; 4001 x 1201 x 617 with unaligned rows 83, now 58.)
 template <int MODE, bool VEC>
-__device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uint32_t ta, int n_mine, int m0, int rows, int nb0, int lane, unsigned& mag) {
+__device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uint32_t ta, int n_mine, int m0, int rows, int nb0, int lane) {
   constexpr int W = VEC ? 4 : 1, STEP = VEC ? 4 : 1, IT = 32 / STEP;
   constexpr bool ONE_OP = MODE == 2 || MODE == 3;
   const int col = VEC ? (lane & 7) * 4 : lane, r_first = VEC ? lane >> 3 : 0;
@@ -201,15 +211,8 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uin
           xs[i][q] = t;
         }
       }
-      // (the record and the stores in loops of their own, whole chunks without a test per row: with rows that are no
-      // multiple of four floats every element is a store of its own, and what surrounds it counts)
-      if (e.amax_out) {
-#pragma unroll
-        for (int i = 0; i < IT; ++i)
-#pragma unroll
-          for (int q = 0; q < W; ++q)
-            if (r_first + i * STEP < rows) mag = max(mag, finite_magnitude(xs[i][q]));
-      }
+      // (the stores in a loop of their own, whole chunks without a test per row: with rows that are no multiple of four
+      // floats every element is a store of its own, and what surrounds it counts)
       float* d = e.D + (long long)(m0 + r_first) * e.ldd + n;
       const long long step = STEP * e.ldd;
       if (rows == 32) {
@@ -230,20 +233,17 @@ __device__ __forceinline__ void store_tile(const HEpilogue& e, uint32_t stg, uin
   }
 }
 
-// Piece `i` of the chunk list of a K range: chunks of chunk_kb k-blocks that never straddle the two operand pairs.
+// Piece `i` of the chunk list of a K range: chunks of 1 or 2 k-blocks that never straddle the two operand pairs.
 struct ChunkPos { int pair, kb0, kb1; };
 __device__ __forceinline__ ChunkPos chunk_at(const HParams& p, int i) {
-  const int n0 = (p.kblocks[0] + p.chunk_kb - 1) / p.chunk_kb;
   ChunkPos c;
-  c.pair = i >= n0 ? 1 : 0;
-  c.kb0 = (i - (c.pair ? n0 : 0)) * p.chunk_kb;
-  c.kb1 = min(p.kblocks[c.pair], c.kb0 + p.chunk_kb);
+  c.pair = i >= p.chunks0 ? 1 : 0;
+  c.kb0 = (i - (c.pair ? p.chunks0 : 0)) << p.chunk_log;
+  c.kb1 = min(p.kblocks[c.pair], c.kb0 + (1 << p.chunk_log));
   return c;
 }
 __device__ __forceinline__ int chunk_count(const HParams& p) {
-  int n = (p.kblocks[0] + p.chunk_kb - 1) / p.chunk_kb;
-  if (p.n_pairs > 1) n += (p.kblocks[1] + p.chunk_kb - 1) / p.chunk_kb;
-  return n;
+  return p.chunks0 + (p.n_pairs > 1 ? (p.kblocks[1] + p.chunk_log) >> p.chunk_log : 0);
 }
 
 // Item of the work list: its tile, its chunks c0 .. c1 - 1, and, for a K slice, where its partial sums go (else -1).
@@ -252,6 +252,105 @@ __device__ __forceinline__ Item item_at(const HParams& p, int i, int n_chunks) {
   if (i < p.whole) return Item{i, 0, n_chunks, -1};
   const int k = i - p.whole, sl = k / p.rem;
   return Item{p.whole + k - sl * p.rem, (int)((long long)n_chunks * sl / p.slices), (int)((long long)n_chunks * (sl + 1) / p.slices), k};
+}
+
+// Where a lane finds the exponents of the chunks it looks up for its warp in this tile: lanes 0..3 of the cells of B under the
+// warp's four 32-column groups, lane 4 of A's cell of the CTA's rows (lanes without a cell repeat a neighbour's).
+struct CellWalk { const int8_t* at[2]; int step[2]; };
+__device__ __forceinline__ CellWalk cell_walk(const HParams& p, int m_cta, int n_warp, int n_cc_mine, int lane) {
+  const bool is_a = lane >= 4;
+  const int c = (is_a ? min(m_cta, p.e.M - 1) : min(n_warp + 64 * min(lane, max(n_cc_mine, 1) - 1), p.e.N - 1)) / CELL;
+  CellWalk w;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int op = 2 * s + (is_a ? 0 : 1), ld = p.cells_ld[op];
+    const bool k_rows = is_a ? p.a_mn : p.b_mn;            // K runs over the rows of the stored matrix
+    w.step[s] = k_rows ? ld : 1;
+    w.at[s] = p.cells[op] + (k_rows ? (long long)c : (long long)c * ld);
+  }
+  return w;
+}
+__device__ __forceinline__ int cell_exponent(const HParams& p, const CellWalk& w, int ch) {
+  const int s = ch >= p.chunks0 ? 1 : 0, k = ((ch - (s ? p.chunks0 : 0)) << p.chunk_log) >> 1;      // (two k-blocks per cell)
+  return __ldcg((s ? w.at[1] : w.at[0]) + (long long)k * (s ? w.step[1] : w.step[0]));
+}
+
+__device__ __forceinline__ void stg_put1(uint32_t a, float x) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory"); }
+
+// A chunk of K as FP32 FMAs: sum_k A(m, k) B(k, n) for the warp's 32 rows from m_warp on and its groups of 32 columns, 64 apart
+// from n_warp on, added to the running sums at `sums` in tensor memory (lane = row).  16 terms at a time go through the warp's
+// staging tile, A's and B's 16 x 32 each; a thread takes 4 rows x 8 columns, three 16-byte reads for 32 FMAs.  Not meant
+// to be fast: 12000 x 2000 x 2000 takes 0.21 ms with no cell marked, 0.71 ms with one column of A far below the others and
+// 7.5 ms with every cell marked (the FMA GEMM: 2.3 ms).
+__device__ __forceinline__ void fma_chunk(const HParams& p, const ChunkPos cp, uint32_t stg, int m_warp, int n_warp, int n_groups, int lane, uint32_t sums) {
+  const float* const A = dep(p.src[2 * cp.pair]);
+  const float* const B = dep(p.src[2 * cp.pair + 1]);
+  const long long lda = p.ld_src[2 * cp.pair], ldb = p.ld_src[2 * cp.pair + 1];
+  const int k_end = min(p.K[cp.pair], cp.kb1 * H_BK), M = p.e.M, N = p.e.N;
+  const int k_of = lane & 15, mn_of = lane >> 4;           // K-major operands: 16 terms of two rows per access
+#pragma unroll 1
+  for (int j = 0; j < n_groups; ++j) {
+    const int n0 = n_warp + 64 * j;
+    float acc[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+    float a[16], b[16];
+    const auto fetch = [&](int k0) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int ka = p.a_mn ? k0 + i : k0 + k_of, m = m_warp + (p.a_mn ? lane : 2 * i + mn_of);
+        a[i] = ka < k_end && m < M ? __ldg(A + (p.a_mn ? ka * lda + m : m * lda + ka)) : 0.f;
+        const int kb = p.b_mn ? k0 + i : k0 + k_of, n = n0 + (p.b_mn ? lane : 2 * i + mn_of);
+        b[i] = kb < k_end && n < N ? __ldg(B + (p.b_mn ? kb * ldb + n : n * ldb + kb)) : 0.f;
+      }
+    };
+    fetch(cp.kb0 * H_BK);
+#pragma unroll 1
+    for (int k0 = cp.kb0 * H_BK; k0 < k_end; k0 += 16) {
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int ra = p.a_mn ? i : k_of, m = p.a_mn ? lane : 2 * i + mn_of;
+        stg_put1(stg_at(stg, ra, m >> 2) + (m & 3) * 4u, a[i]);
+        const int rb = p.b_mn ? i : k_of, n = p.b_mn ? lane : 2 * i + mn_of;
+        stg_put1(stg_at(stg, 16 + rb, n >> 2) + (n & 3) * 4u, b[i]);
+      }
+      __syncwarp();
+      if (k0 + 16 < k_end) fetch(k0 + 16);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        float x[4], y[8];
+        stg_get<4>(stg_at(stg, k, lane >> 2), x);
+        stg_get<4>(stg_at(stg, 16 + k, 2 * (lane & 3)), y);
+        stg_get<4>(stg_at(stg, 16 + k, 2 * (lane & 3) + 1), y + 4);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(x[u], y[v], acc[u][v]);
+      }
+    }
+    __syncwarp();                                          // the block's sums, turned to lane = row
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        stg_put(stg_at(stg, (lane >> 2) * 4 + u, 2 * (lane & 3) + h), acc[u][4 * h], acc[u][4 * h + 1], acc[u][4 * h + 2], acc[u][4 * h + 3]);
+    __syncwarp();
+    float run[32];
+    tmem_ld32(sums + (uint32_t)(64 * j), run);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      float x[4];
+      stg_get<4>(stg_at(stg, lane, q), x);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) run[4 * q + u] += x[u];
+    }
+    tmem_st32(sums + (uint32_t)(64 * j), run);
+    tmem_st_wait();
+    __syncwarp();
+  }
 }
 
 template <int MODE, bool VEC>
@@ -293,7 +392,6 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(H_REGS_LOW));
     if (warp == 0) {
       // ---------------------------------------------------------------- producer (both CTAs)
-      if (blockIdx.x == 0 && lane < 4 && p.reset[lane]) *p.reset[lane] = 0u;
       const int b_chunks = p.b_mn ? (hb + 63) / 64 : 0;    // MN-major B: 64-column boxes
       const uint32_t b_bytes = p.b_mn ? (uint32_t)b_chunks * 8192u : (uint32_t)hb * 128u;
       const uint32_t pair_tx = 4u * (H_PART_BYTES + b_bytes);            // two CTAs x (hi + lo) x (A + B half)
@@ -391,15 +489,7 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
     const uint32_t stg = smem_u32(smem + H_STAGES * H_STAGE_BYTES) + (uint32_t)(warp - 4) * 4096u;
-    // what undoes the operands' scales: pair i's products are true values times 2^-E_i; sums are kept relative to
-    // the largest E (the other pair's factor is a power of two below one), which is undone once per tile
-    const int E0 = -(scale_exponent(__ldcg(p.amax[0])) + scale_exponent(__ldcg(p.amax[1])));
-    const int E1 = p.n_pairs > 1 ? -(scale_exponent(__ldcg(p.amax[2])) + scale_exponent(__ldcg(p.amax[3]))) : E0;
-    const int E = max(E0, E1);
-    const float f0 = exp2_int(E0 - E), f1 = exp2_int(E1 - E);
-    const float u0 = exp2_int(E / 2), u1 = exp2_int(E - E / 2);
     const HEpilogue& e = p.e;
-    unsigned mag = 0u;
     int ci = 0;
     bool alive = true;
     for (int item = pair; item < p.items && alive; item += p.P) {
@@ -411,10 +501,17 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int i = 0; i < 32; ++i) run[j][i] = 0.f;
+      const CellWalk walk = cell_walk(p, m0 - quad * 32, n0 + half * 32, (n_cc - half + 1) / 2, lane);
+      int exps = cell_exponent(p, walk, w.c0);                   // exponents of the cells of the chunk to come
       for (int ch = w.c0; ch < w.c1; ++ch, ++ci) {
         const int buf = ci & 1;
         const uint32_t aph = (ci >> 1) & 1;
-        const float f = chunk_at(p, ch).pair ? f1 : f0;
+        const bool by_fma = __any_sync(0xffffffffu, exps == kMarked);
+        // what undoes the scales of this chunk's cells, per 32-column group: 2^-shift
+        int shift[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) shift[j] = __shfl_sync(0xffffffffu, exps, 4) + __shfl_sync(0xffffffffu, exps, j);
+        if (ch + 1 < w.c1) exps = cell_exponent(p, walk, ch + 1);       // (on its way while this chunk is waited for)
         int good = 1;
         if (lane == 0) good = wait_or_abort(&acc_full[buf], aph, abort_flag, p.err, 3) ? 1 : 0;
         good = __shfl_sync(0xffffffffu, good, 0);
@@ -422,17 +519,34 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
         tc_fence_after();
         // two 32-column reads in flight at a time (a read of columns past the tile is harmless: it is never stored)
         const uint32_t ta = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * H_BN_MAX + half * 32);
+        if (by_fma) {                                            // (the sums wait in tensor memory: the buffer is free)
 #pragma unroll
-        for (int j = 0; j < 4; j += 2) {
-          if (half + 2 * j < n_cc) {                             // warp-uniform
-            float v[64];
-            tmem_ld_32x32b_x32(ta + (uint32_t)(j * 64), v);
-            tmem_ld_32x32b_x32(ta + (uint32_t)(j * 64 + 64), v + 32);
-            tmem_ld_wait();
+          for (int j = 0; j < 4; ++j) tmem_st32(ta + (uint32_t)(j * 64), run[j]);
+          tmem_st_wait();
+          fma_chunk(p, chunk_at(p, ch), stg, m0, n0 + half * 32, (n_cc - half + 1) / 2, lane, ta);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              run[j][i] = fmaf(v[i], f, run[j][i]);
-              run[j + 1][i] = fmaf(v[32 + i], f, run[j + 1][i]);
+          for (int j = 0; j < 4; ++j) tmem_ld_32x32b_x32(ta + (uint32_t)(j * 64), run[j]);
+          tmem_ld_wait();
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; j += 2) {
+            if (half + 2 * j < n_cc) {                           // warp-uniform
+              float v[64];
+              tmem_ld_32x32b_x32(ta + (uint32_t)(j * 64), v);
+              tmem_ld_32x32b_x32(ta + (uint32_t)(j * 64 + 64), v + 32);
+              tmem_ld_wait();
+              if (abs(shift[j]) > 126 || abs(shift[j + 1]) > 126) {      // (out of a factor's range: in two steps)
+                const float g0 = exp2_int(-shift[j] / 2), g1 = exp2_int(-shift[j + 1] / 2);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) { v[i] *= g0; v[32 + i] *= g1; }
+                shift[j] += -shift[j] / 2; shift[j + 1] += -shift[j + 1] / 2;
+              }
+              const float f0 = exp2_int(-shift[j]), f1 = exp2_int(-shift[j + 1]);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                run[j][i] = fmaf(v[i], f0, run[j][i]);
+                run[j + 1][i] = fmaf(v[32 + i], f1, run[j + 1][i]);
+              }
             }
           }
         }
@@ -448,11 +562,7 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
       const int n_mine = (n_cc - half + 1) / 2;
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (j < n_mine) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) run[j][i] = run[j][i] * u0 * u1;
-          tmem_st32(ta + (uint32_t)(j * 64), run[j]);
-        }
+        if (j < n_mine) tmem_st32(ta + (uint32_t)(j * 64), run[j]);
       tmem_st_wait();
       if (m0 < e.M) {                                            // warp-uniform
         const int rows = min(32, e.M - m0), nb0 = n0 + half * 32;
@@ -475,16 +585,12 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
               __stcg(reinterpret_cast<float4*>(o + 4 * r * bn + 64 * j), make_float4(x[r][0], x[r][1], x[r][2], x[r][3]));
           }
         } else {
-          store_tile<MODE, VEC>(e, stg, ta, n_mine, m0, rows, nb0, lane, mag);
+          store_tile<MODE, VEC>(e, stg, ta, n_mine, m0, rows, nb0, lane);
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
-    }
-    if (e.amax_out) {
-      mag = __reduce_max_sync(0xffffffffu, mag);
-      if (lane == 0 && mag) atomicMax(e.amax_out, mag);
     }
   }
   tc_fence_before();
@@ -506,7 +612,6 @@ __global__ void __launch_bounds__(256) slice_sum_kernel(const HEpilogue e, const
   const int j = blockIdx.x / per_tile, c = (blockIdx.x - j * per_tile) * 32 + lane;
   const int t = whole + j;
   const int m0 = (t / tiles_n) * (2 * H_BM), n = (t % tiles_n) * bn + c;
-  unsigned mag = 0u;
   if (n < e.N) {
     const float bz = e.bias ? __ldg(e.bias + n) : 0.f;
     const long long step = (long long)rem * (2 * H_BM) * bn;
@@ -519,38 +624,37 @@ __global__ void __launch_bounds__(256) slice_sum_kernel(const HEpilogue e, const
       float s = 0.f;
 #pragma unroll 8
       for (int k = 0; k < slices; ++k) s += __ldcg(w + k * step);
-      const float x = finish(e, s, bz, z, cv);
-      e.D[(long long)m * e.ldd + n] = x;
-      mag = max(mag, finite_magnitude(x));
+      e.D[(long long)m * e.ldd + n] = finish(e, s, bz, z, cv);
     }
-  }
-  if (e.amax_out) {
-    mag = __reduce_max_sync(0xffffffffu, mag);
-    if (lane == 0 && mag) atomicMax(e.amax_out, mag);
   }
 }
 
 // ---- splitting -----------------------------------------------------------------------------------
-// Up to kSplitSegs matrices per launch.  A thread takes 4 consecutive columns; a block of 256 threads covers 256 / per_row
-// rows at a time (or one row in several steps), with the thread's place in that pattern fixed so that the loop
-// has no division.  Four rows are requested before the first is used.
+// Up to kSplitSegs matrices per launch, a cluster of four blocks per cell: a block holds 32 rows of it in registers (4 groups of
+// 4 columns per thread, all requested before the first is used), the cluster finds its largest element, and every block writes
+// its parts, so a matrix is read once.  (A last column of cells of at most 32 columns has a block per cell, four to a cluster.)  Bound by its memory traffic where there is some and by the chain of load, exchange
+// and store where there is not.  12000 x 2000:
+// 43 us (192 MB; a pass for one maximum of the whole matrix and one for the parts took 22 + 45), 2500 x 1000: 6.2 us (3.9 +
+// 5.3), 300 x 300: 3.5 us (2.3 + 2.8).  A block of 512 threads per cell: 36, 8.4 and 4.9 us.
+constexpr int SPLIT_THREADS = 256, SPLIT_BLOCKS = 4, SPLIT_ROWS = CELL / SPLIT_BLOCKS / (SPLIT_THREADS / 32);   // rows of a warp
 struct SplitSeg {
   const float* src; long long rows; int cols; long long ld;
   __half* hi; __half* lo; long long ld_out;
-  unsigned* part; int n_part;                // maxima of the blocks of the first pass (or the producer's one maximum)
-  unsigned* bits;                            // the operand's maximum, for the contraction
-  int block0, blocks, vec;
+  int8_t* cells; int cells_ld;
+  int rows_ld;                               // 128-row panels
+  int wide, wide_ld;                         // clusters with a cell each, of them per panel; then clusters of four narrow cells
+  int cluster0, vec;
 };
 struct SplitList { int n; SplitSeg s[kSplitSegs]; };
 
-__device__ __forceinline__ float4 load_group(const SplitSeg& s, long long r, int c) {
-  const float* q = s.src + r * s.ld + c;
-  if (s.vec) return __ldg(reinterpret_cast<const float4*>(q));
+// columns c .. c + 3 of a row of which `left` are there
+__device__ __forceinline__ float4 load_group(const float* q, int left, int vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(q));
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
   x.x = __ldg(q);
-  if (c + 1 < s.cols) x.y = __ldg(q + 1);
-  if (c + 2 < s.cols) x.z = __ldg(q + 2);
-  if (c + 3 < s.cols) x.w = __ldg(q + 3);
+  if (left > 1) x.y = __ldg(q + 1);
+  if (left > 2) x.z = __ldg(q + 2);
+  if (left > 3) x.w = __ldg(q + 3);
   return x;
 }
 
@@ -563,66 +667,117 @@ __device__ __forceinline__ void split4(float4 x, float sc, uint2& h, uint2& l) {
   l.x = *reinterpret_cast<const unsigned*>(&la); l.y = *reinterpret_cast<const unsigned*>(&lb);
 }
 
-template <bool SPLIT>
-__global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ SplitList list) {
-  __shared__ unsigned sh[8];
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void put_remote(const void* at, uint32_t rank, unsigned x) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(smem_u32(at), rank)), "r"(x) : "memory");
+}
+
+__device__ __forceinline__ unsigned magnitude(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+
+__global__ void __cluster_dims__(SPLIT_BLOCKS, 1, 1) __launch_bounds__(SPLIT_THREADS) split_f16_kernel(const __grid_constant__ SplitList list) {
+  constexpr int WARPS = SPLIT_THREADS / 32;
+  __shared__ unsigned col_max[CELL];                       // of this block's rows: largest magnitude per column,
+  __shared__ unsigned warp_max[WARPS], warp_row[WARPS];    // largest, and smallest of the rows' largest (less one, so that a row of zeros is the largest)
+  __shared__ unsigned all_max[SPLIT_BLOCKS];               // what the blocks tell every block, and block 0
+  __shared__ unsigned all_row[SPLIT_BLOCKS], all_col[SPLIT_BLOCKS][CELL];
+  cluster_arrive();                                        // (no block writes to another before that one runs)
   grid_dep_wait();
   grid_dep_launch();
+  const int cluster = blockIdx.x / SPLIT_BLOCKS;
+  const int rank = (int)cluster_ctarank();
   int k = 0;
-  while (k + 1 < list.n && (int)blockIdx.x >= list.s[k + 1].block0) ++k;
+  while (k + 1 < list.n && cluster >= list.s[k + 1].cluster0) ++k;
   const SplitSeg& s = list.s[k];
-  const int blk = blockIdx.x - s.block0;
-  const int tid = threadIdx.x;
-  float sc = 1.f;
-  if (SPLIT) {
-    unsigned m = 0u;
-    for (int i = tid; i < s.n_part; i += 256) m = max(m, __ldcg(s.part + i));
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((tid & 31) == 0) sh[tid >> 5] = m;
-    __syncthreads();
+  const float* const src = dep(s.src);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the cluster's cell, or (narrow, at most 32 columns: a block holds all of one) this block's
+  const int at_seg = cluster - s.cluster0;
+  const bool solo = at_seg >= s.wide;
+  const int panel = solo ? (at_seg - s.wide) * SPLIT_BLOCKS + rank : at_seg / s.wide_ld, ct = solo ? s.cells_ld - 1 : at_seg - panel * s.wide_ld;
+  // lanes that share a row (8, 16 or 32 groups of 4 columns, as the cell has columns), rows of an access
+  const int width = s.cols - ct * CELL, lanes_log = solo ? 3 : width <= 64 ? 4 : 5, lanes = 1 << lanes_log, rpi = 32 >> lanes_log;
+  const int g = lane & (lanes - 1), c = ct * CELL + 4 * g, left = s.cols - c;
+  const int warp_rows = solo ? 4 * SPLIT_ROWS : SPLIT_ROWS;
+  const long long r0 = (long long)panel * CELL + (solo ? warp : rank * WARPS + warp) * warp_rows + (lane >> lanes_log);
+  const int n_mine = left > 0 ? (int)min((s.rows - r0 + rpi - 1) >> (5 - lanes_log), (long long)(warp_rows >> (5 - lanes_log))) : 0;   // this thread's groups
+  float4 x[SPLIT_ROWS];
+  {
+    const float* q = src + r0 * s.ld + c;
+    const long long step = rpi * s.ld;
+    const int vec = s.vec;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) m = max(m, sh[i]);
-    if (blk == 0 && tid == 0) *s.bits = m;
-    sc = exp2_int(scale_exponent(m));
+    for (int i = 0; i < SPLIT_ROWS; ++i, q += step)
+      x[i] = i < n_mine ? load_group(q, left, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  const int per_row = (s.cols + 3) >> 2;
-  const int rpb = per_row < 256 ? 256 / per_row : 1;       // rows a block covers at a time
-  const int r_off = per_row < 256 ? tid / per_row : 0;
-  const int g0 = per_row < 256 ? tid - r_off * per_row : tid;
-  unsigned mag = 0u;
-  if (r_off < rpb) {
-    const long long step = (long long)s.blocks * rpb;
-    for (long long r0 = (long long)blk * rpb + r_off; r0 < s.rows; r0 += 4 * step) {
-      for (int g = g0; g < per_row; g += 256) {
-        float4 x[4];
+  if (tid < CELL) col_max[tid] = 0u;
+  __syncthreads();
+  unsigned largest = 0u, row_min = 0xffffffffu, col[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          x[i] = r0 + i * step < s.rows ? load_group(s, r0 + i * step, 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = 0; i < SPLIT_ROWS; ++i) {
+    const unsigned m[4] = {magnitude(x[i].x), magnitude(x[i].y), magnitude(x[i].z), magnitude(x[i].w)};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (!SPLIT) {
-            mag = max(mag, max(max(finite_magnitude(x[i].x), finite_magnitude(x[i].y)),
-                               max(finite_magnitude(x[i].z), finite_magnitude(x[i].w))));
-          } else if (r0 + i * step < s.rows) {
-            uint2 h, l;
-            split4(x[i], sc, h, l);                        // (ld_out is a multiple of 8: a whole group always fits)
-            *reinterpret_cast<uint2*>(s.hi + (r0 + i * step) * s.ld_out + 4 * g) = h;
-            *reinterpret_cast<uint2*>(s.lo + (r0 + i * step) * s.ld_out + 4 * g) = l;
-          }
-        }
+    for (int q = 0; q < 4; ++q) col[q] = max(col[q], m[q]);
+    unsigned row = max(max(m[0], m[1]), max(m[2], m[3]));
+    if (lanes == 32) {
+      row = __reduce_max_sync(0xffffffffu, row);
+    } else {
+      for (int o = lanes >> 1; o > 0; o >>= 1) row = max(row, __shfl_xor_sync(0xffffffffu, row, o));
+    }
+    largest = max(largest, row);
+    row_min = min(row_min, row - 1u);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (col[q]) atomicMax(&col_max[4 * g + q], col[q]);
+  if (lanes < 32) {
+    largest = __reduce_max_sync(0xffffffffu, largest);
+    row_min = __reduce_min_sync(0xffffffffu, row_min);
+  }
+  if (lane == 0) { warp_max[warp] = largest; warp_row[warp] = row_min; }
+  cluster_wait();
+  __syncthreads();
+  if (warp == 0) {
+    largest = __reduce_max_sync(0xffffffffu, warp_max[lane & (WARPS - 1)]);
+    row_min = __reduce_min_sync(0xffffffffu, warp_row[lane & (WARPS - 1)]);
+    // (a block that has a cell to itself fills all places, its own)
+    if (lane < SPLIT_BLOCKS) put_remote(&all_max[solo ? lane : rank], solo ? rank : lane, largest);
+    else if (lane < 2 * SPLIT_BLOCKS && (solo || lane == SPLIT_BLOCKS)) put_remote(&all_row[solo ? lane - SPLIT_BLOCKS : rank], solo ? rank : 0, row_min);
+  } else if (tid >= SPLIT_THREADS - CELL) {
+    const int t = tid & (CELL - 1);
+    if (!solo) put_remote(&all_col[rank][t], 0, col_max[t]);
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  largest = max(max(all_max[0], all_max[1]), max(all_max[2], all_max[3]));
+  const int e = scale_exponent(largest);
+  if (largest < 0x7f800000u) {                             // (infinities, NaN: nobody reads the parts)
+    const float sc = exp2_int(e);
+    long long at = r0 * s.ld_out + c;
+    const long long step = rpi * s.ld_out;
+    __half* const hi = s.hi;
+    __half* const lo = s.lo;
+#pragma unroll
+    for (int i = 0; i < SPLIT_ROWS; ++i, at += step)
+      if (i < n_mine) {
+        uint2 h, l;
+        split4(x[i], sc, h, l);                            // (ld_out is a multiple of 8: a whole group always fits)
+        *reinterpret_cast<uint2*>(hi + at) = h;
+        *reinterpret_cast<uint2*>(lo + at) = l;
       }
-    }
   }
-  if (!SPLIT) {
-    mag = __reduce_max_sync(0xffffffffu, mag);
-    if ((tid & 31) == 0) sh[tid >> 5] = mag;
-    __syncthreads();
-    if (tid == 0) {
-#pragma unroll
-      for (int i = 1; i < 8; ++i) mag = max(mag, sh[i]);
-      s.part[blk] = mag;
-    }
+  if (solo ? panel >= s.rows_ld : rank != 0) return;
+  // Marked: a row or a column whose largest element is not zero but below 2^-20 of the cell's, or anything infinite or NaN.
+  const unsigned least = largest > (FAR_LOG << 23) ? largest - (FAR_LOG << 23) : 1u;
+  bool far = largest >= 0x7f800000u;
+  if (tid < CELL) {
+    const unsigned m = solo ? col_max[tid] : max(max(all_col[0][tid], all_col[1][tid]), max(all_col[2][tid], all_col[3][tid]));
+    far = far || (m != 0u && m < least);
   }
+  if (tid < SPLIT_BLOCKS) far = far || all_row[tid] < least - 1u;                 // (0xffffffff: only zeros)
+  far = __syncthreads_or(far) != 0;
+  if (tid == 0) s.cells[(long long)panel * s.cells_ld + ct] = (int8_t)(far ? kMarked : e);
 }
 
 // 2-D map over a row-major [rows][cols] FP16 matrix with leading dimension ld; box = 64 columns x box_r rows.
@@ -641,7 +796,7 @@ bool make_half_map(CUtensorMap* m, const void* base, long long rows, long long c
 struct HPlan { int bn, whole, rem, slices; double us; };
 
 int chunks_of(const GemmArgs& g, int chunk_kb) {
-  const int kc = chunk_kb * H_BK;
+  const int kc = chunk_kb * H_BK;                          // (1 or 2 k-blocks)
   return (g.K1 + kc - 1) / kc + (g.A2 ? (g.K2 + kc - 1) / kc : 0);
 }
 
@@ -674,7 +829,7 @@ HPlan plan_f16x3(const GemmArgs& g) {
   return best;
 }
 
-HEpilogue make_epilogue(const GemmArgs& g, unsigned* amax_out) {
+HEpilogue make_epilogue(const GemmArgs& g) {
   HEpilogue e{};
   e.M = g.M; e.N = g.N; e.D = g.D; e.ldd = g.ldd; e.bias = g.bias; e.sigmoid = g.sigmoid ? 1 : 0;
   e.dsig = g.dsig; e.ld_dsig = g.ld_dsig; e.dsig_rows = g.dsig_rows > 0 ? g.dsig_rows : 1; e.dsig_div = g.dsig_div > 0 ? g.dsig_div : 1;
@@ -682,7 +837,6 @@ HEpilogue make_epilogue(const GemmArgs& g, unsigned* amax_out) {
   e.alpha = g.alpha; e.cin = g.cin; e.ld_cin = g.ld_cin; e.beta = g.beta;
   e.vec = g.N % 4 == 0 && aligned16(g.D) && g.ldd % 4 == 0 && (!g.bias || aligned16(g.bias)) && (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
           (!g.cin || (aligned16(g.cin) && g.ld_cin % 4 == 0));
-  e.amax_out = amax_out;
   return e;
 }
 
@@ -719,7 +873,7 @@ int64_t gemm_f16x3_workspace_floats(const GemmArgs& g) {
   return (int64_t)(pl.slices > 1 ? pl.slices : 0) * pl.rem * (2 * H_BM) * pl.bn;
 }
 
-int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, unsigned* amax_out, int* err_flag, cudaStream_t st) {
+int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, int* err_flag, cudaStream_t st) {
   if (!gemm_f16x3_usable()) return -1;
   const HPlan pl = plan_f16x3(g);
   if (pl.slices > 1 && !ws) return -1;
@@ -742,16 +896,20 @@ int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, uns
     }
     p.kblocks[s] = s < n_pairs ? (Ks[s] + H_BK - 1) / H_BK : 0;
     for (int q = 0; q < 2; ++q) {
-      p.amax[2 * s + q] = ops[2 * src + q].amax;
-      p.reset[2 * s + q] = s < n_pairs ? ops[2 * s + q].reset : nullptr;
+      p.cells[2 * s + q] = ops[2 * src + q].cells;
+      p.cells_ld[2 * s + q] = ops[2 * src + q].cells_ld;
     }
+    p.src[2 * s] = src ? g.A2 : g.A1; p.ld_src[2 * s] = src ? g.lda2 : g.lda1;
+    p.src[2 * s + 1] = src ? g.B2 : g.B1; p.ld_src[2 * s + 1] = src ? g.ldb2 : g.ldb1;
+    p.K[s] = Ks[src];
   }
-  p.e = make_epilogue(g, amax_out);
+  p.e = make_epilogue(g);
   p.n_pairs = n_pairs;
   p.a_mn = g.a_kmajor ? 0 : 1; p.b_mn = g.b_kmajor ? 0 : 1;
   p.bn = pl.bn;
   p.tiles_n = (g.N + pl.bn - 1) / pl.bn;
-  p.chunk_kb = g.chunk_kb;
+  p.chunk_log = g.chunk_kb - 1;
+  p.chunks0 = (p.kblocks[0] + p.chunk_log) >> p.chunk_log;
   p.whole = pl.whole; p.rem = pl.rem; p.slices = pl.slices;
   p.items = p.whole + p.rem * p.slices;
   const int pairs = num_sms() / 2;
@@ -771,44 +929,28 @@ int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, uns
   return 2;
 }
 
-int launch_split_f16(const SplitJob* jobs, int n, unsigned* part, cudaStream_t st) {
+int launch_split_f16(const SplitJob* jobs, int n, cudaStream_t st) {
   if (n < 1 || n > kSplitSegs) return -1;
-  SplitList all{}, need{};
-  int blocks_all = 0, blocks_need = 0;
+  SplitList list{};
+  long long clusters = 0;
   for (int i = 0; i < n; ++i) {
     const SplitJob& j = jobs[i];
-    SplitSeg s{};
+    SplitSeg& s = list.s[list.n++];
     s.src = j.src; s.rows = j.rows; s.cols = j.cols; s.ld = j.ld;
     s.hi = static_cast<__half*>(j.hi); s.lo = static_cast<__half*>(j.lo); s.ld_out = j.ld_out;
-    s.bits = j.bits;
+    s.cells = j.cells; s.cells_ld = (j.cols + CELL - 1) / CELL;
     s.vec = j.cols % 4 == 0 && j.ld % 4 == 0 && aligned16(j.src);
-    const int per_row = (j.cols + 3) / 4;
-    const int rpb = per_row < 256 ? 256 / per_row : 1;
-    long long b = (j.rows + rpb - 1) / rpb;
-    b = (b + 3) / 4;                                       // (four rows in flight per thread)
-    if (b < 1) b = 1;
-    if (b > kSplitBlocks / n) b = kSplitBlocks / n;
-    s.blocks = (int)b;
-    s.block0 = blocks_all;
-    blocks_all += s.blocks;
-    if (j.acc) {                                           // the producer's epilogue has left the maximum
-      s.part = j.acc; s.n_part = 1;
-    } else {
-      s.part = part + s.block0; s.n_part = s.blocks;
-      SplitSeg q = s;
-      q.block0 = blocks_need;
-      blocks_need += q.blocks;
-      need.s[need.n++] = q;
-    }
-    all.s[all.n++] = s;
+    const bool narrow = j.cols - (s.cells_ld - 1) * CELL <= 32;
+    const long long panels = (j.rows + CELL - 1) / CELL;
+    if (panels * s.cells_ld > 0x7fffffff / SPLIT_BLOCKS) return -1;
+    s.rows_ld = (int)panels;
+    s.wide_ld = s.cells_ld - (narrow ? 1 : 0);
+    s.wide = (int)panels * s.wide_ld;
+    s.cluster0 = (int)clusters;
+    clusters += s.wide + (narrow ? (panels + SPLIT_BLOCKS - 1) / SPLIT_BLOCKS : 0);
+    if (clusters > 0x7fffffff / SPLIT_BLOCKS) return -1;
   }
-  int launches = 0;
-  if (need.n) {
-    if (launch_pdl(split_f16_kernel<false>, blocks_need, 256, 0, st, need) != cudaSuccess) return -1;
-    ++launches;
-  }
-  if (launch_pdl(split_f16_kernel<true>, blocks_all, 256, 0, st, all) != cudaSuccess) return -1;
-  return launches + 1;
+  return launch_pdl(split_f16_kernel, (int)clusters * SPLIT_BLOCKS, SPLIT_THREADS, 0, st, list) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace gn

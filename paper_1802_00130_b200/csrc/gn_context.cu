@@ -95,8 +95,12 @@ struct gn_ctx {
   int acc_method = 0;        // 0 choose (tensor cores where they are faster), 1 FP32 FMA only, 2 as 0
   bool x3_usable = true;     // cleared if the tensor-core kernel could not be launched
   uint64_t theta_epoch = 1, sub_epoch = 1;   // bumped whenever theta / the stored activations are rewritten
-  // [hi part: cap elements][lo part: cap elements][bit pattern of the largest magnitude]
-  struct SplitBuf { uint16_t* p = nullptr; int64_t cap = 0; unsigned* bits() const { return reinterpret_cast<unsigned*>(p + 2 * cap); } };
+  // [hi part: cap elements][lo part: cap elements][exponents of the cells, in whole 16 bytes]
+  struct SplitBuf {
+    uint16_t* p = nullptr; int64_t cap = 0;
+    int8_t* cells() const { return reinterpret_cast<int8_t*>(p + 2 * cap); }
+    static int64_t elements(int64_t cap) { return 2 * cap + (split_cell_bytes(cap) + 15) / 16 * 8; }
+  };
   // Parts kept until the matrix changes: of matrices inside theta (kind 1) and the stored Z_m (kind 2), and, for the
   // length of one launch sequence, inside the product's v (kind 3) and the row batch's X and Z_m (kind 4).  The key is
   // the matrix's place in those, never an address of the caller's.  Whole layers' matrices have their place in one
@@ -111,15 +115,9 @@ struct gn_ctx {
     uint64_t seq = 0;        // contraction (gemm_seq) that wrote these parts
   };
   SplitSlot split_slot[4];
-  unsigned* split_part = nullptr;                          // scratch of the splitting pass, then kMaxRecords maxima
-  SplitOperand h_ops[4]; unsigned* h_amax_out = nullptr;   // of the contraction being launched
-  // max|D| accumulated by the contraction that produced D, for the splitting pass of a later contraction of the SAME
-  // launch sequence (R z^m, delta s^m, Z_m): valid only while parts_epoch stands (every launch sequence that may
-  // rewrite those buffers bumps it).  dirty: the word has not been cleared by a consumer yet.
-  struct AmaxEntry { const float* src = nullptr; int64_t rows = 0; int cols = 0; int64_t ld = 0; uint64_t epoch = 0; unsigned* acc = nullptr; bool dirty = false; };
-  std::vector<AmaxEntry> amax;
+  SplitOperand h_ops[4];                                   // of the contraction being launched
   uint64_t parts_epoch = 1;
-  bool amax_enabled = true;
+  bool split_together = true;                              // a contraction's operands in one splitting launch (else one each)
   bool own_capture = false, foreign_capture = false;       // the solver's step / the caller is capturing the stream
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
   float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
@@ -332,7 +330,7 @@ void run_gemm_kind(gn_ctx* c, const GemmArgs& g, int kind, cudaStream_t st = nul
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "cuTensorMapEncodeTiled failed"; }
     else c->launches += r;
   } else if (kind == 3) {
-    const int r = launch_gemm_f16x3(g, c->h_ops, c->sk_ws, c->h_amax_out, c->err_flag + 1, st);
+    const int r = launch_gemm_f16x3(g, c->h_ops, c->sk_ws, c->err_flag + 1, st);
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "the FP32-accurate tensor-core kernel could not be launched"; c->x3_usable = false; ++c->dispatch_gen; }
     else c->launches += r;
   } else if (kind == 2) {
@@ -361,19 +359,9 @@ bool split_buf_reserve(gn_ctx* c, gn_ctx::SplitBuf& b, int64_t need) {
   cudaStreamSynchronize(c->st);   // an earlier contraction may still be reading the old buffer
   dev_free(c, b.p);
   b.cap = 0;
-  if (dev_alloc(c, &b.p, 2 * need + 8) != GN_OK) return false;
+  if (dev_alloc(c, &b.p, gn_ctx::SplitBuf::elements(need)) != GN_OK) return false;
   b.cap = need;
   return true;
-}
-
-// The matrices whose maxima are recorded live in the subsample and row-batch workspaces: when those move, the records
-// kept for their old addresses go.
-constexpr size_t kMaxRecords = 256;
-void drop_amax(gn_ctx* c) { c->amax.clear(); }
-
-gn_status ensure_split_scratch(gn_ctx* c) {
-  if (c->split_part) return GN_OK;
-  return dev_alloc(c, &c->split_part, kSplitBlocks + (int64_t)kMaxRecords);
 }
 
 // The parts of kind `kind` go (their workspace is about to move or to change size).
@@ -401,7 +389,7 @@ bool arena_buffer(gn_ctx* c, int kind, int64_t key, int64_t rows, int cols, int6
     const int64_t n = vec ? (int64_t)c->w[m + 1] * round8(c->w[m]) : cap_rows * round8(c->w[m]);
     const int64_t k = vec ? c->w_off[m + 1] : (int64_t)m << 48;
     if (key == k && cols == c->w[m] && ld == c->w[m] && rows <= (vec ? c->w[m + 1] : cap_rows)) { at = total; size = n; }
-    total += 2 * n + 8;
+    total += gn_ctx::SplitBuf::elements(n);
   }
   if (at < 0) return false;
   if (!c->arena[kind]) {
@@ -491,25 +479,20 @@ bool split_operand(gn_ctx* c, const float* src, int64_t rows, int cols, int64_t 
     sl.seq = c->gemm_seq;
     buf = &sl.buf;
   }
-  out->hi = buf->p; out->lo = buf->p + buf->cap; out->ld = ldo; out->amax = buf->bits(); out->reset = nullptr;
+  out->hi = buf->p; out->lo = buf->p + buf->cap; out->ld = ldo; out->cells = buf->cells(); out->cells_ld = (cols + 127) / 128;
   if (!fresh) {
     SplitJob j{};
     j.src = src; j.rows = rows; j.cols = cols; j.ld = ld;
-    j.hi = buf->p; j.lo = buf->p + buf->cap; j.ld_out = ldo; j.bits = buf->bits();
-    for (auto& e : c->amax)
-      if (e.src == src && e.dirty && e.epoch == c->parts_epoch && e.rows == rows && e.cols == cols && e.ld == ld) {
-        j.acc = e.acc;                       // recorded by the contraction that produced this operand
-        out->reset = e.acc;
-        e.dirty = false;
-      }
+    j.hi = buf->p; j.lo = buf->p + buf->cap; j.ld_out = ldo; j.cells = buf->cells();
     jobs.push_back(j);
   }
   return true;
 }
 
 void run_splits(gn_ctx* c, const std::vector<SplitJob>& jobs) {
-  for (size_t i = 0; i < jobs.size(); i += kSplitSegs) {
-    const int r = launch_split_f16(jobs.data() + i, (int)std::min<size_t>(kSplitSegs, jobs.size() - i), c->split_part, c->st);
+  const size_t together = c->split_together ? kSplitSegs : 1;
+  for (size_t i = 0; i < jobs.size(); i += together) {
+    const int r = launch_split_f16(jobs.data() + i, (int)std::min<size_t>(together, jobs.size() - i), c->st);
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "an operand could not be split"; return; }
     c->launches += r;
   }
@@ -538,38 +521,18 @@ bool run_gemm_f16x3(gn_ctx* c, const GemmArgs& args) {
   if (!c->x3_usable || !gemm_f16x3_usable() || g.K1 < 1 || (g.A2 && g.K2 < 1)) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   c->foreign_capture = !c->own_capture && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
-  if (ensure_split_scratch(c) != GN_OK) return false;
   if (!c->sk_enabled || (gemm_f16x3_workspace_floats(g) > 0 && ensure_sk_workspace(c) != GN_OK)) g.whole_tiles = true;
-  // (the record of the result's maximum first: what follows takes records away, and must not be undone)
-  gn_ctx::AmaxEntry* ae = nullptr;
-  if (g.emit_amax && c->amax_enabled) {
-    for (auto& e : c->amax)
-      if (e.src == g.D) { ae = &e; break; }
-    if (!ae && c->amax.size() < kMaxRecords) {
-      gn_ctx::AmaxEntry e;
-      e.acc = c->split_part + kSplitBlocks + c->amax.size();
-      e.src = g.D; e.dirty = true;
-      c->amax.push_back(e);
-      ae = &c->amax.back();
-    }
-  }
   std::vector<SplitJob> jobs;
   SplitOperand ops[4];
   for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
     const OperandView v = operand_view(g, role);
     if (!split_operand(c, v.p, v.rows, v.cols, v.ld, role, role == 0 && g.a1_split_fresh, &ops[role], jobs)) {
       run_splits(c, jobs);                       // (what has been recorded as split must be)
-      for (auto& e : c->amax) { e.epoch = 0; e.dirty = true; }
       return false;
     }
   }
   run_splits(c, jobs);
-  if (ae) {
-    if (ae->dirty) cudaMemsetAsync(ae->acc, 0, sizeof(unsigned), c->st);   // (new, or nobody read the last record)
-    ae->rows = g.M; ae->cols = g.N; ae->ld = g.ldd; ae->epoch = c->parts_epoch; ae->dirty = true;
-  }
   for (int k = 0; k < 4; ++k) c->h_ops[k] = ops[k];
-  c->h_amax_out = ae ? ae->acc : nullptr;
   run_gemm_kind(c, g, 3);
   return true;
 }
@@ -638,7 +601,6 @@ void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
   for (int i = 0; i < n; ++i) {
     const GemmArgs& g = gs[i];
     if (!goes_f16x3(c, g)) continue;
-    if (ensure_split_scratch(c) != GN_OK) return;
     for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
       const OperandView v = operand_view(g, role);
       int64_t key = 0;
@@ -848,7 +810,6 @@ void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>&
     g.sigmoid = m < c->L;
     dep[(size_t)m - 1] = m - 2;          // layer m reads the rows layer m - 1 writes
   }
-  for (int m = 1; m < c->L; ++m) gs[(size_t)m - 1].emit_amax = goes_f16x3(c, gs[(size_t)m]);   // Z_m feeds layer m + 1
   presplit(c, gs.data(), c->L, 0x2);       // theta's weights
   run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), c->L);
 }
@@ -899,7 +860,6 @@ GemmArgs backward_data_args(const gn_ctx* c, int m, const float* ds, int64_t row
   g.dsig = Zprev; g.ld_dsig = c->w[m - 1]; g.dsig_rows = (int)z_rows;
   g.D = dst; g.ldd = c->w[m - 1];
   g.mn_padded = true;     // B is the context's own (padded) copy of theta
-  g.emit_amax = ds_just_used;   // in the full product and the gradient, delta s^{m-1} feeds the two contractions of layer m - 1
   return g;
 }
 
@@ -1006,7 +966,6 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
       g.D = c->RZ[m]; g.ldd = c->w[m];
       dep[(size_t)m - 1] = m - 2;        // R z^{m-1} of the layer below
     }
-    for (int m = 1; m < L; ++m) gs[(size_t)m - 1].emit_amax = goes_f16x3(c, gs[(size_t)m]);   // R z^m feeds layer m + 1
     presplit(c, gs.data(), L, 0xf);
     run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), L, 2);
   }
@@ -1027,7 +986,6 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
 gn_status ensure_stacked(gn_ctx* c) {
   if (c->stacked) return GN_OK;
   quiesce(c);
-  drop_amax(c);
   for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m]); dev_free(c, c->DS[m]); }
   c->stacked = true;
   for (int m = 1; m <= c->L; ++m) {
@@ -1321,7 +1279,6 @@ gn_status ensure_batch(gn_ctx* c) {
   const int64_t rows = c->batch_rows < c->l ? c->batch_rows : c->l;
   if (rows <= c->capB) return GN_OK;
   quiesce(c);
-  drop_amax(c);
   drop_kept_parts(c, 4);
   for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
   c->capB = 0;
@@ -1585,8 +1542,7 @@ gn_status gn_set_batch_rows(gn_ctx* c, int64_t rows) {
   if ((rows < c->l ? rows : c->l) != c->capB && c->capB > 0) {
     // shrink or grow on next use: drop the old workspace now so memory stays bounded
     quiesce(c);
-    drop_amax(c);
-    drop_kept_parts(c, 4);
+      drop_kept_parts(c, 4);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
     c->capB = 0;
   }
@@ -1680,8 +1636,7 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   if (nS > c->capS) {
     GN_TRY(sync(c, "set_subsample"));
     drop_kept_parts(c, 2);      // the stored activations move: their parts are made anew
-    drop_amax(c);
-    dev_free(c, c->idx, c->capS);
+      dev_free(c, c->idx, c->capS);
     for (int m = 0; m <= c->L; ++m) dev_free(c, c->Z[m], c->capS * c->w[m]);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m], m * c->capS * c->w[m]); dev_free(c, c->DS[m], m * c->capS * c->w[m]); }
     c->capS = 0;
@@ -2066,7 +2021,7 @@ gn_status gn_debug_option(gn_ctx* c, int option, int value) {
   if (option == 10) { c->small_enabled = value != 0; return GN_OK; }
   if (option == 9) { c->fly_enabled = value != 0; return GN_OK; }
   if (option == 6) { c->graph_enabled = value != 0; return GN_OK; }
-  if (option == 5) { c->amax_enabled = value != 0; return GN_OK; }
+  if (option == 5) { c->split_together = value != 0; return GN_OK; }
   if (option == 4) { c->chain_level = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }
   if (option == 0) c->group_enabled = value != 0;
   else if (option == 1) c->sk_enabled = value != 0 && c->sk_enabled;

@@ -25,7 +25,6 @@ struct GemmArgs {
   bool a1_split_fresh = false;   // caller's word that A1 is, unchanged, the A1 of the previous contraction
   int chunk_kb = 1;              // FP32-accurate tensor-core form: 64-term k-blocks per accumulation in tensor memory
   bool whole_tiles = false;      // ... without K slices (no workspace)
-  bool emit_amax = false;        // the result is an operand of a later contraction of this launch sequence
   bool a_kmajor = true, b_kmajor = true;
   bool mn_padded = false;  // every MN-major operand is followed by >= 128 readable bytes
   int two_cta = -1;        // tensor-core kernel: -1 choose, 0 one CTA per tile, 1 CTA pair per 256-row tile
@@ -75,26 +74,26 @@ double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K,
 
 // FP32-accurate contraction on the FP16 tensor cores (gemm_f16x3.cu): any shape and alignment, because it reads
 // split copies of its operands.
-//   SplitOperand  the two FP16 parts of a stored matrix X (X 2^e = hi + lo; leading dimension a multiple of 8, 16-byte
-//                 aligned) and the device word with the bit pattern of max|X| that e follows from; `reset`, if set, is a
-//                 word the contraction clears (see SplitJob::acc).
-//   SplitJob      one matrix to be split.  acc: a device word into which the contraction that produced the matrix has
-//                 accumulated max|X| (amax_out below), or nullptr to have it found in a pass of its own.
+//   SplitOperand  the two FP16 parts of a stored matrix X (leading dimension a multiple of 8, 16-byte aligned) and one
+//                 byte per 128 x 128 cell of it, cells_ld of them per 128 rows: the exponent e of X 2^e = hi + lo, or the mark
+//                 that the parts do not hold the cell and the contraction is to read X itself, which GemmArgs points to.
+//   SplitJob      one matrix to be split.
 // ops: A1, B1, A2, B2.  ws: gemm_f16x3_workspace_floats(g) floats (K slices; never more than
-// gemm_tf32_workspace_floats()).  amax_out: if set, atomically raised to the bit pattern of the largest finite |D|.
-// Both return launches made, or -1 if the launch failed.
-struct SplitOperand { const void* hi = nullptr; const void* lo = nullptr; int64_t ld = 0; const unsigned* amax = nullptr; unsigned* reset = nullptr; };
+// gemm_tf32_workspace_floats()).  Both return launches made, or -1 if the launch failed.
+struct SplitOperand { const void* hi = nullptr; const void* lo = nullptr; int64_t ld = 0; const int8_t* cells = nullptr; int cells_ld = 0; };
 struct SplitJob {
   const float* src; int64_t rows; int cols; int64_t ld;
-  void* hi; void* lo; int64_t ld_out; unsigned* bits; unsigned* acc;
+  void* hi; void* lo; int64_t ld_out; int8_t* cells;
 };
+// Bytes that hold the cells of any matrix of at most `cap` elements with its rows rounded up to 8: cap / 4096 where it has a
+// cell's rows and columns or more, else one per 128 rows (of 8 elements at least) or columns.
+inline int64_t split_cell_bytes(int64_t cap) { return cap / 128 + 16; }
 constexpr int kSplitSegs = 8;
-constexpr int kSplitBlocks = 148 * 8;   // blocks of a splitting launch at most; `part` holds that many words
 bool gemm_f16x3_usable();
 double gemm_f16x3_estimate_us(const GemmArgs& g);
 int64_t gemm_f16x3_workspace_floats(const GemmArgs& g);
-int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, unsigned* amax_out, int* err_flag, cudaStream_t st);
-int launch_split_f16(const SplitJob* jobs, int n, unsigned* part, cudaStream_t st);
+int launch_gemm_f16x3(const GemmArgs& g, const SplitOperand* ops, float* ws, int* err_flag, cudaStream_t st);
+int launch_split_f16(const SplitJob* jobs, int n, cudaStream_t st);
 
 // Whole passes of a small network (small_net.cu).  kind 0: G^S v, 1: block-diagonal G^S v, 2: loss and gradient, 3: loss,
 // 4: row gather and stored forward pass.  The blocks' sums go to scratch (small_net_blocks(rows) * n floats) and their losses to

@@ -64,28 +64,121 @@ def test_scales_of_the_operands(ctx, ea, eb):
         assert np.linalg.norm(np.ldexp(D, ea + eb - 4) - E) <= 1e-5 * np.linalg.norm(E)
 
 
-def test_wide_range_inside_an_operand(ctx):
-    """Rows of A over twelve decades: every row is as accurate as an absolute error of 2^-40 max|A| per element leaves it."""
-    A, B, _ = operands(256, 64, 320, True, False)
-    scale = 10.0 ** -np.linspace(0, 12, 256)
-    A = (A * scale[:, None]).astype(np.float32)
-    ref = A.astype(np.float64) @ B.astype(np.float64)
-    err = np.linalg.norm(product(ctx, A, B, True, False) - ref, axis=1)
-    bound = 1e-6 * np.linalg.norm(ref, axis=1) + 2.0 ** -40 * np.abs(A).max() * np.linalg.norm(B)
-    assert np.all(err <= bound)
+def decades(n, d):
+    return 10.0 ** -np.linspace(0, d, n)
 
 
-def test_zero_operands_and_non_finite_elements(ctx):
-    A, B, ref = operands(300, 140, 200, True, True)
+# what is scaled, over how many decades, and whether the other operand is scaled the other way (so that all terms of a sum
+# are of one size); "one" = a single row of 10^-d, "half" = the first half of K
+RANGES = [("m", 12, False), ("m", 30, False), ("n", 12, False), ("k", 6, True), ("k", 8, True), ("k", 10, True), ("k", 16, True),
+          ("k", 30, True), ("k", 12, False), ("large m", 55, False), ("one m", 12, False), ("one k", 10, True), ("half k", 20, True)]
+
+
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, False)])
+@pytest.mark.parametrize("which,d,compensated", RANGES)
+def test_wide_range_inside_an_operand(ctx, which, d, compensated, a_k, b_k):
+    """Element by element as accurate as any FP32 sum, whatever the range of an operand."""
+    M, N, K = 300, 200, 333
+    A, B, _ = operands(M, N, K, a_k, b_k)
+    Am, Bm = (A if a_k else A.T), (B.T if b_k else B)          # views: [M][K], [K][N]
+    ax = which.split()[-1]
+    n = {"m": M, "n": N, "k": K}[ax]
+    f = decades(n, d)
+    if which.startswith("one"):
+        f = np.where(np.arange(n) == n // 3, 10.0 ** -d, 1.0)
+    elif which.startswith("half"):
+        f = np.where(np.arange(n) < n // 2, 10.0 ** -d, 1.0)
+    elif which.startswith("large"):
+        f *= 1e35
+    if ax == "m":
+        Am *= f.astype(np.float32)[:, None]
+    elif ax == "n":
+        Bm *= f.astype(np.float32)[None, :]
+    else:
+        Am *= f.astype(np.float32)[None, :]
+        if compensated:
+            Bm *= (1.0 / f).astype(np.float32)[:, None]
+    D = product(ctx, A, B, a_k, b_k)
+    ref = Am.astype(np.float64) @ Bm.astype(np.float64)
+    bound = np.abs(Am).astype(np.float64) @ np.abs(Bm).astype(np.float64)
+    assert np.all(np.abs(D - ref) <= 2e-6 * bound)             # (the bound of test_against_float64)
+    rows, cols = np.linalg.norm(D - ref, axis=1), np.linalg.norm(D - ref, axis=0)
+    assert np.all(rows <= 2e-6 * np.linalg.norm(ref, axis=1)) and np.all(cols <= 2e-6 * np.linalg.norm(ref, axis=0))
+
+
+@pytest.mark.parametrize("shape", [(300, 200, 333), (26, 803, 4001), (700, 65, 64)])
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, True), (False, False)])
+def test_sparse_operands_with_a_small_row_or_column(ctx, shape, a_k, b_k):
+    """Mostly zeros, and one column of A of 10^-12 against a row of B of 10^12: (also where K is cut into slices)."""
+    M, N, K = shape
+    A, B, _ = operands(M, N, K, a_k, b_k)
+    Am, Bm = (A if a_k else A.T), (B.T if b_k else B)
+    Am *= np.random.Generator(np.random.PCG64(1)).random((M, K)) < 0.2
+    Am[:, K // 2] *= np.float32(1e-12)
+    Bm[K // 2] *= np.float32(1e12)
+    D = product(ctx, A, B, a_k, b_k)
+    ref = Am.astype(np.float64) @ Bm.astype(np.float64)
+    bound = np.abs(Am).astype(np.float64) @ np.abs(Bm).astype(np.float64)
+    assert np.all(np.abs(D - ref) <= 2e-6 * bound)
+
+
+def test_zero_operands(ctx):
+    A, B, _ = operands(300, 140, 200, True, True)
     assert not product(ctx, np.zeros_like(A), B, True, True).any()
     assert not product(ctx, A, np.zeros_like(B), True, True).any()
-    A[7, 11], A[290, 3], B[100, 5] = np.inf, np.nan, -np.inf
-    D = product(ctx, A, B, True, True)
-    bad = np.zeros(D.shape, bool)
-    bad[[7, 290], :] = True
-    bad[:, 100] = True
-    assert not np.isfinite(D[bad]).any()      # as in any FP32 sum: the rows and the column that meet them, and no others
-    assert np.linalg.norm(D[~bad] - ref[~bad]) <= 1e-6 * np.linalg.norm(ref[~bad])
+
+
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, True), (False, False)])
+def test_infinities_and_nan_as_in_any_fp32_sum(ctx, a_k, b_k):
+    A, B, _ = operands(300, 140, 200, a_k, b_k)
+    Am, Bm = (A if a_k else A.T), (B.T if b_k else B)
+    Am[7, 11], Am[290, 3], Am[130, 199], Bm[5, 100] = np.inf, np.nan, -np.inf, -np.inf
+    Bm[11, 20] = 0.0                          # inf * 0
+    D = product(ctx, A, B, a_k, b_k)
+    with np.errstate(invalid="ignore"):
+        ref = np.stack([(Am[i].astype(np.float64)[:, None] * Bm.astype(np.float64)).sum(0) for i in range(300)])
+    ok = np.isfinite(ref)
+    assert ok.sum() == (300 - 3) * 139
+    assert np.array_equal(D[~ok], ref[~ok], equal_nan=True)
+    assert np.linalg.norm(D[ok] - ref[ok]) <= 1e-6 * np.linalg.norm(ref[ok])
+
+
+def test_an_infinite_pre_activation_is_a_saturated_unit(ctx):
+    """... through the epilogue: the sigmoid of an infinite sum is 0 or 1."""
+    import torch
+    A, B, ref = operands(260, 130, 100, True, True)
+    A[3, 4], A[200, 9] = np.inf, -np.inf
+    D = ctx.debug_gemm_epilogue(8, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), sigmoid=True).cpu().numpy()
+    want = 1.0 / (1.0 + np.exp(-ref))
+    want[3], want[200] = B[:, 4] > 0, B[:, 9] < 0
+    assert np.max(np.abs(D - want)) <= 1e-5
+
+
+@pytest.mark.parametrize("d", [4, 6, 8, 10])
+def test_unnormalised_features(d):
+    """Features over d decades with the first layer's weights scaled the other way: the gradient and the product, column by
+    column of the first weight block (each belongs to one feature)."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    from oracle import gn_oracle as orc
+    w = (200, 164, 5)
+    p = wl.make_custom(w, 1500, 1100, 15.0, seed=4)
+    f = decades(200, d)
+    X = (p["X"] * f[None, :]).astype(np.float32)
+    th, v = p["theta"].copy(), p["v"].copy()
+    for t in (th, v):
+        t[: 200 * 164] = (t[: 200 * 164].reshape(164, 200) / f[None, :]).astype(np.float32).ravel()
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    C = 1e30                                  # (the regularisation terms would hide the small columns)
+    c = gn.GnContext(list(w), C, dev(X), dev(p["Y"]))
+    c.profile(True)
+    c.set_theta(dev(th))
+    c.set_subsample(dev(p["idx"]))
+    for got, want in ((c.grad(), orc.grad(th, w, C, X, p["Y"])), (c.Gv(dev(v)), orc.Gv(th, w, C, X[p["idx"]], v))):
+        got, want = (np.asarray(a, np.float64)[: 200 * 164].reshape(164, 200) for a in (got.cpu().numpy(), want))
+        assert np.all(np.linalg.norm(got - want, axis=0) <= 1e-5 * np.linalg.norm(want, axis=0))
+    assert c.profile_read()["tensor_x3"]["launches"] > 0
+    c.close()
 
 
 @pytest.mark.parametrize("widths", [(37, 129, 131, 3), (617, 203, 150, 26), (50, 300, 17)])

@@ -60,9 +60,8 @@ def test_grouped_launches_give_the_bits_of_single_launches(name):
 
 @pytest.mark.parametrize("name", ["mid", "deep", "mnist2000_5"])
 def test_parts_written_by_the_epilogue_are_the_parts_a_separate_pass_would_write(name):
-    """FP32-accurate mode: the error-compensated kernel writes the hi / lo TF32 parts of a result that a later
-    contraction of the same product (or row batch) takes as an operand.  Same bits as splitting that result in a pass
-    of its own, fewer launches, and the mode's bound against the float64 checker."""
+    """FP32-accurate mode: the operands of a contraction are split by one launch.  Same bits as a launch per operand,
+    fewer launches, and the mode's bound against the float64 checker."""
     import torch
     p = CASES[name]()
     outs = []
