@@ -100,6 +100,13 @@ __device__ __forceinline__ void mma2_f16(uint32_t tmem_d, uint64_t adesc, uint64
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
 
+// The epilogue as it is after grid_dep_wait (see dep()).
+__device__ __forceinline__ HEpilogue after_wait(const HEpilogue& in) {
+  HEpilogue e = in;
+  e.bias = dep(e.bias); e.dsig = dep(e.dsig); e.cin = dep(e.cin);
+  return e;
+}
+
 __device__ __forceinline__ long long dsig_row(const HEpilogue& e, int m) {
   return e.dsig_direct ? m : (m / e.dsig_div) % e.dsig_rows;
 }
@@ -489,13 +496,12 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
     const uint32_t stg = smem_u32(smem + H_STAGES * H_STAGE_BYTES) + (uint32_t)(warp - 4) * 4096u;
-    const HEpilogue& e = p.e;
     int ci = 0;
     bool alive = true;
     for (int item = pair; item < p.items && alive; item += p.P) {
       const Item w = item_at(p, item, n_chunks);
       const int m0 = (w.tile / p.tiles_n) * (2 * H_BM) + (int)rank * H_BM + quad * 32, n0 = (w.tile % p.tiles_n) * bn;
-      const int n_cc = min(bn / 32, (e.N - n0 + 31) / 32);       // column chunks of this tile that exist
+      const int n_cc = min(bn / 32, (p.e.N - n0 + 31) / 32);     // column chunks of this tile that exist
       float run[4][32];                                          // this warp's chunks: half, half + 2, half + 4, half + 6
 #pragma unroll
       for (int j = 0; j < 4; ++j)
@@ -564,8 +570,8 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
       for (int j = 0; j < 4; ++j)
         if (j < n_mine) tmem_st32(ta + (uint32_t)(j * 64), run[j]);
       tmem_st_wait();
-      if (m0 < e.M) {                                            // warp-uniform
-        const int rows = min(32, e.M - m0), nb0 = n0 + half * 32;
+      if (m0 < p.e.M) {                                          // warp-uniform
+        const int rows = min(32, p.e.M - m0), nb0 = n0 + half * 32;
         if (w.slot >= 0) {                                       // (the workspace holds whole tiles)
           float* o = p.ws + ((long long)w.slot * (2 * H_BM) + (int)rank * H_BM + quad * 32 + (lane >> 3)) * bn + half * 32 + (lane & 7) * 4;
 #pragma unroll 1
@@ -585,7 +591,7 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
               __stcg(reinterpret_cast<float4*>(o + 4 * r * bn + 64 * j), make_float4(x[r][0], x[r][1], x[r][2], x[r][3]));
           }
         } else {
-          store_tile<MODE, VEC>(e, stg, ta, n_mine, m0, rows, nb0, lane);
+          store_tile<MODE, VEC>(after_wait(p.e), stg, ta, n_mine, m0, rows, nb0, lane);
         }
       }
       tc_fence_before();
@@ -603,10 +609,12 @@ gemm_f16x3_kernel(const __grid_constant__ HMaps maps, const __grid_constant__ HP
 
 // Sum of the K slices of the left-over tiles, slice 0 first, and the epilogue.  blockIdx.x = 32-column chunk of a left-over
 // tile, warp = row, lane = column; bound by the reads of the workspace, which the kernel before it has left in L2.
-__global__ void __launch_bounds__(256) slice_sum_kernel(const HEpilogue e, const float* __restrict__ ws, int whole, int rem, int slices,
+__global__ void __launch_bounds__(256) slice_sum_kernel(const HEpilogue epi, const float* __restrict__ ws, int whole, int rem, int slices,
                                                         int tiles_n, int bn) {
   grid_dep_wait();
   grid_dep_launch();
+  const HEpilogue e = after_wait(epi);
+  ws = dep(ws);
   const int lane = threadIdx.x & 31;
   const int per_tile = bn / 32;
   const int j = blockIdx.x / per_tile, c = (blockIdx.x - j * per_tile) * 32 + lane;

@@ -131,11 +131,14 @@ __global__ void __launch_bounds__(NT, 2) gemm_ffma_kernel(const FfmaParams p) {
   }
 
   // ---- epilogue
+  const float* const bias = dep(p.bias);
+  const float* const dsig = dep(p.dsig);
+  const float* const cin = dep(p.cin);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int m = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
     if (m >= p.M) continue;
-    const long long zrow = p.dsig ? (long long)((m / p.dsig_div) % p.dsig_rows) * p.ld_dsig : 0;
+    const long long zrow = dsig ? (long long)((m / p.dsig_div) % p.dsig_rows) * p.ld_dsig : 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int n = n0 + h * 64 + tx * 4;
@@ -145,23 +148,23 @@ __global__ void __launch_bounds__(NT, 2) gemm_ffma_kernel(const FfmaParams p) {
       const int cnt = min(4, p.N - n);
       float bz[4] = {0.f, 0.f, 0.f, 0.f}, zc[4] = {0.f, 0.f, 0.f, 0.f}, ci[4] = {0.f, 0.f, 0.f, 0.f};
       if (v4) {
-        if (p.bias) { const float4 x = __ldg(reinterpret_cast<const float4*>(p.bias + n)); bz[0] = x.x; bz[1] = x.y; bz[2] = x.z; bz[3] = x.w; }
-        if (p.dsig) { const float4 x = __ldg(reinterpret_cast<const float4*>(p.dsig + zrow + n)); zc[0] = x.x; zc[1] = x.y; zc[2] = x.z; zc[3] = x.w; }
-        if (p.cin)  { const float4 x = __ldg(reinterpret_cast<const float4*>(p.cin + (long long)m * p.ld_cin + n)); ci[0] = x.x; ci[1] = x.y; ci[2] = x.z; ci[3] = x.w; }
+        if (bias) { const float4 x = __ldg(reinterpret_cast<const float4*>(bias + n)); bz[0] = x.x; bz[1] = x.y; bz[2] = x.z; bz[3] = x.w; }
+        if (dsig) { const float4 x = __ldg(reinterpret_cast<const float4*>(dsig + zrow + n)); zc[0] = x.x; zc[1] = x.y; zc[2] = x.z; zc[3] = x.w; }
+        if (cin)  { const float4 x = __ldg(reinterpret_cast<const float4*>(cin + (long long)m * p.ld_cin + n)); ci[0] = x.x; ci[1] = x.y; ci[2] = x.z; ci[3] = x.w; }
       } else {
         for (int j = 0; j < cnt; ++j) {
-          if (p.bias) bz[j] = __ldg(p.bias + n + j);
-          if (p.dsig) zc[j] = __ldg(p.dsig + zrow + n + j);
-          if (p.cin)  ci[j] = __ldg(p.cin + (long long)m * p.ld_cin + n + j);
+          if (bias) bz[j] = __ldg(bias + n + j);
+          if (dsig) zc[j] = __ldg(dsig + zrow + n + j);
+          if (cin)  ci[j] = __ldg(cin + (long long)m * p.ld_cin + n + j);
         }
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         float x = t[j] + bz[j];
         if (p.sigmoid) x = 1.f / (1.f + expf(-x));
-        if (p.dsig) x *= zc[j] * (1.f - zc[j]);
+        if (dsig) x *= zc[j] * (1.f - zc[j]);
         x *= p.alpha;
-        if (p.cin) x = fmaf(p.beta, ci[j], x);
+        if (cin) x = fmaf(p.beta, ci[j], x);
         t[j] = x;
       }
       float* dp = p.D + (long long)m * p.ldd + n;

@@ -208,6 +208,9 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
     // Two warps per tensor-memory quadrant; the pair alternates over the tile's 32-column chunks.
     const int quad = warp & 3;            // tensor-memory lanes 32*quad .. 32*quad+31 are this warp's
     const int half = (warp - 2) >> 2;     // 0 or 1: which chunks of the tile this warp takes
+    const float* const bias = dep(p.bias);
+    const float* const dsig = dep(p.dsig);
+    const float* const cin = dep(p.cin);
     int ti = 0;
     for (int t = blockIdx.x; t < p.tiles; t += gridDim.x, ++ti) {
       const int m0 = (t / p.tiles_n) * BM, n0 = (t % p.tiles_n) * bn;
@@ -223,8 +226,8 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
       // moves 16 bytes per access and a row's 128 bytes are completed by consecutive accesses.
       const int m = m0 + quad * 32 + lane;
       const bool m_ok = m < p.M;
-      const float* zrow = p.dsig ? p.dsig + (long long)((m / p.dsig_div) % p.dsig_rows) * p.ld_dsig : nullptr;
-      const float* crow = p.cin ? p.cin + (long long)m * p.ld_cin : nullptr;
+      const float* zrow = dsig ? dsig + (long long)((m / p.dsig_div) % p.dsig_rows) * p.ld_dsig : nullptr;
+      const float* crow = cin ? cin + (long long)m * p.ld_cin : nullptr;
       float* drow = p.D + (long long)m * p.ldd;
       for (int c = half; c < bn / 32; c += 2) {
         const int nb = n0 + c * 32;
@@ -245,7 +248,7 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             float4 bz = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p.bias) bz = __ldg(reinterpret_cast<const float4*>(p.bias + nb) + q);
+            if (bias) bz = __ldg(reinterpret_cast<const float4*>(bias + nb) + q);
             float x[4] = {v[4 * q] + bz.x, v[4 * q + 1] + bz.y, v[4 * q + 2] + bz.z, v[4 * q + 3] + bz.w};
             const float z[4] = {zc[q].x, zc[q].y, zc[q].z, zc[q].w};
             const float cc[4] = {ci[q].x, ci[q].y, ci[q].z, ci[q].w};
@@ -263,7 +266,7 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
           for (int j = 0; j < 32; ++j) {
             const int n = nb + j;
             if (n < p.N) {
-              float x = v[j] + (p.bias ? __ldg(p.bias + n) : 0.f);
+              float x = v[j] + (bias ? __ldg(bias + n) : 0.f);
               if (p.sigmoid) x = 1.f / (1.f + __expf(-x));
               if (zrow) { const float z = __ldg(zrow + n); x *= z * (1.f - z); }
               x *= p.alpha;
@@ -662,7 +665,7 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       {
         const int mq = m0 + quad * 32 + rsub;                    // this thread's rows are mq + 16h + 8e
         EpiArgs ea;
-        ea.dsig = p.dsig; ea.cin = p.cin; ea.bias = p.bias; ea.D = p.D;
+        ea.dsig = dep(p.dsig); ea.cin = dep(p.cin); ea.bias = dep(p.bias); ea.D = p.D;
         ea.ldd = p.ldd; ea.ld_dsig = p.ld_dsig; ea.ld_cin = p.ld_cin;
         ea.dsig_rows = p.dsig_rows; ea.dsig_div = p.dsig_div;
         ea.dsig_direct = p.dsig_div == 1 && p.dsig_rows >= p.M;

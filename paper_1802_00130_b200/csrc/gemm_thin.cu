@@ -32,6 +32,13 @@ Epi make_epi(const GemmArgs& g) {
   return e;
 }
 
+// The epilogue as it is after grid_dep_wait (see dep()).
+__device__ __forceinline__ Epi after_wait(const Epi& in) {
+  Epi e = in;
+  e.bias = dep(e.bias); e.dsig = dep(e.dsig); e.cin = dep(e.cin);
+  return e;
+}
+
 __device__ __forceinline__ float apply_epi(const Epi& e, float x, int m, int n) {
   if (e.bias) x += __ldg(e.bias + n);
   if (e.sigmoid) x = 1.f / (1.f + expf(-x));
@@ -61,6 +68,7 @@ template <int NMAX>
 __global__ void __launch_bounds__(128, 3) gemm_thin_n_kernel(const ThinNParams p) {
   grid_dep_wait();
   grid_dep_launch();
+  const Epi e = after_wait(p.e);
   const int lane = threadIdx.x & 31;
   const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int m0 = warp * TR;
@@ -117,7 +125,7 @@ __global__ void __launch_bounds__(128, 3) gemm_thin_n_kernel(const ThinNParams p
       if (lane == n) mine = s;
     }
     const int m = m0 + r;
-    if (m < p.M && lane < p.N) p.e.D[(long long)m * p.e.ldd + lane] = apply_epi(p.e, mine, m, lane);
+    if (m < p.M && lane < p.N) e.D[(long long)m * e.ldd + lane] = apply_epi(e, mine, m, lane);
   }
 }
 
@@ -196,9 +204,10 @@ __global__ void __launch_bounds__(256) gemm_thin_m_partial_kernel(const ThinMPar
 // One block per 32 consecutive elements of the [M][N] result (lane = element); warp w adds chunks w, w + 8, ...
 // and the eight warp sums are added in warp order: a fixed order, and eight short chains instead of one long one.
 __global__ void __launch_bounds__(256) gemm_thin_m_final_kernel(const float* __restrict__ scratch, int chunks, int M, int N,
-                                                                const Epi e) {
+                                                                const Epi epi) {
   grid_dep_wait();
   grid_dep_launch();
+  const Epi e = after_wait(epi);
   __shared__ float sh[8][33];
   scratch = dep(scratch);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -243,12 +252,13 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
   const bool n_ok = n < p.N;
   const float* const pA = dep(p.A);
   const float* const pB = dep(p.B);
+  const Epi e = after_wait(p.e);
   float4 b[KMAX];
 #pragma unroll
   for (int k = 0; k < KMAX; ++k)
     b[k] = (n_ok && k < p.K) ? __ldg(reinterpret_cast<const float4*>(pB + (long long)k * p.ldb + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
   float4 bz = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (p.e.bias && n_ok) bz = __ldg(reinterpret_cast<const float4*>(p.e.bias + n));
+  if (e.bias && n_ok) bz = __ldg(reinterpret_cast<const float4*>(e.bias + n));
   const int m_begin = blockIdx.y * p.rows_per_block;
   const int m_end = min(p.M, m_begin + p.rows_per_block);
   for (int mb = m_begin; mb < m_end; mb += RB) {
@@ -266,7 +276,7 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
       for (int i = 0; i < RG; ++i) {
         const int m = mb + r0 + i;
         const bool ok = r0 + i < cnt;
-        z[i] = (p.e.dsig && ok) ? __ldg(reinterpret_cast<const float4*>(p.e.dsig + (long long)((m / p.e.dsig_div) % p.e.dsig_rows) * p.e.ld_dsig + n))
+        z[i] = (e.dsig && ok) ? __ldg(reinterpret_cast<const float4*>(e.dsig + (long long)((m / e.dsig_div) % e.dsig_rows) * e.ld_dsig + n))
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
@@ -286,22 +296,22 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
           }
         }
         float t[4] = {acc.x, acc.y, acc.z, acc.w};
-        if (p.e.sigmoid) {
+        if (e.sigmoid) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) t[j] = 1.f / (1.f + expf(-t[j]));
         }
-        if (p.e.dsig) {
+        if (e.dsig) {
           t[0] *= z[i].x * (1.f - z[i].x); t[1] *= z[i].y * (1.f - z[i].y);
           t[2] *= z[i].z * (1.f - z[i].z); t[3] *= z[i].w * (1.f - z[i].w);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) t[j] *= p.e.alpha;
-        if (p.e.cin) {   // not on the path's hot use of this kernel: read in place
-          const float4 c = __ldg(reinterpret_cast<const float4*>(p.e.cin + (long long)m * p.e.ld_cin + n));
-          t[0] = fmaf(p.e.beta, c.x, t[0]); t[1] = fmaf(p.e.beta, c.y, t[1]);
-          t[2] = fmaf(p.e.beta, c.z, t[2]); t[3] = fmaf(p.e.beta, c.w, t[3]);
+        for (int j = 0; j < 4; ++j) t[j] *= e.alpha;
+        if (e.cin) {   // not on the path's hot use of this kernel: read in place
+          const float4 c = __ldg(reinterpret_cast<const float4*>(e.cin + (long long)m * e.ld_cin + n));
+          t[0] = fmaf(e.beta, c.x, t[0]); t[1] = fmaf(e.beta, c.y, t[1]);
+          t[2] = fmaf(e.beta, c.z, t[2]); t[3] = fmaf(e.beta, c.w, t[3]);
         }
-        *reinterpret_cast<float4*>(p.e.D + (long long)m * p.e.ldd + n) = make_float4(t[0], t[1], t[2], t[3]);
+        *reinterpret_cast<float4*>(e.D + (long long)m * e.ldd + n) = make_float4(t[0], t[1], t[2], t[3]);
       }
     }
   }

@@ -107,6 +107,9 @@ __global__ void __launch_bounds__(SN_THREADS) small_net_kernel(const __grid_cons
   extern __shared__ __align__(16) float sm[];
   grid_dep_wait();
   grid_dep_launch();
+  const float* const theta = dep(a.theta);
+  const float* const v = dep(a.v);
+  const float* const Y = dep(a.Y);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int L = a.L;
   const long long row0 = (long long)blockIdx.x * SN_ROWS;
@@ -133,16 +136,16 @@ __global__ void __launch_bounds__(SN_THREADS) small_net_kernel(const __grid_cons
       const int np = a.w[m - 1], ldw = np | 1;
       for (int j = warp; j < a.w[m]; j += SN_THREADS / 32)
         for (int k = lane; k < np; k += 32) {
-          const float t = __ldg(a.theta + a.w_off[m] + j * np + k);
+          const float t = __ldg(theta + a.w_off[m] + j * np + k);
           ws[wo[m] + j * ldw + k] = t;
           if (KIND == SN_GRAD || KIND == SN_FUN) tt += (double)t * t;
-          if (sn_has_v(KIND)) vs[wo[m] + j * ldw + k] = __ldg(a.v + a.w_off[m] + j * np + k);
+          if (sn_has_v(KIND)) vs[wo[m] + j * ldw + k] = __ldg(v + a.w_off[m] + j * np + k);
         }
       for (int j = tid; j < a.w[m]; j += SN_THREADS) {
-        const float t = __ldg(a.theta + a.b_off[m] + j);
+        const float t = __ldg(theta + a.b_off[m] + j);
         ws[wo[m] + a.w[m] * ldw + j] = t;
         if (KIND == SN_GRAD || KIND == SN_FUN) tt += (double)t * t;
-        if (sn_has_v(KIND)) vs[wo[m] + a.w[m] * ldw + j] = __ldg(a.v + a.b_off[m] + j);
+        if (sn_has_v(KIND)) vs[wo[m] + a.w[m] * ldw + j] = __ldg(v + a.b_off[m] + j);
       }
     }
   if ((KIND == SN_GRAD || KIND == SN_FUN) && blockIdx.x == 0) {
@@ -151,9 +154,10 @@ __global__ void __launch_bounds__(SN_THREADS) small_net_kernel(const __grid_cons
   }
 #pragma unroll
   for (int m = 0; m < (sn_has_v(KIND) ? kSmallLayers : 1); ++m)
-    if (m < L)
+    if (m < L) {
+      const float* const zm = dep(a.z[m]);
       for (int r = warp; r < SN_ROWS; r += SN_THREADS / 32) {
-        const float* src = a.z[m];
+        const float* src = zm;
         bool ok = r < cnt;
         if (KIND == SN_FORWARD && ok) {
           const long long s = a.idx[row0 + r];
@@ -169,6 +173,7 @@ __global__ void __launch_bounds__(SN_THREADS) small_net_kernel(const __grid_cons
           if (KIND == SN_FORWARD && r < cnt) a.z_out[0][(row0 + r) * a.w[0] + k] = x;
         }
       }
+    }
   __syncthreads();
 
   if (KIND == SN_GRAD || KIND == SN_FUN || KIND == SN_FORWARD) {
@@ -197,7 +202,7 @@ __global__ void __launch_bounds__(SN_THREADS) small_net_kernel(const __grid_cons
       for (int j = lane; j < a.w[L]; j += 32) {
         float d = 0.f;
         if (r < cnt) {
-          d = cur[j * SN_LD + r] - __ldg(a.Y + (row0 + r) * a.w[L] + j);
+          d = cur[j * SN_LD + r] - __ldg(Y + (row0 + r) * a.w[L] + j);
           loss += (double)d * d;
         }
         cur[j * SN_LD + r] = 2.f * d;
@@ -295,6 +300,7 @@ __global__ void __launch_bounds__(256) small_sum_kernel(const float* __restrict_
   __shared__ double sh[8][33];
   grid_dep_wait();
   grid_dep_launch();
+  part = dep(part); loss = dep(loss);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (out) {
     const int i = blockIdx.x * 32 + lane;
