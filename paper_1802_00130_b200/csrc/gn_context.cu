@@ -109,7 +109,7 @@ struct gn_ctx {
   std::vector<SplitEntry> split_cache;
   uint16_t* arena[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; int64_t arena_rows[5] = {0, 0, 0, 0, 0};
   const float* cur_v = nullptr;                            // the vector of the product in progress
-  const float* cur_x = nullptr; int64_t cur_x_count = 0;   // the rows of X of the batch in progress
+  const float* cur_x = nullptr;                            // the rows of X of the batch in progress
   struct SplitSlot {         // parts of any other operand: one slot per operand role, overwritten by the next use
     const float* src = nullptr; int64_t rows = 0; int cols = 0; int64_t ld = 0; SplitBuf buf;
     uint64_t seq = 0;        // contraction (gemm_seq) that wrote these parts
@@ -364,16 +364,18 @@ bool split_buf_reserve(gn_ctx* c, gn_ctx::SplitBuf& b, int64_t need) {
   return true;
 }
 
-// The parts of kind `kind` go (their workspace is about to move or to change size).
-void drop_kept_parts(gn_ctx* c, int kind) {
+// The parts of kind `kind` (0: of every kind) that have a buffer of their own go, and, with `all`, the whole kind's.
+void drop_kept_parts(gn_ctx* c, int kind, bool all) {
   for (size_t i = 0; i < c->split_cache.size();) {
-    if (c->split_cache[i].kind == kind) {
-      if (!c->split_cache[i].in_arena) dev_free(c, c->split_cache[i].buf.p);
+    const gn_ctx::SplitEntry& e = c->split_cache[i];
+    if ((kind == 0 || e.kind == kind) && (all || !e.in_arena)) {
+      if (!e.in_arena) dev_free(c, c->split_cache[i].buf.p);
       c->split_cache.erase(c->split_cache.begin() + (long)i);
     } else {
       ++i;
     }
   }
+  if (!all) return;
   dev_free(c, c->arena[kind]);
   c->arena_rows[kind] = 0;
 }
@@ -402,19 +404,20 @@ bool arena_buffer(gn_ctx* c, int kind, int64_t key, int64_t rows, int cols, int6
   return true;
 }
 
-// Place of `src` in a matrix set whose parts are kept (SplitEntry::kind), or 0.
+// Place of `src` in a matrix set whose parts are kept (SplitEntry::kind), or 0.  Of the activations only what starts in the
+// first row has one: a place per row offset would be one per subsample size.
 int split_kind(const gn_ctx* c, const float* src, int64_t* key, uint64_t* epoch) {
   if (src >= c->theta && src < c->theta + c->n) { *key = src - c->theta; *epoch = c->theta_epoch; return 1; }
   for (int m = 0; m <= c->L; ++m)
-    if (c->Z[m] && src >= c->Z[m] && src < c->Z[m] + c->capS * c->w[m]) {
+    if (c->Z[m] && src >= c->Z[m] && src < c->Z[m] + c->w[m]) {
       *key = ((int64_t)m << 48) + (src - c->Z[m]); *epoch = c->sub_epoch;
       return 2;
     }
   *epoch = c->parts_epoch;
   if (c->cur_v && src >= c->cur_v && src < c->cur_v + c->n) { *key = src - c->cur_v; return 3; }
-  if (c->cur_x && src >= c->cur_x && src < c->cur_x + c->cur_x_count) { *key = src - c->cur_x; return 4; }
+  if (c->cur_x && src >= c->cur_x && src < c->cur_x + c->w[0]) { *key = src - c->cur_x; return 4; }
   for (int m = 1; m <= c->L; ++m)
-    if (c->Zb[m] && src >= c->Zb[m] && src < c->Zb[m] + c->capB * c->w[m]) { *key = ((int64_t)m << 48) + (src - c->Zb[m]); return 4; }
+    if (c->Zb[m] && src >= c->Zb[m] && src < c->Zb[m] + c->w[m]) { *key = ((int64_t)m << 48) + (src - c->Zb[m]); return 4; }
   return 0;
 }
 
@@ -994,7 +997,7 @@ gn_status ensure_stacked(gn_ctx* c) {
     if (st != GN_OK) {
       // leave a consistent, empty state: the next set_subsample allocates afresh
       for (int k = 1; k <= c->L; ++k) { dev_free(c, c->RZ[k]); dev_free(c, c->DS[k]); }
-      drop_kept_parts(c, 2);
+      drop_kept_parts(c, 2, true);
       for (int k = 0; k <= c->L; ++k) dev_free(c, c->Z[k]);
       dev_free(c, c->idx);
       c->capS = 0; c->have_sub = false; c->factors_valid = false;
@@ -1279,7 +1282,7 @@ gn_status ensure_batch(gn_ctx* c) {
   const int64_t rows = c->batch_rows < c->l ? c->batch_rows : c->l;
   if (rows <= c->capB) return GN_OK;
   quiesce(c);
-  drop_kept_parts(c, 4);
+  drop_kept_parts(c, 4, true);
   for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
   c->capB = 0;
   for (int m = 1; m <= c->L; ++m) {
@@ -1315,12 +1318,12 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
   GN_TRY(ensure_partials(c, per_batch * nb + (c->n + kCgChunk - 1) / kCgChunk + 16));
   const float inv_l = (float)(1.0 / (double)c->l);
   const float inv_C = (float)(1.0 / c->C);
-  struct CurrentBatch { gn_ctx* c; ~CurrentBatch() { c->cur_x = nullptr; c->cur_x_count = 0; } } current{c};
+  struct CurrentBatch { gn_ctx* c; ~CurrentBatch() { c->cur_x = nullptr; } } current{c};
   for (int64_t b = 0; b < nb; ++b) {
     const int64_t r0 = b * Rb;
     const int64_t rows = (c->l - r0 < Rb) ? c->l - r0 : Rb;
     const float* X0 = c->dX + r0 * c->w[0];
-    c->cur_x = X0; c->cur_x_count = rows * c->w[0];
+    c->cur_x = X0;
     ++c->parts_epoch;           // the batch buffers are rewritten
     forward_pass(c, X0, rows, c->Zb);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
@@ -1542,7 +1545,7 @@ gn_status gn_set_batch_rows(gn_ctx* c, int64_t rows) {
   if ((rows < c->l ? rows : c->l) != c->capB && c->capB > 0) {
     // shrink or grow on next use: drop the old workspace now so memory stays bounded
     quiesce(c);
-      drop_kept_parts(c, 4);
+      drop_kept_parts(c, 4, true);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->Zb[m], c->capB * c->w[m]); dev_free(c, c->Db[m], c->capB * c->w[m]); }
     c->capB = 0;
   }
@@ -1586,6 +1589,7 @@ gn_status gn_set_split(gn_ctx* c, const int32_t* split) {
   c->has_split = any;
   c->P = (int)P;
   const gn_status st = build_chunks(c, true);
+  if (st == GN_OK) drop_kept_parts(c, 0, false);     // (of the sub-blocks of the structure that has gone)
   if (st != GN_OK) { c->split = old_split; c->has_split = old_has; c->P = old_P; }   // the old tables are still in place
   return st;
 }
@@ -1635,7 +1639,7 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   ++c->parts_epoch;
   if (nS > c->capS) {
     GN_TRY(sync(c, "set_subsample"));
-    drop_kept_parts(c, 2);      // the stored activations move: their parts are made anew
+    drop_kept_parts(c, 2, true);      // the stored activations move: their parts are made anew
       dev_free(c, c->idx, c->capS);
     for (int m = 0; m <= c->L; ++m) dev_free(c, c->Z[m], c->capS * c->w[m]);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m], m * c->capS * c->w[m]); dev_free(c, c->DS[m], m * c->capS * c->w[m]); }

@@ -266,3 +266,46 @@ def test_a_kept_solver_step_follows_the_accurate_method(blockdiag, first, second
         # products within 1e-6, multiplied a few times by the five steps (systems of condition below 100)
         assert np.linalg.norm(d.cpu().numpy() - ref) <= 1e-4 * np.linalg.norm(ref)
     ctx.close()
+
+
+def test_kept_parts_do_not_accumulate():
+    """Parts of theta and of the activations are kept per place: neither new variable partitions nor new subsample sizes may
+    leave the parts of the old ones behind."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    p = wl.make_custom((1201, 802, 605, 5), 1500, 900, 15.0, seed=3)
+    ctx = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]))
+    ctx.set_theta(dev(p["theta"]))
+    ctx.set_subsample(dev(p["idx"]))
+    ctx.profile(True)
+    v, seen = dev(p["v"]), []
+    for s in [[2, 2, 2, 1], [3, 2, 1, 1], [2, 3, 4, 1], [5, 4, 3, 1], [2, 2, 2, 1], [3, 2, 1, 1]]:
+        ctx.set_split(s)
+        ctx.Gv_blockdiag(v)
+        torch.cuda.synchronize()
+        seen.append(ctx.workspace_bytes)
+    assert ctx.profile_read()["tensor_x3"]["launches"] > 0
+    # (once the largest structure has grown the shared workspaces) the same structure takes the same memory as before
+    ctx.set_split([5, 4, 3, 1])
+    ctx.Gv_blockdiag(v)
+    assert ctx.workspace_bytes == seen[3] and seen[4] <= seen[3] and seen[5] <= seen[3]
+    ctx.close()
+
+
+def test_parts_of_narrow_layers_do_not_accumulate_over_subsample_sizes():
+    import torch
+    import paper_1802_00130_b200 as gn
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    p = wl.make_custom((96, 64, 60, 10), 9000, 9000, 15.0, seed=3)
+    ctx = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32)
+    ctx.debug_option(10, 0)
+    ctx.set_blockdiag_method(2)
+    ctx.set_theta(dev(p["theta"]))
+    v, seen = dev(p["v"]), []
+    for nS in (9000, 8800, 8600, 8400, 8200):
+        ctx.set_subsample(dev(p["idx"][:nS]))
+        ctx.Gv_blockdiag(v)
+        seen.append(ctx.workspace_bytes)
+    assert len(set(seen)) == 1
+    ctx.close()
