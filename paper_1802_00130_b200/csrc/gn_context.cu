@@ -381,8 +381,9 @@ void drop_kept_parts(gn_ctx* c, int kind, bool all) {
 }
 
 // Buffer of the kept parts of a whole layer's matrix inside the kind's arena: kinds 1 and 3 hold every W^m-shaped
-// matrix, kinds 2 and 4 the operands z^0 .. z^{L-1} of the subsample and of the row batch at their workspaces' capacity.
-// False if the matrix has no place there.
+// matrix, kinds 2 and 4 the operands z^0 .. z^{L-1} of the subsample and of the row batch at their workspaces' capacity - on a
+// TF32 context only those that TMA cannot address in one of their contractions (the layer's two widths, and where its weights
+// start), since nothing else is split there.  False if the matrix has no place there.
 bool arena_buffer(gn_ctx* c, int kind, int64_t key, int64_t rows, int cols, int64_t ld, gn_ctx::SplitBuf* out) {
   const bool vec = kind == 1 || kind == 3;
   const int64_t cap_rows = kind == 2 ? c->capS : kind == 4 ? c->capB : 0;
@@ -390,6 +391,7 @@ bool arena_buffer(gn_ctx* c, int kind, int64_t key, int64_t rows, int cols, int6
   for (int m = 0; m < c->L; ++m) {
     const int64_t n = vec ? (int64_t)c->w[m + 1] * round8(c->w[m]) : cap_rows * round8(c->w[m]);
     const int64_t k = vec ? c->w_off[m + 1] : (int64_t)m << 48;
+    if (c->prec == GN_TF32 && c->w[m] % 4 == 0 && c->w[m + 1] % 4 == 0 && (!vec || c->w_off[m + 1] % 4 == 0)) continue;
     if (key == k && cols == c->w[m] && ld == c->w[m] && rows <= (vec ? c->w[m + 1] : cap_rows)) { at = total; size = n; }
     total += gn_ctx::SplitBuf::elements(n);
   }

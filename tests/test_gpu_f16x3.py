@@ -309,3 +309,23 @@ def test_parts_of_narrow_layers_do_not_accumulate_over_subsample_sizes():
         seen.append(ctx.workspace_bytes)
     assert len(set(seen)) == 1
     ctx.close()
+
+
+def test_parts_take_the_memory_of_the_layers_that_are_split():
+    """A TF32 context with one odd layer: the parts of that layer's activations, not of all."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    w, nS = (30, 1024, 1024, 20), 20000
+    p = wl.make_custom(w, 500, 500, 15.0, seed=3)
+    ctx = gn.GnContext(list(w), p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32)
+    ctx.set_theta(dev(p["theta"]))
+    ctx.profile(True)
+    ctx.set_subsample(dev(np.resize(p["idx"], nS)))
+    v = dev(p["v"])
+    ctx.Gv(v)
+    assert ctx.profile_read()["tensor_x3"]["launches"] > 0
+    activations = 4 * nS * (2 * sum(w) + sum(w[:-1]))          # Z, RZ, DS
+    odd = 2 * 4 * nS * 32 + 4 * nS * 1024                      # parts of X_S (rows of 8), and of delta s^1 for the length of a contraction
+    assert ctx.workspace_bytes <= activations + odd + 100e6    # (weights, vectors, the K slices' workspace: 50 MB)
+    ctx.close()
