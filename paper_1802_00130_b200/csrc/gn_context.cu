@@ -434,10 +434,11 @@ constexpr int64_t kMaxTransientSplitFloats = 1500LL * 1000 * 1000;   // 6 GB for
 bool split_operand(gn_ctx* c, const float* src, int64_t rows, int cols, int64_t ld, int role, bool reuse,
                    SplitOperand* out, std::vector<SplitJob>& jobs) {
   const int64_t ldo = round8(cols);
-  if (rows * ldo > kMaxTransientSplitFloats) return false;
   int64_t key = 0;
   uint64_t epoch = 0;
   const int kind = split_kind(c, src, &key, &epoch);
+  // (theta and the stored activations are split whatever their size: their parts serve many contractions)
+  if (kind != 1 && kind != 2 && rows * ldo > kMaxTransientSplitFloats) return false;
   gn_ctx::SplitBuf* buf = nullptr;
   bool fresh = false;
   if (kind != 0) {

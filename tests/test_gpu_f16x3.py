@@ -280,16 +280,14 @@ def test_kept_parts_do_not_accumulate():
     ctx.set_subsample(dev(p["idx"]))
     ctx.profile(True)
     v, seen = dev(p["v"]), []
-    for s in [[2, 2, 2, 1], [3, 2, 1, 1], [2, 3, 4, 1], [5, 4, 3, 1], [2, 2, 2, 1], [3, 2, 1, 1]]:
+    for s in [[4, 1, 1, 1], [3, 1, 1, 1], [2, 1, 1, 1]]:      # (the largest workspaces first; the parts take about the same each time)
         ctx.set_split(s)
         ctx.Gv_blockdiag(v)
         torch.cuda.synchronize()
         seen.append(ctx.workspace_bytes)
     assert ctx.profile_read()["tensor_x3"]["launches"] > 0
-    # (once the largest structure has grown the shared workspaces) the same structure takes the same memory as before
-    ctx.set_split([5, 4, 3, 1])
-    ctx.Gv_blockdiag(v)
-    assert ctx.workspace_bytes == seen[3] and seen[4] <= seen[3] and seen[5] <= seen[3]
+    parts = 4 * 900 * 1201
+    assert max(seen) <= seen[0] + parts // 4
     ctx.close()
 
 
@@ -329,3 +327,25 @@ def test_parts_take_the_memory_of_the_layers_that_are_split():
     odd = 2 * 4 * nS * 32 + 4 * nS * 1024                      # parts of X_S (rows of 8), and of delta s^1 for the length of a contraction
     assert ctx.workspace_bytes <= activations + odd + 100e6    # (weights, vectors, the K slices' workspace: 50 MB)
     ctx.close()
+
+
+def test_stored_activations_beyond_the_limit_of_passing_operands():
+    """Z^1 of 1.6e9 elements (6.5 GB): its contractions stay on the tensor cores."""
+    import torch
+    import paper_1802_00130_b200 as gn
+    from oracle import gn_oracle as orc
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    w, nS = (64, 4096, 20), 400000
+    p = wl.make_custom(w, 1000, 1000, 15.0, seed=3)
+    ctx = gn.GnContext(list(w), p["C"], dev(p["X"]), dev(p["Y"]))
+    ctx.set_theta(dev(p["theta"]))
+    ctx.profile(True)
+    ctx.set_subsample(dev(np.resize(np.arange(1000, dtype=np.int32), nS)))
+    kinds = ctx.profile_read()
+    assert kinds["ffma"]["launches"] == 0 and kinds["tensor_x3"]["launches"] == 2
+    z = ctx.debug_activations(2).reshape(nS, 20)
+    ref = orc.forward(p["theta"], list(w), p["X"])[2]
+    for at in (0, 200000, nS - 1000):
+        assert np.linalg.norm(z[at:at + 1000].cpu().numpy() - ref) <= 1e-6 * np.linalg.norm(ref)
+    ctx.close()
+    torch.cuda.empty_cache()
