@@ -49,6 +49,40 @@ def test_against_float64(widths, nS, l, mode):
     ctx.close()
 
 
+@pytest.mark.parametrize("mode", ["fp32", "tf32"])
+@pytest.mark.parametrize("nS,l", [(1, 3), (33, 1000), (500, 700)])
+@pytest.mark.parametrize("widths", NETS)
+def test_the_chain_of_kernels_at_the_same_sizes(widths, nS, l, mode):
+    """The same networks with the one-launch passes switched off: the contraction, streaming, column-sum, gather, loss and
+    vector kernels at odd and tiny sizes, in every pass and in both solves."""
+    import paper_1802_00130_b200 as gn
+    p = wl.make_custom(widths, l, nS, 0.3 * l, seed=sum(widths) + l)
+    ctx = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32 if mode == "tf32" else gn.GN_FP32_ACCURATE)
+    ctx.debug_option(10, 0)
+    th, w, C, XS, v = p["theta"], p["widths"], p["C"], p["X"][p["idx"]], p["v"]
+    tol = 1e-5 if mode == "fp32" else 2e-3    # the modes' bounds
+    rel = lambda a, b: np.linalg.norm(np.asarray(a.cpu().numpy() if hasattr(a, "cpu") else a) - b) / np.linalg.norm(b)
+    ctx.set_theta(dev(th))
+    before = ctx.kernel_launches
+    ctx.set_subsample(dev(p["idx"]))
+    assert ctx.kernel_launches - before > 1
+    Z = orc.forward(th, w, XS)
+    for m in range(1, len(w)):
+        assert rel(ctx.debug_activations(m).reshape(nS, w[m]), Z[m]) <= tol
+    g, f = ctx.grad(with_f=True)
+    ref_g, ref_f = orc.grad(th, w, C, p["X"], p["Y"]), orc.fun(th, w, C, p["X"], p["Y"])
+    assert rel(g, ref_g) <= tol and abs(f - ref_f) <= tol * abs(ref_f) and ctx.fun() == f
+    assert rel(ctx.Gv(dev(v)), orc.Gv(th, w, C, XS, v)) <= tol
+    ref_b = orc.Gv_blockdiag(th, w, C, XS, v)
+    for method in [1, 2] if len(w) > 2 and w[-1] <= 16 else [1]:
+        ctx.set_blockdiag_method(method)
+        assert rel(ctx.Gv_blockdiag(dev(v)), ref_b) <= tol
+    for block in (False, True):               # two steps: what a product's rounding does to them is a few times that rounding
+        d, _, _ = ctx.cg_solve(dev(ref_g.astype(np.float32)), 1.0, blockdiag=block, max_iter=2, tol=0.0)
+        assert rel(d, orc.cg_solve(th, w, C, XS, ref_g, 1.0, block, 2, 0.0)[0]) <= 10 * tol
+    ctx.close()
+
+
 def test_an_index_out_of_range_is_still_refused():
     import paper_1802_00130_b200 as gn
     p = wl.make("tiny")
@@ -80,5 +114,5 @@ def test_tf32_solves_round_one_operator(widths, nS, l):
     d, _, _ = ctx.cg_solve(ctx.grad(), 1.0, max_iter=2, tol=0.0)
     th, w, C, XS = p["theta"], p["widths"], p["C"], p["X"][p["idx"]]
     ref = orc.cg_solve(th, w, C, XS, orc.grad(th, w, C, p["X"], p["Y"]), 1.0, False, 2, 0.0)[0]
-    assert np.linalg.norm(d.cpu().numpy() - ref) <= 6e-4 * np.linalg.norm(ref)
+    assert np.linalg.norm(d.cpu().numpy() - ref) <= 4e-4 * np.linalg.norm(ref)
     ctx.close()
