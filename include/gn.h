@@ -339,10 +339,10 @@ gn_status gn_debug_activations(gn_ctx* ctx, int m, float* d_out);
  * every GEMM launch is bracketed by a pair of CUDA events on the context's stream.
  * gn_profile_read - synchronise the stream and return, for the CTA-pair tensor-core kernel that carries the large
  * contractions (index 0), the FP32 FMA GEMM (index 1), the streaming kernels for n_L-wide shapes (index 2), the
- * error-compensated tensor-core kernel of GN_FP32_ACCURATE contexts (index 3) and the one-CTA tensor-core kernel
- * that takes the n_L-wide and small-M shapes in TF32 mode (index 4): summed device time in milliseconds,
+ * error-compensated tensor-core kernel of GN_FP32_ACCURATE contexts (index 3) and the TF32 kernels at the n_L-wide, narrow
+ * and small-M shapes (index 4; mostly the one-CTA kernel): summed device time in milliseconds,
  * floating-point operations of the contractions (2 M N K per launch, summed over the problems of a grouped
- * launch; for index 3 the three TF32 products per term count once) and number of launches; then reset the
+ * launch; for index 3 the three FP16 products per term count once) and number of launches; then reset the
  * counters.  Each output is an array of FIVE entries and may be NULL.
  */
 gn_status gn_profile(gn_ctx* ctx, int enable);

@@ -545,7 +545,8 @@ bool run_gemm_f16x3(gn_ctx* c, const GemmArgs& args) {
 
 // Whether the tensor-core form is the faster way to FP32 accuracy.  The FP32 FMA GEMM walks K alone in 128 x 128
 // tiles: about 10 us plus 0.12 us per unit of K and round of tiles (17 us at K = 37, 53 at 333).  The tensor-core form
-// pays for splitting its operands before it starts (two launches, about 8 us, and their bytes) and about 6 us of ramp.
+// pays for splitting its operands before it starts (a launch, 4 to 6 us, and its bytes) and about 6 us of ramp; the 14 us
+// charged here date from when a split took two launches, so the line lies a little on the FMA GEMM's side.
 bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
   if (!c->x3_usable || !gemm_f16x3_usable()) return false;
   if (c->prec == GN_FP32_ACCURATE && c->acc_method == 1) return false;
@@ -557,9 +558,9 @@ bool wants_f16x3(const gn_ctx* c, const GemmArgs& g) {
 }
 
 // Whether a contraction goes to the TF32 kernels: on a TF32 context every one whose operands TMA can address, whatever its
-// sizes.  The gradient (K or M up to a row batch) and the products (|S|) of one solve have to round the same operator: with
-// the weight blocks of narrow layers in FP32 accuracy from some K on (an earlier rule, 96-100-50-200-1, |S| = 554,
-// l = 5540) the first residual holds an error that is not along the gradient, and conjugate gradient amplifies it.
+// sizes.  The gradient (K or M up to a row batch) and the products (|S|) of one solve have to round the same operator (see
+// small_pass); with the weight blocks of narrow layers in FP32 accuracy from some K on, as an earlier rule had it, they did not
+// (300-120-80-40: the 80 x 120 block above about 1150 rows).
 bool on_tf32(const gn_ctx* c, const GemmArgs& g) { return c->prec == GN_TF32 && gemm_tf32_eligible(g); }
 
 // Whether run_gemm will send a contraction to that form.
