@@ -64,7 +64,9 @@ typedef enum {
 } gn_status;
 
 typedef enum {
-  GN_TF32 = 0,         /* contractions on the tensor cores with TF32 operands, FP32 accumulate;  */
+  GN_TF32 = 0,         /* contractions on the tensor cores with operands rounded to TF32's 11    */
+                       /* significant bits (held as TF32 or, in large passes and where that is  */
+                       /* the same number up to a power of two, as FP16), FP32 accumulate;      */
                        /* to FP32 accuracy where TMA cannot address the operands (rows that are */
                        /* no multiple of four floats)                                           */
   GN_FP32_ACCURATE = 1 /* results at FP32 accuracy: error-compensated tensor-core contractions  */
@@ -356,7 +358,8 @@ gn_status gn_profile_read(gn_ctx* ctx, double* gemm_ms, double* gemm_flop, int64
  * 4 and 5 = as 3 with one CTA per 128-row tile, respectively a CTA pair per 256-row tile, forced;
  * 6 = as 5 but whole tiles only, i.e. without the stream-K split of tiles between CTA pairs;
  * 7 = the error-compensated tensor-core form, see gn_set_accurate_method, for results of more than 128 rows and at
- * least 128 columns; 8 = the same for any shape).  a_kmajor: A is [M][K]
+ * least 128 columns; 8 = the same for any shape; 9 = as 5 on FP16 copies of the operands, which are made first: leading
+ * dimensions must be the row lengths, M > 128, N >= 128).  a_kmajor: A is [M][K]
  * (else [K][M]); b_kmajor: B is [N][K] (else [K][N]); all row-major with the given leading
  * dimensions.  GN_EINVAL if the chosen kernel cannot take the operands (alignment, shape).
  */
@@ -396,7 +399,8 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* ctx, int kind, int M, int N, int K, con
  * stored-factor block product the factor of the last hidden layer, W^L * sigma'(z^{L-1}), is formed on the fly from
  * W^L and the stored activations instead of being read back (value 0 = read back; same bits either way).  Option 10:
  * whole passes of small networks as one launch (value 0 = one contraction per layer and operand; the forms differ by
- * rounding).  Results do not depend on options 0, 3, 4, 5, 6, 9 and, with whole tiles (option 1 off), 8 (tiles, sums
+ * rounding).  Option 11: FP16 copies of TF32 operands (value 0 = never, 1 = in passes large enough, the default, 2 = wherever
+ * an operand can have one; the forms differ in the order of sums).  Results do not depend on options 0, 3, 4, 5, 6, 9 and, with whole tiles (option 1 off), 8 (tiles, sums
  * and parts are computed identically); GN_EINVAL for an unknown option.
  */
 gn_status gn_debug_option(gn_ctx* ctx, int option, int value);

@@ -1,7 +1,10 @@
 // TF32 tensor-core GEMM for sm_100a: tcgen05.mma with the accumulator in tensor memory, operands
 // staged in shared memory by TMA (128-byte swizzle), fused epilogue read back with tcgen05.ld.
 //
-// Persistent kernel, one CTA per SM, each walking 128 x bn output tiles.  Warp roles:
+// Operands of the CTA-pair kernel may also be FP16 copies (see HalfInfo in gn_kernels.h): the same numbers up to a power of two, in
+// half the bytes and at twice the rate.  18944 x 2048 x 2048: 255 us with TF32 operands, 140 us with copies.
+//
+// Persistent kernels.  One CTA per SM, each walking 128 x bn output tiles (the CTA-pair kernel further down).  Warp roles:
 //   warp 0      TMA producer: fills a ring of STAGES operand buffers (issue spread over lanes)
 //   warp 1      MMA issuer   (one elected lane): 4 x (128 x bn x 8) tcgen05.mma per ring slot
 //   warps 2..9  epilogue: two warps per 32-lane quadrant of tensor memory, alternating over the
@@ -23,7 +26,10 @@
 //              advances 1024 B.
 // Every wait on an mbarrier is bounded: after about two seconds the waiting role records an error
 // code in global memory and the CTA drains and exits (tensor memory is always released).
+#include <cuda_fp16.h>
+
 #include "gn_kernels.h"
+#include "half_common.cuh"
 #include "tc_common.cuh"
 
 namespace gn {
@@ -33,23 +39,34 @@ constexpr int BM = 128, BK = 32, BN_MAX = 256;
 constexpr int A_STAGE_BYTES = BM * BK * 4;  // 16 KB
 
 struct Tf32Params {
+  // (what the producer and the MMA issuer look at before their first instruction stands together: parameters are read through
+  // the constant cache, and every line of it that is new to an SM costs some hundred cycles)
   int M, N;
   int kblocks[2];
   int a_mn, b_mn;
   int a_3d, b_3d;       // MN-major operand fetched with one 3-D box per stage (needs a padded operand)
-  float* D; long long ldd;
-  const float* bias; int sigmoid;
-  const float* dsig; long long ld_dsig; int dsig_rows, dsig_div;
-  float alpha;
-  const float* cin; long long ld_cin; float beta;
-  int vec_epi;          // D, bias, dsig, cin all 16-byte aligned with leading dimensions % 4 == 0
   int bn;               // tile width: multiple of 32, 32 <= bn <= 256
   int tiles_n, tiles;
-  int* err;
   // work list of the two-CTA kernel: pair q runs tiles q, q + P, ... for `waves` full waves of P tiles;
   // the `rem` tiles left over are each cut along K into `slices` parts, one per pair, done before the
   // pair's whole tiles (slices == 1: whole tiles, done last)
   int P, waves, rem, slices;
+  // FP16 copies (CTA-pair kernel): half = every operand has one, k-blocks of 64 terms, K; further down the infos of A1, B1, A2, B2,
+  // where the copy of D goes (copy_out), its info, and the infos of GemmArgs::h_next
+  int half, copy_out;
+  int khalf[2];
+  int K[2];
+  float alpha;
+  int sigmoid;
+  int vec_epi;          // D, bias, dsig, cin all 16-byte aligned with leading dimensions % 4 == 0, N % 4 == 0
+  float* D; long long ldd;
+  const float* bias;
+  const float* dsig; long long ld_dsig; int dsig_rows, dsig_div;
+  const float* cin; long long ld_cin; float beta;
+  const HalfInfo* hin[4];
+  __half* Dh; long long ldh; HalfInfo* hout;
+  const HalfInfo* hnext[3];
+  int* err;
   float* sk_ws;          // [P][2][128][256] raw partial accumulators of the sliced tiles, slot = pair
   int* sk_flags;         // [P] arrival counters, one per sliced tile; zero between launches (the kernel resets them)
 };
@@ -74,10 +91,11 @@ struct GroupParams {
   int dep_prob[MAX_GROUP];
   int dep_all[MAX_GROUP];
   int signal[MAX_GROUP];
+  // (bit 30 of a counter: a copy written by these tiles may not be used)
   int* done;                 // [n_prob][done_stride]: entry i < done_stride - 1 counts panel i, the last entry all tiles
   int done_stride;
 };
-struct GroupMaps { CUtensorMap m[MAX_GROUP][4]; };   // per problem: A0, B0, A1, B1
+struct GroupMaps { CUtensorMap m[MAX_GROUP][4], h[MAX_GROUP][4]; };   // per problem: A0, B0, A1, B1, and their FP16 copies
 
 __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile(
@@ -299,7 +317,9 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
 // Protocol: both producers wait on their own empty[s] (released in both CTAs by a multicast commit),
 // only the leader (rank 0) arms full[s] with the bytes of both CTAs, and both CTAs' TMA loads complete
 // on the leader's full[s].  MMAs are issued by the leader only.  acc_full[b] is multicast to both
-// CTAs; all 16 epilogue warps of the pair arrive on the leader's acc_empty[b].
+// CTAs; all 32 epilogue warps of the pair arrive on the leader's acc_empty[b].  Sixteen epilogue warps per CTA, four per scheduler,
+// because their time is latency (12000 x 2000 x 784 with the sigmoid: 105 us with eight, 75 us with sixteen), at 96 registers,
+// which leaves room on the SM for a block of the column-sum kernel that runs beside this one (576 x 96 + 256 x 40 = 65536).
 //
 // Work list: with T tiles on P pairs, pair q runs tiles q, q + P, ... for the floor(T / P) full waves, so
 // that all pairs move through neighbouring tiles together (tiles of one A panel are read at the same
@@ -317,7 +337,110 @@ __device__ __forceinline__ void mma2_tf32(uint32_t tmem_d, uint64_t adesc, uint6
       "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
-struct Work { int prob, tile, kb0, kb1, sliced; };
+// The same with FP16 operands (K = 16 per instruction: as many bytes of operands and as long, twice the terms).
+__device__ __forceinline__ void mma2_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
+}
+// ... adding to the accumulator times 2^-S
+template <int S>
+__device__ __forceinline__ void mma2_f16_scaled(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.eq.b32 p, 0, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p, %4;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "n"(S) : "memory");
+}
+__device__ __forceinline__ void mma2_f16_shift(int s, uint32_t d, uint64_t a, uint64_t b, uint32_t i) {
+  switch (s) {
+    case 1: mma2_f16_scaled<1>(d, a, b, i); break;
+    case 2: mma2_f16_scaled<2>(d, a, b, i); break;
+    case 3: mma2_f16_scaled<3>(d, a, b, i); break;
+    case 4: mma2_f16_scaled<4>(d, a, b, i); break;
+    case 5: mma2_f16_scaled<5>(d, a, b, i); break;
+    case 6: mma2_f16_scaled<6>(d, a, b, i); break;
+    case 7: mma2_f16_scaled<7>(d, a, b, i); break;
+    case 8: mma2_f16_scaled<8>(d, a, b, i); break;
+    case 9: mma2_f16_scaled<9>(d, a, b, i); break;
+    case 10: mma2_f16_scaled<10>(d, a, b, i); break;
+    case 11: mma2_f16_scaled<11>(d, a, b, i); break;
+    case 12: mma2_f16_scaled<12>(d, a, b, i); break;
+    case 13: mma2_f16_scaled<13>(d, a, b, i); break;
+    case 14: mma2_f16_scaled<14>(d, a, b, i); break;
+    default: mma2_f16_scaled<15>(d, a, b, i); break;
+  }
+}
+
+constexpr int BK_HALF = 64;                    // K elements of a 128-byte row of FP16
+constexpr unsigned kBadPanel = 1u << 30;       // in a counter of finished tiles: their rows of the copy may not be used
+
+// What the producer finds out about a problem from the copies' infos (all of them in a few lines of L2, which thousands of
+// warps must not read per tile).  use: its tiles are computed from the copies; 2^sum0, 2^sum1: scale of A1 B1 and of A2 B2.  With
+// two operand pairs the second goes first, and where the first begins the sums are brought to its scale (scale-input-d: exact, but
+// downwards only).  out: exponent of the scale of D's copy.
+struct HalfUse { int use, sum0, sum1, out; };
+
+// Exponent of the scale of D's copy: |D| is bounded from the operands' largest magnitudes m, and 2^e takes the bound below 2^15.
+// (The bound is reached by operands without any cancellation; sums of K terms of random sign stay about sqrt(K) / 2 below it, so
+// at K = 4096 the largest element comes to lie near 2^9, 22 binary orders above what kHalfLeast lets pass.)  Sigmoids need no
+// bound.  Where the next contraction adds A2 B2 to the product of this copy with W (hnext: infos of A2, B2, W), its scale must not
+// be above theirs.
+constexpr int kSigmoidExp = 15;
+__device__ __forceinline__ int out_exponent(const Tf32Params& p, const unsigned (&m)[4]) {
+  if (p.sigmoid) return kSigmoidExp;
+  float bound = (float)p.K[0] * __uint_as_float(m[0]) * __uint_as_float(m[1]) + (float)p.K[1] * __uint_as_float(m[2]) * __uint_as_float(m[3]);
+  if (p.bias) bound += __uint_as_float(p.K[1] > 0 ? m[3] : m[1]);
+  bound *= fabsf(p.alpha) * (p.dsig ? 0.25f : 1.f);
+  int e = half_exponent(__float_as_uint(bound) & 0x7fffffffu);
+  if (p.hnext[0]) e = min(e, max(-kHalfMaxExp, __ldcg(&p.hnext[0]->e) + __ldcg(&p.hnext[1]->e) - __ldcg(&p.hnext[2]->e)));
+  return e;
+}
+// a1_here: A1's copy is written by this very launch (a sigmoid's; the tiles say with the counter whether it may be used).
+__device__ __forceinline__ HalfUse half_use(const Tf32Params& p, bool a1_here) {
+  HalfUse u{0, 0, 0, 0};
+  if (!p.half && !p.copy_out) return u;
+  const int n = p.K[1] > 0 ? 4 : 2;
+  int e[4] = {0, 0, 0, 0};
+  unsigned amax[4] = {0u, 0u, 0u, 0u}, bad = 0u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (k < n) {
+      const int4 i = __ldcg(reinterpret_cast<const int4*>(p.hin[k]));
+      const bool here = k == 0 && a1_here;
+      e[k] = here ? kSigmoidExp : i.x;
+      amax[k] = here ? __float_as_uint(1.f) : (unsigned)i.y;
+      if (!here) bad |= (unsigned)i.z;
+    }
+  if (p.half) {
+    u.sum0 = e[0] + e[1]; u.sum1 = n == 4 ? e[2] + e[3] : u.sum0;
+    u.use = bad == 0u && abs(u.sum0) <= kHalfMaxExp && abs(u.sum1) <= kHalfMaxExp && u.sum1 >= u.sum0 && u.sum1 - u.sum0 <= 60;
+  }
+  if (p.copy_out) u.out = out_exponent(p, amax);
+  return u;
+}
+
+// Word from the producer to its CTA's epilogue warps, one per tile, tagged with the tile's place in the pair's work list: form of
+// the operands, exponent that undoes the scale of the sums, exponent of the scale of D's copy.  The ring of words is longer
+// than the producer can be ahead: two tiles in tensor memory, the operand slots, the tile it is at.
+constexpr int TILE_WORDS = 16;
+__device__ __forceinline__ int tile_word(int wi, int use, int un, int out) { return use | (un + 128) << 1 | (out + 128) << 9 | ((wi + 1) & 0x3fff) << 17; }
+
+struct Work { int prob, tile, sl, sliced; };
+
+// Its k-blocks: all, or slice sl of them.
+__device__ __forceinline__ void k_range(const Tf32Params& p, const Work& w, bool half, int& kb0, int& kb1) {
+  const int total = half ? p.khalf[0] + p.khalf[1] : p.kblocks[0] + p.kblocks[1];
+  kb0 = w.sliced ? (int)((long long)total * w.sl / p.slices) : 0;
+  kb1 = w.sliced ? (int)((long long)total * (w.sl + 1) / p.slices) : total;
+}
+// Counter of finished tiles that a tile's first A operand (its row panel) or K operand (all) waits for.
+__device__ __forceinline__ const int* dep_counter(const GroupParams& gp, const Work& w) {
+  const int d = gp.dep_prob[w.prob];
+  return gp.done + (long long)d * gp.done_stride + (gp.dep_all[w.prob] ? gp.done_stride - 1 : w.tile / gp.pr[w.prob].tiles_n);
+}
 
 // idx-th piece of work of CTA pair `pair` (see Tf32Params and GroupParams); false when the pair has no more.
 // A single problem whose left-over tiles are cut along K: the pair does its slice FIRST; the store of the partial
@@ -326,28 +449,26 @@ struct Work { int prob, tile, kb0, kb1, sliced; };
 __device__ __forceinline__ bool next_work(const GroupParams& gp, int pair, int idx, Work& w) {
   if (gp.pr[0].slices >= 2) {                  // (only ever set for a launch with one problem)
     const Tf32Params& p = gp.pr[0];
-    const int total_kb = p.kblocks[0] + p.kblocks[1];
     w.prob = 0;
     if (pair < p.rem * p.slices) {
       if (idx == 0) {
-        const int j = pair / p.slices, sl = pair - j * p.slices;
+        const int j = pair / p.slices;
         w.tile = p.waves * p.P + j;
-        w.kb0 = (int)((long long)total_kb * sl / p.slices);
-        w.kb1 = (int)((long long)total_kb * (sl + 1) / p.slices);
+        w.sl = pair - j * p.slices;
         w.sliced = 1;
         return true;
       }
       --idx;
     }
     if (idx >= p.waves) return false;
-    w.tile = idx * p.P + pair; w.kb0 = 0; w.kb1 = total_kb; w.sliced = 0;
+    w.tile = idx * p.P + pair; w.sl = 0; w.sliced = 0;
     return true;
   }
   for (int g = 0; g < gp.n_prob; ++g) {
     const Tf32Params& p = gp.pr[g];
     const int r0 = gp.rstart[g][pair], n_rem = gp.rstart[g][pair + 1] - r0;
     if (idx < p.waves + n_rem) {
-      w.prob = g; w.kb0 = 0; w.kb1 = p.kblocks[0] + p.kblocks[1]; w.sliced = 0;
+      w.prob = g; w.sl = 0; w.sliced = 0;
       w.tile = idx < p.waves ? idx * p.P + pair : p.waves * p.P + r0 + (idx - p.waves);
       return true;
     }
@@ -356,14 +477,12 @@ __device__ __forceinline__ bool next_work(const GroupParams& gp, int pair, int i
   return false;
 }
 
-// Epilogue of one whole, 16-byte-aligned 32 x 32 chunk of a warp's quadrant in the fragment layout of
-// tmem_ld_16x256b_x4: value v[4j + 2e + i] of half h is element (row 16h + 8e + lane / 4, column 8j + 2 (lane % 4) + i).
-// The epilogue warps are few (two per scheduler) and run beside the main loop, so what bounds them is their own
-// instruction stream, not the memory system: the same chunk took 10.7 us with every option tested per element
-// and 3.6 us as a plain store.  MODE fixes the options at compile time: 0 = alpha * acc (+ bias), 1 = sigmoid,
-// 2 = times the sigmoid derivative of `dsig`, 3 = plus beta * cin; 4 = any combination, tested at run time (its operands
-// are read where they are used, so that it needs no more registers than the others: the kernel is at its limit
-// of 168 and a spill here would be paid by every mode).
+// Epilogue of a warp's 16 x 32 pieces of a tile, on 16-byte aligned rows, in the fragment layout of tmem_ld_16x256b_x4: value
+// v[4j + 2e + i] is element (row 8e + lane / 4, column 8j + 2 (lane % 4) + i).  Sixteen warps run this beside the main loop, four per
+// scheduler; each waits for its operands most of the time, so the warps' number and the loads they keep in flight are
+// what counts (a piece's operands are requested before the piece before it is computed), and after that the instruction stream.
+// MODE fixes the options at compile time: 0 = alpha * acc (+ bias), 1 = sigmoid, 2 = times the sigmoid derivative of `dsig`,
+// 3 = plus beta * cin.  (Combinations, none of them on the path, go element by element: epilogue_ragged.)
 struct EpiArgs {
   const float* dsig; const float* cin; const float* bias; float* D;
   long long ldd, ld_dsig, ld_cin;
@@ -371,94 +490,163 @@ struct EpiArgs {
   int dsig_direct;           // ... which is m itself when dsig_div == 1 and dsig_rows >= M (no division per row)
   float alpha, beta;
   int M, sigm;
+  float un;                  // what undoes the scale of the sums (1 for TF32 operands)
+  __half* Dh; long long ldh; float hsc;      // copy of D, and its scale
 };
+
 
 __device__ __forceinline__ long long dsig_row(const EpiArgs& a, int m) {
   return a.dsig_direct ? m : (m / a.dsig_div) % a.dsig_rows;
 }
 
-template <int MODE>
-__device__ __forceinline__ void epilogue_full_chunk(const EpiArgs& a, uint32_t taddr, int mq, int nb, int lane,
-                                                    const float* ws, int slices) {
-  const bool use_sigm = MODE == 4 ? a.sigm != 0 : MODE == 1;
-  const bool use_dsig = MODE == 4 ? a.dsig != nullptr : MODE == 2;
-  const bool use_cin = MODE == 4 ? a.cin != nullptr : MODE == 3;
-  float2 op[2][8];                             // [h][4e + j]: the chunk of dsig (mode 2) or of cin (mode 3)
-  if (MODE == 2 || MODE == 3) {                // all global reads of the chunk in flight before anything waits
+// This warp's pieces of a tile: column chunks first, first + step, ... below end of the 16 rows whose element 0 this thread holds in
+// row m (and m + 8); column nb0 + 32 c of this thread in chunk c.  slices > 0: a tile cut along K, its partial sums at ws.
+struct PieceRun { uint32_t taddr; int m, nb0, first, step, end; const float* ws; int slices; };
+
+// The sums of a piece: from tensor memory, or of the slices' partials, slice 0 first.
+__device__ __forceinline__ void piece_sums(const PieceRun& r, int c, float (&v)[16]) {
+  if (r.slices == 0) {
+    tmem_ld_16x256b_x4(r.taddr + (uint32_t)(c * 32), v);
+    tmem_ld_wait();
+    return;
+  }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+  for (int i = 0; i < 16; ++i) v[i] = 0.f;
+  for (int s2 = 0; s2 < r.slices; ++s2) {
+    const float* wsr = r.ws + c * 32 + (long long)s2 * (2 * BM * BN_MAX);
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int m = mq + 16 * h + 8 * e;
-        const float* row = nullptr;
-        if (m < a.M) row = MODE == 3 ? a.cin + (long long)m * a.ld_cin + nb
-                                     : a.dsig + dsig_row(a, m) * a.ld_dsig + nb;
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 x = __ldcg(reinterpret_cast<const float2*>(wsr + (8 * e) * BN_MAX + 8 * j));
+        v[4 * j + 2 * e] += x.x; v[4 * j + 2 * e + 1] += x.y;
+      }
+  }
+}
+
+// HALF: D's FP16 copy is written too.  The runs of it that are looked at are a thread's 8 elements of a row and 2 of a column of
+// the piece; two threads swap halves of what they hold so that a store covers whole 32-byte sectors.
+template <int MODE, bool HALF>
+__device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun& r, int N, int lane, HalfCheck& check) {
+  constexpr bool ONE_OP = MODE == 2 || MODE == 3;
+  const bool ok[2] = {r.m < a.M, r.m + 8 < a.M};
+  const float* orow[2] = {nullptr, nullptr};   // this thread's rows of dsig (mode 2) or of cin (mode 3)
+  if (ONE_OP) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (ok[e]) orow[e] = (MODE == 3 ? a.cin + (long long)(r.m + 8 * e) * a.ld_cin : a.dsig + dsig_row(a, r.m + 8 * e) * a.ld_dsig) + r.nb0;
+  }
+  float* const drow = a.D + (long long)r.m * a.ldd + r.nb0;
+#pragma unroll 1
+  for (int c = r.first; c < r.end; c += r.step) {
+    bool in[4];                                // (N is a multiple of four: a thread's pair, and what it stores of a copy, is in or out)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) in[j] = r.nb0 + c * 32 + 8 * j < N;
+    float2 op[ONE_OP ? 8 : 1];                 // [4e + j], requested before anything is waited for
+    if (ONE_OP) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           float2 x = make_float2(0.f, 0.f);
           // (cin: L2-coherent read, in a chained launch it may have been written by another pair of this very launch)
-          if (row) x = MODE == 3 ? __ldcg(reinterpret_cast<const float2*>(row + 8 * j)) : __ldg(reinterpret_cast<const float2*>(row + 8 * j));
-          op[h][4 * e + j] = x;
+          if (ok[e] && in[j]) x = MODE == 3 ? __ldcg(reinterpret_cast<const float2*>(orow[e] + c * 32 + 8 * j)) : __ldg(reinterpret_cast<const float2*>(orow[e] + c * 32 + 8 * j));
+          op[ONE_OP ? 4 * e + j : 0] = x;
         }
-      }
-  }
-  float2 bz[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) bz[j] = a.bias ? __ldg(reinterpret_cast<const float2*>(a.bias + nb + 8 * j)) : make_float2(0.f, 0.f);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {                // one 16-row half of the chunk at a time (16 accumulator registers live)
-    float v[16];
-    if (slices == 0) {
-      tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * h) << 16), v);
-      tmem_ld_wait();
-    } else {                                   // a tile cut along K: sum of the slices' partials, slice 0 first
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = 0.f;
-      for (int s2 = 0; s2 < slices; ++s2) {
-        const float* wsr = ws + (long long)s2 * (2 * BM * BN_MAX) + (16 * h) * BN_MAX;
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float2 x = __ldcg(reinterpret_cast<const float2*>(wsr + (8 * e) * BN_MAX + 8 * j));
-            v[4 * j + 2 * e] += x.x; v[4 * j + 2 * e + 1] += x.y;
-          }
-      }
     }
+    float2 bz[4];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int m = mq + 16 * h + 8 * e;
-      if (m >= a.M) continue;
-      float* drow = a.D + (long long)m * a.ldd + nb;
-      const float* crow = (MODE == 4 && use_cin) ? a.cin + (long long)m * a.ld_cin + nb : nullptr;
-      const float* zrow = (MODE == 4 && use_dsig) ? a.dsig + dsig_row(a, m) * a.ld_dsig + nb : nullptr;
+    for (int j = 0; j < 4; ++j) bz[j] = a.bias && in[j] ? __ldg(reinterpret_cast<const float2*>(a.bias + r.nb0 + c * 32 + 8 * j)) : make_float2(0.f, 0.f);
+    float v[16];
+    piece_sums(r, c, v);
+    unsigned hv[2][HALF ? 4 : 1];
+    float row[2] = {0.f, 0.f};
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float x0 = v[4 * j + 2 * e] + bz[j].x, x1 = v[4 * j + 2 * e + 1] + bz[j].y;
-        if (use_sigm) { x0 = 1.f / (1.f + __expf(-x0)); x1 = 1.f / (1.f + __expf(-x1)); }
-        if (use_dsig) {
-          const float2 z = MODE == 4 ? __ldg(reinterpret_cast<const float2*>(zrow + 8 * j)) : op[h][4 * e + j];
+    for (int j = 0; j < 4; ++j) {
+      float c0 = 0.f, c1 = 0.f;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        float x0 = fmaf(v[4 * j + 2 * e], a.un, bz[j].x), x1 = fmaf(v[4 * j + 2 * e + 1], a.un, bz[j].y);
+        if (MODE == 1) { x0 = sigmoid_from(__expf(-x0)); x1 = sigmoid_from(__expf(-x1)); }
+        if (MODE == 2) {
+          const float2 z = op[ONE_OP ? 4 * e + j : 0];
           x0 *= z.x * (1.f - z.x); x1 *= z.y * (1.f - z.y);
         }
         x0 *= a.alpha; x1 *= a.alpha;
         if (MODE == 3) {
-          const float2 cc = op[h][4 * e + j];
-          x0 = fmaf(a.beta, cc.x, x0); x1 = fmaf(a.beta, cc.y, x1);
-        } else if (MODE == 4 && use_cin) {
-          const float2 cc = __ldcg(reinterpret_cast<const float2*>(crow + 8 * j));
+          const float2 cc = op[ONE_OP ? 4 * e + j : 0];
           x0 = fmaf(a.beta, cc.x, x0); x1 = fmaf(a.beta, cc.y, x1);
         }
-        *reinterpret_cast<float2*>(drow + 8 * j) = make_float2(x0, x1);
+        if (ok[e] && in[j]) *reinterpret_cast<float2*>(drow + 8 * e * a.ldd + c * 32 + 8 * j) = make_float2(x0, x1);
+        if (HALF) {
+          const float y0 = ok[e] && in[j] ? x0 * a.hsc : 0.f, y1 = ok[e] && in[j] ? x1 * a.hsc : 0.f;
+          row[e] = max3_abs(row[e], y0, y1);
+          if (e == 0) { c0 = y0; c1 = y1; } else { check.run(max3_abs(c0, y0, y0)); check.run(max3_abs(c1, y1, y1)); }
+          const __half2 y = __floats2half2_rn(y0, y1);
+          hv[e][HALF ? j : 0] = *reinterpret_cast<const unsigned*>(&y);
+        }
+      }
+    }
+    if (HALF) {
+      const bool odd = lane & 1;
+      __half* const hrow = a.Dh + (long long)r.m * a.ldh + r.nb0 + c * 32 + (odd ? 6 : 0);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        check.run(row[e]);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2) {       // even lanes: columns 8 j + 0..3 or 4..7, odd lanes the same of 8 (j + 1)
+          const unsigned mine = odd ? hv[e][HALF ? j + 1 : 0] : hv[e][HALF ? j : 0];
+          const unsigned other = __shfl_xor_sync(0xffffffffu, odd ? hv[e][HALF ? j : 0] : hv[e][HALF ? j + 1 : 0], 1);
+          if (ok[e] && (odd ? in[j + 1] : in[j])) *reinterpret_cast<uint2*>(hrow + 8 * e * a.ldh + 8 * j) = odd ? make_uint2(other, mine) : make_uint2(mine, other);
+        }
       }
     }
   }
 }
 
+// The same of pieces that are ragged or unaligned, or that combine options, element by element.
+__device__ __forceinline__ void epilogue_ragged(const EpiArgs& a, const PieceRun& r, int N, HalfCheck& check) {
+#pragma unroll 1
+  for (int c = r.first; c < r.end; c += r.step) {
+    float v[16];
+    piece_sums(r, c, v);
+    float row[2] = {0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int n = r.nb0 + c * 32 + 8 * j + i;
+        float col = 0.f;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int m = r.m + 8 * e;
+          if (n < N && m < a.M) {
+            float x = fmaf(v[4 * j + 2 * e + i], a.un, a.bias ? __ldg(a.bias + n) : 0.f);
+            if (a.sigm) x = sigmoid_from(__expf(-x));
+            if (a.dsig) { const float z = __ldg(a.dsig + dsig_row(a, m) * a.ld_dsig + n); x *= z * (1.f - z); }
+            x *= a.alpha;
+            if (a.cin) x = fmaf(a.beta, __ldcg(a.cin + (long long)m * a.ld_cin + n), x);
+            a.D[(long long)m * a.ldd + n] = x;
+            if (a.Dh) {
+              const float y = x * a.hsc;
+              row[e] = max3_abs(row[e], y, y);
+              col = max3_abs(col, y, y);
+              a.Dh[(long long)m * a.ldh + n] = __float2half_rn(y);
+            }
+          }
+        }
+        if (a.Dh) check.run(col);
+      }
+    if (a.Dh) { check.run(row[0]); check.run(row[1]); }
+  }
+}
+
+constexpr int PAIR_EPI_WARPS = 16, PAIR_THREADS = 64 + 32 * PAIR_EPI_WARPS;
 constexpr int B2_STAGE_MAX = (BN_MAX / 2) * BK * 4;          // 16 KB: this CTA's half of the B tile
 constexpr int STAGE2_BYTES = A_STAGE_BYTES + B2_STAGE_MAX;   // 32 KB
 
 template <int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
 gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constant__ GroupParams gp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -468,7 +656,9 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
   uint64_t* acc_empty = acc_full + 2;    // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
+  volatile int* tile_words = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [TILE_WORDS]
+  volatile int* tile_form = tile_words + TILE_WORDS;   // [STAGES], from the producer to the MMA issuer with a
+                                                                              // tile's first slot: 1 = FP16 copies, + 2 x scale step
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1;
@@ -476,8 +666,9 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 16); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * PAIR_EPI_WARPS); }
     *abort_flag = 0;
+    for (int i = 0; i < TILE_WORDS; ++i) tile_words[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 2) {  // both CTAs of the pair allocate all 512 columns, same warp, same destination offset
@@ -493,50 +684,120 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (both CTAs)
-    int it = 0;
+    int s = 0;                                 // ring slot and its phase
+    uint32_t ph = 0;
     bool ok = true;
     Work w;
+    HalfUse hu{0, 0, 0, 0};
+    int hu_prob = -1;
     for (int wi = 0; ok && next_work(gp, pair, wi, w); ++wi) {
       const Tf32Params& p = gp.pr[w.prob];
       const int bn = p.bn, hb = p.bn >> 1;                     // hb: B rows staged by each CTA
-      const uint32_t pair_tx = 2u * (A_STAGE_BYTES + (uint32_t)hb * BK * 4);
-      const int t = w.tile, kb0 = w.kb0, kb1 = w.kb1;
+      const int t = w.tile;
       const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM;
       const int n0 = (t % p.tiles_n) * bn + (int)rank * hb;
-      if (gp.dep_prob[w.prob] >= 0) {
+      const int dp = gp.dep_prob[w.prob];
+      const bool a1_here = dp >= 0 && p.half && gp.pr[dp].hout == p.hin[0];
+      int bad_panel = 0;
+      if (dp >= 0) {
         // an operand of this tile is written by an earlier problem of this launch: wait until its tiles are stored
-        const int d = gp.dep_prob[w.prob];
-        const int* ctr = gp.done + (long long)d * gp.done_stride + (gp.dep_all[w.prob] ? gp.done_stride - 1 : t / p.tiles_n);
-        const int want = 16 * (gp.dep_all[w.prob] ? gp.pr[d].tiles : gp.pr[d].tiles_n);
+        const int* const ctr = dep_counter(gp, w);
+        const int want = 2 * PAIR_EPI_WARPS * (gp.dep_all[w.prob] ? gp.pr[dp].tiles : gp.pr[dp].tiles_n);
         int good = 1;
         if (lane == 0) {
           const unsigned long long t0 = globaltimer();
-          while (ld_acquire_gpu(ctr) < want) {
+          int seen;
+          while (((seen = ld_acquire_gpu(ctr)) & (int)(kBadPanel - 1u)) < want) {
             if (*abort_flag || globaltimer() - t0 > WAIT_LIMIT_NS) { atomicCAS(err, 0, 6); *abort_flag = 1; good = 0; break; }
             __nanosleep(100);
           }
+          if (seen & (int)kBadPanel) good |= 2;
         }
         good = __shfl_sync(0xffffffffu, good, 0);
-        if (!good) { ok = false; break; }
+        if (!(good & 1)) { ok = false; break; }
+        bad_panel = good >> 1;
         asm volatile("fence.proxy.async.global;" ::: "memory");   // the stores were generic, the loads below are TMA's
         __syncwarp();
       }
-      for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        const int s = it % STAGES;
-        const uint32_t ph = (it / STAGES) & 1;
+      if (w.prob != hu_prob) { hu = half_use(p, a1_here); hu_prob = w.prob; }
+      const bool half = hu.use != 0 && !(a1_here && bad_panel);
+      int kb0, kb1;
+      k_range(p, w, half, kb0, kb1);
+      if (lane == 0)             // (a slice may end before the first operand pair)
+        tile_words[wi % TILE_WORDS] = tile_word(wi, half ? 1 : 0, half ? -(p.khalf[1] > 0 && kb1 <= p.khalf[1] ? hu.sum1 : hu.sum0) : 0, hu.out);
+      const int first = half && p.khalf[1] > 0 ? 1 : 0;        // operand pair that goes first
+      const int n_first = half ? p.khalf[first] : p.kblocks[0];
+      // (an FP16 box covers 128 bytes of a row too: a slot holds 64 terms instead of 32.  MN-major copies are staged in chunks of 64
+      // columns: a half tile of 96 takes two, each with a box of its own because it does not start on a multiple of 64)
+      const int b_boxes = half && p.b_mn ? (hb + 63) / 64 : 0;
+      const uint32_t pair_tx = 2u * (A_STAGE_BYTES + (b_boxes ? (uint32_t)b_boxes * 8192u : (uint32_t)hb * BK * 4));
+      const int a_boxes = half || !p.a_mn || p.a_3d ? 1 : BM / 32;
+      const bool one_box = a_boxes == 1 && (half ? b_boxes < 2 || hb % 64 == 0 : !p.b_mn || p.b_3d);
+      if (one_box) {
+        // one thread, and nothing in the loop that need not be there (as for the MMA issuer)
+        int good = 1;
+        if (lane == 0) {
+          const CUtensorMap* const maps = half ? gm.h[w.prob] : gm.m[w.prob];
+          const int bk = half ? BK_HALF : BK, am = m0 / (half ? 64 : 32), bm = n0 / (half ? 64 : 32);
+          const bool a3 = p.a_mn != 0, b3 = p.b_mn != 0;
+          for (int kb = kb0; kb < kb1; ++kb) {
+            if (!wait_or_abort(&empty[s], ph ^ 1, abort_flag, err, 1)) { good = 0; break; }
+            if (rank == 0) {
+              if (kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
+              mbar_expect_tx(&full[s], pair_tx);
+            }
+            const uint32_t full_leader = map_to_cta(smem_u32(&full[s]), 0);
+            const int pr = kb < n_first ? first : first ^ 1;
+            const int k0 = (kb < n_first ? kb : kb - n_first) * bk;
+            uint8_t* sa = smem + s * STAGE2_BYTES;
+            if (a3) tma2_load_3d(sa, maps + 2 * pr, 0, k0, am, full_leader);
+            else tma2_load_2d(sa, maps + 2 * pr, k0, m0, full_leader);
+            if (b3) tma2_load_3d(sa + A_STAGE_BYTES, maps + 2 * pr + 1, 0, k0, bm, full_leader);
+            else tma2_load_2d(sa + A_STAGE_BYTES, maps + 2 * pr + 1, k0, n0, full_leader);
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+          }
+        }
+        good = __shfl_sync(0xffffffffu, good, 0);
+        s = __shfl_sync(0xffffffffu, s, 0);
+        ph = __shfl_sync(0xffffffffu, ph, 0);
+        if (!good) { ok = false; break; }
+        continue;
+      }
+      for (int kb = kb0; kb < kb1; ++kb) {
         int good = 1;
         if (lane == 0) good = wait_or_abort(&empty[s], ph ^ 1, abort_flag, err, 1) ? 1 : 0;
         good = __shfl_sync(0xffffffffu, good, 0);
         if (!good) { ok = false; break; }
-        if (rank == 0 && lane == 0) mbar_expect_tx(&full[s], pair_tx);
+        if (rank == 0 && lane == 0) {
+          if (kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
+          mbar_expect_tx(&full[s], pair_tx);
+        }
         __syncwarp();
         const uint32_t full_leader = map_to_cta(smem_u32(&full[s]), 0);
-        const int pr = kb < p.kblocks[0] ? 0 : 1;
-        const int k0 = (pr == 0 ? kb : kb - p.kblocks[0]) * BK;
-        const CUtensorMap* ma = &gm.m[w.prob][2 * pr];
-        const CUtensorMap* mb = &gm.m[w.prob][2 * pr + 1];
+        const int pr = kb < n_first ? first : first ^ 1;
+        const int kk = kb < n_first ? kb : kb - n_first;
         uint8_t* sa = smem + s * STAGE2_BYTES;
         uint8_t* sb = sa + A_STAGE_BYTES;
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        if (half) {
+          const CUtensorMap* ma = &gm.h[w.prob][2 * pr];
+          const CUtensorMap* mb = &gm.h[w.prob][2 * pr + 1];
+          const int k0 = kk * BK_HALF;
+          if (lane == 0) {
+            if (!p.a_mn) tma2_load_2d(sa, ma, k0, m0, full_leader);
+            else tma2_load_3d(sa, ma, 0, k0, m0 / 64, full_leader);
+          } else if (lane == 8) {
+            if (!p.b_mn) tma2_load_2d(sb, mb, k0, n0, full_leader);
+            else if (hb % 64 == 0) tma2_load_3d(sb, mb, 0, k0, n0 / 64, full_leader);
+            else tma2_load_2d(sb, mb, n0, k0, full_leader);
+          } else if (lane == 9 && p.b_mn && hb % 64 != 0) {
+            tma2_load_2d(sb + 8192, mb, n0 + 64, k0, full_leader);
+          }
+          continue;
+        }
+        const int k0 = kk * BK;
+        const CUtensorMap* ma = &gm.m[w.prob][2 * pr];
+        const CUtensorMap* mb = &gm.m[w.prob][2 * pr + 1];
         if (!p.a_mn) {
           if (lane == 0) tma2_load_2d(sa, ma, k0, m0, full_leader);
         } else if (p.a_3d) {
@@ -557,39 +818,88 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
   } else if (warp == 1) {
     if (rank == 0 && lane == 0) {
       // ---------------------------------------------------------------- MMA issuer (leader CTA only)
-      int it = 0, ti = 0;
+      int s = 0, ti = 0;                       // ring slot and its phase, tiles done
+      uint32_t ph = 0;
       bool ok = true;
       Work w;
       for (int wi = 0; ok && next_work(gp, pair, wi, w); ++wi, ++ti) {
         const Tf32Params& p = gp.pr[w.prob];
-        const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(p.a_mn ? 1 : 0) << 15) |
-                               ((uint32_t)(p.b_mn ? 1 : 0) << 16) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-        const uint32_t a_lbo = p.a_mn ? BK * 128 : 16, b_lbo = p.b_mn ? BK * 128 : 16;
-        const uint32_t a_step = p.a_mn ? 1024 : 32, b_step = p.b_mn ? 1024 : 32;
-        const uint32_t a_sbo = p.a_mn ? 512 : 1024, b_sbo = p.b_mn ? 512 : 1024;
-        const uint32_t a_lay = p.a_mn ? 1 : 2, b_lay = p.b_mn ? 1 : 2;
-        const int kb0 = w.kb0, kb1 = w.kb1;
+        const uint32_t shape = (1u << 4) | ((uint32_t)(p.a_mn ? 1 : 0) << 15) | ((uint32_t)(p.b_mn ? 1 : 0) << 16) |
+                               ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
         const int buf = ti & 1;
         const uint32_t aph = (ti >> 1) & 1;
         ok = wait_or_abort(&acc_empty[buf], aph ^ 1, abort_flag, err, 4);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN_MAX);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
+        int form = 0;
+        if (p.half) {                          // (comes with the tile's first operands)
           ok = wait_or_abort(&full[s], ph, abort_flag, err, 2);
           if (!ok) break;
-          tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * STAGE2_BYTES);
-          const uint32_t sb = sa + A_STAGE_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / 8; ++k) {
-            const uint64_t ad = make_desc(sa + k * a_step, a_lbo, a_sbo, a_lay);
-            const uint64_t bd = make_desc(sb + k * b_step, b_lbo, b_sbo, b_lay);
-            mma2_tf32(tmem_d, ad, bd, idesc, (kb > kb0 || k != 0) ? 1u : 0u);
+          form = tile_form[s];
+        }
+        const bool half = form != 0;
+        int kb0, kb1;
+        k_range(p, w, half, kb0, kb1);
+        // scale step: before the first k-block of the first operand pair, where one of the second went before it
+        const int step_at = (form >> 1) > 0 && p.khalf[1] > kb0 && p.khalf[1] < kb1 ? p.khalf[1] : -1;
+        const uint32_t idesc = shape | (half ? 0u : (2u << 7) | (2u << 10));       // operands: FP16 or TF32
+        // MN-major: chunks of 64 (32) columns, BK_HALF (BK) rows of 128 bytes each
+        const uint32_t chunk = half ? BK_HALF * 128 : BK * 128, mn_sbo = half ? 1024 : 512, mn_lay = half ? 2 : 1;
+        const uint64_t mn_step = (half ? 2048 : 1024) >> 4;
+        const uint64_t a_step = p.a_mn ? mn_step : 32 >> 4, b_step = p.b_mn ? mn_step : 32 >> 4;       // (descriptors count in 16 bytes)
+        const uint32_t base = smem_u32(smem);
+        const uint64_t a0 = make_desc(base, p.a_mn ? chunk : 16, p.a_mn ? mn_sbo : 1024, p.a_mn ? mn_lay : 2);
+        const uint64_t b0 = make_desc(base + A_STAGE_BYTES, p.b_mn ? chunk : 16, p.b_mn ? mn_sbo : 1024, p.b_mn ? mn_lay : 2);
+        uint32_t acc = 0u;
+        // One thread issues everything, and what it takes per k-block (descriptors made anew, ring arithmetic, all forms of the
+        // scale step in the loop: 680 cycles with TF32 operands, 900 with FP16) was what bounded the main loop, where the
+        // instructions themselves need 512: so nothing is in the loop that need not be there.
+        for (int kb = kb0; ok && kb < kb1;) {
+          const int end = kb < step_at ? step_at : kb1;
+          if (half) {
+            if (kb == step_at) {
+              if (!wait_or_abort(&full[s], ph, abort_flag, err, 2)) { ok = false; break; }
+              tc_fence_after();
+              const uint64_t ad = a0 + (uint64_t)(s * (STAGE2_BYTES >> 4)), bd = b0 + (uint64_t)(s * (STAGE2_BYTES >> 4));
+              int down = form >> 1;
+#pragma unroll 1
+              for (int k = 0; k < 4; ++k, down -= 15) {
+                if (down > 0) mma2_f16_shift(min(down, 15), tmem_d, ad + k * a_step, bd + k * b_step, idesc);
+                else mma2_f16(tmem_d, ad + k * a_step, bd + k * b_step, idesc, 1u);
+              }
+              mma2_commit_both(&empty[s]);
+              if (++s == STAGES) { s = 0; ph ^= 1u; }
+              ++kb;
+            }
+#pragma unroll 1
+            for (; kb < end; ++kb) {
+              if (!wait_or_abort(&full[s], ph, abort_flag, err, 2)) { ok = false; break; }
+              tc_fence_after();
+              const uint64_t ad = a0 + (uint64_t)(s * (STAGE2_BYTES >> 4)), bd = b0 + (uint64_t)(s * (STAGE2_BYTES >> 4));
+              mma2_f16(tmem_d, ad, bd, idesc, acc);
+              acc = 1u;
+              mma2_f16(tmem_d, ad + a_step, bd + b_step, idesc, 1u);
+              mma2_f16(tmem_d, ad + 2 * a_step, bd + 2 * b_step, idesc, 1u);
+              mma2_f16(tmem_d, ad + 3 * a_step, bd + 3 * b_step, idesc, 1u);
+              mma2_commit_both(&empty[s]);
+              if (++s == STAGES) { s = 0; ph ^= 1u; }
+            }
+          } else {
+#pragma unroll 1
+            for (; kb < end; ++kb) {
+              if (!wait_or_abort(&full[s], ph, abort_flag, err, 2)) { ok = false; break; }
+              tc_fence_after();
+              const uint64_t ad = a0 + (uint64_t)(s * (STAGE2_BYTES >> 4)), bd = b0 + (uint64_t)(s * (STAGE2_BYTES >> 4));
+              mma2_tf32(tmem_d, ad, bd, idesc, acc);
+              acc = 1u;
+              mma2_tf32(tmem_d, ad + a_step, bd + b_step, idesc, 1u);
+              mma2_tf32(tmem_d, ad + 2 * a_step, bd + 2 * b_step, idesc, 1u);
+              mma2_tf32(tmem_d, ad + 3 * a_step, bd + 3 * b_step, idesc, 1u);
+              mma2_commit_both(&empty[s]);
+              if (++s == STAGES) { s = 0; ph ^= 1u; }
+            }
           }
-          mma2_commit_both(&empty[s]);
         }
         if (ok) mma2_commit_both(&acc_full[buf]);
       }
@@ -599,14 +909,18 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
     // Fragment layout of tmem_ld_16x256b_x4: this thread's 32 values of a 32 x 32 chunk are v[h][4j + 2e + i] =
     // element (row 16h + 8e + lane/4, column 8j + 2 (lane%4) + i) of the warp's quadrant.
     const int quad = warp & 3;
-    const int half = (warp - 2) >> 2;
-    const int rsub = lane >> 2, csub = (lane & 3) * 2;
+    const int sub = (warp - 2) >> 2;             // of the quadrant's four warps: rows 16 (sub % 2) .., every other column chunk
+    const int hh = sub & 1, half = sub >> 1;
+    const int rsub = 16 * hh + (lane >> 2), csub = (lane & 3) * 2;
     int ti = 0;
     Work w;
+    int amax_prob = -1;
+    unsigned amax_seen = 0u;                     // largest magnitude this warp has reported of that problem's copy
     for (int wi = 0; next_work(gp, pair, wi, w); ++wi, ++ti) {
       const Tf32Params& p = gp.pr[w.prob];
       const int bn = p.bn;
       const int t = w.tile;
+
       const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (t % p.tiles_n) * bn;
       const int buf = ti & 1;
       const uint32_t aph = (ti >> 1) & 1;
@@ -615,43 +929,57 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       good = __shfl_sync(0xffffffffu, good, 0);
       if (!good) break;
       tc_fence_after();
+      // (the producer has left the tile's word before it asked for the first operands: this loop ends at once)
+      int word = 0;
+      if (lane == 0) {
+        const unsigned long long t0 = globaltimer();
+        while (((word = tile_words[wi % TILE_WORDS]) >> 17) != ((wi + 1) & 0x3fff)) {
+          if (*abort_flag || globaltimer() - t0 > WAIT_LIMIT_NS) { atomicCAS(err, 0, 7); *abort_flag = 1; word = 0; break; }
+        }
+      }
+      word = __shfl_sync(0xffffffffu, word, 0);
+      if (word == 0) break;
+      const float un = word & 1 ? half_scale((word >> 1 & 0xff) - 128) : 1.f;
+      const int out_e = (word >> 9 & 0xff) - 128;
       const int n_chunks = min(bn / 32, (p.N - n0 + 31) / 32);   // column chunks of this tile that exist
-      const uint32_t tq = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN_MAX);
+      const uint32_t tq = tmem_base + ((uint32_t)(quad * 32 + 16 * hh) << 16) + (uint32_t)(buf * BN_MAX);
       int sl = 0, grp = 0;                                       // slice index and first pair of the tile's group
       if (w.sliced) {
         grp = (pair / p.slices) * p.slices;
         sl = pair - grp;
+        // (a tile of few rows or columns is few warps' work, and the others take no part in the count)
+        if (m0 + quad * 32 + 16 * hh >= p.M || half >= n_chunks) {
+          if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+          continue;
+        }
         // 1. raw accumulator of this slice to the workspace slot of this pair
         float* wsw = p.sk_ws + (((long long)pair * 2 + rank) * BM + quad * 32 + rsub) * BN_MAX + csub;
         for (int c = half; c < n_chunks; c += 2) {
-          float v[2][16];
-          tmem_ld_16x256b_x4(tq + (uint32_t)(c * 32), v[0]);
-          tmem_ld_16x256b_x4(tq + (16u << 16) + (uint32_t)(c * 32), v[1]);
+          float v[16];
+          tmem_ld_16x256b_x4(tq + (uint32_t)(c * 32), v);
           tmem_ld_wait();
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
+          for (int e = 0; e < 2; ++e)
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                __stcg(reinterpret_cast<float2*>(wsw + (long long)(16 * h + 8 * e) * BN_MAX + c * 32 + 8 * j),
-                       make_float2(v[h][4 * j + 2 * e], v[h][4 * j + 2 * e + 1]));
+            for (int j = 0; j < 4; ++j)
+              __stcg(reinterpret_cast<float2*>(wsw + (long long)(8 * e) * BN_MAX + c * 32 + 8 * j),
+                     make_float2(v[4 * j + 2 * e] * un, v[4 * j + 2 * e + 1] * un));
         }
         // the accumulator is free again; the tensor pipe has no further use for it in this pair
         tc_fence_before();
         __threadfence();
         __syncwarp();
         if (lane == 0) {
-          mbar_arrive_cluster(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+          mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
           int* flag_w = p.sk_flags + pair / p.slices;
           atomicAdd(flag_w, 1);
-          // 2. wait until the 16 warps of every slice of this tile have stored theirs
+          // 2. wait until the warps of both CTAs of every slice of this tile have stored theirs (16 rows, every other chunk each)
           const volatile int* flag = flag_w;
-          const int want = 16 * p.slices;
+          const int want = (min(2 * BM, p.M - (t / p.tiles_n) * (2 * BM)) + 15) / 16 * min(2, n_chunks) * p.slices;
           const unsigned long long t0 = globaltimer();
           while (*flag < want) {
             if (*abort_flag || globaltimer() - t0 > WAIT_LIMIT_NS) { atomicCAS(err, 0, 5); *abort_flag = 1; good = 0; break; }
-            __nanosleep(200);   // sixteen warps per pair poll the same word: keep them off the L2 while the pair's MMAs run
+            __nanosleep(200);   // up to thirty-two warps per pair poll the same word: keep them off the L2 while the pair's MMAs run
           }
           __threadfence();
           // 3. count out again: the last of the tile's warps to have seen the full count puts the flag back to
@@ -662,14 +990,18 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         good = __shfl_sync(0xffffffffu, good, 0);
         if (!good) break;
       }
+      bool bad_out = false;
       {
-        const int mq = m0 + quad * 32 + rsub;                    // this thread's rows are mq + 16h + 8e
+        const int mq = m0 + quad * 32 + rsub;                    // this thread's rows are mq and mq + 8
         EpiArgs ea;
         ea.dsig = dep(p.dsig); ea.cin = dep(p.cin); ea.bias = dep(p.bias); ea.D = p.D;
         ea.ldd = p.ldd; ea.ld_dsig = p.ld_dsig; ea.ld_cin = p.ld_cin;
         ea.dsig_rows = p.dsig_rows; ea.dsig_div = p.dsig_div;
         ea.dsig_direct = p.dsig_div == 1 && p.dsig_rows >= p.M;
         ea.alpha = p.alpha; ea.beta = p.beta; ea.M = p.M; ea.sigm = p.sigmoid;
+        ea.un = w.sliced ? 1.f : un;
+        ea.Dh = p.copy_out ? p.Dh : nullptr; ea.ldh = p.ldh; ea.hsc = half_scale(out_e);
+        HalfCheck check;
         const int N = p.N, vec_epi = p.vec_epi;
         const int n_opt = (p.sigmoid ? 1 : 0) + (p.dsig ? 1 : 0) + (p.cin ? 1 : 0);
         const int mode = n_opt == 0 ? 0 : n_opt > 1 ? 4 : p.sigmoid ? 1 : p.dsig ? 2 : 3;
@@ -679,70 +1011,42 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         const int c_step = w.sliced ? 2 * p.slices : 2;
         const int n_slices = w.sliced ? p.slices : 0;
         const float* const ws0 = w.sliced ? p.sk_ws + (((long long)grp * 2 + rank) * BM + quad * 32 + rsub) * BN_MAX + csub : nullptr;
-        for (int c = c_first; c < n_chunks; c += c_step) {
-          const int nb = n0 + c * 32 + csub;                     // this thread's columns are nb + 8j, nb + 8j + 1
-          const uint32_t taddr = tq + (uint32_t)(c * 32);
-          if (vec_epi && n0 + c * 32 + 32 <= N) {                // warp-uniform: whole chunk in range, 16-byte aligned rows
-            const float* ws = ws0 + c * 32;
-            switch (mode) {
-              case 0: epilogue_full_chunk<0>(ea, taddr, mq, nb, lane, ws, n_slices); break;
-              case 1: epilogue_full_chunk<1>(ea, taddr, mq, nb, lane, ws, n_slices); break;
-              case 2: epilogue_full_chunk<2>(ea, taddr, mq, nb, lane, ws, n_slices); break;
-              case 3: epilogue_full_chunk<3>(ea, taddr, mq, nb, lane, ws, n_slices); break;
-              default: epilogue_full_chunk<4>(ea, taddr, mq, nb, lane, ws, n_slices); break;
-            }
-            continue;
+        // (options of one kind on 16-byte aligned rows; anything else element by element)
+        const PieceRun run{tq, mq, n0 + csub, c_first, c_step, n_chunks, ws0, n_slices};
+        if (!vec_epi || mode == 4) {
+          epilogue_ragged(ea, run, N, check);
+        } else if (p.copy_out) {                                            // (only ever set with mode 1 or 2)
+          if (mode == 1) epilogue_pieces<1, true>(ea, run, N, lane, check);
+          else epilogue_pieces<2, true>(ea, run, N, lane, check);
+        } else {
+          switch (mode) {
+            case 0: epilogue_pieces<0, false>(ea, run, N, lane, check); break;
+            case 1: epilogue_pieces<1, false>(ea, run, N, lane, check); break;
+            case 2: epilogue_pieces<2, false>(ea, run, N, lane, check); break;
+            case 3: epilogue_pieces<3, false>(ea, run, N, lane, check); break;
+            default: break;
           }
-          // ragged or unaligned chunk: element by element
-#pragma unroll 1
-          for (int h = 0; h < 2; ++h) {
-            float v[16];
-            if (!w.sliced) {
-              tmem_ld_16x256b_x4(taddr + ((uint32_t)(16 * h) << 16), v);
-              tmem_ld_wait();
-            } else {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = 0.f;
-              for (int s2 = 0; s2 < n_slices; ++s2) {
-                const float* wsr = ws0 + c * 32 + (long long)s2 * (2 * BM * BN_MAX) + (16 * h) * BN_MAX;
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    const float2 x = __ldcg(reinterpret_cast<const float2*>(wsr + (8 * e) * BN_MAX + 8 * j));
-                    v[4 * j + 2 * e] += x.x; v[4 * j + 2 * e + 1] += x.y;
-                  }
-              }
+        }
+        if (p.copy_out) {
+          // this warp's word on the copy: the largest magnitude, and whether it may be used (the scale is said once)
+          const unsigned high = __reduce_max_sync(0xffffffffu, check.high);
+          bad_out = __any_sync(0xffffffffu, check.bad());
+          if (w.prob != amax_prob) { amax_prob = w.prob; amax_seen = 0u; }
+          if (lane == 0) {
+            if (t == 0 && warp == 2 && rank == 0) {
+              __stcg(&p.hout->e, out_e);
+              if (p.sigmoid) __stcg(&p.hout->amax, __float_as_uint(1.f));
             }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const int m = mq + 16 * h + 8 * e;
-              if (m >= ea.M) continue;
-              const float* zrow = ea.dsig ? ea.dsig + dsig_row(ea, m) * ea.ld_dsig : nullptr;
-              const float* crow = ea.cin ? ea.cin + (long long)m * ea.ld_cin : nullptr;
-              float* drow = ea.D + (long long)m * ea.ldd;
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                  const int n = nb + 8 * j + i;
-                  if (n < N) {
-                    float x = v[4 * j + 2 * e + i] + (ea.bias ? __ldg(ea.bias + n) : 0.f);
-                    if (ea.sigm) x = 1.f / (1.f + __expf(-x));
-                    if (zrow) { const float z = __ldg(zrow + n); x *= z * (1.f - z); }
-                    x *= ea.alpha;
-                    if (crow) x = fmaf(ea.beta, __ldcg(crow + n), x);
-                    drow[n] = x;
-                  }
-                }
-            }
+            if (!p.sigmoid && high > amax_seen) atomicMax(&p.hout->amax, __float_as_uint(__uint_as_float(high) * half_scale(-out_e)));
+            if (bad_out) atomicOr(&p.hout->bad, 1u);
           }
+          amax_seen = max(amax_seen, high);
         }
       }
       if (!w.sliced) {       // (a sliced tile released its accumulator right after storing it)
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+        if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
       }
       if (gp.signal[w.prob]) {
         // a later problem of this launch reads this tile: publish this warp's stores, then count the warp in
@@ -751,8 +1055,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         __syncwarp();
         if (lane == 0) {
           int* base = gp.done + (long long)w.prob * gp.done_stride;
-          if (gp.signal[w.prob] & 1) atomicAdd(base + t / p.tiles_n, 1);
-          if (gp.signal[w.prob] & 2) atomicAdd(base + gp.done_stride - 1, 1);
+          if (gp.signal[w.prob] & 1) { if (bad_out) atomicOr(base + t / p.tiles_n, (int)kBadPanel); atomicAdd(base + t / p.tiles_n, 1); }
+          if (gp.signal[w.prob] & 2) { if (bad_out) atomicOr(base + gp.done_stride - 1, (int)kBadPanel); atomicAdd(base + gp.done_stride - 1, 1); }
         }
       }
     }
@@ -800,6 +1104,30 @@ bool make_map(CUtensorMap* m, const float* base, long long rows, long long cols,
 // One box (32, BK, chunks) lands in shared memory as `chunks` consecutive [BK][32] blocks.  The last
 // chunk of a row may extend past MN (into the next row, or up to 124 bytes past the last row), so the
 // operand must be followed by that much readable memory.
+// The same of FP16 copies: 2-D, box = 64 columns x box_r rows, and 3-D, chunks of 64 columns, BK_HALF rows.
+bool make_half_map(CUtensorMap* m, const void* base, long long rows, long long cols, long long ld, int box_r) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+  cuuint32_t box[2] = {64, (cuuint32_t)box_r};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool make_half_map_mn3d(CUtensorMap* m, const void* base, long long K, long long MN, long long ld, int chunks) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {64, (cuuint64_t)K, (cuuint64_t)((MN + 63) / 64)};
+  cuuint64_t strides[2] = {(cuuint64_t)ld * 2, 128};
+  cuuint32_t box[3] = {64, (cuuint32_t)BK_HALF, (cuuint32_t)chunks};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool make_map_mn3d(CUtensorMap* m, const float* base, long long K, long long MN, long long ld, int chunks) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
@@ -851,7 +1179,7 @@ bool gemm_tf32_eligible(const GemmArgs& g) {
 
 constexpr int kStages2 = 6;
 constexpr int kMaxSlices = 16;   // K slices per left-over tile
-constexpr int kSmemBytes2 = kStages2 * STAGE2_BYTES + 1024 + 256;
+constexpr int kSmemBytes2 = kStages2 * STAGE2_BYTES + 1024 + 512;
 
 // Two-CTA tile width (a multiple of 64 so that each CTA's half is whole 32-column chunks).  With the
 // work split evenly over the pairs (stream-K) only the padding of N to whole tiles costs anything;
@@ -876,7 +1204,7 @@ int gemm_tf32_workspace_flags() { return num_sms() / 2; }
 namespace {
 
 // Tensor maps and kernel parameters of one problem for a given tile width (two_cta: 256 x bn tiles of a CTA pair).
-bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUtensorMap* maps, Tf32Params& p) {
+bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUtensorMap* maps, CUtensorMap* half_maps, Tf32Params& p) {
   const int b_rows = two_cta ? bn / 2 : bn;      // B rows staged per CTA
   const float* As[2] = {g.A1, g.A2};
   const float* Bs[2] = {g.B1, g.B2};
@@ -905,9 +1233,31 @@ bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUten
   p.dsig = g.dsig; p.ld_dsig = g.ld_dsig; p.dsig_rows = g.dsig_rows > 0 ? g.dsig_rows : 1; p.dsig_div = g.dsig_div > 0 ? g.dsig_div : 1;
   p.alpha = g.alpha;
   p.cin = g.cin; p.ld_cin = g.ld_cin; p.beta = g.beta;
-  p.vec_epi = aligned16(g.D) && (g.ldd % 4 == 0) && (!g.bias || aligned16(g.bias)) &&
+  p.vec_epi = g.N % 4 == 0 && aligned16(g.D) && (g.ldd % 4 == 0) && (!g.bias || aligned16(g.bias)) &&
               (!g.dsig || (aligned16(g.dsig) && g.ld_dsig % 4 == 0)) &&
               (!g.cin || (aligned16(g.cin) && g.ld_cin % 4 == 0));
+  for (int s = 0; s < 2; ++s) p.K[s] = Ks[s];
+  if (two_cta && (g.half || g.hout.p)) {
+    for (int k = 0; k < (g.A2 ? 4 : 2); ++k) p.hin[k] = g.h[k].info;
+    if (g.half) {
+      for (int s = 0; s < (g.A2 ? 2 : 1); ++s) {
+        const HalfMat& a = g.h[2 * s];
+        const HalfMat& b = g.h[2 * s + 1];
+        bool ok = g.a_kmajor ? make_half_map(&half_maps[2 * s], a.p, g.M, Ks[s], a.ld, BM)
+                             : make_half_map_mn3d(&half_maps[2 * s], a.p, Ks[s], g.M, a.ld, BM / 64);
+        if (g.b_kmajor) ok = ok && make_half_map(&half_maps[2 * s + 1], b.p, g.N, Ks[s], b.ld, b_rows);
+        else if (b_rows % 64 == 0) ok = ok && make_half_map_mn3d(&half_maps[2 * s + 1], b.p, Ks[s], g.N, b.ld, b_rows / 64);
+        else ok = ok && make_half_map(&half_maps[2 * s + 1], b.p, Ks[s], g.N, b.ld, BK_HALF);
+        if (!ok) return false;
+        p.khalf[s] = (Ks[s] + BK_HALF - 1) / BK_HALF;
+      }
+      p.half = 1;
+    }
+    if (g.hout.p) {
+      p.Dh = static_cast<__half*>(g.hout.p); p.ldh = g.hout.ld; p.hout = g.hout.info; p.copy_out = 1;
+      for (int k = 0; k < 3; ++k) p.hnext[k] = g.h_next[k];
+    }
+  }
   p.bn = bn;
   p.tiles_n = (g.N + bn - 1) / bn;
   p.tiles = ((g.M + (two_cta ? 2 : 1) * BM - 1) / ((two_cta ? 2 : 1) * BM)) * p.tiles_n;
@@ -929,6 +1279,11 @@ inline bool suits_pair_kernel(const GemmArgs& g) { return g.M > BM && g.N >= 128
 }  // namespace
 
 namespace {
+// k-blocks of a tile: 128 bytes of a row each, whatever the operands' type, and as long to multiply
+int kblocks_of(const GemmArgs& g) {
+  const int bk = g.half ? BK_HALF : BK;
+  return (g.K1 + bk - 1) / bk + (g.A2 ? (g.K2 + bk - 1) / bk : 0);
+}
 // K slices for the tiles left over after the whole waves of a problem with `tiles` tiles of `total_kb` k-blocks on
 // `pairs` CTA pairs (1 = whole tiles).  A sliced tile pays for a store and a re-read of its partial accumulators
 // and for the wait between them, about as much as 25 to 30 k-blocks of main loop (measured: a 25-k-block tile is
@@ -950,7 +1305,7 @@ int choose_slices(int tiles, int total_kb, int pairs) {
 int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_flags, cudaStream_t st) {
   set_kernel_attributes();
   const int pairs = num_sms() / 2;
-  const int total_kb_all = (g.K1 + BK - 1) / BK + (g.A2 ? (g.K2 + BK - 1) / BK : 0);
+  const int total_kb_all = kblocks_of(g);
   bool two_cta = g.two_cta >= 0 ? g.two_cta != 0 : suits_pair_kernel(g);
   if (!two_cta && g.two_cta < 0 && sk_ws && sk_flags) {
     // A result of at most 128 rows or fewer than 128 columns leaves part of a pair's tile empty, but the pair kernel can
@@ -975,8 +1330,8 @@ int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_fla
     for (int k = 0; k < MAX_GROUP; ++k) gp.dep_prob[k] = -1;
     gp.n_prob = 1;
     Tf32Params& p = gp.pr[0];
-    if (!setup_problem(g, true, bn, err_flag, gm.m[0], p)) return -1;
-    const int total_kb = p.kblocks[0] + p.kblocks[1];
+    if (!setup_problem(g, true, bn, err_flag, gm.m[0], gm.h[0], p)) return -1;
+    const int total_kb = total_kb_all;
     p.sk_ws = sk_ws; p.sk_flags = sk_flags;
     p.P = p.tiles < pairs ? p.tiles : pairs;
     p.waves = p.tiles / p.P;
@@ -991,11 +1346,11 @@ int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_fla
       }
     }
     for (int q = 0; q <= MAX_PAIRS_LAUNCH; ++q) gp.rstart[0][q] = (unsigned short)(q < p.rem ? q : p.rem);
-    launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * launch_pairs, 320, kSmemBytes2, st, gm, gp);
+    launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * launch_pairs, PAIR_THREADS, kSmemBytes2, st, gm, gp);
   } else {
     CUtensorMap maps[4];
     Tf32Params p;
-    if (!setup_problem(g, false, bn, err_flag, maps, p)) return -1;
+    if (!setup_problem(g, false, bn, err_flag, maps, nullptr, p)) return -1;
     const int grid = p.tiles < num_sms() ? p.tiles : num_sms();
     launch_pdl(gemm_tf32_kernel<kStages>, grid, 320, kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], p);
   }
@@ -1053,7 +1408,9 @@ void deal_tiles(GroupParams& gp, int k, double cost, int P, double* load) {
 }
 
 // time of one tile in k-blocks of a 256-wide tile: operand bytes per k-block (the feed bounds the main loop) plus a fixed part
-double tile_cost(const Tf32Params& p) { return (p.kblocks[0] + p.kblocks[1]) * (256.0 + p.bn) / 512.0 + 8.0; }
+double tile_cost(const Tf32Params& p) {
+  return (p.half ? p.khalf[0] + p.khalf[1] : p.kblocks[0] + p.kblocks[1]) * (256.0 + p.bn) / 512.0 + 8.0;
+}
 
 }  // namespace
 
@@ -1074,11 +1431,11 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
   struct Item { int src; double cost; };
   Item order[MAX_GROUP];
   Tf32Params tmp[MAX_GROUP];
-  CUtensorMap tmaps[MAX_GROUP][4];
+  CUtensorMap tmaps[MAX_GROUP][4], thalf[MAX_GROUP][4];
   long long total_tiles = 0;
   for (int i = 0; i < n; ++i) {
     const int bn = choose_bn2(gs[i].M, gs[i].N, true);
-    if (!setup_problem(gs[i], true, bn, err_flag, tmaps[i], tmp[i])) return -1;
+    if (!setup_problem(gs[i], true, bn, err_flag, tmaps[i], thalf[i], tmp[i])) return -1;
     if (tmp[i].tiles > 60000) return -1;       // (left-over tile indices are 16-bit)
     order[i].src = i;
     order[i].cost = tile_cost(tmp[i]);
@@ -1105,7 +1462,7 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
   for (int k = 0; k < n; ++k) {
     const int i = order[k].src;
     gp.pr[k] = tmp[i];
-    for (int j = 0; j < 4; ++j) gm.m[k][j] = tmaps[i][j];
+    for (int j = 0; j < 4; ++j) { gm.m[k][j] = tmaps[i][j]; gm.h[k][j] = thalf[i][j]; }
     deal_tiles(gp, k, order[k].cost, P, load);
     if (chain && dep_prob[i] >= 0) {            // (a chain keeps its order: slot == index)
       gp.dep_prob[k] = dep_prob[i];
@@ -1114,7 +1471,7 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
     }
   }
   if (chain && cudaMemsetAsync(done, 0, sizeof(int) * (size_t)n * done_stride, st) != cudaSuccess) return -1;
-  launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * P, 320, kSmemBytes2, st, gm, gp);
+  launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * P, PAIR_THREADS, kSmemBytes2, st, gm, gp);
   return 1;
 }
 

@@ -120,6 +120,22 @@ struct gn_ctx {
   bool split_together = true;                              // a contraction's operands in one splitting launch (else one each)
   bool own_capture = false, foreign_capture = false;       // the solver's step / the caller is capturing the stream
   uint64_t gemm_seq = 0;     // counts contractions (run_gemm calls)
+  // FP16 copies of the matrices that TF32 contractions of a large pass read (HalfInfo in gn_kernels.h): of the stored activations
+  // and theta's weights until these change, of everything else for the length of a pass.  One entry per FP32 matrix it stands for.
+  struct HalfBuf {
+    uint16_t* p = nullptr; int64_t cap = 0;                  // (cap: elements of an allocation of its own, 0: borrowed memory)
+    const float* base = nullptr; int64_t rows = 0; int cols = 0;   // the matrix the copy is of
+    int info = 0;                                            // index into half_info
+    bool valid = false, info_valid = false;                  // the copy, and its info, belong to what the matrix now holds
+  };
+  enum HalfSet { kHZ, kHRZ, kHDS, kHZb, kHDb, kHW, kHV, kHF, kHalfSets };   // (kHZb[0]: the rows of X of a batch; kHF: factors)
+  std::vector<HalfBuf> half_buf[kHalfSets];
+  HalfInfo* half_info = nullptr; unsigned* half_acc = nullptr;
+  uint16_t* half_weights = nullptr; std::vector<int64_t> half_at;   // the copies of theta's weights, then of a vector's; where layer m's starts
+  int half_mode = 1;         // 0 never, 1 where a pass is large enough, 2 wherever it can be done
+  bool half_usable = true;   // cleared if a copy's memory could not be had
+  bool half_now = false;     // the pass in progress works with copies
+  uint64_t half_theta_epoch = 0;
   float* small_scratch = nullptr; int64_t small_cap = 0;     // blocks' sums of a small network's pass
   bool small_enabled = true;
   int small_tf32 = -1;         // a TF32 context's passes are all small ones (-1: not looked at yet)
@@ -619,6 +635,208 @@ void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
   run_splits(c, jobs);
 }
 
+// ---- FP16 copies ---------------------------------------------------------------------------------
+using HalfBuf = gn_ctx::HalfBuf;
+
+int half_info_index(const gn_ctx* c, int set, int m) { return set * (c->L + 1) + (set == gn_ctx::kHV ? 0 : m); }   // (one scale for all of v)
+
+bool half_setup(gn_ctx* c) {
+  if (c->half_info) return true;
+  const int64_t n = (int64_t)gn_ctx::kHalfSets * (c->L + 1);
+  if (dev_alloc(c, &c->half_info, n) != GN_OK) return false;
+  c->half_at.assign((size_t)c->L + 2, 0);
+  for (int m = 1; m <= c->L; ++m) c->half_at[(size_t)m + 1] = c->half_at[(size_t)m] + c->w[m] * round8(c->w[m - 1]);
+  if (dev_alloc(c, &c->half_acc, (int64_t)kHalfSegs + 1) != GN_OK || dev_alloc(c, &c->half_weights, 2 * c->half_at.back()) != GN_OK) {
+    dev_free(c, c->half_acc); dev_free(c, c->half_info);
+    return false;
+  }
+  cudaMemsetAsync(c->half_info, 0, sizeof(HalfInfo) * (size_t)n, c->st);
+  cudaMemsetAsync(c->half_acc, 0, sizeof(unsigned) * (kHalfSegs + 1), c->st);
+  return true;
+}
+
+// Where the copy of entry m of a set has its place in memory that is there anyway: weights and vectors in theirs, and in FP32
+// memory of the context that holds nothing meanwhile, with as many rows and columns: a copy of R z^m is read before delta s^m is
+// written, and one of delta s^m is written when R z^m has been read for the last time.
+uint16_t* half_lender(const gn_ctx* c, int set, int m) {
+  if (set == gn_ctx::kHW) return c->half_weights + c->half_at[(size_t)m];
+  if (set == gn_ctx::kHV) return c->half_weights + c->half_at.back() + c->half_at[(size_t)m];
+  if (m < 1 || m >= c->L) return nullptr;
+  return reinterpret_cast<uint16_t*>(set == gn_ctx::kHRZ ? c->DS[(size_t)m] : set == gn_ctx::kHDS ? c->RZ[(size_t)m] : nullptr);
+}
+
+// Room for a copy of a rows x cols matrix at `base`.
+bool half_reserve(gn_ctx* c, HalfBuf& b, int set, int m, const float* base, int64_t rows, int cols, int64_t cap_rows) {
+  if (!half_setup(c)) return false;
+  const int64_t need = std::max(rows, cap_rows) * round8(cols);
+  if (uint16_t* lent = half_lender(c, set, m)) {
+    b.p = lent;
+  } else if (need > b.cap) {
+    if (b.cap > 0) { quiesce(c); dev_free(c, b.p); }
+    b.p = nullptr; b.cap = 0; b.valid = false;
+    if (dev_alloc(c, &b.p, need) != GN_OK) return false;
+    b.cap = need;
+  }
+  b.base = base; b.rows = rows; b.cols = cols; b.info = half_info_index(c, set, m);
+  b.valid = b.info_valid = false;
+  return true;
+}
+
+void half_invalidate(gn_ctx* c, int set) {
+  for (auto& b : c->half_buf[set]) b.valid = b.info_valid = false;
+}
+void half_drop(gn_ctx* c, int set) {
+  for (auto& b : c->half_buf[set]) {
+    if (b.cap > 0) dev_free(c, b.p);
+    b.p = nullptr; b.cap = 0; b.valid = b.info_valid = false;
+  }
+}
+// No room: the passes go on without copies.
+void half_give_up(gn_ctx* c) {
+  quiesce(c);
+  for (int set = 0; set < gn_ctx::kHalfSets; ++set) half_drop(c, set);
+  dev_free(c, c->half_weights); dev_free(c, c->half_acc); dev_free(c, c->half_info);
+  c->half_usable = false; c->half_now = false; ++c->dispatch_gen;
+}
+
+HalfMat half_mat(const gn_ctx* c, const HalfBuf& b) {
+  HalfMat h;
+  h.p = b.p; h.ld = round8(b.cols); h.info = c->half_info + b.info;
+  return h;
+}
+// The copy of the matrix at `src` with leading dimension ld, possibly a part of a larger one that starts on a copy's 16 bytes.
+bool half_find(const gn_ctx* c, const float* src, int64_t ld, HalfMat* out, bool info_only) {
+  for (int set = 0; set < gn_ctx::kHalfSets; ++set)
+    for (const HalfBuf& b : c->half_buf[set]) {
+      if (!(info_only ? b.info_valid : b.valid) || b.cols != ld || src < b.base || src >= b.base + b.rows * b.cols) continue;
+      const int64_t off = src - b.base, r = off / ld, col = off - r * ld;
+      if (!info_only && col % 8 != 0) return false;
+      *out = half_mat(c, b);
+      out->p = info_only ? nullptr : b.p + r * out->ld + col;
+      return true;
+    }
+  return false;
+}
+
+bool suits_half(const GemmArgs& g) {
+  return gemm_thin_kind(g) == THIN_NONE && g.M > 128 && g.N >= 128 && g.two_cta != 0 && gemm_tf32_eligible(g);
+}
+// The copies of a contraction's operands, if it can be computed from them and all are there.
+void attach_half(const gn_ctx* c, GemmArgs& g) {
+  if (!c->half_now || !suits_half(g)) return;
+  bool all = true;
+  for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
+    const float* p = role == 0 ? g.A1 : role == 1 ? g.B1 : role == 2 ? g.A2 : g.B2;
+    const int64_t ld = role == 0 ? g.lda1 : role == 1 ? g.ldb1 : role == 2 ? g.lda2 : g.ldb2;
+    if (!half_find(c, p, ld, &g.h[role], false)) {
+      all = false;
+      if (!half_find(c, p, ld, &g.h[role], true)) g.h[role] = HalfMat{};
+    }
+  }
+  g.half = all;
+}
+// ... and the copy of its result, which it writes (attach_half comes first).  The result is the matrix of `b`.
+void attach_half_out(const gn_ctx* c, GemmArgs& g, HalfBuf& b) {
+  b.valid = b.info_valid = false;
+  if (!c->half_now || !suits_half(g) || !b.p || b.base != g.D || b.cols != g.ldd) return;
+  for (int role = 0; role < (g.A2 ? 4 : 2); ++role)
+    if (!g.h[role].info) return;
+  g.hout = half_mat(c, b);
+  b.valid = b.info_valid = true;
+}
+
+// Copies by passes of their own.  infos: one largest-magnitude job per scale; every matrix of `bufs` is then copied.  The infos
+// from `reset` on are cleared on the way.
+bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::vector<HalfBuf*>& bufs, int reset = 0, int n_reset = 0) {
+  for (size_t i = 0; i < amax.size(); i += kHalfSegs) {
+    const int r = launch_half_amax(amax.data() + i, (int)std::min<size_t>(kHalfSegs, amax.size() - i), c->half_acc, c->half_info + reset, i == 0 ? n_reset : 0, c->st);
+    if (r < 0) { c->sticky = GN_ECUDA; c->err = "FP16 copies could not be made"; return false; }
+    c->launches += r;
+  }
+  std::vector<HalfCopyJob> jobs;
+  for (HalfBuf* b : bufs) jobs.push_back(HalfCopyJob{b->base, b->rows, b->cols, (int64_t)b->cols, half_mat(c, *b)});
+  for (size_t i = 0; i < jobs.size(); i += kHalfSegs) {
+    const int r = launch_half_copy(jobs.data() + i, (int)std::min<size_t>(kHalfSegs, jobs.size() - i), c->st);
+    if (r < 0) { c->sticky = GN_ECUDA; c->err = "FP16 copies could not be made"; return false; }
+    c->launches += r;
+  }
+  for (HalfBuf* b : bufs) b->valid = b->info_valid = true;
+  return true;
+}
+
+// Layers whose weights are an operand of a contraction that suits_half.
+bool half_layer(const gn_ctx* c, int m) { return c->w[m] >= 128 && c->w[m] % 4 == 0 && c->w[m - 1] % 4 == 0 && c->w_off[m] % 4 == 0; }
+// Whether a pass over `rows` rows is to work with copies.  They cost launches of their own (v, X, the output layer's delta) and
+// bytes; what they save grows with the weights.  Products, per mille of the time without copies: 784-300-300-10 (0.33e6 weights) 970 to
+// 1090 at 500 to 12000 rows, 784-500-500-10 (0.64e6) 920 to 970, 3072-1000-1000-10 (4.1e6) 850 to 950, 784-2000-2000-2000-10
+// 930 at 1000 rows and 690 at 12000.
+bool half_wanted(gn_ctx* c, int64_t rows) {
+  if (c->prec != GN_TF32 || c->half_mode == 0 || !c->half_usable || rows <= 128 || c->L < 2) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  // (what a caller captures is replayed after theta has changed: such a graph reads the FP32 matrices)
+  if (!c->own_capture && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) return false;
+  double weights = 0.0;
+  for (int m = 1; m <= c->L; ++m)
+    if (half_layer(c, m)) weights += (double)c->w[m - 1] * c->w[m];
+  return weights > 0.0 && (c->half_mode == 2 || (weights >= 5e5 && rows * weights >= 1e9));
+}
+struct HalfPass {                       // a pass that works with copies, or not
+  gn_ctx* c; bool before;
+  HalfPass(gn_ctx* ctx, bool on) : c(ctx), before(ctx->half_now) { c->half_now = on; }
+  ~HalfPass() { c->half_now = before; }
+};
+
+// theta's weights, once per theta.
+void half_theta(gn_ctx* c) {
+  if (!c->half_now || c->half_theta_epoch == c->theta_epoch) return;
+  std::vector<HalfAmaxJob> amax;
+  std::vector<HalfBuf*> bufs;
+  half_invalidate(c, gn_ctx::kHW);
+  for (int m = 1; m <= c->L; ++m) {
+    HalfBuf& b = c->half_buf[gn_ctx::kHW][(size_t)m];
+    const bool copy = half_layer(c, m) || (c->w[m - 1] >= 128 && c->w[m] > 16 && c->w[m] % 4 == 0 && c->w[m - 1] % 4 == 0 && c->w_off[m] % 4 == 0);
+    if (!copy) continue;
+    if (!half_reserve(c, b, gn_ctx::kHW, m, c->theta + c->w_off[m], c->w[m], c->w[m - 1], 0)) { half_give_up(c); return; }
+    amax.push_back(HalfAmaxJob{b.base, b.rows * b.cols, c->half_info + b.info});
+    bufs.push_back(&b);
+  }
+  if (half_convert(c, amax, bufs)) c->half_theta_epoch = c->theta_epoch;
+}
+
+// The vector of a product; the infos of what the product computes start afresh.
+void half_vector(gn_ctx* c, const float* v) {
+  if (!c->half_now) return;
+  std::vector<HalfBuf*> bufs;
+  half_invalidate(c, gn_ctx::kHV); half_invalidate(c, gn_ctx::kHRZ); half_invalidate(c, gn_ctx::kHDS);
+  for (int m = 1; m <= c->L; ++m) {
+    if (!half_layer(c, m)) continue;
+    HalfBuf& b = c->half_buf[gn_ctx::kHV][(size_t)m];
+    if (!half_reserve(c, b, gn_ctx::kHV, m, v + c->w_off[m], c->w[m], c->w[m - 1], 0)) { half_give_up(c); return; }
+    bufs.push_back(&b);
+  }
+  const std::vector<HalfAmaxJob> amax{HalfAmaxJob{v, c->n, c->half_info + half_info_index(c, gn_ctx::kHV, 0)}};
+  half_convert(c, amax, bufs, half_info_index(c, gn_ctx::kHRZ, 0), 2 * (c->L + 1));
+}
+
+// A copy of one matrix that something else than a contraction with a copy of its own has written.
+void half_matrix(gn_ctx* c, int set, int m, const float* base, int64_t rows, int cols, int64_t cap_rows, bool copy, int reset = 0, int n_reset = 0) {
+  if (!c->half_now) return;
+  HalfBuf& b = c->half_buf[set][(size_t)m];
+  if (!half_reserve(c, b, set, m, base, rows, cols, copy ? cap_rows : 0)) { half_give_up(c); return; }
+  std::vector<HalfBuf*> bufs;
+  if (copy) bufs.push_back(&b);
+  if (half_convert(c, {HalfAmaxJob{base, rows * cols, c->half_info + b.info}}, bufs, reset, n_reset)) b.info_valid = true;
+}
+
+// Room for the copies of the layers' matrices `mats` (1 .. top) that a pass over `rows` rows writes.
+bool half_room(gn_ctx* c, int set, const std::vector<float*>& mats, int top, int64_t rows, int64_t cap_rows) {
+  if (!c->half_now) return false;
+  for (int m = 1; m <= top; ++m)
+    if (c->w[m] >= 128 && c->w[m] % 4 == 0 &&
+        !half_reserve(c, c->half_buf[set][(size_t)m], set, m, mats[(size_t)m], rows, c->w[m], cap_rows)) { half_give_up(c); return false; }
+  return true;
+}
+
 // Independent contractions issued together (any order is allowed).  In TF32 mode those that suit the CTA-pair
 // kernel go out in launches of up to three problems with a common work list (the tiles of one fill the partial
 // last wave of another); everything else runs one after the other, in the order given.
@@ -803,7 +1021,18 @@ const float* Wm(const gn_ctx* c, const float* vec, int m) { return vec + c->w_of
 const float* bm(const gn_ctx* c, const float* vec, int m) { return vec + c->b_off[m]; }
 
 // Eq. (xtoz): Zout[m] = sigma(Zout[m-1] W^m + 1 b^mT), m = 1..L, over `rows` rows; Zout[0] = Z0.
-void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout) {
+// With copies (half_now): of Z0 as `set`'s entry 0, of the Z_m, all written here; cap_rows as of the buffers Zout.
+void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>& Zout, int set, int64_t cap_rows) {
+  half_theta(c);
+  half_invalidate(c, set);
+  if (c->half_now) {
+    // infos of what is about to be written, to be cleared: of Z_1 .. Z_L, and of a batch's deltas, which follow
+    const int reset = half_info_index(c, set, 1), n_reset = set == gn_ctx::kHZb ? 2 * c->L + 1 : c->L;
+    if (half_layer(c, 1)) half_matrix(c, set, 0, Z0, rows, c->w[0], cap_rows, true, reset, n_reset);
+    else cudaMemsetAsync(c->half_info + reset, 0, sizeof(HalfInfo) * (size_t)n_reset, c->st);
+    // (z^{L-1} is an operand of the output layer's contractions alone)
+    half_room(c, set, Zout, half_layer(c, c->L) ? c->L - 1 : c->L - 2, rows, cap_rows);
+  }
   std::vector<GemmArgs> gs((size_t)c->L);
   std::vector<int> dep((size_t)c->L), dep_all((size_t)c->L, 0);
   for (int m = 1; m <= c->L; ++m) {
@@ -815,6 +1044,8 @@ void forward_pass(gn_ctx* c, const float* Z0, int64_t rows, std::vector<float*>&
     g.D = Zout[m]; g.ldd = c->w[m];
     g.bias = bm(c, c->theta, m);
     g.sigmoid = m < c->L;
+    attach_half(c, g);
+    if (m < c->L) attach_half_out(c, g, c->half_buf[set][(size_t)m]);
     dep[(size_t)m - 1] = m - 2;          // layer m reads the rows layer m - 1 writes
   }
   presplit(c, gs.data(), c->L, 0x2);       // theta's weights
@@ -834,6 +1065,7 @@ GemmArgs weight_block_args(const gn_ctx* c, int m, const float* ds, const float*
   g.alpha = alpha;
   g.cin = cin + c->w_off[m]; g.ld_cin = c->w[m - 1]; g.beta = beta;
   g.D = out + c->w_off[m]; g.ldd = c->w[m - 1];
+  attach_half(c, g);
   return g;
 }
 
@@ -856,7 +1088,7 @@ gn_status weight_block(gn_ctx* c, int m, const float* ds, const float* Zprev, in
 
 // Activation-space half (Eq. communi-g / communi-jaco followed by Eq. ztox-g):
 // dst = (ds W^mT) * sigma'(z^{m-1}), rows stacked modulo z_rows.
-GemmArgs backward_data_args(const gn_ctx* c, int m, const float* ds, int64_t rows, const float* Zprev, int64_t z_rows,
+GemmArgs backward_data_args(gn_ctx* c, int m, const float* ds, int64_t rows, const float* Zprev, int64_t z_rows,
                             float* dst, bool ds_just_used = false) {
   GemmArgs g;
   g.a1_split_fresh = ds_just_used;   // the weight block of the same layer has just read these very rows of ds
@@ -867,6 +1099,11 @@ GemmArgs backward_data_args(const gn_ctx* c, int m, const float* ds, int64_t row
   g.dsig = Zprev; g.ld_dsig = c->w[m - 1]; g.dsig_rows = (int)z_rows;
   g.D = dst; g.ldd = c->w[m - 1];
   g.mn_padded = true;     // B is the context's own (padded) copy of theta
+  attach_half(c, g);
+  for (int set : {(int)gn_ctx::kHDS, (int)gn_ctx::kHDb}) {
+    HalfBuf& b = c->half_buf[set][(size_t)m - 1];
+    if (b.p && b.base == dst) attach_half_out(c, g, b);
+  }
   return g;
 }
 
@@ -904,7 +1141,8 @@ gn_status backward_hidden_layers(gn_ctx* c, int m_top, const float* ds_top, cons
   int widest = 0;
   for (int m = 1; m <= m_top; ++m) widest = std::max(widest, c->w[m]);
   const bool chain = c->back_chain == 1 || (c->back_chain == 2 && (double)rows * widest <= 7.0e6);
-  if (!(c->prec == GN_TF32 && chain && m_top >= 2)) {
+  // (with copies never as a chain: a copy's scale comes from the largest delta of the layer above, known when that is complete)
+  if (!(c->prec == GN_TF32 && chain && m_top >= 2) || c->half_now) {
     const float* ds = ds_top;
     for (int m = m_top; m >= 1; --m) {
       const int64_t wr = m == 1 ? w1_rows : rows;
@@ -940,6 +1178,19 @@ gn_status backward_hidden_layers(gn_ctx* c, int m_top, const float* ds_top, cons
   return GN_OK;
 }
 
+// Copies of a backward pass (`deltas` as of set kHDS or kHDb): room for those that contractions write, with the largest
+// magnitude of the output layer's delta where the first of them has to bound its result from it ...
+void half_deltas(gn_ctx* c, int set, const float* top, const std::vector<float*>& deltas, int64_t rows, int64_t cap_rows) {
+  if (!c->half_now || !half_room(c, set, deltas, c->L - 1, rows, cap_rows)) return;
+  if (c->w[c->L] > 16) half_matrix(c, set, c->L, top, rows, c->w[c->L], cap_rows, false);
+}
+// ... and of the last hidden layer's delta, if it was written by something that writes no copy.
+void half_top_delta(gn_ctx* c, int set, const std::vector<float*>& deltas, int64_t rows, int64_t cap_rows) {
+  const int m = c->L - 1;
+  if (!c->half_now || c->half_buf[set][(size_t)m].valid || c->w[m] < 128 || c->w[m] % 4 != 0) return;
+  half_matrix(c, set, m, deltas[(size_t)m], rows, c->w[m], cap_rows, true);
+}
+
 // out = coef v + (1/|S|) J^T (2 J v) over the stored subsample (Eq. sampled-Gauss).
 gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("G v");
@@ -955,6 +1206,10 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
   ++c->parts_epoch;
   const int L = c->L;
   const int64_t nS = c->nS;
+  HalfPass half_guard(c, half_wanted(c, nS));
+  half_theta(c);
+  half_vector(c, v);
+  half_room(c, gn_ctx::kHRZ, c->RZ, L - 1, nS, c->capS);
   {
     std::vector<GemmArgs> gs((size_t)L);
     std::vector<int> dep((size_t)L), dep_all((size_t)L, 0);
@@ -971,17 +1226,29 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
       if (m < L) { g.dsig = c->Z[m]; g.ld_dsig = c->w[m]; g.dsig_rows = (int)nS; }
       else g.alpha = 2.f;                                   // B = 2I
       g.D = c->RZ[m]; g.ldd = c->w[m];
+      attach_half(c, g);
+      if (m < L && half_layer(c, m + 1)) {
+        g.h_next[0] = c->half_info + half_info_index(c, gn_ctx::kHZ, m);
+        g.h_next[1] = c->half_info + half_info_index(c, gn_ctx::kHV, m + 1);
+        g.h_next[2] = c->half_info + half_info_index(c, gn_ctx::kHW, m + 1);
+        attach_half_out(c, g, c->half_buf[gn_ctx::kHRZ][(size_t)m]);
+      }
       dep[(size_t)m - 1] = m - 2;        // R z^{m-1} of the layer below
     }
     presplit(c, gs.data(), L, 0xf);
-    run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), L, 2);
+    // (with copies never as a chain, see backward_hidden_layers)
+    run_gemm_chain(c, gs.data(), dep.data(), dep_all.data(), L, c->half_now ? 3 : 2);
   }
   const float inv = (float)(1.0 / (double)nS);
   std::vector<const float*> zprev((size_t)L);
   for (int m = 1; m <= L; ++m) zprev[(size_t)m - 1] = c->Z[m - 1];
   // the output layer (streaming kernels at n_L <= 16) on its own, the hidden layers as one pass
+  half_deltas(c, gn_ctx::kHDS, c->RZ[L], c->DS, nS, c->capS);
   GN_TRY(layer_backward(c, L, c->RZ[L], nS, c->RZ[L], nS, c->Z[L - 1], nS, inv, v, coef, out, L > 1 ? c->DS[L - 1] : nullptr));
-  if (L > 1) GN_TRY(backward_hidden_layers(c, L - 1, c->DS[L - 1], zprev, c->DS, nS, inv, v, coef, out, nS, true));
+  if (L > 1) {
+    half_top_delta(c, gn_ctx::kHDS, c->DS, nS, c->capS);
+    GN_TRY(backward_hidden_layers(c, L - 1, c->DS[L - 1], zprev, c->DS, nS, inv, v, coef, out, nS, true));
+  }
   return check_launch(c, "G v");
 }
 
@@ -1075,6 +1342,11 @@ gn_status ensure_factors(gn_ctx* c) {
     c->capF = nS;
   }
   c->launches += launch_factor_last(Wm(c, c->theta, L), c->Z[L - 1], nS, nL, c->w[L - 1], c->DF[L - 1], c->st);
+  HalfPass half_guard(c, L >= 3 && half_wanted(c, nS * nL));
+  half_theta(c);
+  half_invalidate(c, gn_ctx::kHF);
+  if (L >= 3 && c->w[L - 1] >= 128)
+    half_matrix(c, gn_ctx::kHF, L - 1, c->DF[L - 1], nS * nL, c->w[L - 1], 0, true, half_info_index(c, gn_ctx::kHF, 0), L - 1);
   for (int m = L - 1; m >= 2; --m) {
     GemmArgs g;
     g.M = (int)(nS * nL); g.N = c->w[m - 1];
@@ -1084,8 +1356,15 @@ gn_status ensure_factors(gn_ctx* c) {
     g.dsig = c->Z[m - 1]; g.ld_dsig = c->w[m - 1]; g.dsig_rows = (int)nS; g.dsig_div = nL;
     g.D = c->DF[m - 1]; g.ldd = c->w[m - 1];
     g.mn_padded = true;
+    attach_half(c, g);
+    if (m - 1 >= 2 && c->half_now && c->w[m - 1] >= 128 && c->w[m - 1] % 4 == 0) {
+      HalfBuf& b = c->half_buf[gn_ctx::kHF][(size_t)m - 1];
+      if (half_reserve(c, b, gn_ctx::kHF, m - 1, c->DF[m - 1], nS * nL, c->w[m - 1], 0)) attach_half_out(c, g, b);
+      else { half_give_up(c); g.half = false; }
+    }
     run_gemm(c, g);
   }
+  half_invalidate(c, gn_ctx::kHF);
   c->factors_valid = true;
   return check_launch(c, "Jacobian factors");
 }
@@ -1098,6 +1377,8 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   const int L = c->L, nL = c->w[L];
   const int64_t nS = c->nS;
   const float inv = (float)(1.0 / (double)nS);
+  HalfPass half_guard(c, half_wanted(c, nS));
+  half_vector(c, v);
   constexpr int kGroup = 3;
   // The layers' chains are independent of one another, so each stage is issued for all layers together.
   // 1. u_i = V^{mT} z^{m-1,i} + c^m for every row (the inner sum of Eq. direct-JV-cost); at m = L, D = I and B = 2I
@@ -1111,6 +1392,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
       g.bias = bm(c, v, m);
       if (m == L) g.alpha = 2.f;
       g.D = c->RZ[m]; g.ldd = c->w[m];
+      attach_half(c, g);
     }
     run_gemm_group(c, gs, n);
   }
@@ -1123,6 +1405,18 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
       done = launch_factor_apply_last(Wm(c, c->theta, L), c->Z[L - 1], c->RZ[m], nS, nL, c->w[m], c->DS[m], c->st);
     if (!done) done = launch_factor_apply(c->DF[m], c->RZ[m], nS, nL, c->w[m], 1, 1, 0, c->DS[m], c->st);
     c->launches += done;
+  }
+  if (c->half_now) {
+    std::vector<HalfAmaxJob> amax;
+    std::vector<HalfBuf*> bufs;
+    for (int m = 1; m < L && c->half_now; ++m) {
+      if (c->w[m] <= 128 || c->w[m] % 4 != 0 || c->w[m - 1] < 128 || c->w[m - 1] % 4 != 0) continue;
+      HalfBuf& b = c->half_buf[gn_ctx::kHDS][(size_t)m];
+      if (!half_reserve(c, b, gn_ctx::kHDS, m, c->DS[m], nS, c->w[m], c->capS)) { half_give_up(c); break; }
+      amax.push_back(HalfAmaxJob{b.base, b.rows * b.cols, c->half_info + b.info});
+      bufs.push_back(&b);
+    }
+    if (c->half_now && !bufs.empty()) half_convert(c, amax, bufs);
   }
   // 3. the weight and bias blocks.  The bias sums and the n_L-row weight block go first: they run on the side
   // stream beside the large weight blocks, which is only possible if they are forked before those are enqueued.
@@ -1146,17 +1440,18 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
     if (c->cut_for_nS != nS) {
       double best = -1.0;
       for (int eighths = 4; eighths <= 6; ++eighths) {
-        const int64_t r = (nS * eighths / 8 + 31) / 32 * 32;  // first part: a whole number of k-blocks
+        const int64_t r = (nS * eighths / 8 + 63) / 64 * 64;  // first part: a whole number of k-blocks
         int Ms[2 * kGroup], Ns[2 * kGroup], Ks[2 * kGroup];
         for (int part = 0; part < 2; ++part)
           for (int m = 1; m <= nl; ++m) {
             const int k = part * nl + m - 1;
             Ms[k] = c->w[m]; Ns[k] = c->w[m - 1]; Ks[k] = (int)(part == 0 ? r : nS - r);
+            if (c->half_now) Ks[k] = (Ks[k] + 1) / 2;         // (k-blocks of twice the terms)
           }
         const double t = gemm_tf32_group_makespan(2 * nl, Ms, Ns, Ks, 1);
         if (t >= 0.0 && (best < 0.0 || t < best)) { best = t; c->cut_rows = r; }
       }
-      if (best < 0.0) c->cut_rows = (nS / 2 + 31) / 32 * 32;
+      if (best < 0.0) c->cut_rows = (nS / 2 + 63) / 64 * 64;
       c->cut_for_nS = nS;
     }
     const int64_t h0 = c->cut_rows;
@@ -1329,7 +1624,9 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
     const float* X0 = c->dX + r0 * c->w[0];
     c->cur_x = X0;
     ++c->parts_epoch;           // the batch buffers are rewritten
-    forward_pass(c, X0, rows, c->Zb);
+    HalfPass half_guard(c, half_wanted(c, rows));
+    half_invalidate(c, gn_ctx::kHDb);
+    forward_pass(c, X0, rows, c->Zb, gn_ctx::kHZb, c->capB);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
                                      c->partial + b * per_batch, c->st);
     {
@@ -1347,10 +1644,14 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
       // layer 1 reads the caller's X, which has no slack after its last row: in the last batch all but the final
       // 32 rows use the TF32 kernel's padded fast path, the rest is added by a second, unpadded contraction
       const bool last = r0 + rows == c->l;
-      const bool tail = last && rows > 64 && c->prec == GN_TF32 && c->w[0] % 4 == 0 && c->w[1] % 4 == 0;
+      // (a copy of X has the slack)
+      const bool tail = last && rows > 64 && c->prec == GN_TF32 && c->w[0] % 4 == 0 && c->w[1] % 4 == 0 &&
+                        !(c->half_now && c->half_buf[gn_ctx::kHZb][0].valid && c->w[1] > 128 && c->w[0] >= 128);
       const int64_t head = tail ? rows - 32 : rows;
       if (L > 1) {
+        half_deltas(c, gn_ctx::kHDb, c->Db[L], c->Db, rows, c->capB);
         GN_TRY(layer_backward(c, L, c->Db[L], rows, c->Db[L], rows, c->Zb[L - 1], rows, inv_l, cin0, beta0, d_grad, c->Db[L - 1]));
+        half_top_delta(c, gn_ctx::kHDb, c->Db, rows, c->capB);
         GN_TRY(backward_hidden_layers(c, L - 1, c->Db[L - 1], zprev, c->Db, rows, inv_l, cin0, beta0, d_grad, head, tail || !last));
       } else {
         GN_TRY(weight_block(c, 1, c->Db[1], X0, head, inv_l, cin0, beta0, d_grad, tail || !last));
@@ -1495,6 +1796,7 @@ gn_status gn_create(gn_ctx** out, int L, const int32_t* widths, double C, int64_
   c->Z.assign(L + 1, nullptr); c->RZ.assign(L + 1, nullptr); c->DS.assign(L + 1, nullptr);
   c->DF.assign(L + 1, nullptr);
   c->Zb.assign(L + 1, nullptr); c->Db.assign(L + 1, nullptr);
+  for (auto& set : c->half_buf) set.resize((size_t)L + 1);
   c->split.assign(L + 1, 1); c->has_split = false; c->P = L;
   gn_status s = GN_OK;
   do {
@@ -1640,10 +1942,12 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   c->factors_valid = false;
   c->bd_count = 0;
   ++c->sub_epoch;             // the stored activations are about to be rewritten
+  half_invalidate(c, gn_ctx::kHZ);
   ++c->parts_epoch;
   if (nS > c->capS) {
     GN_TRY(sync(c, "set_subsample"));
     drop_kept_parts(c, 2, true);      // the stored activations move: their parts are made anew
+    half_drop(c, gn_ctx::kHZ);
       dev_free(c, c->idx, c->capS);
     for (int m = 0; m <= c->L; ++m) dev_free(c, c->Z[m], c->capS * c->w[m]);
     for (int m = 1; m <= c->L; ++m) { dev_free(c, c->RZ[m], m * c->capS * c->w[m]); dev_free(c, c->DS[m], m * c->capS * c->w[m]); }
@@ -1667,7 +1971,8 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
     GN_TRY(run_small_pass(c, kSmallForward, small, 0.f, nullptr, 0.f, nullptr, nullptr));
   } else {
     c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
-    forward_pass(c, c->Z[0], nS, c->Z);
+    HalfPass half_guard(c, half_wanted(c, nS));
+    forward_pass(c, c->Z[0], nS, c->Z, gn_ctx::kHZ, c->capS);
   }
   GN_TRY(check_launch(c, "set_subsample"));
   GN_TRY(sync(c, "set_subsample"));
@@ -1912,7 +2217,7 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* c, int kind, int M, int N, int K, const
                                  int sigmoid, const float* d_dsig, int64_t ld_dsig, float alpha, const float* d_cin,
                                  int64_t ld_cin, float beta) {
   if (!c) return GN_EINVAL;
-  if (!dA || !dB || !dD || M < 1 || N < 1 || K < 1 || kind < 0 || kind > 8) return fail(c, GN_EINVAL, "bad GEMM arguments");
+  if (!dA || !dB || !dD || M < 1 || N < 1 || K < 1 || kind < 0 || kind > 9) return fail(c, GN_EINVAL, "bad GEMM arguments");
   if ((d_dsig && ld_dsig < N) || (d_cin && ld_cin < N)) return fail(c, GN_EINVAL, "leading dimension of an epilogue operand below N");
   GemmArgs g;
   g.M = M; g.N = N; g.K1 = K;
@@ -1936,6 +2241,21 @@ static gn_status debug_gemm_impl(gn_ctx* c, int kind, GemmArgs g) {
     if ((kind == 7 && (g.M <= 128 || g.N < 128)) || !run_gemm_f16x3(c, g)) return fail(c, GN_EINVAL, "the FP32-accurate tensor-core form does not take this problem");
     GN_TRY(check_launch(c, "debug_gemm"));
     return sync(c, "debug_gemm");
+  }
+  if (kind == 9) {                // CTA pair per tile, FP16 copies of the operands
+    HalfPass half_guard(c, true);
+    if (!suits_half(g)) return fail(c, GN_EINVAL, "operands do not qualify for FP16 copies");
+    for (int role = 0; role < 2; ++role) {
+      const OperandView v = operand_view(g, role);
+      if (v.ld != v.cols) return fail(c, GN_EINVAL, "FP16 copies are of whole matrices");
+      half_matrix(c, gn_ctx::kHF, role, v.p, v.rows, v.cols, 0, true);
+    }
+    if (!c->half_now) return fail(c, GN_ENOMEM, "no room for FP16 copies");
+    attach_half(c, g);
+    c->factors_valid = false;
+    half_invalidate(c, gn_ctx::kHF);
+    if (!g.half) return fail(c, GN_EINVAL, "operands do not qualify for FP16 copies");
+    kind = 5;
   }
   g.mn_padded = (kind >= 3);
   if (kind == 4) g.two_cta = 0;
@@ -2022,7 +2342,8 @@ gn_status gn_newton_iter(gn_ctx* c, float* d_theta, const int32_t* d_idx, int64_
 gn_status gn_debug_option(gn_ctx* c, int option, int value) {
   if (!c) return GN_EINVAL;
   if (option == 2) { if (value < 0) return fail(c, GN_EINVAL, "count must be >= 0"); c->fail_alloc_in = value; return GN_OK; }
-  if (option >= 0 && option <= 10) ++c->dispatch_gen;
+  if (option >= 0 && option <= 11) ++c->dispatch_gen;
+  if (option == 11) { c->half_mode = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }
   if (option == 3) { quiesce(c); c->side_enabled = value != 0; return GN_OK; }
   if (option == 7) { c->split_k_enabled = value != 0; return GN_OK; }
   if (option == 8) { c->back_chain = value < 0 ? 0 : (value > 2 ? 2 : value); return GN_OK; }

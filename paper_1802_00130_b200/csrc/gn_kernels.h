@@ -18,6 +18,20 @@ namespace gn {
 // A operands: a_kmajor -> A(m,k) = A[m * lda + k], else A(m,k) = A[k * lda + m].
 // B operands: b_kmajor -> B(k,n) = B[n * ldb + k], else B(k,n) = B[k * ldb + n].
 // Both pairs share layouts but have their own K and leading dimensions.
+//
+// FP16 copies.  The tensor core reads a TF32 operand as its 11 leading significant bits.  FP16 has as many, so a copy
+// X 2^e in FP16, rounded to nearest as TMA rounds on its way to TF32, holds the same operand (up to the power of two) wherever
+// X 2^e is a normal FP16 number, takes half the bytes and is multiplied at twice the rate.  HalfInfo, in device memory, says
+// which power of two, how large the matrix's largest magnitude is, and whether the copy may be used: `bad` is set by whoever
+// writes it when an element overflows, is infinite or NaN, or when a whole run of a row or of a column lies so low that FP16's
+// denormals would cost it precision (kHalfLeast).  The contraction kernels look at it and read the FP32 matrix instead.
+struct HalfInfo { int e; unsigned amax; unsigned bad; unsigned pad; };
+// Copy of a matrix, stored with leading dimension ld (a multiple of 8, 16-byte aligned, followed by >= 128 readable bytes).
+struct HalfMat { void* p = nullptr; int64_t ld = 0; HalfInfo* info = nullptr; };
+// A run of elements of a row or column whose largest scaled magnitude is below this (and not zero) makes a copy bad: above it
+// the rounding of a denormal, at most 2^-25, stays below the 2^-12 by which rounding to 11 bits changes the run's largest element.
+constexpr float kHalfLeast = 1.220703125e-4f;   // 2^-13
+
 struct GemmArgs {
   int M = 0, N = 0;
   const float* A1 = nullptr; const float* B1 = nullptr; int K1 = 0; int64_t lda1 = 0, ldb1 = 0;
@@ -34,6 +48,13 @@ struct GemmArgs {
   const float* dsig = nullptr; int64_t ld_dsig = 0; int dsig_rows = 1; int dsig_div = 1;
   float alpha = 1.f;
   const float* cin = nullptr; int64_t ld_cin = 0; float beta = 0.f;
+  // CTA-pair kernel only.  half: every operand has a copy in h (A1, B1, A2, B2).  hout: a copy of D is written as well, scaled
+  // by a bound on D from the operands' infos (all in h, with or without copies; the second pair's matrices, or the only pair's,
+  // bound the bias too); h_next: infos of what the next contraction adds to hout's product (see out_exponent).
+  bool half = false;
+  HalfMat h[4];
+  HalfMat hout;
+  const HalfInfo* h_next[3] = {nullptr, nullptr, nullptr};
 };
 
 // FP32 fused-multiply-add GEMM (any shape, any alignment).  Returns launches made.
@@ -71,6 +92,16 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
 int gemm_tf32_plan_group(int n, const int* M, const int* N, const int* K, int pairs, int keep_order, int* counts,
                          int* waves, int* order_out, int* tiles_out);
 double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K, int keep_order);
+
+// FP16 copies by passes of their own (half_copy.cu), at most kHalfSegs matrices a launch.  launch_half_amax starts an info
+// afresh from the largest magnitude of `count` consecutive floats and clears the n_reset infos from `reset` on; acc:
+// kHalfSegs + 1 words, zero before the first launch and after every one.  launch_half_copy writes the copies and marks the bad
+// ones.  Both return launches made, or -1.
+constexpr int kHalfSegs = 8;
+struct HalfAmaxJob { const float* src; int64_t count; HalfInfo* info; };
+struct HalfCopyJob { const float* src; int64_t rows; int cols; int64_t ld; HalfMat out; };
+int launch_half_amax(const HalfAmaxJob* jobs, int n, unsigned* acc, HalfInfo* reset, int n_reset, cudaStream_t st);
+int launch_half_copy(const HalfCopyJob* jobs, int n, cudaStream_t st);
 
 // FP32-accurate contraction on the FP16 tensor cores (gemm_f16x3.cu): any shape and alignment, because it reads
 // split copies of its operands.

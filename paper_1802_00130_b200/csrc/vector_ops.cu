@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const float* __rest
 
 // 16-byte version: grid (ceil(cols/128), ceil(rows/CS_ROWS)); a warp covers 128 columns of a row,
 // 8 warps stride rows with four rows in flight per thread.  Held to 40 registers so that a block fits on an SM
-// beside a CTA of the tensor-core kernel (320 threads x 168 registers): the sums run on a side stream under it.
+// beside a CTA of the tensor-core kernel (576 threads x 96 registers): the sums run on a side stream under it.
 __global__ void __launch_bounds__(256, 6) colsum_partial_vec_kernel(const float* __restrict__ A, long long rows, int cols,
                                                                  long long lda, float* __restrict__ scratch) {
   grid_dep_wait();

@@ -1,0 +1,158 @@
+"""FP16 copies of TF32 operands: the operands are the same, so a contraction computed from copies is the product of the operands
+rounded to 11 bits; a copy that cannot hold its matrix is not used."""
+import numpy as np
+import pytest
+
+import gn_workloads as wl
+from oracle import gn_oracle as orc
+from test_gpu_parity import TOL, dev, make_ctx, relb
+
+pytestmark = pytest.mark.gpu
+HALF, PAIR = 9, 5                    # debug_gemm kinds: the CTA-pair kernel on copies, and on the FP32 matrices
+
+
+def round11(a):
+    """To nearest even, 11 significant bits: what TMA makes of a float on its way to TF32, and FP16 of a scaled one."""
+    bits = a.view(np.uint32)
+    return ((bits + 0xFFF + ((bits >> 13) & 1)) & 0xFFFFE000).astype(np.uint32).view(np.float32)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_1802_00130_b200 as gn
+    p = wl.make("tiny")
+    c = gn.GnContext(p["widths"], p["C"], dev(p["X"]), dev(p["Y"]), gn.GN_TF32)
+    yield c
+    c.close()
+
+
+def operands(M, N, K, a_k, b_k, seed, scale=1.0):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    A = scale * rng.standard_normal((M, K) if a_k else (K, M), dtype=np.float32)
+    B = rng.standard_normal((N, K) if b_k else (K, N), dtype=np.float32)
+    return A, B
+
+
+# tile edges in M (256), N (tiles of 128, 192 and 256) and K (blocks of 64), K slices, several rounds of tiles
+SHAPES = [(132, 128, 20), (256, 256, 64), (260, 132, 68), (512, 384, 1000), (640, 192, 520), (300, 520, 200), (260, 2000, 3000),
+          (2000, 784, 3000), (12000, 2000, 196)]
+
+
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, True), (False, False)])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_contraction_of_copies_is_the_product_of_the_rounded_operands(ctx, shape, a_k, b_k):
+    M, N, K = shape
+    A, B = operands(M, N, K, a_k, b_k, M + 3 * N + 5 * K)
+    D = ctx.debug_gemm(HALF, dev(A), dev(B), a_kmajor=a_k, b_kmajor=b_k).cpu().numpy()
+    ra, rb = round11(A).astype(np.float64), round11(B).astype(np.float64)
+    ref = (ra if a_k else ra.T) @ (rb.T if b_k else rb)
+    # the tensor core truncates each addition of 16 terms into its accumulator: at most 2^-23 of it a step, and the products are exact
+    bound = (K / 16 + 1) * 2.0 ** -23
+    assert np.linalg.norm(D - ref) <= bound * np.linalg.norm(ref)
+    assert np.max(np.abs(D - ref)) <= 8 * bound * np.sqrt(K)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-12, 1e12, 1e30])
+def test_scales_of_whole_matrices_cost_nothing(ctx, scale):
+    A, B = operands(300, 260, 500, True, True, 11, scale)
+    D = ctx.debug_gemm(HALF, dev(A), dev(B)).cpu().numpy().astype(np.float64)
+    ref = round11(A).astype(np.float64) @ round11(B).astype(np.float64).T
+    assert np.linalg.norm(D - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def far_column(A):
+    A[:, 3] *= 1e-11
+
+
+def far_row(A):
+    A[7] *= 1e-11
+
+
+def infinity(A):
+    A[5, 9] = np.inf
+
+
+def not_a_number(A):
+    A[5, 9] = np.nan
+
+
+@pytest.mark.parametrize("spoil", [far_column, far_row, infinity, not_a_number])
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (True, False), (False, False)])
+def test_a_copy_that_cannot_hold_its_matrix_is_not_used(ctx, spoil, a_k, b_k):
+    A, B = operands(520, 392, 300, a_k, b_k, 13)
+    spoil(A)
+    got = ctx.debug_gemm(HALF, dev(A), dev(B), a_kmajor=a_k, b_kmajor=b_k).cpu().numpy()
+    want = ctx.debug_gemm(PAIR, dev(A), dev(B), a_kmajor=a_k, b_kmajor=b_k).cpu().numpy()
+    # (with TF32 operands the K slices are cut at other places: the order of sums may differ, nothing else)
+    fin = np.isfinite(want)
+    assert np.array_equal(fin, np.isfinite(got))
+    assert np.linalg.norm(got[fin] - want[fin]) <= 1e-5 * np.linalg.norm(want[fin])
+    if spoil in (far_column, far_row):          # the far row or column itself
+        ref = round11(A).astype(np.float64)
+        ref = (ref if a_k else ref.T) @ (round11(B).astype(np.float64).T if b_k else round11(B).astype(np.float64))
+        rows = np.linalg.norm(got - ref, axis=1) <= 1e-5 * np.linalg.norm(ref, axis=1)
+        assert rows.all()
+
+
+NETS = {
+    "mid": lambda: wl.make("mid"),
+    "wide_output": lambda: wl.make_custom([260, 392, 520, 260, 132], l=1500, nS=1100, C=15.0, seed=51, x="normal"),
+    "ragged_tiles": lambda: wl.make_custom([300, 520, 392, 264, 10], l=2300, nS=1700, C=23.0, seed=53, x="sparse80"),
+    "two_layers": lambda: wl.make_custom([784, 516, 7], l=1200, nS=900, C=12.0, seed=55, x="uniform"),
+}
+
+
+@pytest.mark.parametrize("v_scale", [1.0, 1e-15])
+@pytest.mark.parametrize("name", sorted(NETS))
+def test_passes_with_copies_against_the_checker(name, v_scale):
+    """Products, block products, gradient and loss with copies wherever they can be made and with none: both within the mode's
+    bound, the same from run to run, and no further from the checker with copies than without."""
+    import torch
+    p = NETS[name]()
+    w, th, C = p["widths"], p["theta"], p["C"]
+    XS, v = p["X"][p["idx"]], (v_scale * p["v"]).astype(np.float32)
+    refs = [orc.Gv(th, w, C, XS, v), orc.Gv_blockdiag(th, w, C, XS, v), orc.grad(th, w, C, p["X"], p["Y"])]
+    err = {}
+    for mode in (0, 2):
+        c = make_ctx(p, "tf32")
+        c.debug_option(10, 0)
+        c.debug_option(11, mode)
+        if w[-1] <= 16:
+            c.set_blockdiag_method(2)
+        c.set_subsample(dev(p["idx"]))
+        first = [c.Gv(dev(v)).clone(), c.Gv_blockdiag(dev(v)).clone(), c.grad().clone()]
+        again = [c.Gv(dev(v)).clone(), c.Gv_blockdiag(dev(v)).clone(), c.grad().clone()]
+        assert all(torch.equal(a, b) for a, b in zip(first, again))
+        err[mode] = [relb(a.cpu().numpy(), r, w) for a, r in zip(first, refs)]
+        assert max(err[mode]) <= TOL["tf32"]
+        f = c.fun()
+        assert abs(f - orc.fun(th, w, C, p["X"], p["Y"])) <= TOL["tf32"] * abs(f)
+        c.close()
+    assert all(a <= 1.02 * b + 1e-6 for a, b in zip(err[2], err[0]))
+
+
+def test_saturated_neurons_and_far_features():
+    """Activations and deltas of saturated neurons lie many orders below the others, and so do features with compensating weights:
+    whole rows of the result depend on them, and have the mode's accuracy."""
+    p = wl.make_custom([260, 392, 264, 10], l=1500, nS=1100, C=15.0, seed=57, x="uniform")
+    w, th = p["widths"], p["theta"].copy()
+    W1 = th[:260 * 392].reshape(392, 260)
+    p["X"][:, 5] *= np.float32(1e-12)
+    W1[:, 5] *= np.float32(1e12)
+    th[260 * 392 + 9] -= 30.0           # b^1 of neuron 9: z about 1e-13
+    p["theta"] = th
+    XS = p["X"][p["idx"]]
+    v = p["v"]
+    ref = orc.Gv(th, w, p["C"], XS, v)
+    gref = orc.grad(th, w, p["C"], p["X"], p["Y"])
+    for mode in (0, 2):
+        c = make_ctx(p, "tf32")
+        c.debug_option(11, mode)
+        c.set_subsample(dev(p["idx"]))
+        assert relb(c.Gv(dev(v)).cpu().numpy(), ref, w) <= TOL["tf32"]
+        g = c.grad().cpu().numpy()
+        assert relb(g, gref, w) <= TOL["tf32"]
+        reg = th / p["C"]               # the loss's own part of the rows in question
+        got, want = (g - reg)[:260 * 392].reshape(392, 260), (gref - reg)[:260 * 392].reshape(392, 260)
+        assert np.linalg.norm(got[:, 5] - want[:, 5]) <= 1e-2 * np.linalg.norm(want[:, 5]) + 1e-6 * np.linalg.norm(reg[:260 * 392])
+        c.close()
