@@ -2,7 +2,8 @@
 // staged in shared memory by TMA (128-byte swizzle), fused epilogue read back with tcgen05.ld.
 //
 // Operands of the CTA-pair kernel may also be FP16 copies (see HalfInfo in gn_kernels.h): the same numbers up to a power of two, in
-// half the bytes and at twice the rate.  18944 x 2048 x 2048: 255 us with TF32 operands, 140 us with copies.
+// half the bytes and at twice the rate.  18944 x 2048 x 2048: 241 us with TF32 operands, 141 us with copies; 16384 x
+// 4096 x 4096: 801 and 433 us, 1270 TFLOP/s.
 //
 // Persistent kernels.  One CTA per SM, each walking 128 x bn output tiles (the CTA-pair kernel further down).  Warp roles:
 //   warp 0      TMA producer: fills a ring of STAGES operand buffers (issue spread over lanes)
@@ -318,7 +319,7 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant
 // only the leader (rank 0) arms full[s] with the bytes of both CTAs, and both CTAs' TMA loads complete
 // on the leader's full[s].  MMAs are issued by the leader only.  acc_full[b] is multicast to both
 // CTAs; all 32 epilogue warps of the pair arrive on the leader's acc_empty[b].  Sixteen epilogue warps per CTA, four per scheduler,
-// because their time is latency (12000 x 2000 x 784 with the sigmoid: 105 us with eight, 75 us with sixteen), at 96 registers,
+// because their time is latency (12000 x 2000 x 784 on copies with the sigmoid: 105 us with eight, 63 us with sixteen), at 96 registers,
 // which leaves room on the SM for a block of the column-sum kernel that runs beside this one (576 x 96 + 256 x 40 = 65536).
 //
 // Work list: with T tiles on P pairs, pair q runs tiles q, q + P, ... for the floor(T / P) full waves, so
