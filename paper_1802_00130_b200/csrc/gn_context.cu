@@ -747,6 +747,7 @@ void attach_half_out(const gn_ctx* c, GemmArgs& g, HalfBuf& b) {
 
 // Copies by passes of their own.  infos: one largest-magnitude job per scale; every matrix of `bufs` is then copied.  The infos
 // from `reset` on are cleared on the way.
+// (With no such job the infos hold what the matrices' writers have reported.)
 bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::vector<HalfBuf*>& bufs, int reset = 0, int n_reset = 0) {
   for (size_t i = 0; i < amax.size(); i += kHalfSegs) {
     const int r = launch_half_amax(amax.data() + i, (int)std::min<size_t>(kHalfSegs, amax.size() - i), c->half_acc, c->half_info + reset, i == 0 ? n_reset : 0, c->st);
@@ -754,7 +755,7 @@ bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::ve
     c->launches += r;
   }
   std::vector<HalfCopyJob> jobs;
-  for (HalfBuf* b : bufs) jobs.push_back(HalfCopyJob{b->base, b->rows, b->cols, (int64_t)b->cols, half_mat(c, *b)});
+  for (HalfBuf* b : bufs) jobs.push_back(HalfCopyJob{b->base, b->rows, b->cols, (int64_t)b->cols, half_mat(c, *b), amax.empty()});
   for (size_t i = 0; i < jobs.size(); i += kHalfSegs) {
     const int r = launch_half_copy(jobs.data() + i, (int)std::min<size_t>(kHalfSegs, jobs.size() - i), c->st);
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "FP16 copies could not be made"; return false; }
@@ -1401,22 +1402,21 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   // the stored copy being needed only as the operand of the recurrence that builds the factors below it)
   for (int m = 1; m < L; ++m) {
     int done = 0;
+    HalfInfo* const info = c->half_now ? c->half_info + half_info_index(c, gn_ctx::kHDS, m) : nullptr;
     if (m == L - 1 && c->fly_enabled)
-      done = launch_factor_apply_last(Wm(c, c->theta, L), c->Z[L - 1], c->RZ[m], nS, nL, c->w[m], c->DS[m], c->st);
-    if (!done) done = launch_factor_apply(c->DF[m], c->RZ[m], nS, nL, c->w[m], 1, 1, 0, c->DS[m], c->st);
+      done = launch_factor_apply_last(Wm(c, c->theta, L), c->Z[L - 1], c->RZ[m], nS, nL, c->w[m], c->DS[m], info, c->st);
+    if (!done) done = launch_factor_apply(c->DF[m], c->RZ[m], nS, nL, c->w[m], 1, 1, 0, c->DS[m], info, c->st);
     c->launches += done;
   }
   if (c->half_now) {
-    std::vector<HalfAmaxJob> amax;
     std::vector<HalfBuf*> bufs;
     for (int m = 1; m < L && c->half_now; ++m) {
       if (c->w[m] <= 128 || c->w[m] % 4 != 0 || c->w[m - 1] < 128 || c->w[m - 1] % 4 != 0) continue;
       HalfBuf& b = c->half_buf[gn_ctx::kHDS][(size_t)m];
       if (!half_reserve(c, b, gn_ctx::kHDS, m, c->DS[m], nS, c->w[m], c->capS)) { half_give_up(c); break; }
-      amax.push_back(HalfAmaxJob{b.base, b.rows * b.cols, c->half_info + b.info});
       bufs.push_back(&b);
     }
-    if (c->half_now && !bufs.empty()) half_convert(c, amax, bufs);
+    if (c->half_now && !bufs.empty()) half_convert(c, {}, bufs);
   }
   // 3. the weight and bias blocks.  The bias sums and the n_L-row weight block go first: they run on the side
   // stream beside the large weight blocks, which is only possible if they are forked before those are enqueued.
@@ -1528,7 +1528,7 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     const float* Q = c->SU;
     if (m < L) {
       side_join(c);                                         // (the layer below's bias sums read what this overwrites)
-      c->launches += launch_factor_apply(c->DF[m], c->SU, nS, nL, nm, sb, sa, stride, c->SQ, c->st);
+      c->launches += launch_factor_apply(c->DF[m], c->SU, nS, nL, nm, sb, sa, stride, c->SQ, nullptr, c->st);
       Q = c->SQ;
     }
     // the bias sums on the side stream, beside this layer's weight blocks and the next layer's first contractions

@@ -99,7 +99,8 @@ double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K,
 // ones.  Both return launches made, or -1.
 constexpr int kHalfSegs = 8;
 struct HalfAmaxJob { const float* src; int64_t count; HalfInfo* info; };
-struct HalfCopyJob { const float* src; int64_t rows; int cols; int64_t ld; HalfMat out; };
+// fresh: the info holds the largest magnitude alone (whoever wrote the matrix has reported it): the scale is said here.
+struct HalfCopyJob { const float* src; int64_t rows; int cols; int64_t ld; HalfMat out; bool fresh = false; };
 int launch_half_amax(const HalfAmaxJob* jobs, int n, unsigned* acc, HalfInfo* reset, int n_reset, cudaStream_t st);
 int launch_half_copy(const HalfCopyJob* jobs, int n, cudaStream_t st);
 
@@ -189,11 +190,11 @@ int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL
 // factor_apply, for every neuron group T_b of the layer (groups contiguous, boundaries floor(b n / groups)) and
 // every stream a (U and Q hold `streams` matrices [rows][n], stream_stride floats apart):
 //   p_u = sum_{j in T_b} D[(i,u)][j] U_a[i][j];  Q_a[i][j] = 2 sum_u D[(i,u)][j] p_u for j in T_b
-// (Eqs. direct-JV-cost, JTv; B = 2I).  n_L <= 32.
+// (Eqs. direct-JV-cost, JTv; B = 2I).  n_L <= 32.  info (may be null): its amax is raised to Q's largest magnitude.
 int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, int n, int groups, int streams,
-                        int64_t stream_stride, float* Q, cudaStream_t st);
+                        int64_t stream_stride, float* Q, HalfInfo* info, cudaStream_t st);
 int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U, int64_t rows, int nL, int n, float* Q,
-                             cudaStream_t st);
+                             HalfInfo* info, cudaStream_t st);
 
 // ---- conjugate gradient ------------------------------------------------------------------------
 // The n coordinates are cut into chunks, each inside one segment (one segment for the full system,

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(512) half_amax_kernel(const __grid_constant__ 
 // A block copies 128 rows x 128 columns, a warp 16 of the rows, a thread 4 of the columns (all requested before the first is
 // used).  The runs looked at for kHalfLeast are a row's 128 and a column's 16 elements.
 constexpr int COPY_CELL = 128, COPY_ROWS = 16;
-struct CopySeg { const float* src; long long rows; int cols; long long ld; __half* out; long long ld_out; HalfInfo* info; int cells_ld, cell0, vec; };
+struct CopySeg { const float* src; long long rows; int cols; long long ld; __half* out; long long ld_out; HalfInfo* info; int cells_ld, cell0, vec, fresh; };
 struct CopyList { int n; CopySeg s[kHalfSegs]; };
 
 __global__ void __launch_bounds__(256) half_copy_kernel(const __grid_constant__ CopyList list) {
@@ -104,7 +104,18 @@ __global__ void __launch_bounds__(256) half_copy_kernel(const __grid_constant__ 
       }
     }
   }
-  const float sc = half_scale(__ldcg(&s.info->e));
+  int e = 0;
+  if (s.fresh) {
+    const unsigned m = __ldcg(&s.info->amax);
+    e = half_exponent(m);
+    if (cell == 0 && threadIdx.x == 0) {
+      __stcg(&s.info->e, e);
+      if (m >= 0x7f800000u) atomicOr(&s.info->bad, 1u);
+    }
+  } else {
+    e = __ldcg(&s.info->e);
+  }
+  const float sc = half_scale(e);
   float col[4] = {0.f, 0.f, 0.f, 0.f};
   HalfCheck check;
   __half* o = s.out + r0 * s.ld_out + c;
@@ -151,7 +162,7 @@ int launch_half_copy(const HalfCopyJob* jobs, int n, cudaStream_t st) {
     s.src = j.src; s.rows = j.rows; s.cols = j.cols; s.ld = j.ld;
     s.out = static_cast<__half*>(j.out.p); s.ld_out = j.out.ld; s.info = j.out.info;
     s.cells_ld = (j.cols + COPY_CELL - 1) / COPY_CELL;
-    s.cell0 = (int)cells;
+    s.cell0 = (int)cells; s.fresh = j.fresh ? 1 : 0;
     s.vec = j.cols % 4 == 0 && j.ld % 4 == 0 && aligned16(j.src);
     cells += (j.rows + COPY_CELL - 1) / COPY_CELL * s.cells_ld;
     if (cells > 0x7fffffff) return -1;

@@ -6,6 +6,7 @@
 #include <initializer_list>
 
 #include "gn_kernels.h"
+#include "half_common.cuh"
 #include "tc_common.cuh"
 
 namespace gn {
@@ -204,6 +205,16 @@ __global__ void __launch_bounds__(256) axpby_kernel(long long n, float a, const 
     out[i] = fmaf(a, x[i], b * y[i]);
 }
 
+// What a block has to say about the matrix it has written for a copy of it: the largest magnitude (HalfInfo::amax; null: nobody asks).
+// `seen` is what was known of it when the block began (asked for then: at a block's end the answer would be waited for, 14 us of
+// factor_apply's 164 at 12000 rows).
+__device__ __forceinline__ unsigned seen_amax(const HalfInfo* info) { return info ? __ldcg(&info->amax) : 0xffffffffu; }
+__device__ __forceinline__ void report_amax(HalfInfo* info, unsigned seen, float largest) {
+  if (!info) return;
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(largest));
+  if ((threadIdx.x & 31) == 0 && m > seen) atomicMax(&info->amax, m);
+}
+
 // ---------------------------------------------------------------------------------- stored Jacobian factors
 // D[(i, u)][t] = WL[u][t] * z (1 - z): one block per sample row i, threads over t (16-byte accesses when n % 4 == 0).
 __global__ void __launch_bounds__(256) factor_last_kernel(const float* __restrict__ WL, const float* __restrict__ Zprev,
@@ -229,10 +240,12 @@ __global__ void __launch_bounds__(256) factor_last_kernel(const float* __restric
 template <int NLMAX>
 __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restrict__ D, const float* __restrict__ U,
                                                            int nL, int n, int groups, int streams, long long stream_stride,
-                                                           float* __restrict__ Q) {
+                                                           float* __restrict__ Q, HalfInfo* info) {
   grid_dep_wait();
   grid_dep_launch();
-  D = dep(D); U = dep(U); Q = dep(Q);
+  D = dep(D); U = dep(U); Q = dep(Q); info = dep(info);
+  float largest = 0.f;
+  const unsigned seen = seen_amax(info);
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
@@ -269,9 +282,11 @@ __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restri
 #pragma unroll
       for (int u = 0; u < NLMAX; ++u)
         if (u < nL) q = fmaf(__ldg(d + (long long)u * n + j), pu[u], q);
+      largest = max3_abs(largest, q, q);
       q_row[j] = q;
     }
   }
+  report_amax(info, seen, largest);
 }
 
 // ---------------------------------------------------------------------------------- CG
@@ -545,46 +560,30 @@ int launch_sum_partials(const double* partial, int count, double* out, bool accu
 
 // Register-resident form for groups of at most 1024 * STRIPS columns (n and every group boundary multiples
 // of 4): every thread keeps its n_L x 4 x STRIPS slice of D_i in registers across the passes and the streams,
-// so D is read exactly once.  FLY: the factor of the last hidden layer has the closed form D_i[u][t] = W^L[u][t] *
-// z (1 - z) (what factor_last_kernel stores); it is formed here, with the same two multiplications, from W^L (80 KB,
-// cache-resident) and the sample's row of Z instead of being streamed from memory: 8 KB instead of 80 KB per sample
-// at n_L = 10, the same bits.
-template <int NLMAX, int STRIPS, bool FLY>
+// so D is read exactly once.
+template <int NLMAX, int STRIPS>
 __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __restrict__ D, const float* __restrict__ U,
                                                                int nL, int n, int groups, int streams,
-                                                               long long stream_stride, float* __restrict__ Q,
-                                                               const float* __restrict__ WL, const float* __restrict__ Zprev) {
+                                                               long long stream_stride, float* __restrict__ Q, HalfInfo* info) {
   grid_dep_wait();
   grid_dep_launch();
-  D = dep(D); U = dep(U); Q = dep(Q); WL = dep(WL); Zprev = dep(Zprev);
+  D = dep(D); U = dep(U); Q = dep(Q); info = dep(info);
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
   const int col0 = (int)(((long long)blockIdx.y * n) / groups), col1 = (int)(((long long)(blockIdx.y + 1) * n) / groups);
   const float* d = D + i * nL * n;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float largest = 0.f;
+  const unsigned seen = seen_amax(info);
   float4 dv[STRIPS][NLMAX];
 #pragma unroll
   for (int s = 0; s < STRIPS; ++s) {
     const int j = col0 + (s * 256 + threadIdx.x) * 4;
     const bool ok = j < col1;
-    if (FLY) {
-      float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (ok) {
-        const float4 z = __ldg(reinterpret_cast<const float4*>(Zprev + i * n + j));
-        ds = make_float4(z.x * (1.f - z.x), z.y * (1.f - z.y), z.z * (1.f - z.z), z.w * (1.f - z.w));
-      }
 #pragma unroll
-      for (int u = 0; u < NLMAX; ++u) {
-        float4 wv = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ok && u < nL) wv = __ldg(reinterpret_cast<const float4*>(WL + (long long)u * n + j));
-        dv[s][u] = make_float4(wv.x * ds.x, wv.y * ds.y, wv.z * ds.z, wv.w * ds.w);
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < NLMAX; ++u)
-        dv[s][u] = (ok && u < nL) ? __ldg(reinterpret_cast<const float4*>(d + (long long)u * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int u = 0; u < NLMAX; ++u)
+      dv[s][u] = (ok && u < nL) ? __ldg(reinterpret_cast<const float4*>(d + (long long)u * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (int a = 0; a < streams; ++a) {
     const float* u_row = U + a * stream_stride + i * n;
@@ -624,10 +623,96 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
           q.x = fmaf(dv[s][u].x, pv, q.x); q.y = fmaf(dv[s][u].y, pv, q.y);
           q.z = fmaf(dv[s][u].z, pv, q.z); q.w = fmaf(dv[s][u].w, pv, q.w);
         }
+        largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
         *reinterpret_cast<float4*>(q_row + j) = q;
       }
     }
   }
+  report_amax(info, seen, largest);
+}
+
+// The same for the last hidden layer, whose factor has the closed form D_i[u][t] = W^L[u][t] * z (1 - z) (what factor_last_kernel
+// stores), one group and one stream: formed here, with the same two multiplications, instead of being streamed from memory (the
+// same bits).  Blocks stay and take sample after sample, W^L in their registers: with a block per sample the 80 KB of W^L at
+// n_L = 10, n = 2000 came from L2 for every sample and bounded it (12000 samples: 124 us, now 82).  What bounds it now is its
+// FMAs and the two barriers per sample, behind which the next sample's rows are already on their way.
+template <int NLMAX, int STRIPS>
+__global__ void __launch_bounds__(256, NLMAX * STRIPS <= 16 ? 2 : 1) factor_apply_fly_kernel(const float* __restrict__ WL, const float* __restrict__ Zprev,
+                                                                  const float* __restrict__ U, long long rows, int nL, int n,
+                                                                  float* __restrict__ Q, HalfInfo* info) {
+  grid_dep_wait();
+  grid_dep_launch();
+  WL = dep(WL); Zprev = dep(Zprev); U = dep(U); Q = dep(Q); info = dep(info);
+  __shared__ float red[2][8][NLMAX];
+  __shared__ float pu[2][NLMAX];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float largest = 0.f;
+  const unsigned seen = seen_amax(info);
+  float4 wv[STRIPS][NLMAX], z[STRIPS], x[STRIPS];
+#pragma unroll
+  for (int s = 0; s < STRIPS; ++s) {
+    const int j = (s * 256 + threadIdx.x) * 4;
+#pragma unroll
+    for (int u = 0; u < NLMAX; ++u)
+      wv[s][u] = (j < n && u < nL) ? __ldg(reinterpret_cast<const float4*>(WL + (long long)u * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const auto fetch = [&](long long i) {
+#pragma unroll
+    for (int s = 0; s < STRIPS; ++s) {
+      const int j = (s * 256 + threadIdx.x) * 4;
+      const bool ok = j < n && i < rows;
+      z[s] = ok ? __ldg(reinterpret_cast<const float4*>(Zprev + i * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[s] = ok ? __ldg(reinterpret_cast<const float4*>(U + i * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  fetch(blockIdx.x);
+  int par = 0;                                                // (scratch of alternate samples, so that two barriers are enough)
+  for (long long i = blockIdx.x; i < rows; i += gridDim.x, par ^= 1) {
+    float4 ds[STRIPS];
+    float acc[NLMAX];
+#pragma unroll
+    for (int u = 0; u < NLMAX; ++u) acc[u] = 0.f;
+#pragma unroll
+    for (int s = 0; s < STRIPS; ++s) {
+      ds[s] = make_float4(z[s].x * (1.f - z[s].x), z[s].y * (1.f - z[s].y), z[s].z * (1.f - z[s].z), z[s].w * (1.f - z[s].w));
+      const float4 uj = x[s];
+#pragma unroll
+      for (int u = 0; u < NLMAX; ++u) {
+        const float4 d = make_float4(wv[s][u].x * ds[s].x, wv[s][u].y * ds[s].y, wv[s][u].z * ds[s].z, wv[s][u].w * ds[s].w);
+        acc[u] += d.x * uj.x + d.y * uj.y + d.z * uj.z + d.w * uj.w;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NLMAX; ++u) {
+      const float s = warp_sum(acc[u]);
+      if (lane == 0) red[par][w][u] = s;
+    }
+    __syncthreads();
+    fetch(i + gridDim.x);
+    if (threadIdx.x < NLMAX) {
+      float s = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += red[par][k][threadIdx.x];
+      pu[par][threadIdx.x] = 2.f * s;                         // B = 2I
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < STRIPS; ++s) {
+      const int j = (s * 256 + threadIdx.x) * 4;
+      if (j < n) {
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < NLMAX; ++u) {
+          const float pv = pu[par][u];
+          q.x = fmaf(wv[s][u].x * ds[s].x, pv, q.x); q.y = fmaf(wv[s][u].y * ds[s].y, pv, q.y);
+          q.z = fmaf(wv[s][u].z * ds[s].z, pv, q.z); q.w = fmaf(wv[s][u].w * ds[s].w, pv, q.w);
+        }
+        largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
+        *reinterpret_cast<float4*>(Q + i * n + j) = q;
+      }
+    }
+  }
+  report_amax(info, seen, largest);
 }
 
 int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL, int n, float* D, cudaStream_t st) {
@@ -636,7 +721,7 @@ int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL
 }
 
 int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, int n, int groups, int streams,
-                        int64_t stream_stride, float* Q, cudaStream_t st) {
+                        int64_t stream_stride, float* Q, HalfInfo* info, cudaStream_t st) {
   bool vec = (n % 4 == 0) && (stream_stride % 4 == 0) && ((reinterpret_cast<uintptr_t>(D) & 15) == 0) &&
              ((reinterpret_cast<uintptr_t>(U) & 15) == 0) && ((reinterpret_cast<uintptr_t>(Q) & 15) == 0);
   int widest = 0;
@@ -647,29 +732,29 @@ int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, in
   }
   const dim3 grid((unsigned)rows, (unsigned)groups);
   const long long ss = stream_stride;
-#define GN_FA_REG(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, nullptr, nullptr); return 1; }
+#define GN_FA_REG(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info); return 1; }
   if (vec && widest <= 1024 && nL <= 4)  GN_FA_REG(4, 1)
   if (vec && widest <= 1024 && nL <= 10) GN_FA_REG(10, 1)
   if (vec && widest <= 2048 && nL <= 4)  GN_FA_REG(4, 2)
   if (vec && widest <= 2048 && nL <= 10) GN_FA_REG(10, 2)
   if (vec && widest <= 1024 && nL <= 16) GN_FA_REG(16, 1)
 #undef GN_FA_REG
-  if (nL <= 4) launch_pdl_grid(factor_apply_kernel<4>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
-  else if (nL <= 10) launch_pdl_grid(factor_apply_kernel<10>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
-  else if (nL <= 16) launch_pdl_grid(factor_apply_kernel<16>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
-  else launch_pdl_grid(factor_apply_kernel<32>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q);
+  if (nL <= 4) launch_pdl_grid(factor_apply_kernel<4>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else if (nL <= 10) launch_pdl_grid(factor_apply_kernel<10>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else if (nL <= 16) launch_pdl_grid(factor_apply_kernel<16>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else launch_pdl_grid(factor_apply_kernel<32>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
   return 1;
 }
 
 // The same product for the last hidden layer without its stored factor (see factor_apply_reg_kernel): one group, one
 // stream.  Returns 0, having launched nothing, if the register-resident form does not take the shape.
 int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U, int64_t rows, int nL, int n, float* Q,
-                             cudaStream_t st) {
+                             HalfInfo* info, cudaStream_t st) {
   const bool vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(WL) & 15) == 0) && ((reinterpret_cast<uintptr_t>(Zprev) & 15) == 0) &&
                    ((reinterpret_cast<uintptr_t>(U) & 15) == 0) && ((reinterpret_cast<uintptr_t>(Q) & 15) == 0);
   if (!vec) return 0;
-  const dim3 grid((unsigned)rows, 1);
-#define GN_FA_FLY(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR, true>, dim3(grid), 256, 0, st, nullptr, U, nL, n, 1, 1, 0, Q, WL, Zprev); return 1; }
+  // (as many blocks as are resident: two per SM where W^L and the products with it leave the registers for that)
+#define GN_FA_FLY(NL, STR) { const long long blocks = (NL * STR <= 16 ? 2LL : 1LL) * num_sms(); const dim3 grid((unsigned)(rows < blocks ? rows : blocks), 1); launch_pdl_grid(factor_apply_fly_kernel<NL, STR>, dim3(grid), 256, 0, st, WL, Zprev, U, rows, nL, n, Q, info); return 1; }
   if (n <= 1024 && nL <= 4)  GN_FA_FLY(4, 1)
   if (n <= 1024 && nL <= 10) GN_FA_FLY(10, 1)
   if (n <= 2048 && nL <= 4)  GN_FA_FLY(4, 2)
