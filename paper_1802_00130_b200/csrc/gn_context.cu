@@ -1508,10 +1508,14 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     c->capSplit = need;
   }
   const float inv = (float)(1.0 / (double)nS);
+  HalfPass half_guard(c, half_wanted(c, nS));
+  half_vector(c, v);
   std::vector<GemmArgs> batch;
   for (int m = 1; m <= L; ++m) {
     const int sa = c->split[m - 1], sb = c->split[m], np = c->w[m - 1], nm = c->w[m];
     const int64_t stride = nS * nm;
+    // (the copy of the layer's results lies in R z^m's memory, which has room for two streams' in FP16)
+    const bool copy = c->half_now && m < L && sa <= 2 && nm > 128 && nm % 8 == 0;
     for (int a = 0; a < sa; ++a) {
       const int t0 = group_lo(np, sa, a), t1 = group_lo(np, sa, a + 1);
       GemmArgs g;
@@ -1520,6 +1524,7 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
       if (a == 0) g.bias = bm(c, v, m);
       if (m == L) g.alpha = 2.f;                          // B = 2I
       g.D = c->SU + a * stride; g.ldd = nm;
+      attach_half(c, g);
       batch.push_back(g);
     }
     // the groups' contractions are independent of one another: up to sixteen at a time to the group launcher
@@ -1528,8 +1533,14 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     const float* Q = c->SU;
     if (m < L) {
       side_join(c);                                         // (the layer below's bias sums read what this overwrites)
-      c->launches += launch_factor_apply(c->DF[m], c->SU, nS, nL, nm, sb, sa, stride, c->SQ, nullptr, c->st);
+      c->launches += launch_factor_apply(c->DF[m], c->SU, nS, nL, nm, sb, sa, stride, c->SQ,
+                                         copy ? c->half_info + half_info_index(c, gn_ctx::kHDS, m) : nullptr, c->st);
       Q = c->SQ;
+    }
+    if (copy) {
+      HalfBuf& b = c->half_buf[gn_ctx::kHDS][(size_t)m];
+      if (half_reserve(c, b, gn_ctx::kHDS, m, Q, sa * nS, nm, 0)) half_convert(c, {}, {&b});
+      else half_give_up(c);
     }
     // the bias sums on the side stream, beside this layer's weight blocks and the next layer's first contractions
     GN_TRY(ensure_colsum(c, nS, nm));
@@ -1545,10 +1556,12 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
       g.alpha = inv;
       g.cin = v + c->w_off[m] + t0; g.ld_cin = np; g.beta = coef;
       g.D = out + c->w_off[m] + t0; g.ldd = np;
+      attach_half(c, g);
       batch.push_back(g);
     }
     for (size_t b0 = 0; b0 < batch.size(); b0 += 16) run_gemm_group(c, batch.data() + b0, (int)std::min<size_t>(16, batch.size() - b0));
     batch.clear();
+    half_invalidate(c, gn_ctx::kHDS);                       // (the next layer's results take the same place)
   }
   return check_launch(c, "partition-wise G v");
 }

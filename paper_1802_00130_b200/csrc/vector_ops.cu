@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(256) axpby_kernel(long long n, float a, const 
 }
 
 // What a block has to say about the matrix it has written for a copy of it: the largest magnitude (HalfInfo::amax; null: nobody asks).
-// `seen` is what was known of it when the block began (asked for then: at a block's end the answer would be waited for, 14 us of
-// factor_apply's 164 at 12000 rows).
+// `seen` is what was known of it when the block began (asked for then, and by one thread: at a block's end the answer would be
+// waited for, 14 us of factor_apply's 164 at 12000 rows, and thousands of warps that read one line stand in each other's way).
 __device__ __forceinline__ unsigned seen_amax(const HalfInfo* info) { return info ? __ldcg(&info->amax) : 0xffffffffu; }
 __device__ __forceinline__ void report_amax(HalfInfo* info, unsigned seen, float largest) {
   if (!info) return;
@@ -245,7 +245,8 @@ __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restri
   grid_dep_launch();
   D = dep(D); U = dep(U); Q = dep(Q); info = dep(info);
   float largest = 0.f;
-  const unsigned seen = seen_amax(info);
+  __shared__ unsigned seen;
+  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
@@ -575,7 +576,8 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
   const float* d = D + i * nL * n;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float largest = 0.f;
-  const unsigned seen = seen_amax(info);
+  __shared__ unsigned seen;
+  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   float4 dv[STRIPS][NLMAX];
 #pragma unroll
   for (int s = 0; s < STRIPS; ++s) {
@@ -647,7 +649,8 @@ __global__ void __launch_bounds__(256, NLMAX * STRIPS <= 16 ? 2 : 1) factor_appl
   __shared__ float pu[2][NLMAX];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float largest = 0.f;
-  const unsigned seen = seen_amax(info);
+  __shared__ unsigned seen;
+  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   float4 wv[STRIPS][NLMAX], z[STRIPS], x[STRIPS];
 #pragma unroll
   for (int s = 0; s < STRIPS; ++s) {

@@ -156,3 +156,20 @@ def test_saturated_neurons_and_far_features():
         got, want = (g - reg)[:260 * 392].reshape(392, 260), (gref - reg)[:260 * 392].reshape(392, 260)
         assert np.linalg.norm(got[:, 5] - want[:, 5]) <= 1e-2 * np.linalg.norm(want[:, 5]) + 1e-6 * np.linalg.norm(reg[:260 * 392])
         c.close()
+
+
+@pytest.mark.parametrize("split", [[1, 2, 2, 1, 1], [2, 2, 1, 2, 1], [1, 3, 2, 2, 1], [1, 4, 3, 1, 1]])
+def test_split_structures_with_copies_against_the_checker(split):
+    """Sub-blocks of stored matrices as operands: groups that start on a copy's 16 bytes use it, others do not, streams beyond two
+    have none of their results."""
+    p = wl.make_custom([304, 528, 392, 264, 10], l=2300, nS=1700, C=23.0, seed=59, x="sparse80")
+    w = p["widths"]
+    ref = orc.Gv_partition(p["theta"], w, p["C"], p["X"][p["idx"]], p["v"], split)
+    for mode in (0, 2):
+        c = make_ctx(p, "tf32")
+        c.debug_option(11, mode)
+        c.set_split(split)
+        c.set_subsample(dev(p["idx"]))
+        for _ in range(2):
+            assert relb(c.Gv_blockdiag(dev(p["v"])).cpu().numpy(), ref, w) <= TOL["tf32"]
+        c.close()
