@@ -9,7 +9,10 @@
 #include <cstdio>
 
 #include "../../include/gn.h"
+#include <cuda_fp16.h>
+
 #include "gn_kernels.h"
+#include "half_common.cuh"
 #include "tc_common.cuh"
 
 namespace gn {
@@ -236,9 +239,14 @@ struct ThinKParams {
   const float* A; long long lda;
   const float* B; long long ldb;
   Epi e;
+  __half* Dh; long long ldh; HalfInfo* hout;           // copy of D (null: none), and its info
+  const HalfInfo* hin[2];                              // infos of A and B, which bound D
 };
 
-template <int KMAX>
+// With a copy (COPY): the scale comes from |D| <= K max|A| max|B| / 4 (the sigmoid derivative), the runs looked at are a thread's 4
+// elements of a row and the block's rows of a column.  (A pass of its own for the largest magnitude and one for the copy
+// took 20 + 24 us at 12000 x 2000; written here it costs 7, and 5 for the largest magnitude of A.)
+template <int KMAX, bool COPY>
 __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p) {
   grid_dep_wait();
   grid_dep_launch();
@@ -248,11 +256,22 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
   // otherwise pin their order, since D may alias the inputs as far as the compiler knows).
   constexpr int RB = 64, RG = 8;
   __shared__ __align__(16) float As[RB][KMAX];         // (KMAX is a multiple of 4: a row is read back as 16-byte groups)
+  __shared__ int scale_exp;
+  __shared__ unsigned seen;                            // (both are used behind a barrier)
+  float largest = 0.f, col[4] = {0.f, 0.f, 0.f, 0.f};
+  HalfCheck check;
   const int n = (blockIdx.x * 128 + threadIdx.x) * 4;
   const bool n_ok = n < p.N;
   const float* const pA = dep(p.A);
   const float* const pB = dep(p.B);
   const Epi e = after_wait(p.e);
+  if (COPY && threadIdx.x == 0) {
+    const float bound = (float)p.K * __uint_as_float(__ldcg(&p.hin[0]->amax)) * __uint_as_float(__ldcg(&p.hin[1]->amax)) *
+                        fabsf(e.alpha) * (e.dsig ? 0.25f : 1.f);
+    scale_exp = half_exponent(__float_as_uint(bound) & 0x7fffffffu);
+    seen = __ldcg(&p.hout->amax);
+    if (blockIdx.x == 0 && blockIdx.y == 0) __stcg(&p.hout->e, scale_exp);
+  }
   float4 b[KMAX];
 #pragma unroll
   for (int k = 0; k < KMAX; ++k)
@@ -312,8 +331,27 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
           t[2] = fmaf(e.beta, c.z, t[2]); t[3] = fmaf(e.beta, c.w, t[3]);
         }
         *reinterpret_cast<float4*>(e.D + (long long)m * e.ldd + n) = make_float4(t[0], t[1], t[2], t[3]);
+        if (COPY) {
+          const float sc = half_scale(scale_exp);
+          const float y[4] = {t[0] * sc, t[1] * sc, t[2] * sc, t[3] * sc};
+          const float row = max3_abs(max3_abs(0.f, y[0], y[1]), y[2], y[3]);
+          check.run(row);
+          largest = max3_abs(largest, row, row);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) col[j] = max3_abs(col[j], y[j], y[j]);
+          const __half2 a = __floats2half2_rn(y[0], y[1]), b2 = __floats2half2_rn(y[2], y[3]);
+          *reinterpret_cast<uint2*>(p.Dh + (long long)m * p.ldh + n) = make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b2));
+        }
       }
     }
+  }
+  if (COPY) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) check.run(col[j]);
+    const unsigned high = __reduce_max_sync(0xffffffffu, __float_as_uint(largest));
+    const unsigned amax = __float_as_uint(__uint_as_float(high) * half_scale(-scale_exp));
+    if (__any_sync(0xffffffffu, check.bad()) && (threadIdx.x & 31) == 0) atomicOr(&p.hout->bad, 1u);
+    if ((threadIdx.x & 31) == 0 && amax > seen) atomicMax(&p.hout->amax, amax);
   }
 }
 
@@ -391,10 +429,17 @@ int launch_gemm_thin(const GemmArgs& g, float* scratch, cudaStream_t st) {
     if (row_blocks > g.M) row_blocks = g.M;
     p.rows_per_block = (g.M + row_blocks - 1) / row_blocks;
     dim3 grid(col_tiles, (g.M + p.rows_per_block - 1) / p.rows_per_block);
-    if (g.K1 <= 4) launch_pdl_grid(gemm_thin_k_kernel<4>, dim3(grid), 128, 0, st, p);
-    else if (g.K1 <= 8) launch_pdl_grid(gemm_thin_k_kernel<8>, dim3(grid), 128, 0, st, p);
-    else if (g.K1 <= 12) launch_pdl_grid(gemm_thin_k_kernel<12>, dim3(grid), 128, 0, st, p);
-    else launch_pdl_grid(gemm_thin_k_kernel<16>, dim3(grid), 128, 0, st, p);
+    const bool copy = g.hout.p != nullptr;
+    if (copy) {
+      p.Dh = static_cast<__half*>(g.hout.p); p.ldh = g.hout.ld; p.hout = g.hout.info;
+      p.hin[0] = g.h[0].info; p.hin[1] = g.h[1].info;
+    }
+#define GN_THIN_K(KM) launch_pdl_grid(copy ? gemm_thin_k_kernel<KM, true> : gemm_thin_k_kernel<KM, false>, dim3(grid), 128, 0, st, p)
+    if (g.K1 <= 4) GN_THIN_K(4);
+    else if (g.K1 <= 8) GN_THIN_K(8);
+    else if (g.K1 <= 12) GN_THIN_K(12);
+    else GN_THIN_K(16);
+#undef GN_THIN_K
     return 1;
   }
   return 0;

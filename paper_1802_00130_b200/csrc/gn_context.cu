@@ -721,9 +721,16 @@ bool half_find(const gn_ctx* c, const float* src, int64_t ld, HalfMat* out, bool
 bool suits_half(const GemmArgs& g) {
   return gemm_thin_kind(g) == THIN_NONE && g.M > 128 && g.N >= 128 && g.two_cta != 0 && gemm_tf32_eligible(g);
 }
+// The streaming kernel of a short K reads FP32 and can write its result's copy.
+bool thin_with_copy(const GemmArgs& g) { return gemm_thin_kind(g) == THIN_K && !g.bias && !g.cin && !g.sigmoid; }
 // The copies of a contraction's operands, if it can be computed from them and all are there.
 void attach_half(const gn_ctx* c, GemmArgs& g) {
-  if (!c->half_now || !suits_half(g)) return;
+  if (!c->half_now) return;
+  if (thin_with_copy(g)) {                  // (what bounds its result)
+    if (!half_find(c, g.A1, g.lda1, &g.h[0], true) || !half_find(c, g.B1, g.ldb1, &g.h[1], true)) g.h[0] = g.h[1] = HalfMat{};
+    return;
+  }
+  if (!suits_half(g)) return;
   bool all = true;
   for (int role = 0; role < (g.A2 ? 4 : 2); ++role) {
     const float* p = role == 0 ? g.A1 : role == 1 ? g.B1 : role == 2 ? g.A2 : g.B2;
@@ -738,7 +745,7 @@ void attach_half(const gn_ctx* c, GemmArgs& g) {
 // ... and the copy of its result, which it writes (attach_half comes first).  The result is the matrix of `b`.
 void attach_half_out(const gn_ctx* c, GemmArgs& g, HalfBuf& b) {
   b.valid = b.info_valid = false;
-  if (!c->half_now || !suits_half(g) || !b.p || b.base != g.D || b.cols != g.ldd) return;
+  if (!c->half_now || !(suits_half(g) || thin_with_copy(g)) || !b.p || b.base != g.D || b.cols != g.ldd) return;
   for (int role = 0; role < (g.A2 ? 4 : 2); ++role)
     if (!g.h[role].info) return;
   g.hout = half_mat(c, b);
@@ -796,12 +803,15 @@ void half_theta(gn_ctx* c) {
   for (int m = 1; m <= c->L; ++m) {
     HalfBuf& b = c->half_buf[gn_ctx::kHW][(size_t)m];
     const bool copy = half_layer(c, m) || (c->w[m - 1] >= 128 && c->w[m] > 16 && c->w[m] % 4 == 0 && c->w[m - 1] % 4 == 0 && c->w_off[m] % 4 == 0);
-    if (!copy) continue;
+    // (of the output layer's weights at least the largest magnitude, which bounds the last hidden layer's delta)
+    if (!copy && m < c->L) continue;
     if (!half_reserve(c, b, gn_ctx::kHW, m, c->theta + c->w_off[m], c->w[m], c->w[m - 1], 0)) { half_give_up(c); return; }
     amax.push_back(HalfAmaxJob{b.base, b.rows * b.cols, c->half_info + b.info});
-    bufs.push_back(&b);
+    if (copy) bufs.push_back(&b);
   }
-  if (half_convert(c, amax, bufs)) c->half_theta_epoch = c->theta_epoch;
+  if (!half_convert(c, amax, bufs)) return;
+  c->half_buf[gn_ctx::kHW][(size_t)c->L].info_valid = true;
+  c->half_theta_epoch = c->theta_epoch;
 }
 
 // The vector of a product; the infos of what the product computes start afresh.
@@ -1183,9 +1193,9 @@ gn_status backward_hidden_layers(gn_ctx* c, int m_top, const float* ds_top, cons
 // magnitude of the output layer's delta where the first of them has to bound its result from it ...
 void half_deltas(gn_ctx* c, int set, const float* top, const std::vector<float*>& deltas, int64_t rows, int64_t cap_rows) {
   if (!c->half_now || !half_room(c, set, deltas, c->L - 1, rows, cap_rows)) return;
-  if (c->w[c->L] > 16) half_matrix(c, set, c->L, top, rows, c->w[c->L], cap_rows, false);
+  half_matrix(c, set, c->L, top, rows, c->w[c->L], cap_rows, false);
 }
-// ... and of the last hidden layer's delta, if it was written by something that writes no copy.
+// ... and of the last hidden layer's delta, if it was written by something that wrote no copy.
 void half_top_delta(gn_ctx* c, int set, const std::vector<float*>& deltas, int64_t rows, int64_t cap_rows) {
   const int m = c->L - 1;
   if (!c->half_now || c->half_buf[set][(size_t)m].valid || c->w[m] < 128 || c->w[m] % 4 != 0) return;

@@ -48,7 +48,7 @@ struct GemmArgs {
   const float* dsig = nullptr; int64_t ld_dsig = 0; int dsig_rows = 1; int dsig_div = 1;
   float alpha = 1.f;
   const float* cin = nullptr; int64_t ld_cin = 0; float beta = 0.f;
-  // CTA-pair kernel only.  half: every operand has a copy in h (A1, B1, A2, B2).  hout: a copy of D is written as well, scaled
+  // CTA-pair kernel, and for hout the streaming kernel of a short K as well (no bias, no cin).  half: every operand has a copy in h (A1, B1, A2, B2).  hout: a copy of D is written as well, scaled
   // by a bound on D from the operands' infos (all in h, with or without copies; the second pair's matrices, or the only pair's,
   // bound the bias too); h_next: infos of what the next contraction adds to hout's product (see out_exponent).
   bool half = false;

@@ -147,7 +147,7 @@ int launch_half_amax(const HalfAmaxJob* jobs, int n, unsigned* acc, HalfInfo* re
     list.s[i] = AmaxSeg{jobs[i].src, (long long)jobs[i].count, jobs[i].info, aligned16(jobs[i].src) ? 1 : 0};
     total += jobs[i].count;
   }
-  long long blocks = (total + 16383) / 16384;      // (8 groups of 4 per thread at least)
+  long long blocks = (total + 4095) / 4096;        // (two groups of 4 per thread at least: a small matrix is a chain of round trips)
   if (blocks > 2LL * num_sms()) blocks = 2LL * num_sms();
   return launch_pdl(half_amax_kernel, (int)blocks, 512, 0, st, list) == cudaSuccess ? 1 : -1;
 }

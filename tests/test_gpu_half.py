@@ -98,6 +98,9 @@ NETS = {
     "mid": lambda: wl.make("mid"),
     "wide_output": lambda: wl.make_custom([260, 392, 520, 260, 132], l=1500, nS=1100, C=15.0, seed=51, x="normal"),
     "ragged_tiles": lambda: wl.make_custom([300, 520, 392, 264, 10], l=2300, nS=1700, C=23.0, seed=53, x="sparse80"),
+    "one_output": lambda: wl.make_custom([260, 392, 264, 1], l=1500, nS=1100, C=15.0, seed=61, x="normal"),
+    "three_outputs": lambda: wl.make_custom([260, 392, 268, 3], l=1500, nS=1037, C=15.0, seed=63, x="normal"),
+    "sixteen_outputs": lambda: wl.make_custom([260, 392, 132, 16], l=1500, nS=1100, C=15.0, seed=65, x="uniform"),
     "two_layers": lambda: wl.make_custom([784, 516, 7], l=1200, nS=900, C=12.0, seed=55, x="uniform"),
 }
 
