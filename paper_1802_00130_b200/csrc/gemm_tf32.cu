@@ -380,8 +380,10 @@ constexpr unsigned kBadPanel = 1u << 30;       // in a counter of finished tiles
 
 // What the producer finds out about a problem from the copies' infos (all of them in a few lines of L2, which thousands of
 // warps must not read per tile).  use: its tiles are computed from the copies; 2^sum0, 2^sum1: scale of A1 B1 and of A2 B2.  With
-// two operand pairs the second goes first, and where the first begins the sums are brought to its scale (scale-input-d: exact, but
-// downwards only).  out: exponent of the scale of D's copy.
+// two operand pairs the second goes first, and the first instruction of the first brings the sums to its scale (scale-input-d: exact,
+// but downwards only, and by at most 2^-15: a second scaled instruction would scale the first one's own products as well).  A
+// pair of pairs further apart is computed from the FP32 matrices.  out: exponent of the scale of D's copy.
+constexpr int kMaxScaleStep = 15;
 struct HalfUse { int use, sum0, sum1, out; };
 
 // Exponent of the scale of D's copy: |D| is bounded from the operands' largest magnitudes m, and 2^e takes the bound below 2^15.
@@ -417,7 +419,7 @@ __device__ __forceinline__ HalfUse half_use(const Tf32Params& p, bool a1_here) {
     }
   if (p.half) {
     u.sum0 = e[0] + e[1]; u.sum1 = n == 4 ? e[2] + e[3] : u.sum0;
-    u.use = bad == 0u && abs(u.sum0) <= kHalfMaxExp && abs(u.sum1) <= kHalfMaxExp && u.sum1 >= u.sum0 && u.sum1 - u.sum0 <= 60;
+    u.use = bad == 0u && abs(u.sum0) <= kHalfMaxExp && abs(u.sum1) <= kHalfMaxExp && u.sum1 >= u.sum0 && u.sum1 - u.sum0 <= kMaxScaleStep;
   }
   if (p.copy_out) u.out = out_exponent(p, amax);
   return u;
@@ -863,12 +865,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
               if (!wait_or_abort(&full[s], ph, abort_flag, err, 2)) { ok = false; break; }
               tc_fence_after();
               const uint64_t ad = a0 + (uint64_t)(s * (STAGE2_BYTES >> 4)), bd = b0 + (uint64_t)(s * (STAGE2_BYTES >> 4));
-              int down = form >> 1;
-#pragma unroll 1
-              for (int k = 0; k < 4; ++k, down -= 15) {
-                if (down > 0) mma2_f16_shift(min(down, 15), tmem_d, ad + k * a_step, bd + k * b_step, idesc);
-                else mma2_f16(tmem_d, ad + k * a_step, bd + k * b_step, idesc, 1u);
-              }
+              mma2_f16_shift(form >> 1, tmem_d, ad, bd, idesc);
+              for (int k = 1; k < 4; ++k) mma2_f16(tmem_d, ad + k * a_step, bd + k * b_step, idesc, 1u);
               mma2_commit_both(&empty[s]);
               if (++s == STAGES) { s = 0; ph ^= 1u; }
               ++kb;

@@ -176,3 +176,22 @@ def test_split_structures_with_copies_against_the_checker(split):
         for _ in range(2):
             assert relb(c.Gv_blockdiag(dev(p["v"])).cpu().numpy(), ref, w) <= TOL["tf32"]
         c.close()
+
+
+@pytest.mark.parametrize("slices", [0, 1])
+@pytest.mark.parametrize("k", list(range(-1, 13)) + [16, 20, 24, 31, 40, 60])
+def test_scales_of_the_two_operand_pairs_lie_any_distance_apart(k, slices):
+    """One weight of 2^k in every hidden layer above the first: each doubling takes the scale of R z W one power of two further
+    below that of z V (5 to 8 with the other weights alone), through the 15 that one instruction can bridge."""
+    p = wl.make_custom([260, 392, 520, 392, 10], l=1500, nS=1100, C=1e6, seed=67, x="sparse80")
+    w, th = p["widths"], p["theta"]
+    for m, (w_off, _, _) in enumerate(wl.layer_offsets(w), 1):
+        if 2 <= m < 4:
+            th[w_off + 7 * w[m - 1] + 11] = 2.0 ** k
+    ref = orc.Gv(th, w, p["C"], p["X"][p["idx"]], p["v"])
+    c = make_ctx(p, "tf32")
+    c.debug_option(11, 2)
+    c.debug_option(1, slices)
+    c.set_subsample(dev(p["idx"]))
+    assert relb(c.Gv(dev(p["v"])).cpu().numpy(), ref, w) <= TOL["tf32"]
+    c.close()
