@@ -788,10 +788,17 @@ bool half_wanted(gn_ctx* c, int64_t rows) {
     if (half_layer(c, m)) weights += (double)c->w[m - 1] * c->w[m];
   return weights > 0.0 && (c->half_mode == 2 || (weights >= 5e5 && rows * weights >= 1e9));
 }
-struct HalfPass {                       // a pass that works with copies, or not
-  gn_ctx* c; bool before;
-  HalfPass(gn_ctx* ctx, bool on) : c(ctx), before(ctx->half_now) { c->half_now = on; }
-  ~HalfPass() { c->half_now = before; }
+// A pass that works with copies, or not.  What is known at its end beyond theta and the stored activations is forgotten: a copy is
+// found by the address of its matrix, and the next pass may meet another matrix there (of the caller, or in memory that the
+// context has let go and got again).
+struct HalfPass {
+  gn_ctx* c;
+  HalfPass(gn_ctx* ctx, bool on) : c(ctx) { c->half_now = on; }
+  ~HalfPass() {
+    c->half_now = false;
+    for (int set = 0; set < gn_ctx::kHalfSets; ++set)
+      if (set != gn_ctx::kHZ && set != gn_ctx::kHW) half_invalidate(c, set);
+  }
 };
 
 // theta's weights, once per theta.
@@ -818,7 +825,6 @@ void half_theta(gn_ctx* c) {
 void half_vector(gn_ctx* c, const float* v) {
   if (!c->half_now) return;
   std::vector<HalfBuf*> bufs;
-  half_invalidate(c, gn_ctx::kHV); half_invalidate(c, gn_ctx::kHRZ); half_invalidate(c, gn_ctx::kHDS);
   for (int m = 1; m <= c->L; ++m) {
     if (!half_layer(c, m)) continue;
     HalfBuf& b = c->half_buf[gn_ctx::kHV][(size_t)m];
@@ -1280,6 +1286,7 @@ gn_status ensure_stacked(gn_ctx* c) {
       // leave a consistent, empty state: the next set_subsample allocates afresh
       for (int k = 1; k <= c->L; ++k) { dev_free(c, c->RZ[k]); dev_free(c, c->DS[k]); }
       drop_kept_parts(c, 2, true);
+      half_invalidate(c, gn_ctx::kHZ);
       for (int k = 0; k <= c->L; ++k) dev_free(c, c->Z[k]);
       dev_free(c, c->idx);
       c->capS = 0; c->have_sub = false; c->factors_valid = false;
@@ -1355,7 +1362,6 @@ gn_status ensure_factors(gn_ctx* c) {
   c->launches += launch_factor_last(Wm(c, c->theta, L), c->Z[L - 1], nS, nL, c->w[L - 1], c->DF[L - 1], c->st);
   HalfPass half_guard(c, L >= 3 && half_wanted(c, nS * nL));
   half_theta(c);
-  half_invalidate(c, gn_ctx::kHF);
   if (L >= 3 && c->w[L - 1] >= 128)
     half_matrix(c, gn_ctx::kHF, L - 1, c->DF[L - 1], nS * nL, c->w[L - 1], 0, true, half_info_index(c, gn_ctx::kHF, 0), L - 1);
   for (int m = L - 1; m >= 2; --m) {
@@ -1375,7 +1381,6 @@ gn_status ensure_factors(gn_ctx* c) {
     }
     run_gemm(c, g);
   }
-  half_invalidate(c, gn_ctx::kHF);
   c->factors_valid = true;
   return check_launch(c, "Jacobian factors");
 }
@@ -1648,7 +1653,6 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
     c->cur_x = X0;
     ++c->parts_epoch;           // the batch buffers are rewritten
     HalfPass half_guard(c, half_wanted(c, rows));
-    half_invalidate(c, gn_ctx::kHDb);
     forward_pass(c, X0, rows, c->Zb, gn_ctx::kHZb, c->capB);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
                                      c->partial + b * per_batch, c->st);
@@ -2276,7 +2280,6 @@ static gn_status debug_gemm_impl(gn_ctx* c, int kind, GemmArgs g) {
     if (!c->half_now) return fail(c, GN_ENOMEM, "no room for FP16 copies");
     attach_half(c, g);
     c->factors_valid = false;
-    half_invalidate(c, gn_ctx::kHF);
     if (!g.half) return fail(c, GN_EINVAL, "operands do not qualify for FP16 copies");
     kind = 5;
   }

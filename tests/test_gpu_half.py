@@ -195,3 +195,47 @@ def test_scales_of_the_two_operand_pairs_lie_any_distance_apart(k, slices):
     c.set_subsample(dev(p["idx"]))
     assert relb(c.Gv(dev(p["v"])).cpu().numpy(), ref, w) <= TOL["tf32"]
     c.close()
+
+
+def test_a_copy_ends_with_its_pass():
+    """The memory of a product's vector comes back with other numbers: they are what a contraction reads there."""
+    p = wl.make_custom([260, 392, 264, 10], l=1500, nS=1100, C=15.0, seed=69, x="uniform")
+    w = p["widths"]
+    c = make_ctx(p, "tf32")
+    c.debug_option(11, 2)
+    c.set_subsample(dev(p["idx"]))
+    v = dev(p["v"])
+    c.Gv(v)
+    fresh = np.random.Generator(np.random.PCG64(71)).standard_normal(p["n"], dtype=np.float32)
+    v.copy_(dev(fresh))
+    w_off, b_off, _ = wl.layer_offsets(w)[1]                       # W^2: 264 x 392
+    A, B = fresh[w_off:b_off].reshape(w[2], w[1]), operands(132, 132, w[1], True, True, 73)[1]
+    D = c.debug_gemm(HALF, v[w_off:b_off].view(w[2], w[1]), dev(B)).cpu().numpy()
+    ref = round11(A).astype(np.float64) @ round11(B).astype(np.float64).T
+    assert np.linalg.norm(D - ref) <= 1e-5 * np.linalg.norm(ref)
+    c.close()
+
+
+def test_copies_and_memory_that_changes_hands():
+    """Buffers are let go and got again (a larger subsample, other row batches, factors, the propagate form's deeper buffers,
+    the caller's vector): every result is that of the matrices which are there now."""
+    import torch
+    p = wl.make_custom([392, 392, 392, 392, 10], l=2300, nS=1700, C=23.0, seed=75, x="sparse80")
+    w, th, C, v = p["widths"], p["theta"], p["C"], p["v"]
+    c = make_ctx(p, "tf32")
+    c.debug_option(11, 2)
+    grad_ref = orc.grad(th, w, C, p["X"], p["Y"])
+    for nS, batch, method in [(600, 1000, 2), (1100, 2300, 2), (600, 700, 1), (1700, 1500, 2), (1300, 2000, 1)]:
+        c.set_batch_rows(batch)
+        c.set_blockdiag_method(method)
+        c.set_subsample(dev(p["idx"][:nS]))
+        XS = p["X"][p["idx"][:nS]]
+        dv = dev(v)
+        got = c.Gv(dv).cpu().numpy()
+        del dv
+        torch.cuda.empty_cache()
+        assert relb(got, orc.Gv(th, w, C, XS, v), w) <= TOL["tf32"]
+        assert relb(c.grad().cpu().numpy(), grad_ref, w) <= TOL["tf32"]
+        for _ in range(2):
+            assert relb(c.Gv_blockdiag(dev(v)).cpu().numpy(), orc.Gv_blockdiag(th, w, C, XS, v), w) <= TOL["tf32"]
+    c.close()
