@@ -683,12 +683,12 @@ bool half_reserve(gn_ctx* c, HalfBuf& b, int set, int m, const float* base, int6
 }
 
 void half_invalidate(gn_ctx* c, int set) {
-  for (auto& b : c->half_buf[set]) b.valid = b.info_valid = false;
+  for (auto& b : c->half_buf[set]) { b.base = nullptr; b.valid = b.info_valid = false; }
 }
 void half_drop(gn_ctx* c, int set) {
   for (auto& b : c->half_buf[set]) {
     if (b.cap > 0) dev_free(c, b.p);
-    b.p = nullptr; b.cap = 0; b.valid = b.info_valid = false;
+    b.p = nullptr; b.cap = 0; b.base = nullptr; b.valid = b.info_valid = false;
   }
 }
 // No room: the passes go on without copies.

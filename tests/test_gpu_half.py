@@ -239,3 +239,38 @@ def test_copies_and_memory_that_changes_hands():
         for _ in range(2):
             assert relb(c.Gv_blockdiag(dev(v)).cpu().numpy(), orc.Gv_blockdiag(th, w, C, XS, v), w) <= TOL["tf32"]
     c.close()
+
+
+@pytest.mark.parametrize("widths", [[392] * 4 + [10], [520] * 3 + [10]])
+def test_a_place_ends_with_its_pass(widths):
+    """Row batches' buffers are let go and the subsample's got in their place, in sizes that meet at the same addresses now and
+    then: what a product writes there are its own copies, not those that the gradient kept beside a matrix at that address."""
+    p = wl.make_custom(widths, l=2300, nS=1700, C=23.0, seed=75, x="sparse80")
+    w, v, many, refs = p["widths"], dev(p["v"]), (700, 1000, 1100, 1300, 1700), {}
+    for rows in many:
+        c = make_ctx(p, "tf32")
+        c.debug_option(11, 0)
+        c.set_subsample(dev(p["idx"][:rows]))
+        refs[rows] = c.Gv(v).clone()
+        c.close()
+        ref = orc.Gv(p["theta"], w, p["C"], p["X"][p["idx"][:rows]], p["v"])
+        assert relb(refs[rows].cpu().numpy(), ref, w) <= TOL["tf32"]
+    for first in (0, 300, 600):
+        for batch in (500, 800, 1000, 1300):
+            for rows in many:
+                for blocks in (0, 1):
+                    c = make_ctx(p, "tf32")
+                    c.debug_option(11, 2)
+                    c.set_batch_rows(batch)
+                    c.set_blockdiag_method(2)
+                    if first:
+                        c.set_subsample(dev(p["idx"][:first]))
+                        c.Gv(v)
+                    c.grad()
+                    if first and blocks:
+                        c.Gv_blockdiag(v)
+                    c.set_batch_rows(2300)
+                    c.set_subsample(dev(p["idx"][:rows]))
+                    d = c.Gv(v)
+                    assert float((d - refs[rows]).norm() / refs[rows].norm()) <= TOL["tf32"]
+                    c.close()
