@@ -78,10 +78,16 @@ struct Tf32Params {
 // (longest tiles first), which lets the short tiles of one problem fill the partial last wave of another.
 constexpr int MAX_GROUP = 6;
 constexpr int MAX_PAIRS_LAUNCH = 80;        // >= SMs / 2
+//
+// A launch with one problem may cut left-over tiles along K, one with several may chain them, and neither has the code of the other;
+// one without FP16 copies (HALF false) has nothing of theirs, neither maps nor code.  Parameters are copied at every launch: with 9 KB
+// of them in all launches (six problems and the maps of their copies; one problem without copies takes 1 KB) a full CG step
+// of 54-40-2540-14 with 883 rows took 163 us instead of 155, a 700 x 50 product 4 us more.
+template <int NP>
 struct GroupParams {
   int n_prob;
-  Tf32Params pr[MAX_GROUP];
-  unsigned short rstart[MAX_GROUP][MAX_PAIRS_LAUNCH + 1];
+  Tf32Params pr[NP];
+  unsigned short rstart[NP][MAX_PAIRS_LAUNCH + 1];
   // Dependent problems in one launch (a chain of layers): problem g may read, as an operand, what problem
   // dep_prob[g] (earlier in the list) writes.  dep_all[g] == 0: a tile of g needs the producer's tiles of the
   // same 256-row panel (its A rows are the producer's output rows); dep_all[g] == 1: it needs all of them (its
@@ -89,14 +95,15 @@ struct GroupParams {
   // (signal bit 0) and in total (bit 1) in `done`; the TMA warps of a consumer wait, bounded, for the count.
   // Every pair works through the problems in list order and all pairs are resident, so a wait is always for
   // work that is running or about to run on another pair.
-  int dep_prob[MAX_GROUP];
-  int dep_all[MAX_GROUP];
-  int signal[MAX_GROUP];
+  int dep_prob[NP];
+  int dep_all[NP];
+  int signal[NP];
   // (bit 30 of a counter: a copy written by these tiles may not be used)
   int* done;                 // [n_prob][done_stride]: entry i < done_stride - 1 counts panel i, the last entry all tiles
   int done_stride;
 };
-struct GroupMaps { CUtensorMap m[MAX_GROUP][4], h[MAX_GROUP][4]; };   // per problem: A0, B0, A1, B1, and their FP16 copies
+template <int NP, bool HALF>
+struct GroupMaps { CUtensorMap m[NP][HALF ? 8 : 4]; };   // per problem: A0, B0, A1, B1, then the same of their FP16 copies
 
 __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile(
@@ -440,7 +447,8 @@ __device__ __forceinline__ void k_range(const Tf32Params& p, const Work& w, bool
   kb1 = w.sliced ? (int)((long long)total * (w.sl + 1) / p.slices) : total;
 }
 // Counter of finished tiles that a tile's first A operand (its row panel) or K operand (all) waits for.
-__device__ __forceinline__ const int* dep_counter(const GroupParams& gp, const Work& w) {
+template <int NP>
+__device__ __forceinline__ const int* dep_counter(const GroupParams<NP>& gp, const Work& w) {
   const int d = gp.dep_prob[w.prob];
   return gp.done + (long long)d * gp.done_stride + (gp.dep_all[w.prob] ? gp.done_stride - 1 : w.tile / gp.pr[w.prob].tiles_n);
 }
@@ -449,8 +457,9 @@ __device__ __forceinline__ const int* dep_counter(const GroupParams& gp, const W
 // A single problem whose left-over tiles are cut along K: the pair does its slice FIRST; the store of the partial
 // accumulator, the wait for the other slices and the fix-up epilogue then run on the epilogue warps underneath the
 // MMAs of the pair's first whole tile instead of being exposed at the end of the kernel.
-__device__ __forceinline__ bool next_work(const GroupParams& gp, int pair, int idx, Work& w) {
-  if (gp.pr[0].slices >= 2) {                  // (only ever set for a launch with one problem)
+template <int NP>
+__device__ __forceinline__ bool next_work(const GroupParams<NP>& gp, int pair, int idx, Work& w) {
+  if (NP == 1 && gp.pr[0].slices >= 2) {
     const Tf32Params& p = gp.pr[0];
     w.prob = 0;
     if (pair < p.rem * p.slices) {
@@ -467,7 +476,7 @@ __device__ __forceinline__ bool next_work(const GroupParams& gp, int pair, int i
     w.tile = idx * p.P + pair; w.sl = 0; w.sliced = 0;
     return true;
   }
-  for (int g = 0; g < gp.n_prob; ++g) {
+  for (int g = 0; g < (NP == 1 ? 1 : gp.n_prob); ++g) {
     const Tf32Params& p = gp.pr[g];
     const int r0 = gp.rstart[g][pair], n_rem = gp.rstart[g][pair + 1] - r0;
     if (idx < p.waves + n_rem) {
@@ -487,19 +496,13 @@ __device__ __forceinline__ bool next_work(const GroupParams& gp, int pair, int i
 // MODE fixes the options at compile time: 0 = alpha * acc (+ bias), 1 = sigmoid, 2 = times the sigmoid derivative of `dsig`,
 // 3 = plus beta * cin.  (Combinations, none of them on the path, go element by element: epilogue_ragged.)
 struct EpiArgs {
-  const float* dsig; const float* cin; const float* bias; float* D;
-  long long ldd, ld_dsig, ld_cin;
-  int dsig_rows, dsig_div;   // row m of the tile reads row (m / dsig_div) % dsig_rows of dsig ...
-  int dsig_direct;           // ... which is m itself when dsig_div == 1 and dsig_rows >= M (no division per row)
-  float alpha, beta;
-  int M, sigm;
   float un;                  // what undoes the scale of the sums (1 for TF32 operands)
-  __half* Dh; long long ldh; float hsc;      // copy of D, and its scale
+  float hsc;                 // scale of D's copy
 };
 
-
-__device__ __forceinline__ long long dsig_row(const EpiArgs& a, int m) {
-  return a.dsig_direct ? m : (m / a.dsig_div) % a.dsig_rows;
+// Row of dsig that belongs to row m (m itself without a division where it can be).
+__device__ __forceinline__ long long dsig_row(const Tf32Params& p, int m) {
+  return p.dsig_div == 1 && p.dsig_rows >= p.M ? m : (m / p.dsig_div) % p.dsig_rows;
 }
 
 // This warp's pieces of a tile: column chunks first, first + step, ... below end of the 16 rows whose element 0 this thread holds in
@@ -530,16 +533,18 @@ __device__ __forceinline__ void piece_sums(const PieceRun& r, int c, float (&v)[
 // HALF: D's FP16 copy is written too.  The runs of it that are looked at are a thread's 8 elements of a row and 2 of a column of
 // the piece; two threads swap halves of what they hold so that a store covers whole 32-byte sectors.
 template <int MODE, bool HALF>
-__device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun& r, int N, int lane, HalfCheck& check) {
+__device__ __forceinline__ void epilogue_pieces(const Tf32Params& p, const EpiArgs& a, const PieceRun& r, int lane, HalfCheck& check) {
   constexpr bool ONE_OP = MODE == 2 || MODE == 3;
-  const bool ok[2] = {r.m < a.M, r.m + 8 < a.M};
+  const int N = p.N;
+  const bool ok[2] = {r.m < p.M, r.m + 8 < p.M};
   const float* orow[2] = {nullptr, nullptr};   // this thread's rows of dsig (mode 2) or of cin (mode 3)
   if (ONE_OP) {
 #pragma unroll
     for (int e = 0; e < 2; ++e)
-      if (ok[e]) orow[e] = (MODE == 3 ? a.cin + (long long)(r.m + 8 * e) * a.ld_cin : a.dsig + dsig_row(a, r.m + 8 * e) * a.ld_dsig) + r.nb0;
+      if (ok[e]) orow[e] = (MODE == 3 ? dep(p.cin) + (long long)(r.m + 8 * e) * p.ld_cin : dep(p.dsig) + dsig_row(p, r.m + 8 * e) * p.ld_dsig) + r.nb0;
   }
-  float* const drow = a.D + (long long)r.m * a.ldd + r.nb0;
+  const float* const bias = dep(p.bias);
+  float* const drow = p.D + (long long)r.m * p.ldd + r.nb0;
 #pragma unroll 1
   for (int c = r.first; c < r.end; c += r.step) {
     bool in[4];                                // (N is a multiple of four: a thread's pair, and what it stores of a copy, is in or out)
@@ -559,7 +564,7 @@ __device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun
     }
     float2 bz[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) bz[j] = a.bias && in[j] ? __ldg(reinterpret_cast<const float2*>(a.bias + r.nb0 + c * 32 + 8 * j)) : make_float2(0.f, 0.f);
+    for (int j = 0; j < 4; ++j) bz[j] = bias && in[j] ? __ldg(reinterpret_cast<const float2*>(bias + r.nb0 + c * 32 + 8 * j)) : make_float2(0.f, 0.f);
     float v[16];
     piece_sums(r, c, v);
     unsigned hv[2][HALF ? 4 : 1];
@@ -575,12 +580,12 @@ __device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun
           const float2 z = op[ONE_OP ? 4 * e + j : 0];
           x0 *= z.x * (1.f - z.x); x1 *= z.y * (1.f - z.y);
         }
-        x0 *= a.alpha; x1 *= a.alpha;
+        x0 *= p.alpha; x1 *= p.alpha;
         if (MODE == 3) {
           const float2 cc = op[ONE_OP ? 4 * e + j : 0];
-          x0 = fmaf(a.beta, cc.x, x0); x1 = fmaf(a.beta, cc.y, x1);
+          x0 = fmaf(p.beta, cc.x, x0); x1 = fmaf(p.beta, cc.y, x1);
         }
-        if (ok[e] && in[j]) *reinterpret_cast<float2*>(drow + 8 * e * a.ldd + c * 32 + 8 * j) = make_float2(x0, x1);
+        if (ok[e] && in[j]) *reinterpret_cast<float2*>(drow + 8 * e * p.ldd + c * 32 + 8 * j) = make_float2(x0, x1);
         if (HALF) {
           const float y0 = ok[e] && in[j] ? x0 * a.hsc : 0.f, y1 = ok[e] && in[j] ? x1 * a.hsc : 0.f;
           row[e] = max3_abs(row[e], y0, y1);
@@ -592,7 +597,7 @@ __device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun
     }
     if (HALF) {
       const bool odd = lane & 1;
-      __half* const hrow = a.Dh + (long long)r.m * a.ldh + r.nb0 + c * 32 + (odd ? 6 : 0);
+      __half* const hrow = p.Dh + (long long)r.m * p.ldh + r.nb0 + c * 32 + (odd ? 6 : 0);
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         check.run(row[e]);
@@ -600,7 +605,7 @@ __device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun
         for (int j = 0; j < 4; j += 2) {       // even lanes: columns 8 j + 0..3 or 4..7, odd lanes the same of 8 (j + 1)
           const unsigned mine = odd ? hv[e][HALF ? j + 1 : 0] : hv[e][HALF ? j : 0];
           const unsigned other = __shfl_xor_sync(0xffffffffu, odd ? hv[e][HALF ? j : 0] : hv[e][HALF ? j + 1 : 0], 1);
-          if (ok[e] && (odd ? in[j + 1] : in[j])) *reinterpret_cast<uint2*>(hrow + 8 * e * a.ldh + 8 * j) = odd ? make_uint2(other, mine) : make_uint2(mine, other);
+          if (ok[e] && (odd ? in[j + 1] : in[j])) *reinterpret_cast<uint2*>(hrow + 8 * e * p.ldh + 8 * j) = odd ? make_uint2(other, mine) : make_uint2(mine, other);
         }
       }
     }
@@ -608,7 +613,22 @@ __device__ __forceinline__ void epilogue_pieces(const EpiArgs& a, const PieceRun
 }
 
 // The same of pieces that are ragged or unaligned, or that combine options, element by element.
-__device__ __forceinline__ void epilogue_ragged(const EpiArgs& a, const PieceRun& r, int N, HalfCheck& check) {
+template <bool HALF>
+__device__ __forceinline__ HalfCheck epilogue_ragged(const Tf32Params& p, const EpiArgs& a, const PieceRun& r) {
+  HalfCheck check;
+  const int N = p.N;
+  const float* const bias = p.bias ? dep(p.bias) + r.nb0 : nullptr;
+  const float* const dsig = dep(p.dsig);
+  const float* const cin = dep(p.cin);
+  const float* zrow[2] = {nullptr, nullptr};   // this thread's rows of dsig and cin
+  const float* crow[2] = {nullptr, nullptr};
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (r.m + 8 * e < p.M) {
+      if (dsig) zrow[e] = dsig + dsig_row(p, r.m + 8 * e) * p.ld_dsig + r.nb0;
+      if (cin) crow[e] = cin + (long long)(r.m + 8 * e) * p.ld_cin + r.nb0;
+    }
+  float* const drow = p.D + (long long)r.m * p.ldd + r.nb0;
 #pragma unroll 1
   for (int c = r.first; c < r.end; c += r.step) {
     float v[16];
@@ -618,39 +638,39 @@ __device__ __forceinline__ void epilogue_ragged(const EpiArgs& a, const PieceRun
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const int n = r.nb0 + c * 32 + 8 * j + i;
+        const int n = c * 32 + 8 * j + i;
         float col = 0.f;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const int m = r.m + 8 * e;
-          if (n < N && m < a.M) {
-            float x = fmaf(v[4 * j + 2 * e + i], a.un, a.bias ? __ldg(a.bias + n) : 0.f);
-            if (a.sigm) x = sigmoid_from(__expf(-x));
-            if (a.dsig) { const float z = __ldg(a.dsig + dsig_row(a, m) * a.ld_dsig + n); x *= z * (1.f - z); }
-            x *= a.alpha;
-            if (a.cin) x = fmaf(a.beta, __ldcg(a.cin + (long long)m * a.ld_cin + n), x);
-            a.D[(long long)m * a.ldd + n] = x;
-            if (a.Dh) {
+          if (r.nb0 + n < N && r.m + 8 * e < p.M) {
+            float x = fmaf(v[4 * j + 2 * e + i], a.un, bias ? __ldg(bias + n) : 0.f);
+            if (p.sigmoid) x = sigmoid_from(__expf(-x));
+            if (dsig) { const float z = __ldg(zrow[e] + n); x *= z * (1.f - z); }
+            x *= p.alpha;
+            if (cin) x = fmaf(p.beta, __ldcg(crow[e] + n), x);
+            drow[8 * e * p.ldd + n] = x;
+            if (HALF && p.copy_out) {
               const float y = x * a.hsc;
               row[e] = max3_abs(row[e], y, y);
               col = max3_abs(col, y, y);
-              a.Dh[(long long)m * a.ldh + n] = __float2half_rn(y);
+              p.Dh[(long long)(r.m + 8 * e) * p.ldh + r.nb0 + n] = __float2half_rn(y);
             }
           }
         }
-        if (a.Dh) check.run(col);
+        if (HALF && p.copy_out) check.run(col);
       }
-    if (a.Dh) { check.run(row[0]); check.run(row[1]); }
+    if (HALF && p.copy_out) { check.run(row[0]); check.run(row[1]); }
   }
+  return check;
 }
 
 constexpr int PAIR_EPI_WARPS = 16, PAIR_THREADS = 64 + 32 * PAIR_EPI_WARPS;
 constexpr int B2_STAGE_MAX = (BN_MAX / 2) * BK * 4;          // 16 KB: this CTA's half of the B tile
 constexpr int STAGE2_BYTES = A_STAGE_BYTES + B2_STAGE_MAX;   // 32 KB
 
-template <int STAGES>
+template <int STAGES, int NP, bool HALF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
-gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constant__ GroupParams gp) {
+gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps<NP, HALF> gm, const __grid_constant__ GroupParams<NP> gp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE2_BYTES);
@@ -671,7 +691,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * PAIR_EPI_WARPS); }
     *abort_flag = 0;
-    for (int i = 0; i < TILE_WORDS; ++i) tile_words[i] = 0;
+    if (HALF)
+      for (int i = 0; i < TILE_WORDS; ++i) tile_words[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 2) {  // both CTAs of the pair allocate all 512 columns, same warp, same destination offset
@@ -699,8 +720,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       const int t = w.tile;
       const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM;
       const int n0 = (t % p.tiles_n) * bn + (int)rank * hb;
-      const int dp = gp.dep_prob[w.prob];
-      const bool a1_here = dp >= 0 && p.half && gp.pr[dp].hout == p.hin[0];
+      const int dp = NP > 1 ? gp.dep_prob[w.prob] : -1;
+      const bool a1_here = HALF && dp >= 0 && p.half && gp.pr[dp].hout == p.hin[0];
       int bad_panel = 0;
       if (dp >= 0) {
         // an operand of this tile is written by an earlier problem of this launch: wait until its tiles are stored
@@ -722,11 +743,11 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         asm volatile("fence.proxy.async.global;" ::: "memory");   // the stores were generic, the loads below are TMA's
         __syncwarp();
       }
-      if (w.prob != hu_prob) { hu = half_use(p, a1_here); hu_prob = w.prob; }
-      const bool half = hu.use != 0 && !(a1_here && bad_panel);
+      if (HALF && w.prob != hu_prob) { hu = half_use(p, a1_here); hu_prob = w.prob; }
+      const bool half = HALF && hu.use != 0 && !(a1_here && bad_panel);
       int kb0, kb1;
       k_range(p, w, half, kb0, kb1);
-      if (lane == 0)             // (a slice may end before the first operand pair)
+      if (HALF && lane == 0)     // (a slice may end before the first operand pair)
         tile_words[wi % TILE_WORDS] = tile_word(wi, half ? 1 : 0, half ? -(p.khalf[1] > 0 && kb1 <= p.khalf[1] ? hu.sum1 : hu.sum0) : 0, hu.out);
       const int first = half && p.khalf[1] > 0 ? 1 : 0;        // operand pair that goes first
       const int n_first = half ? p.khalf[first] : p.kblocks[0];
@@ -740,13 +761,13 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         // one thread, and nothing in the loop that need not be there (as for the MMA issuer)
         int good = 1;
         if (lane == 0) {
-          const CUtensorMap* const maps = half ? gm.h[w.prob] : gm.m[w.prob];
+          const CUtensorMap* const maps = gm.m[w.prob] + (half ? 4 : 0);
           const int bk = half ? BK_HALF : BK, am = m0 / (half ? 64 : 32), bm = n0 / (half ? 64 : 32);
           const bool a3 = p.a_mn != 0, b3 = p.b_mn != 0;
           for (int kb = kb0; kb < kb1; ++kb) {
             if (!wait_or_abort(&empty[s], ph ^ 1, abort_flag, err, 1)) { good = 0; break; }
             if (rank == 0) {
-              if (kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
+              if (HALF && kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
               mbar_expect_tx(&full[s], pair_tx);
             }
             const uint32_t full_leader = map_to_cta(smem_u32(&full[s]), 0);
@@ -772,7 +793,7 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         good = __shfl_sync(0xffffffffu, good, 0);
         if (!good) { ok = false; break; }
         if (rank == 0 && lane == 0) {
-          if (kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
+          if (HALF && kb == kb0) tile_form[s] = half ? 1 | (hu.sum1 - hu.sum0) << 1 : 0;
           mbar_expect_tx(&full[s], pair_tx);
         }
         __syncwarp();
@@ -783,8 +804,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         uint8_t* sb = sa + A_STAGE_BYTES;
         if (++s == STAGES) { s = 0; ph ^= 1u; }
         if (half) {
-          const CUtensorMap* ma = &gm.h[w.prob][2 * pr];
-          const CUtensorMap* mb = &gm.h[w.prob][2 * pr + 1];
+          const CUtensorMap* ma = &gm.m[w.prob][HALF ? 4 + 2 * pr : 0];
+          const CUtensorMap* mb = ma + 1;
           const int k0 = kk * BK_HALF;
           if (lane == 0) {
             if (!p.a_mn) tma2_load_2d(sa, ma, k0, m0, full_leader);
@@ -836,12 +857,12 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(buf * BN_MAX);
         int form = 0;
-        if (p.half) {                          // (comes with the tile's first operands)
+        if (HALF && p.half) {                  // (comes with the tile's first operands)
           ok = wait_or_abort(&full[s], ph, abort_flag, err, 2);
           if (!ok) break;
           form = tile_form[s];
         }
-        const bool half = form != 0;
+        const bool half = HALF && form != 0;
         int kb0, kb1;
         k_range(p, w, half, kb0, kb1);
         // scale step: before the first k-block of the first operand pair, where one of the second went before it
@@ -904,9 +925,8 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       }
     }
   } else {
-    // ------------------------------------------------------------------ epilogue (warps 2..9, both CTAs)
-    // Fragment layout of tmem_ld_16x256b_x4: this thread's 32 values of a 32 x 32 chunk are v[h][4j + 2e + i] =
-    // element (row 16h + 8e + lane/4, column 8j + 2 (lane%4) + i) of the warp's quadrant.
+    // ------------------------------------------------------------------ epilogue (warps 2..17, both CTAs)
+    // Fragment layout: see epilogue_pieces.
     const int quad = warp & 3;
     const int sub = (warp - 2) >> 2;             // of the quadrant's four warps: rows 16 (sub % 2) .., every other column chunk
     const int hh = sub & 1, half = sub >> 1;
@@ -919,7 +939,6 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       const Tf32Params& p = gp.pr[w.prob];
       const int bn = p.bn;
       const int t = w.tile;
-
       const int m0 = (t / p.tiles_n) * (2 * BM) + (int)rank * BM, n0 = (t % p.tiles_n) * bn;
       const int buf = ti & 1;
       const uint32_t aph = (ti >> 1) & 1;
@@ -930,20 +949,23 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       tc_fence_after();
       // (the producer has left the tile's word before it asked for the first operands: this loop ends at once)
       int word = 0;
-      if (lane == 0) {
-        const unsigned long long t0 = globaltimer();
-        while (((word = tile_words[wi % TILE_WORDS]) >> 17) != ((wi + 1) & 0x3fff)) {
-          if (*abort_flag || globaltimer() - t0 > WAIT_LIMIT_NS) { atomicCAS(err, 0, 7); *abort_flag = 1; word = 0; break; }
+      if (HALF) {
+        if (lane == 0) {
+          const unsigned long long t0 = globaltimer();
+          while (((word = tile_words[wi % TILE_WORDS]) >> 17) != ((wi + 1) & 0x3fff)) {
+            if (*abort_flag || globaltimer() - t0 > WAIT_LIMIT_NS) { atomicCAS(err, 0, 7); *abort_flag = 1; word = 0; break; }
+          }
         }
+        word = __shfl_sync(0xffffffffu, word, 0);
+        if (word == 0) break;
       }
-      word = __shfl_sync(0xffffffffu, word, 0);
-      if (word == 0) break;
-      const float un = word & 1 ? half_scale((word >> 1 & 0xff) - 128) : 1.f;
+      const float un = HALF && word & 1 ? half_scale((word >> 1 & 0xff) - 128) : 1.f;
       const int out_e = (word >> 9 & 0xff) - 128;
       const int n_chunks = min(bn / 32, (p.N - n0 + 31) / 32);   // column chunks of this tile that exist
       const uint32_t tq = tmem_base + ((uint32_t)(quad * 32 + 16 * hh) << 16) + (uint32_t)(buf * BN_MAX);
       int sl = 0, grp = 0;                                       // slice index and first pair of the tile's group
-      if (w.sliced) {
+      const bool sliced = NP == 1 && w.sliced;
+      if (sliced) {
         grp = (pair / p.slices) * p.slices;
         sl = pair - grp;
         // (a tile of few rows or columns is few warps' work, and the others take no part in the count)
@@ -993,40 +1015,34 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
       {
         const int mq = m0 + quad * 32 + rsub;                    // this thread's rows are mq and mq + 8
         EpiArgs ea;
-        ea.dsig = dep(p.dsig); ea.cin = dep(p.cin); ea.bias = dep(p.bias); ea.D = p.D;
-        ea.ldd = p.ldd; ea.ld_dsig = p.ld_dsig; ea.ld_cin = p.ld_cin;
-        ea.dsig_rows = p.dsig_rows; ea.dsig_div = p.dsig_div;
-        ea.dsig_direct = p.dsig_div == 1 && p.dsig_rows >= p.M;
-        ea.alpha = p.alpha; ea.beta = p.beta; ea.M = p.M; ea.sigm = p.sigmoid;
-        ea.un = w.sliced ? 1.f : un;
-        ea.Dh = p.copy_out ? p.Dh : nullptr; ea.ldh = p.ldh; ea.hsc = half_scale(out_e);
+        const bool copy_out = HALF && p.copy_out;
+        ea.un = sliced ? 1.f : un; ea.hsc = half_scale(out_e);
         HalfCheck check;
-        const int N = p.N, vec_epi = p.vec_epi;
         const int n_opt = (p.sigmoid ? 1 : 0) + (p.dsig ? 1 : 0) + (p.cin ? 1 : 0);
         const int mode = n_opt == 0 ? 0 : n_opt > 1 ? 4 : p.sigmoid ? 1 : p.dsig ? 2 : 3;
         // whole tile: this warp's chunks are half, half + 2, ...; sliced tile: the pair's share of the
-        // chunks is sl, sl + slices, ..., dealt alternately to the two warps of a quadrant
-        const int c_first = w.sliced ? sl + half * p.slices : half;
-        const int c_step = w.sliced ? 2 * p.slices : 2;
-        const int n_slices = w.sliced ? p.slices : 0;
-        const float* const ws0 = w.sliced ? p.sk_ws + (((long long)grp * 2 + rank) * BM + quad * 32 + rsub) * BN_MAX + csub : nullptr;
+        // chunks is sl, sl + slices, ..., dealt alternately to the two warps of these rows
+        const int c_first = sliced ? sl + half * p.slices : half;
+        const int c_step = sliced ? 2 * p.slices : 2;
+        const int n_slices = sliced ? p.slices : 0;
+        const float* const ws0 = sliced ? p.sk_ws + (((long long)grp * 2 + rank) * BM + quad * 32 + rsub) * BN_MAX + csub : nullptr;
         // (options of one kind on 16-byte aligned rows; anything else element by element)
         const PieceRun run{tq, mq, n0 + csub, c_first, c_step, n_chunks, ws0, n_slices};
-        if (!vec_epi || mode == 4) {
-          epilogue_ragged(ea, run, N, check);
-        } else if (p.copy_out) {                                            // (only ever set with mode 1 or 2)
-          if (mode == 1) epilogue_pieces<1, true>(ea, run, N, lane, check);
-          else epilogue_pieces<2, true>(ea, run, N, lane, check);
+        if (!p.vec_epi || mode == 4) {
+          check = epilogue_ragged<HALF>(p, ea, run);
+        } else if (copy_out) {                                            // (only ever set with mode 1 or 2)
+          if (mode == 1) epilogue_pieces<1, true>(p, ea, run, lane, check);
+          else epilogue_pieces<2, true>(p, ea, run, lane, check);
         } else {
           switch (mode) {
-            case 0: epilogue_pieces<0, false>(ea, run, N, lane, check); break;
-            case 1: epilogue_pieces<1, false>(ea, run, N, lane, check); break;
-            case 2: epilogue_pieces<2, false>(ea, run, N, lane, check); break;
-            case 3: epilogue_pieces<3, false>(ea, run, N, lane, check); break;
+            case 0: epilogue_pieces<0, false>(p, ea, run, lane, check); break;
+            case 1: epilogue_pieces<1, false>(p, ea, run, lane, check); break;
+            case 2: epilogue_pieces<2, false>(p, ea, run, lane, check); break;
+            case 3: epilogue_pieces<3, false>(p, ea, run, lane, check); break;
             default: break;
           }
         }
-        if (p.copy_out) {
+        if (copy_out) {
           // this warp's word on the copy: the largest magnitude, and whether it may be used (the scale is said once)
           const unsigned high = __reduce_max_sync(0xffffffffu, check.high);
           bad_out = __any_sync(0xffffffffu, check.bad());
@@ -1042,12 +1058,12 @@ gemm_tf32_2cta_kernel(const __grid_constant__ GroupMaps gm, const __grid_constan
           amax_seen = max(amax_seen, high);
         }
       }
-      if (!w.sliced) {       // (a sliced tile released its accumulator right after storing it)
+      if (!sliced) {       // (a sliced tile released its accumulator right after storing it)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&acc_empty[buf]), 0));
       }
-      if (gp.signal[w.prob]) {
+      if (NP > 1 && gp.signal[w.prob]) {
         // a later problem of this launch reads this tile: publish this warp's stores, then count the warp in
         __threadfence();
         asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -1203,7 +1219,9 @@ int gemm_tf32_workspace_flags() { return num_sms() / 2; }
 namespace {
 
 // Tensor maps and kernel parameters of one problem for a given tile width (two_cta: 256 x bn tiles of a CTA pair).
-bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUtensorMap* maps, CUtensorMap* half_maps, Tf32Params& p) {
+// maps: four, and four more of the copies if there are any.
+bool setup_problem(const GemmArgs& g, bool two_cta, int bn, int* err_flag, CUtensorMap* maps, Tf32Params& p) {
+  CUtensorMap* const half_maps = maps + 4;
   const int b_rows = two_cta ? bn / 2 : bn;      // B rows staged per CTA
   const float* As[2] = {g.A1, g.A2};
   const float* Bs[2] = {g.B1, g.B2};
@@ -1269,8 +1287,20 @@ void set_kernel_attributes() {
   static std::atomic<signed char> state[64];
   once_per_device(state, [] {
     return cudaFuncSetAttribute(gemm_tf32_kernel<kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) == cudaSuccess &&
-           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess;
+           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2, MAX_GROUP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_tf32_2cta_kernel<kStages2, MAX_GROUP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes2) == cudaSuccess;
   });
+}
+
+// One launch of the CTA-pair kernel; maps: eight per problem, the last four unused without copies.
+template <int NP, bool HALF>
+void launch_pair(const GroupParams<NP>& gp, const CUtensorMap (*maps)[8], int ctas, cudaStream_t st) {
+  GroupMaps<NP, HALF> gm;
+  for (int k = 0; k < gp.n_prob; ++k)
+    for (int j = 0; j < (HALF ? 8 : 4); ++j) gm.m[k][j] = maps[k][j];
+  launch_pdl(gemm_tf32_2cta_kernel<kStages2, NP, HALF>, ctas, PAIR_THREADS, kSmemBytes2, st, gm, gp);
 }
 
 inline bool suits_pair_kernel(const GemmArgs& g) { return g.M > BM && g.N >= 128; }
@@ -1324,12 +1354,11 @@ int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_fla
     if (choose_slices(tiles, total_kb_all, pairs) < 2) { stream_k = false; bn = choose_bn2(g.M, g.N, false); }
   }
   if (two_cta) {
-    GroupMaps gm;                              // (host copies; passed to the kernel by value)
-    GroupParams gp = {};                       // (no dependencies, no signals)
-    for (int k = 0; k < MAX_GROUP; ++k) gp.dep_prob[k] = -1;
+    CUtensorMap maps[1][8];
+    GroupParams<1> gp = {};                    // (no dependencies, no signals)
     gp.n_prob = 1;
     Tf32Params& p = gp.pr[0];
-    if (!setup_problem(g, true, bn, err_flag, gm.m[0], gm.h[0], p)) return -1;
+    if (!setup_problem(g, true, bn, err_flag, maps[0], p)) return -1;
     const int total_kb = total_kb_all;
     p.sk_ws = sk_ws; p.sk_flags = sk_flags;
     p.P = p.tiles < pairs ? p.tiles : pairs;
@@ -1345,11 +1374,12 @@ int launch_gemm_tf32(const GemmArgs& g, int* err_flag, float* sk_ws, int* sk_fla
       }
     }
     for (int q = 0; q <= MAX_PAIRS_LAUNCH; ++q) gp.rstart[0][q] = (unsigned short)(q < p.rem ? q : p.rem);
-    launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * launch_pairs, PAIR_THREADS, kSmemBytes2, st, gm, gp);
+    if (p.half || p.copy_out) launch_pair<1, true>(gp, maps, 2 * launch_pairs, st);
+    else launch_pair<1, false>(gp, maps, 2 * launch_pairs, st);
   } else {
     CUtensorMap maps[4];
     Tf32Params p;
-    if (!setup_problem(g, false, bn, err_flag, maps, nullptr, p)) return -1;
+    if (!setup_problem(g, false, bn, err_flag, maps, p)) return -1;
     const int grid = p.tiles < num_sms() ? p.tiles : num_sms();
     launch_pdl(gemm_tf32_kernel<kStages>, grid, 320, kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], p);
   }
@@ -1368,7 +1398,7 @@ namespace {
 // Tiles of problem slot k of a group (cost `cost` each) dealt to the P pairs on top of the loads they carry
 // already: as many whole waves (tiles q, q + P, ... for every pair q) as every pair takes anyway, the rest as
 // contiguous runs of the left-over tiles, so that the loads come out as even as whole tiles allow.
-void deal_tiles(GroupParams& gp, int k, double cost, int P, double* load) {
+void deal_tiles(GroupParams<MAX_GROUP>& gp, int k, double cost, int P, double* load) {
   Tf32Params& p = gp.pr[k];
   p.P = P;
   int cnt[MAX_PAIRS_LAUNCH];
@@ -1424,17 +1454,19 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
                            int done_stride, int* err_flag, cudaStream_t st) {
   if (!gemm_tf32_group_eligible(gs, n)) return -1;
   set_kernel_attributes();
-  GroupMaps gm;
-  GroupParams gp = {};
+  CUtensorMap maps[MAX_GROUP][8];
+  GroupParams<MAX_GROUP> gp = {};
   const int pairs = num_sms() / 2;
   struct Item { int src; double cost; };
   Item order[MAX_GROUP];
   Tf32Params tmp[MAX_GROUP];
-  CUtensorMap tmaps[MAX_GROUP][4], thalf[MAX_GROUP][4];
+  CUtensorMap tmaps[MAX_GROUP][8];
   long long total_tiles = 0;
+  bool half = false;
   for (int i = 0; i < n; ++i) {
     const int bn = choose_bn2(gs[i].M, gs[i].N, true);
-    if (!setup_problem(gs[i], true, bn, err_flag, tmaps[i], thalf[i], tmp[i])) return -1;
+    if (!setup_problem(gs[i], true, bn, err_flag, tmaps[i], tmp[i])) return -1;
+    half = half || tmp[i].half || tmp[i].copy_out;
     if (tmp[i].tiles > 60000) return -1;       // (left-over tile indices are 16-bit)
     order[i].src = i;
     order[i].cost = tile_cost(tmp[i]);
@@ -1461,7 +1493,7 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
   for (int k = 0; k < n; ++k) {
     const int i = order[k].src;
     gp.pr[k] = tmp[i];
-    for (int j = 0; j < 4; ++j) { gm.m[k][j] = tmaps[i][j]; gm.h[k][j] = thalf[i][j]; }
+    for (int j = 0; j < (half ? 8 : 4); ++j) maps[k][j] = tmaps[i][j];
     deal_tiles(gp, k, order[k].cost, P, load);
     if (chain && dep_prob[i] >= 0) {            // (a chain keeps its order: slot == index)
       gp.dep_prob[k] = dep_prob[i];
@@ -1470,7 +1502,8 @@ int launch_gemm_tf32_group(const GemmArgs* gs, int n, const int* dep_prob, const
     }
   }
   if (chain && cudaMemsetAsync(done, 0, sizeof(int) * (size_t)n * done_stride, st) != cudaSuccess) return -1;
-  launch_pdl(gemm_tf32_2cta_kernel<kStages2>, 2 * P, PAIR_THREADS, kSmemBytes2, st, gm, gp);
+  if (half) launch_pair<MAX_GROUP, true>(gp, maps, 2 * P, st);
+  else launch_pair<MAX_GROUP, false>(gp, maps, 2 * P, st);
   return 1;
 }
 
@@ -1483,7 +1516,7 @@ namespace {
 int plan_group_impl(int n, const int* M, const int* N, const int* K, int pairs, int keep_order, int* counts,
                     int* waves, int* order_out, int* tiles_out, double* makespan) {
   if (n < 1 || n > MAX_GROUP || pairs < 1 || pairs > MAX_PAIRS_LAUNCH) return -1;
-  GroupParams gp = {};
+  GroupParams<MAX_GROUP> gp = {};
   struct Item { int src; double cost; };
   Item order[MAX_GROUP];
   Tf32Params tmp[MAX_GROUP];
