@@ -331,6 +331,13 @@ int32_t gn_debug_plan_group(int32_t n, const int32_t* M, const int32_t* N, const
 gn_status gn_debug_check_canaries(gn_ctx* ctx, int64_t* n_checked);
 
 /*
+ * gn_debug_copies - of the matrices that the context has last asked about FP16 copies (option 11 below): how many it knows
+ * the largest magnitude of (*known) and how many of them may not be used, so that contractions read the FP32 matrix
+ * instead (*refused).  Both are 0 before the first pass with copies.  Synchronises.
+ */
+gn_status gn_debug_copies(gn_ctx* ctx, int64_t* known, int64_t* refused);
+
+/*
  * gn_debug_activations - copy the stored Z_m (m in 1..L, [|S|][n_m]) of the current subsample to a
  * device buffer; a test hook for the stored forward pass (Eq. xtoz).
  */
@@ -400,7 +407,8 @@ gn_status gn_debug_gemm_epilogue(gn_ctx* ctx, int kind, int M, int N, int K, con
  * W^L and the stored activations instead of being read back (value 0 = read back; same bits either way).  Option 10:
  * whole passes of small networks as one launch (value 0 = one contraction per layer and operand; the forms differ by
  * rounding).  Option 11: FP16 copies of TF32 operands (value 0 = never, 1 = in passes large enough, the default, 2 = wherever
- * an operand can have one; the forms differ in the order of sums).  Results do not depend on options 0, 3, 4, 5, 6, 9 and, with whole tiles (option 1 off), 8 (tiles, sums
+ * an operand can have one; the forms differ by rounding: in the order of sums, and in elements of a matrix that lie 2^23 or
+ * more below its largest, which FP16 holds with fewer bits).  Results do not depend on options 0, 3, 4, 5, 6, 9 and, with whole tiles (option 1 off), 8 (tiles, sums
  * and parts are computed identically); GN_EINVAL for an unknown option.
  */
 gn_status gn_debug_option(gn_ctx* ctx, int option, int value);

@@ -45,6 +45,7 @@ _SIGNATURES = {
     "gn_debug_timeout_probe": (_i32, [_vp, _dbl]),
     "gn_debug_option": (_i32, [_vp, _i32, _i32]),
     "gn_debug_check_canaries": (_i32, [_vp, C.POINTER(_i64)]),
+    "gn_debug_copies": (_i32, [_vp, C.POINTER(_i64), C.POINTER(_i64)]),
     "gn_debug_plan_group": (_i32, [_i32, C.POINTER(_i32), C.POINTER(_i32), C.POINTER(_i32), _i32, _i32, C.POINTER(_i32),
                                    C.POINTER(_i32), C.POINTER(_i32), C.POINTER(_i32)]),
     "gn_profile": (_i32, [_vp, _i32]),
@@ -383,6 +384,12 @@ class GnContext:
         n = _i64()
         self._check(self._lib.gn_debug_check_canaries(self._h, C.byref(n)))
         return int(n.value)
+
+    def debug_copies(self):
+        """Test hook: matrices asked about FP16 copies, and how many of them may not be used."""
+        known, refused = _i64(), _i64()
+        self._check(self._lib.gn_debug_copies(self._h, C.byref(known), C.byref(refused)))
+        return int(known.value), int(refused.value)
 
     def debug_activations(self, m):
         import torch

@@ -393,20 +393,27 @@ constexpr unsigned kBadPanel = 1u << 30;       // in a counter of finished tiles
 constexpr int kMaxScaleStep = 15;
 struct HalfUse { int use, sum0, sum1, out; };
 
-// Exponent of the scale of D's copy: |D| is bounded from the operands' largest magnitudes m, and 2^e takes the bound below 2^15.
-// (The bound is reached by operands without any cancellation; sums of K terms of random sign stay about sqrt(K) / 2 below it, so
-// at K = 4096 the largest element comes to lie near 2^9, 22 binary orders above what kHalfLeast lets pass.)  Sigmoids need no
+// Exponent of the scale of D's copy: |D| is bounded by A's largest magnitude times the largest sum of magnitudes that an output
+// column of B has (K times B's largest magnitude where that is not known), and 2^e takes the bound below 2^15.  On 784-2000-2000-2000-10
+// with 3000 rows the largest elements then lie at 2^9 to 2^11, with dense and with sparse weights (K times the largest magnitude left them at
+// 2^6 to 2^8 and 2^2 to 2^5: runs below kHalfLeast in five of nine copies of a sparse network).  Sigmoids need no
 // bound.  Where the next contraction adds A2 B2 to the product of this copy with W (hnext: infos of A2, B2, W), its scale must not
 // be above theirs.
 constexpr int kSigmoidExp = 15;
-__device__ __forceinline__ int out_exponent(const Tf32Params& p, const unsigned (&m)[4]) {
+__device__ __forceinline__ int out_exponent(const Tf32Params& p, const int (&e)[4], const unsigned (&m)[4]) {
   if (p.sigmoid) return kSigmoidExp;
-  float bound = (float)p.K[0] * __uint_as_float(m[0]) * __uint_as_float(m[1]) + (float)p.K[1] * __uint_as_float(m[2]) * __uint_as_float(m[3]);
+  float bound = 0.f;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+    if (p.K[s] > 0) {
+      const HalfInfo* const b = p.hin[2 * s + 1];
+      const unsigned long long sum = __ldcg(p.b_mn ? &b->col1 : &b->row1);
+      bound += __uint_as_float(m[2 * s]) * (sum ? half_norm(sum, e[2 * s + 1]) : (float)p.K[s] * __uint_as_float(m[2 * s + 1]));
+    }
   if (p.bias) bound += __uint_as_float(p.K[1] > 0 ? m[3] : m[1]);
   bound *= fabsf(p.alpha) * (p.dsig ? 0.25f : 1.f);
-  int e = half_exponent(__float_as_uint(bound) & 0x7fffffffu);
-  if (p.hnext[0]) e = min(e, max(-kHalfMaxExp, __ldcg(&p.hnext[0]->e) + __ldcg(&p.hnext[1]->e) - __ldcg(&p.hnext[2]->e)));
-  return e;
+  const int out = half_exponent(__float_as_uint(bound) & 0x7fffffffu);
+  return p.hnext[0] ? min(out, max(-kHalfMaxExp, __ldcg(&p.hnext[0]->e) + __ldcg(&p.hnext[1]->e) - __ldcg(&p.hnext[2]->e))) : out;
 }
 // a1_here: A1's copy is written by this very launch (a sigmoid's; the tiles say with the counter whether it may be used).
 __device__ __forceinline__ HalfUse half_use(const Tf32Params& p, bool a1_here) {
@@ -428,7 +435,7 @@ __device__ __forceinline__ HalfUse half_use(const Tf32Params& p, bool a1_here) {
     u.sum0 = e[0] + e[1]; u.sum1 = n == 4 ? e[2] + e[3] : u.sum0;
     u.use = bad == 0u && abs(u.sum0) <= kHalfMaxExp && abs(u.sum1) <= kHalfMaxExp && u.sum1 >= u.sum0 && u.sum1 - u.sum0 <= kMaxScaleStep;
   }
-  if (p.copy_out) u.out = out_exponent(p, amax);
+  if (p.copy_out) u.out = out_exponent(p, e, amax);
   return u;
 }
 
@@ -530,8 +537,45 @@ __device__ __forceinline__ void piece_sums(const PieceRun& r, int c, float (&v)[
   }
 }
 
-// HALF: D's FP16 copy is written too.  The runs of it that are looked at are a thread's 8 elements of a row and 2 of a column of
-// the piece; two threads swap halves of what they hold so that a store covers whole 32-byte sectors.
+// The runs of a copy that are looked at are a piece's 32 elements of a row and 16 of a column.  A thread has 8 and 2 of them; only if
+// these lie low (`check` says so, for some thread of the warp) is the piece looked at as a whole: read back from D, which the
+// same threads have just written, so that the common case pays for a vote and holds nothing more in registers.
+__device__ __noinline__ bool low_piece(const float* drow, long long ldd, int rows, int n, int N, float hsc) {
+  const int lane = threadIdx.x & 31;
+  const bool whole_col = rows + lane / 4 >= 16, whole_row = n - 2 * (lane & 3) + 32 <= N;
+  float y[2][8];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      y[e][j] = 8 * e < rows && n + 8 * (j / 2) + j % 2 < N ? fabsf(drow[8 * e * ldd + 8 * (j / 2) + j % 2] * hsc) : 0.f;
+  HalfCheck check;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    float m = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = fmaxf(m, y[e][j]);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    if (whole_row) check.run(m);
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    float m = fmaxf(y[0][j], y[1][j]);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    if (whole_col) check.run(m);
+  }
+  return __any_sync(0xffffffffu, check.low_run());
+}
+// A piece is done: its low runs, if it has any, belong to longer ones that are not low, or make the copy bad.
+__device__ __forceinline__ void end_piece(const Tf32Params& p, const PieceRun& r, int c, float hsc, HalfCheck& check) {
+  if (!__any_sync(0xffffffffu, check.low_run())) return;
+  check.low = low_piece(p.D + (long long)r.m * p.ldd + r.nb0 + c * 32, p.ldd, p.M - r.m, r.nb0 + c * 32, p.N, hsc) ? 0u : 0xffffffffu;
+}
+
+// HALF: D's FP16 copy is written too.  Two threads swap halves of what they hold so that a store covers whole 32-byte sectors.
 template <int MODE, bool HALF>
 __device__ __forceinline__ void epilogue_pieces(const Tf32Params& p, const EpiArgs& a, const PieceRun& r, int lane, HalfCheck& check) {
   constexpr bool ONE_OP = MODE == 2 || MODE == 3;
@@ -608,6 +652,7 @@ __device__ __forceinline__ void epilogue_pieces(const Tf32Params& p, const EpiAr
           if (ok[e] && (odd ? in[j + 1] : in[j])) *reinterpret_cast<uint2*>(hrow + 8 * e * p.ldh + 8 * j) = odd ? make_uint2(other, mine) : make_uint2(mine, other);
         }
       }
+      end_piece(p, r, c, a.hsc, check);
     }
   }
 }
@@ -659,7 +704,7 @@ __device__ __forceinline__ HalfCheck epilogue_ragged(const Tf32Params& p, const 
         }
         if (HALF && p.copy_out) check.run(col);
       }
-    if (HALF && p.copy_out) { check.run(row[0]); check.run(row[1]); }
+    if (HALF && p.copy_out) { check.run(row[0]); check.run(row[1]); end_piece(p, r, c, a.hsc, check); }
   }
   return check;
 }
@@ -1115,11 +1160,7 @@ bool make_map(CUtensorMap* m, const float* base, long long rows, long long cols,
   return r == CUDA_SUCCESS;
 }
 
-// 3-D view of a row-major [K][MN] matrix (MN contiguous): (32 inner columns, K rows, MN/32 column chunks).
-// One box (32, BK, chunks) lands in shared memory as `chunks` consecutive [BK][32] blocks.  The last
-// chunk of a row may extend past MN (into the next row, or up to 124 bytes past the last row), so the
-// operand must be followed by that much readable memory.
-// The same of FP16 copies: 2-D, box = 64 columns x box_r rows, and 3-D, chunks of 64 columns, BK_HALF rows.
+// The maps of FP16 copies: 2-D as above, box = 64 columns x box_r rows, and 3-D as below, chunks of 64 columns, BK_HALF rows.
 bool make_half_map(CUtensorMap* m, const void* base, long long rows, long long cols, long long ld, int box_r) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
@@ -1143,6 +1184,10 @@ bool make_half_map_mn3d(CUtensorMap* m, const void* base, long long K, long long
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 3-D view of a row-major [K][MN] matrix (MN contiguous): (32 inner columns, K rows, MN/32 column chunks).
+// One box (32, BK, chunks) lands in shared memory as `chunks` consecutive [BK][32] blocks.  The last
+// chunk of a row may extend past MN (into the next row, or up to 124 bytes past the last row), so the
+// operand must be followed by that much readable memory.
 bool make_map_mn3d(CUtensorMap* m, const float* base, long long K, long long MN, long long ld, int chunks) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;

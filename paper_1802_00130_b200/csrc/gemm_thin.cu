@@ -243,7 +243,7 @@ struct ThinKParams {
   const HalfInfo* hin[2];                              // infos of A and B, which bound D
 };
 
-// With a copy (COPY): the scale comes from |D| <= K max|A| max|B| / 4 (the sigmoid derivative), the runs looked at are a thread's 4
+// With a copy (COPY): the scale comes from |D| <= K max|A| max|B| / 4 (the sigmoid derivative), the runs looked at are a warp's 128
 // elements of a row and the block's rows of a column.  (A pass of its own for the largest magnitude and one for the copy
 // took 20 + 24 us at 12000 x 2000; written here it costs 7, and 5 for the largest magnitude of A.)
 template <int KMAX, bool COPY>
@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
   HalfCheck check;
   const int n = (blockIdx.x * 128 + threadIdx.x) * 4;
   const bool n_ok = n < p.N;
+  const unsigned in = __ballot_sync(0xffffffffu, n_ok);
   const float* const pA = dep(p.A);
   const float* const pB = dep(p.B);
   const Epi e = after_wait(p.e);
@@ -278,8 +279,9 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
     b[k] = (n_ok && k < p.K) ? __ldg(reinterpret_cast<const float4*>(pB + (long long)k * p.ldb + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
   float4 bz = make_float4(0.f, 0.f, 0.f, 0.f);
   if (e.bias && n_ok) bz = __ldg(reinterpret_cast<const float4*>(e.bias + n));
-  const int m_begin = blockIdx.y * p.rows_per_block;
-  const int m_end = min(p.M, m_begin + p.rows_per_block);
+  // (with a copy: 16 rows at least, a run of a column)
+  const int m_begin = COPY ? (int)((long long)p.M * blockIdx.y / gridDim.y) : blockIdx.y * p.rows_per_block;
+  const int m_end = COPY ? (int)((long long)p.M * (blockIdx.y + 1) / gridDim.y) : min(p.M, m_begin + p.rows_per_block);
   for (int mb = m_begin; mb < m_end; mb += RB) {
     const int cnt = min(RB, m_end - mb);
     __syncthreads();
@@ -335,7 +337,8 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
           const float sc = half_scale(scale_exp);
           const float y[4] = {t[0] * sc, t[1] * sc, t[2] * sc, t[3] * sc};
           const float row = max3_abs(max3_abs(0.f, y[0], y[1]), y[2], y[3]);
-          check.run(row);
+          const unsigned row_max = __reduce_max_sync(in, __float_as_uint(row));
+          if (in == 0xffffffffu) check.run(__uint_as_float(row_max));
           largest = max3_abs(largest, row, row);
 #pragma unroll
           for (int j = 0; j < 4; ++j) col[j] = max3_abs(col[j], y[j], y[j]);
@@ -426,10 +429,11 @@ int launch_gemm_thin(const GemmArgs& g, float* scratch, cudaStream_t st) {
     p.A = g.A1; p.lda = g.lda1; p.B = g.B1; p.ldb = g.ldb1; p.e = make_epi(g);
     const int col_tiles = (g.N + 511) / 512;
     int row_blocks = (148 * 8 + col_tiles - 1) / col_tiles;
+    const bool copy = g.hout.p != nullptr;
+    if (copy && row_blocks > g.M / 16) row_blocks = g.M / 16 > 0 ? g.M / 16 : 1;
     if (row_blocks > g.M) row_blocks = g.M;
     p.rows_per_block = (g.M + row_blocks - 1) / row_blocks;
-    dim3 grid(col_tiles, (g.M + p.rows_per_block - 1) / p.rows_per_block);
-    const bool copy = g.hout.p != nullptr;
+    dim3 grid(col_tiles, copy ? row_blocks : (g.M + p.rows_per_block - 1) / p.rows_per_block);
     if (copy) {
       p.Dh = static_cast<__half*>(g.hout.p); p.ldh = g.hout.ld; p.hout = g.hout.info;
       p.hin[0] = g.h[0].info; p.hin[1] = g.h[1].info;

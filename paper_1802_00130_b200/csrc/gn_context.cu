@@ -128,10 +128,12 @@ struct gn_ctx {
     int info = 0;                                            // index into half_info
     bool valid = false, info_valid = false;                  // the copy, and its info, belong to what the matrix now holds
   };
-  enum HalfSet { kHZ, kHRZ, kHDS, kHZb, kHDb, kHW, kHV, kHF, kHalfSets };   // (kHZb[0]: the rows of X of a batch; kHF: factors)
+  enum HalfSet { kHZ, kHV, kHRZ, kHDS, kHZb, kHDb, kHW, kHF, kHalfSets };   // (kHV[0]: all of a vector, its scale; kHZb[0]: the rows of X of a batch; kHF: factors)
   std::vector<HalfBuf> half_buf[kHalfSets];
-  HalfInfo* half_info = nullptr; unsigned* half_acc = nullptr;
+  HalfInfo* half_info = nullptr; unsigned* half_acc = nullptr; unsigned long long* half_sums = nullptr;
   uint16_t* half_weights = nullptr; std::vector<int64_t> half_at;   // the copies of theta's weights, then of a vector's; where layer m's starts
+  struct HalfSums { int64_t v_rows, rows, cols; };
+  std::vector<HalfSums> half_sums_at; int64_t half_sums_v = 0, half_sums_n = 0;   // where a layer's sums are in half_sums: a vector's (the first half_sums_v), theta's
   int half_mode = 1;         // 0 never, 1 where a pass is large enough, 2 wherever it can be done
   bool half_usable = true;   // cleared if a copy's memory could not be had
   bool half_now = false;     // the pass in progress works with copies
@@ -638,7 +640,7 @@ void presplit(gn_ctx* c, const GemmArgs* gs, int n, unsigned roles) {
 // ---- FP16 copies ---------------------------------------------------------------------------------
 using HalfBuf = gn_ctx::HalfBuf;
 
-int half_info_index(const gn_ctx* c, int set, int m) { return set * (c->L + 1) + (set == gn_ctx::kHV ? 0 : m); }   // (one scale for all of v)
+int half_info_index(const gn_ctx* c, int set, int m) { return set * (c->L + 1) + m; }
 
 bool half_setup(gn_ctx* c) {
   if (c->half_info) return true;
@@ -646,8 +648,18 @@ bool half_setup(gn_ctx* c) {
   if (dev_alloc(c, &c->half_info, n) != GN_OK) return false;
   c->half_at.assign((size_t)c->L + 2, 0);
   for (int m = 1; m <= c->L; ++m) c->half_at[(size_t)m + 1] = c->half_at[(size_t)m] + c->w[m] * round8(c->w[m - 1]);
-  if (dev_alloc(c, &c->half_acc, (int64_t)kHalfSegs + 1) != GN_OK || dev_alloc(c, &c->half_weights, 2 * c->half_at.back()) != GN_OK) {
-    dev_free(c, c->half_acc); dev_free(c, c->half_info);
+  c->half_sums_at.assign((size_t)c->L + 1, {});
+  c->half_sums_n = 0;
+  for (int m = 1; m <= c->L; ++m) { c->half_sums_at[(size_t)m].v_rows = c->half_sums_n; c->half_sums_n += c->w[m]; }
+  c->half_sums_v = c->half_sums_n;
+  for (int m = 1; m <= c->L; ++m) {
+    c->half_sums_at[(size_t)m].rows = c->half_sums_n;
+    c->half_sums_at[(size_t)m].cols = c->half_sums_n + c->w[m];
+    c->half_sums_n += c->w[m] + c->w[m - 1];
+  }
+  if (dev_alloc(c, &c->half_acc, (int64_t)kHalfSegs + 1) != GN_OK || dev_alloc(c, &c->half_weights, 2 * c->half_at.back()) != GN_OK ||
+      dev_alloc(c, &c->half_sums, c->half_sums_n) != GN_OK) {
+    dev_free(c, c->half_weights); dev_free(c, c->half_acc); dev_free(c, c->half_info);
     return false;
   }
   cudaMemsetAsync(c->half_info, 0, sizeof(HalfInfo) * (size_t)n, c->st);
@@ -695,7 +707,7 @@ void half_drop(gn_ctx* c, int set) {
 void half_give_up(gn_ctx* c) {
   quiesce(c);
   for (int set = 0; set < gn_ctx::kHalfSets; ++set) half_drop(c, set);
-  dev_free(c, c->half_weights); dev_free(c, c->half_acc); dev_free(c, c->half_info);
+  dev_free(c, c->half_weights); dev_free(c, c->half_sums); dev_free(c, c->half_acc); dev_free(c, c->half_info);
   c->half_usable = false; c->half_now = false; ++c->dispatch_gen;
 }
 
@@ -755,14 +767,28 @@ void attach_half_out(const gn_ctx* c, GemmArgs& g, HalfBuf& b) {
 // Copies by passes of their own.  infos: one largest-magnitude job per scale; every matrix of `bufs` is then copied.  The infos
 // from `reset` on are cleared on the way.
 // (With no such job the infos hold what the matrices' writers have reported.)
-bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::vector<HalfBuf*>& bufs, int reset = 0, int n_reset = 0) {
+// set: kHW or kHV, whose copies' rows (and, of theta, columns) are summed as well: they bound what is computed from them.
+bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::vector<HalfBuf*>& bufs, int reset = 0, int n_reset = 0,
+                  int set = gn_ctx::kHalfSets) {
+  const bool theta = set == gn_ctx::kHW, vec = set == gn_ctx::kHV;
+  unsigned long long* const sums = c->half_sums + (theta ? c->half_sums_v : 0);
+  const int64_t n_sums = theta ? c->half_sums_n - c->half_sums_v : vec ? c->half_sums_v : 0;
   for (size_t i = 0; i < amax.size(); i += kHalfSegs) {
-    const int r = launch_half_amax(amax.data() + i, (int)std::min<size_t>(kHalfSegs, amax.size() - i), c->half_acc, c->half_info + reset, i == 0 ? n_reset : 0, c->st);
+    const int r = launch_half_amax(amax.data() + i, (int)std::min<size_t>(kHalfSegs, amax.size() - i), c->half_acc, c->half_info + reset, i == 0 ? n_reset : 0, sums, i == 0 ? n_sums : 0, c->st);
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "FP16 copies could not be made"; return false; }
     c->launches += r;
   }
   std::vector<HalfCopyJob> jobs;
-  for (HalfBuf* b : bufs) jobs.push_back(HalfCopyJob{b->base, b->rows, b->cols, (int64_t)b->cols, half_mat(c, *b), amax.empty()});
+  for (HalfBuf* b : bufs) {
+    HalfCopyJob j{b->base, b->rows, b->cols, (int64_t)b->cols, half_mat(c, *b), amax.empty()};
+    if (theta || vec) {
+      const gn_ctx::HalfSums& at = c->half_sums_at[(size_t)(b->info - half_info_index(c, set, 0))];
+      j.row_sums = c->half_sums + (theta ? at.rows : at.v_rows);
+      if (theta) j.col_sums = c->half_sums + at.cols;
+      if (vec) j.from = c->half_info + half_info_index(c, set, 0);
+    }
+    jobs.push_back(j);
+  }
   for (size_t i = 0; i < jobs.size(); i += kHalfSegs) {
     const int r = launch_half_copy(jobs.data() + i, (int)std::min<size_t>(kHalfSegs, jobs.size() - i), c->st);
     if (r < 0) { c->sticky = GN_ECUDA; c->err = "FP16 copies could not be made"; return false; }
@@ -816,7 +842,7 @@ void half_theta(gn_ctx* c) {
     amax.push_back(HalfAmaxJob{b.base, b.rows * b.cols, c->half_info + b.info});
     if (copy) bufs.push_back(&b);
   }
-  if (!half_convert(c, amax, bufs)) return;
+  if (!half_convert(c, amax, bufs, 0, 0, gn_ctx::kHW)) return;
   c->half_buf[gn_ctx::kHW][(size_t)c->L].info_valid = true;
   c->half_theta_epoch = c->theta_epoch;
 }
@@ -832,7 +858,8 @@ void half_vector(gn_ctx* c, const float* v) {
     bufs.push_back(&b);
   }
   const std::vector<HalfAmaxJob> amax{HalfAmaxJob{v, c->n, c->half_info + half_info_index(c, gn_ctx::kHV, 0)}};
-  half_convert(c, amax, bufs, half_info_index(c, gn_ctx::kHRZ, 0), 2 * (c->L + 1));
+  // (one scale for all of v: that of entry 0, which the layers' infos take over)
+  half_convert(c, amax, bufs, half_info_index(c, gn_ctx::kHV, 1), 3 * (c->L + 1) - 1, gn_ctx::kHV);
 }
 
 // A copy of one matrix that something else than a contraction with a copy of its own has written.
@@ -2388,6 +2415,17 @@ int32_t gn_debug_plan_group(int32_t n, const int32_t* M, const int32_t* N, const
                             int32_t* counts, int32_t* waves, int32_t* order, int32_t* tiles) {
   if (!M || !N || !K || !counts || !waves || !order || !tiles) return -1;
   return gemm_tf32_plan_group(n, M, N, K, pairs, keep_order, counts, waves, order, tiles);
+}
+
+gn_status gn_debug_copies(gn_ctx* c, int64_t* known, int64_t* refused) {
+  if (!c || !known || !refused) return GN_EINVAL;
+  *known = *refused = 0;
+  GN_TRY(sync(c, "copies"));
+  if (!c->half_info) return GN_OK;
+  std::vector<HalfInfo> host((size_t)gn_ctx::kHalfSets * (c->L + 1));
+  GN_CUDA(c, cudaMemcpy(host.data(), c->half_info, sizeof(HalfInfo) * host.size(), cudaMemcpyDeviceToHost));
+  for (const HalfInfo& i : host) { *known += i.amax != 0u; *refused += i.bad != 0u; }
+  return GN_OK;
 }
 
 gn_status gn_debug_check_canaries(gn_ctx* c, int64_t* n_checked) {

@@ -25,11 +25,15 @@ namespace gn {
 // which power of two, how large the matrix's largest magnitude is, and whether the copy may be used: `bad` is set by whoever
 // writes it when an element overflows, is infinite or NaN, or when a whole run of a row or of a column lies so low that FP16's
 // denormals would cost it precision (kHalfLeast).  The contraction kernels look at it and read the FP32 matrix instead.
-struct HalfInfo { int e; unsigned amax; unsigned bad; unsigned pad; };
+// row1, col1: largest sum of the magnitudes of a row and of a column, in units of 2^(-e - 4) (0: not known).
+struct alignas(16) HalfInfo { int e; unsigned amax; unsigned bad; unsigned pad; unsigned long long row1, col1; };
 // Copy of a matrix, stored with leading dimension ld (a multiple of 8, 16-byte aligned, followed by >= 128 readable bytes).
 struct HalfMat { void* p = nullptr; int64_t ld = 0; HalfInfo* info = nullptr; };
-// A run of elements of a row or column whose largest scaled magnitude is below this (and not zero) makes a copy bad: above it
-// the rounding of a denormal, at most 2^-25, stays below the 2^-12 by which rounding to 11 bits changes the run's largest element.
+// A run of elements of a row (32 or 128) or column (16, or more) whose largest scaled magnitude is below this (and not zero) makes
+// a copy bad: above it the rounding of a denormal, at most 2^-25, stays below the 2^-12 by which rounding to 11 bits changes the
+// run's largest element.  (Runs of 2 and 8 elements were too short: a few saturated neurons have them, and one run decides over a
+// whole matrix.  For the same reason what is left over at the end of a row or column, shorter than a run, is not judged by itself: the
+// row's or column's runs are.)
 constexpr float kHalfLeast = 1.220703125e-4f;   // 2^-13
 
 struct GemmArgs {
@@ -95,13 +99,18 @@ double gemm_tf32_group_makespan(int n, const int* M, const int* N, const int* K,
 
 // FP16 copies by passes of their own (half_copy.cu), at most kHalfSegs matrices a launch.  launch_half_amax starts an info
 // afresh from the largest magnitude of `count` consecutive floats and clears the n_reset infos from `reset` on; acc:
-// kHalfSegs + 1 words, zero before the first launch and after every one.  launch_half_copy writes the copies and marks the bad
-// ones.  Both return launches made, or -1.
+// kHalfSegs + 1 words, zero before the first launch and after every one; the n_sums words from `sums` on are cleared as well.
+// launch_half_copy writes the copies and marks the bad ones.  Both return launches made, or -1.
 constexpr int kHalfSegs = 8;
 struct HalfAmaxJob { const float* src; int64_t count; HalfInfo* info; };
 // fresh: the info holds the largest magnitude alone (whoever wrote the matrix has reported it): the scale is said here.
-struct HalfCopyJob { const float* src; int64_t rows; int cols; int64_t ld; HalfMat out; bool fresh = false; };
-int launch_half_amax(const HalfAmaxJob* jobs, int n, unsigned* acc, HalfInfo* reset, int n_reset, cudaStream_t st);
+// from: the info that has the scale, if it is not the copy's own (which is told scale and largest magnitude then).  row_sums,
+// col_sums: `rows` and `cols` words, zero: the sums of magnitudes are formed there, the largest goes into the info.
+struct HalfCopyJob {
+  const float* src; int64_t rows; int cols; int64_t ld; HalfMat out; bool fresh = false;
+  const HalfInfo* from = nullptr; unsigned long long* row_sums = nullptr; unsigned long long* col_sums = nullptr;
+};
+int launch_half_amax(const HalfAmaxJob* jobs, int n, unsigned* acc, HalfInfo* reset, int n_reset, unsigned long long* sums, int64_t n_sums, cudaStream_t st);
 int launch_half_copy(const HalfCopyJob* jobs, int n, cudaStream_t st);
 
 // FP32-accurate contraction on the FP16 tensor cores (gemm_f16x3.cu): any shape and alignment, because it reads

@@ -25,6 +25,10 @@ __device__ __forceinline__ float max3_abs(float a, float b, float c) {
   return d;
 }
 
+// A sum of magnitudes that an info has in units of 2^(-e - kHalfNormExp).
+constexpr int kHalfNormExp = 4;
+__device__ __forceinline__ float half_norm(unsigned long long units, int e) { return (float)units * half_scale(-kHalfNormExp) * half_scale(-e); }
+
 // Collects what decides whether a copy may be used, from the largest scaled magnitudes of runs of a row or column.
 struct HalfCheck {
   unsigned low = 0xffffffffu, high = 0u;     // smallest that is not zero (less one: zeros wrap to the largest), and largest
@@ -33,6 +37,7 @@ struct HalfCheck {
     low = min(low, b - 1u);
     high = max(high, b);
   }
+  __device__ __forceinline__ bool low_run() const { return low < __float_as_uint(kHalfLeast) - 1u; }
   __device__ __forceinline__ bool bad() const { return low < __float_as_uint(kHalfLeast) - 1u || high > __float_as_uint(65504.f); }
 };
 

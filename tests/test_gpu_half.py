@@ -241,6 +241,41 @@ def test_copies_and_memory_that_changes_hands():
     c.close()
 
 
+@pytest.mark.parametrize("theta,outlier,rows", [("sparse", 0.0, 1104), ("sparse", 0.0, 1105), ("dense", 0.0, 1105), ("dense", 8.0, 1100), ("dense", 64.0, 1100)])
+def test_copies_hold_ordinary_networks(theta, outlier, rows):
+    """The initialisation of the paper (a few weights of order one per neuron, saturated neurons), and single large weights: no
+    copy is refused, and results are those without copies."""
+    p = wl.make_custom([392, 1000, 1000, 1000, 10], l=1501, nS=rows, C=15.0, seed=79, x="sparse80", theta=theta)
+    w, th, C, v = p["widths"], p["theta"], p["C"], p["v"]
+    for m, (w_off, _, _) in enumerate(wl.layer_offsets(w), 1):
+        if outlier and 2 <= m < 4:
+            th[w_off + 7 * w[m - 1] + 11] = outlier
+    XS = p["X"][p["idx"]]
+    refs = [orc.Gv(th, w, C, XS, v), orc.Gv_blockdiag(th, w, C, XS, v), orc.grad(th, w, C, p["X"], p["Y"])]
+    c = make_ctx(p, "tf32")
+    c.debug_option(11, 2)
+    c.set_blockdiag_method(2)
+    c.set_subsample(dev(p["idx"]))
+    for call, ref in zip((lambda: c.Gv(dev(v)), lambda: c.Gv_blockdiag(dev(v)), c.grad), refs):
+        got = call().cpu().numpy()
+        known, refused = c.debug_copies()
+        assert known >= 6 and (refused == 0 or outlier > 8.0)       # (64 saturates a neuron: its column lies low as a whole)
+        assert relb(got, ref, w) <= TOL["tf32"]
+    c.close()
+
+
+def test_a_copy_that_cannot_hold_its_matrix_is_refused():
+    """Far features (1e-12 of the others): the copy of X_S loses them, and is refused."""
+    p = wl.make_custom([260, 392, 264, 10], l=1500, nS=1100, C=15.0, seed=57, x="uniform")
+    p["X"][:, 5] *= np.float32(1e-12)
+    c = make_ctx(p, "tf32")
+    c.debug_option(11, 2)
+    c.set_subsample(dev(p["idx"]))
+    c.Gv(dev(p["v"]))
+    assert c.debug_copies()[1] == 1
+    c.close()
+
+
 @pytest.mark.parametrize("widths", [[392] * 4 + [10], [520] * 3 + [10]])
 def test_a_place_ends_with_its_pass(widths):
     """Row batches' buffers are let go and the subsample's got in their place, in sizes that meet at the same addresses now and
