@@ -215,20 +215,26 @@ gn_status cuda_fail(gn_ctx* c, cudaError_t e, const char* where) {
   } while (0)
 
 constexpr int kCanaryByte = 0xA5;
+bool half_release(gn_ctx* c);
 
 template <class T>
 gn_status dev_alloc(gn_ctx* c, T** p, int64_t count) {
   *p = nullptr;
   if (count <= 0) count = 1;
-  if (c->fail_alloc_in > 0 && --c->fail_alloc_in == 0)
-    return fail(c, GN_ENOMEM, std::string("device allocation of ") + std::to_string(count * (int64_t)sizeof(T)) + " bytes refused (injected)");
   void* q = nullptr;
-  // 256 bytes of slack: the tensor-core kernel's 3-D TMA boxes may read up to 124 bytes past the last
-  // row of an MN-major operand
-  cudaError_t e = cudaMalloc(&q, (size_t)count * sizeof(T) + 256);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(c, GN_ENOMEM, std::string("cudaMalloc of ") + std::to_string(count * (int64_t)sizeof(T)) + " bytes: " + cudaGetErrorString(e));
+  for (;;) {
+    std::string why;
+    if (c->fail_alloc_in > 0 && --c->fail_alloc_in == 0) {
+      why = "device allocation of " + std::to_string(count * (int64_t)sizeof(T)) + " bytes refused (injected)";
+    } else {
+      // 256 bytes of slack: the tensor-core kernel's 3-D TMA boxes may read up to 124 bytes past the last
+      // row of an MN-major operand
+      const cudaError_t e = cudaMalloc(&q, (size_t)count * sizeof(T) + 256);
+      if (e == cudaSuccess) break;
+      cudaGetLastError();
+      why = "cudaMalloc of " + std::to_string(count * (int64_t)sizeof(T)) + " bytes: " + cudaGetErrorString(e);
+    }
+    if (!half_release(c)) return fail(c, GN_ENOMEM, why);      // (FP16 copies make room for what is needed)
   }
   // the last 128 bytes of the slack are a canary: nothing of the library may write there (gn_debug_check_canaries)
   if (cudaMemset(static_cast<char*>(q) + (size_t)count * sizeof(T) + 128, kCanaryByte, 128) != cudaSuccess) {
@@ -677,10 +683,10 @@ uint16_t* half_lender(const gn_ctx* c, int set, int m) {
   return reinterpret_cast<uint16_t*>(set == gn_ctx::kHRZ ? c->DS[(size_t)m] : set == gn_ctx::kHDS ? c->RZ[(size_t)m] : nullptr);
 }
 
-// Room for a copy of a rows x cols matrix at `base`.
-bool half_reserve(gn_ctx* c, HalfBuf& b, int set, int m, const float* base, int64_t rows, int cols, int64_t cap_rows) {
+// Room for a copy of a rows x cols matrix at `base` (copy: it will have one, and not an info alone).
+bool half_reserve(gn_ctx* c, HalfBuf& b, int set, int m, const float* base, int64_t rows, int cols, int64_t cap_rows, bool copy = true) {
   if (!half_setup(c)) return false;
-  const int64_t need = std::max(rows, cap_rows) * round8(cols);
+  const int64_t need = copy ? std::max(rows, cap_rows) * round8(cols) : 0;
   if (uint16_t* lent = half_lender(c, set, m)) {
     b.p = lent;
   } else if (need > b.cap) {
@@ -703,12 +709,27 @@ void half_drop(gn_ctx* c, int set) {
     b.p = nullptr; b.cap = 0; b.base = nullptr; b.valid = b.info_valid = false;
   }
 }
-// No room: the passes go on without copies.
+// No room: the passes go on without copies until the next subsample, whose memory may be another.
 void half_give_up(gn_ctx* c) {
   quiesce(c);
   for (int set = 0; set < gn_ctx::kHalfSets; ++set) half_drop(c, set);
   dev_free(c, c->half_weights); dev_free(c, c->half_sums); dev_free(c, c->half_acc); dev_free(c, c->half_info);
-  c->half_usable = false; c->half_now = false; ++c->dispatch_gen;
+  c->half_usable = false; c->half_now = false; c->half_theta_epoch = 0; ++c->dispatch_gen;
+}
+// Something that a call cannot do without has found no room: whether copies could be let go for it.  (Not inside a pass with
+// copies, whose operands point to them: or_without_copies is for that.)
+bool half_release(gn_ctx* c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (!c->half_info || c->half_now) return false;
+  if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  half_give_up(c);
+  return true;
+}
+// A pass, and once more without copies if it has run out of memory with them.
+template <class Pass>
+gn_status or_without_copies(gn_ctx* c, Pass pass) {
+  const gn_status s = pass();
+  return s == GN_ENOMEM && half_release(c) ? pass() : s;
 }
 
 HalfMat half_mat(const gn_ctx* c, const HalfBuf& b) {
@@ -866,7 +887,7 @@ void half_vector(gn_ctx* c, const float* v) {
 void half_matrix(gn_ctx* c, int set, int m, const float* base, int64_t rows, int cols, int64_t cap_rows, bool copy, int reset = 0, int n_reset = 0) {
   if (!c->half_now) return;
   HalfBuf& b = c->half_buf[set][(size_t)m];
-  if (!half_reserve(c, b, set, m, base, rows, cols, copy ? cap_rows : 0)) { half_give_up(c); return; }
+  if (!half_reserve(c, b, set, m, base, rows, cols, cap_rows, copy)) { half_give_up(c); return; }
   std::vector<HalfBuf*> bufs;
   if (copy) bufs.push_back(&b);
   if (half_convert(c, {HalfAmaxJob{base, rows * cols, c->half_info + b.info}}, bufs, reset, n_reset)) b.info_valid = true;
@@ -1236,7 +1257,7 @@ void half_top_delta(gn_ctx* c, int set, const std::vector<float*>& deltas, int64
 }
 
 // out = coef v + (1/|S|) J^T (2 J v) over the stored subsample (Eq. sampled-Gauss).
-gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
+gn_status product_full_pass(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("G v");
   SmallNet small;
   if (small_pass(c, kSmallGv, c->nS, &small)) {
@@ -1294,6 +1315,9 @@ gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
     GN_TRY(backward_hidden_layers(c, L - 1, c->DS[L - 1], zprev, c->DS, nS, inv, v, coef, out, nS, true));
   }
   return check_launch(c, "G v");
+}
+gn_status product_full(gn_ctx* c, const float* v, float* out, float coef) {
+  return or_without_copies(c, [&] { return product_full_pass(c, v, out, coef); });
 }
 
 // Eq. (approx-jaco), one block per layer.  The perturbation of layer k is pushed to the output and
@@ -1389,7 +1413,15 @@ gn_status ensure_factors(gn_ctx* c) {
   c->launches += launch_factor_last(Wm(c, c->theta, L), c->Z[L - 1], nS, nL, c->w[L - 1], c->DF[L - 1], c->st);
   HalfPass half_guard(c, L >= 3 && half_wanted(c, nS * nL));
   half_theta(c);
-  if (L >= 3 && c->w[L - 1] >= 128)
+  // (the factors' copies are the largest: where they find no room the recurrence goes on without, and the other copies stay)
+  const auto room = [&](int m) {
+    if (half_reserve(c, c->half_buf[gn_ctx::kHF][(size_t)m], gn_ctx::kHF, m, c->DF[m], nS * nL, c->w[m], 0)) return true;
+    quiesce(c);
+    half_drop(c, gn_ctx::kHF);
+    c->half_now = false;
+    return false;
+  };
+  if (L >= 3 && c->w[L - 1] >= 128 && c->half_now && room(L - 1))
     half_matrix(c, gn_ctx::kHF, L - 1, c->DF[L - 1], nS * nL, c->w[L - 1], 0, true, half_info_index(c, gn_ctx::kHF, 0), L - 1);
   for (int m = L - 1; m >= 2; --m) {
     GemmArgs g;
@@ -1402,9 +1434,8 @@ gn_status ensure_factors(gn_ctx* c) {
     g.mn_padded = true;
     attach_half(c, g);
     if (m - 1 >= 2 && c->half_now && c->w[m - 1] >= 128 && c->w[m - 1] % 4 == 0) {
-      HalfBuf& b = c->half_buf[gn_ctx::kHF][(size_t)m - 1];
-      if (half_reserve(c, b, gn_ctx::kHF, m - 1, c->DF[m - 1], nS * nL, c->w[m - 1], 0)) attach_half_out(c, g, b);
-      else { half_give_up(c); g.half = false; }
+      if (room(m - 1)) attach_half_out(c, g, c->half_buf[gn_ctx::kHF][(size_t)m - 1]);
+      else g.half = false;
     }
     run_gemm(c, g);
   }
@@ -1614,7 +1645,7 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
 // asked for on the same (theta, S), counting the one at hand; after that every product uses them.
 constexpr int kFactorBreakEven = 8;
 
-gn_status product_blockdiag_any(gn_ctx* c, const float* v, float* out, float coef) {
+gn_status product_blockdiag_pass(gn_ctx* c, const float* v, float* out, float coef) {
   GN_PHASE("block-diagonal G v");
   if (c->has_split) return product_split(c, v, out, coef);
   SmallNet small;
@@ -1630,6 +1661,9 @@ gn_status product_blockdiag_any(gn_ctx* c, const float* v, float* out, float coe
   if (stored && c->L >= 2 && c->w[c->L] <= 16) return product_blockdiag_stored(c, v, out, coef);
   ++c->bd_count;
   return product_blockdiag(c, v, out, coef);
+}
+gn_status product_blockdiag_any(gn_ctx* c, const float* v, float* out, float coef) {
+  return or_without_copies(c, [&] { return product_blockdiag_pass(c, v, out, coef); });
 }
 
 gn_status ensure_batch(gn_ctx* c) {
@@ -1656,7 +1690,7 @@ gn_status read_loss(gn_ctx* c, double* f_host) {
 }
 
 // f and (optionally) the gradient over all rows in row batches (Section 6.1 in its one-GPU form).
-gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
+gn_status fun_grad_pass(gn_ctx* c, float* d_grad, double* f_host) {
   GN_PHASE("f / gradient");
   SmallNet small;
   if (small_pass(c, d_grad ? kSmallGrad : kSmallFun, c->l, &small)) {
@@ -1723,6 +1757,9 @@ gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
     return read_loss(c, f_host);
   }
   return check_launch(c, "grad");
+}
+gn_status fun_grad(gn_ctx* c, float* d_grad, double* f_host) {
+  return or_without_copies(c, [&] { return fun_grad_pass(c, d_grad, f_host); });
 }
 
 gn_status ensure_tmp(gn_ctx* c) {
@@ -1985,9 +2022,8 @@ gn_status gn_set_theta_host(gn_ctx* c, const float* h_theta) {
   return GN_OK;
 }
 
-static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, cudaMemcpyKind kind) {
+static gn_status set_subsample_pass(gn_ctx* c, const int32_t* idx, int64_t nS, cudaMemcpyKind kind) {
   GN_PHASE("set_subsample");
-  if (!c) return GN_EINVAL;
   if (!idx) return fail(c, GN_EINVAL, "idx is NULL");
   if (nS < 1) return fail(c, GN_EINVAL, "the subsample must have at least one row");
   if (!c->have_theta) return fail(c, GN_ESTATE, "theta has not been set");
@@ -2033,6 +2069,12 @@ static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, c
   if (*c->h_err) return fail(c, GN_EINVAL, "a subsample index lies outside [0, l)");
   c->have_sub = true;
   return GN_OK;
+}
+
+static gn_status set_subsample_impl(gn_ctx* c, const int32_t* idx, int64_t nS, cudaMemcpyKind kind) {
+  if (!c) return GN_EINVAL;
+  if (!c->half_usable) { c->half_usable = true; ++c->dispatch_gen; }
+  return or_without_copies(c, [&] { return set_subsample_pass(c, idx, nS, kind); });
 }
 
 gn_status gn_set_subsample(gn_ctx* c, const int32_t* d_idx, int64_t nS) {

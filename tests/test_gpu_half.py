@@ -276,6 +276,33 @@ def test_a_copy_that_cannot_hold_its_matrix_is_refused():
     c.close()
 
 
+def test_copies_make_room_for_what_a_call_cannot_do_without():
+    """One allocation refused at a time, on the host, in contexts that hold copies: what a pass needs gets the room of the copies,
+    a copy without room is done without, and the next subsample has copies again.  No call fails."""
+    p = wl.make_custom([260, 392, 520, 264, 10], l=1500, nS=1100, C=15.0, seed=81, x="sparse80")
+    w, th, C, v = p["widths"], p["theta"], p["C"], dev(p["v"])
+    XS, idx = p["X"][p["idx"]], dev(p["idx"])
+    refs = dict(Gv=orc.Gv(th, w, C, XS, p["v"]), block=orc.Gv_blockdiag(th, w, C, XS, p["v"]), grad=orc.grad(th, w, C, p["X"], p["Y"]))
+    calls = dict(Gv=lambda c: c.Gv(v), block=lambda c: c.Gv_blockdiag(v), grad=lambda c: c.grad())
+    for name, call in calls.items():
+        for n in range(1, 12):
+            c = make_ctx(p, "tf32")
+            c.debug_option(11, 2)
+            c.set_blockdiag_method(2)
+            c.set_subsample(idx)
+            c.debug_option(2, n)
+            got = call(c).cpu().numpy()
+            c.debug_option(2, 0)
+            assert relb(got, refs[name], w) <= TOL["tf32"]
+            for other, again in calls.items():
+                assert relb(again(c).cpu().numpy(), refs[other], w) <= TOL["tf32"]
+            c.set_subsample(idx)
+            for other, again in calls.items():
+                assert relb(again(c).cpu().numpy(), refs[other], w) <= TOL["tf32"]
+            assert c.debug_copies()[0] > 0
+            c.close()
+
+
 @pytest.mark.parametrize("widths", [[392] * 4 + [10], [520] * 3 + [10]])
 def test_a_place_ends_with_its_pass(widths):
     """Row batches' buffers are let go and the subsample's got in their place, in sizes that meet at the same addresses now and
