@@ -88,6 +88,7 @@ struct gn_ctx {
   int chain_level = 1;
   bool split_k_enabled = true; // weight blocks of the stored-factor product as two chained parts of the rows
   int64_t cut_for_nS = -1, cut_rows = 0;   // rows of the first part, chosen once per subsample size
+  bool cut_for_half = false;                 // ... and kind of operands
   bool fly_enabled = true;                 // last hidden layer's factor formed on the fly in the stored-factor product
   int back_chain = 2;                      // hidden layers of a backward pass as one chained launch: 0 never, 1 always, 2 where it pays
   int* chain_ctr = nullptr; int64_t chain_ctr_cap = 0;   // finished-tile counters of such a launch
@@ -1510,7 +1511,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
     int dep[2 * kGroup], dep_all[2 * kGroup];
     int n = 0;
     const int nl = L - 1;                                     // the hidden layers' blocks (the n_L-row block is a streaming kernel)
-    if (c->cut_for_nS != nS) {
+    if (c->cut_for_nS != nS || c->cut_for_half != c->half_now) {
       double best = -1.0;
       for (int eighths = 4; eighths <= 6; ++eighths) {
         const int64_t r = (nS * eighths / 8 + 63) / 64 * 64;  // first part: a whole number of k-blocks
@@ -1525,7 +1526,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
         if (t >= 0.0 && (best < 0.0 || t < best)) { best = t; c->cut_rows = r; }
       }
       if (best < 0.0) c->cut_rows = (nS / 2 + 63) / 64 * 64;
-      c->cut_for_nS = nS;
+      c->cut_for_nS = nS; c->cut_for_half = c->half_now;
     }
     const int64_t h0 = c->cut_rows;
     for (int part = 0; part < 2; ++part)
