@@ -1476,7 +1476,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   // the stored copy being needed only as the operand of the recurrence that builds the factors below it)
   for (int m = 1; m < L; ++m) {
     int done = 0;
-    HalfInfo* const info = c->half_now ? c->half_info + half_info_index(c, gn_ctx::kHDS, m) : nullptr;
+    HalfInfo* const info = c->half_now && factor_apply_reports(nL, c->w[m]) ? c->half_info + half_info_index(c, gn_ctx::kHDS, m) : nullptr;
     if (m == L - 1 && c->fly_enabled)
       done = launch_factor_apply_last(Wm(c, c->theta, L), c->Z[L - 1], c->RZ[m], nS, nL, c->w[m], c->DS[m], info, c->st);
     if (!done) done = launch_factor_apply(c->DF[m], c->RZ[m], nS, nL, c->w[m], 1, 1, 0, c->DS[m], info, c->st);
@@ -1485,7 +1485,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   if (c->half_now) {
     std::vector<HalfBuf*> bufs;
     for (int m = 1; m < L && c->half_now; ++m) {
-      if (c->w[m] <= 128 || c->w[m] % 4 != 0 || c->w[m - 1] < 128 || c->w[m - 1] % 4 != 0) continue;
+      if (c->w[m] <= 128 || c->w[m] % 4 != 0 || c->w[m - 1] < 128 || c->w[m - 1] % 4 != 0 || !factor_apply_reports(nL, c->w[m])) continue;
       HalfBuf& b = c->half_buf[gn_ctx::kHDS][(size_t)m];
       if (!half_reserve(c, b, gn_ctx::kHDS, m, c->DS[m], nS, c->w[m], c->capS)) { half_give_up(c); break; }
       bufs.push_back(&b);
@@ -1589,7 +1589,7 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     const int sa = c->split[m - 1], sb = c->split[m], np = c->w[m - 1], nm = c->w[m];
     const int64_t stride = nS * nm;
     // (the copy of the layer's results lies in R z^m's memory, which has room for two streams' in FP16)
-    const bool copy = c->half_now && m < L && sa <= 2 && nm > 128 && nm % 8 == 0;
+    const bool copy = c->half_now && m < L && sa <= 2 && nm > 128 && nm % 8 == 0 && factor_apply_reports(nL, (nm + sb - 1) / sb);
     for (int a = 0; a < sa; ++a) {
       const int t0 = group_lo(np, sa, a), t1 = group_lo(np, sa, a + 1);
       GemmArgs g;

@@ -200,6 +200,10 @@ int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL
 // every stream a (U and Q hold `streams` matrices [rows][n], stream_stride floats apart):
 //   p_u = sum_{j in T_b} D[(i,u)][j] U_a[i][j];  Q_a[i][j] = 2 sum_u D[(i,u)][j] p_u for j in T_b
 // (Eqs. direct-JV-cost, JTv; B = 2I).  n_L <= 32.  info (may be null): its amax is raised to Q's largest magnitude.
+// factor_apply_reports: whether asking for it costs less than the copies save (columns of the widest group).  Not where the general form
+// has n_L above 10: fewer registers, more samples in flight, D out of L2 (512-3000-3000-16 at 4000 rows, a product with copies
+// and without: 1156 and 1106 us, 1395 and 1188 split in two; with n_L = 10 700 and 727).
+inline bool factor_apply_reports(int nL, int widest) { return nL <= 10 || widest <= 1024; }
 int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, int n, int groups, int streams,
                         int64_t stream_stride, float* Q, HalfInfo* info, cudaStream_t st);
 int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U, int64_t rows, int nL, int n, float* Q,

@@ -237,16 +237,20 @@ __global__ void __launch_bounds__(256) factor_last_kernel(const float* __restric
 // `stream_stride` floats apart in U and Q, share them.  Pass 1 forms p_u = D_i[u][T_b] . U_i[T_b] (block
 // reduction per u), pass 2 re-reads D_i (just read, so from cache) and writes Q_i[j] = 2 sum_u D_i[u][j] p_u.
 // NLMAX bounds n_L.  With groups = 1 and streams = 1 this is the product of a whole layer block.
-template <int NLMAX>
+// REPORT: `info` is told the largest magnitude.  The loops are not unrolled: how many samples are in flight decides whether pass 2
+// finds D_i in L2, and the compiler's choices went both ways with every change (TF32 products through stored factors, us, before the
+// report / with a report that was tested at run time / now: 513-3001-3001-10 at 4000 rows 1253 / 1007 / 1018, 200-350-750-351-10 at
+// 3000 334 / 280 / 255, 30-950-600-3550-16 at 17796 3824 / 3958 / 3818, 144-50-100-2300-50-16 at 3817 588 / 626 / 588).
+template <int NLMAX, bool REPORT>
 __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restrict__ D, const float* __restrict__ U,
                                                            int nL, int n, int groups, int streams, long long stream_stride,
                                                            float* __restrict__ Q, HalfInfo* info) {
   grid_dep_wait();
   grid_dep_launch();
   D = dep(D); U = dep(U); Q = dep(Q); info = dep(info);
-  float largest = 0.f;
+  unsigned largest = 0u;                                     // (as bits: NaN is the largest of all)
   __shared__ unsigned seen;
-  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
+  if (REPORT && threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   __shared__ float red[8][NLMAX];
   __shared__ float pu[NLMAX];
   const long long i = blockIdx.x;
@@ -259,6 +263,7 @@ __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restri
     float acc[NLMAX];
 #pragma unroll
     for (int u = 0; u < NLMAX; ++u) acc[u] = 0.f;
+#pragma unroll 1
     for (int j = col0 + threadIdx.x; j < col1; j += 256) {
       const float uj = __ldg(u_row + j);
 #pragma unroll
@@ -278,16 +283,17 @@ __global__ void __launch_bounds__(256) factor_apply_kernel(const float* __restri
       pu[threadIdx.x] = 2.f * s;                              // B = 2I
     }
     __syncthreads();
+#pragma unroll 1
     for (int j = col0 + threadIdx.x; j < col1; j += 256) {
       float q = 0.f;
 #pragma unroll
       for (int u = 0; u < NLMAX; ++u)
         if (u < nL) q = fmaf(__ldg(d + (long long)u * n + j), pu[u], q);
-      largest = max3_abs(largest, q, q);
+      if (REPORT) largest = max(largest, magnitude(q));
       q_row[j] = q;
     }
   }
-  report_amax(info, seen, largest);
+  if (REPORT) report_amax(info, seen, __uint_as_float(largest));
 }
 
 // ---------------------------------------------------------------------------------- CG
@@ -562,7 +568,7 @@ int launch_sum_partials(const double* partial, int count, double* out, bool accu
 // Register-resident form for groups of at most 1024 * STRIPS columns (n and every group boundary multiples
 // of 4): every thread keeps its n_L x 4 x STRIPS slice of D_i in registers across the passes and the streams,
 // so D is read exactly once.
-template <int NLMAX, int STRIPS>
+template <int NLMAX, int STRIPS, bool REPORT>
 __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __restrict__ D, const float* __restrict__ U,
                                                                int nL, int n, int groups, int streams,
                                                                long long stream_stride, float* __restrict__ Q, HalfInfo* info) {
@@ -577,7 +583,7 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float largest = 0.f;
   __shared__ unsigned seen;
-  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
+  if (REPORT && threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   float4 dv[STRIPS][NLMAX];
 #pragma unroll
   for (int s = 0; s < STRIPS; ++s) {
@@ -625,21 +631,22 @@ __global__ void __launch_bounds__(256) factor_apply_reg_kernel(const float* __re
           q.x = fmaf(dv[s][u].x, pv, q.x); q.y = fmaf(dv[s][u].y, pv, q.y);
           q.z = fmaf(dv[s][u].z, pv, q.z); q.w = fmaf(dv[s][u].w, pv, q.w);
         }
-        largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
+        if (REPORT) largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
         *reinterpret_cast<float4*>(q_row + j) = q;
       }
     }
   }
-  report_amax(info, seen, largest);
+  if (REPORT) report_amax(info, seen, largest);
 }
 
 // The same for the last hidden layer, whose factor has the closed form D_i[u][t] = W^L[u][t] * z (1 - z) (what factor_last_kernel
 // stores), one group and one stream: formed here, with the same two multiplications, instead of being streamed from memory (the
 // same bits).  Blocks stay and take sample after sample, W^L in their registers: with a block per sample the 80 KB of W^L at
 // n_L = 10, n = 2000 came from L2 for every sample and bounded it (12000 samples: 124 us, now 82).  What bounds it now is its
-// FMAs and the two barriers per sample, behind which the next sample's rows are already on their way.
-template <int NLMAX, int STRIPS>
-__global__ void __launch_bounds__(256, NLMAX * STRIPS <= 16 ? 2 : 1) factor_apply_fly_kernel(const float* __restrict__ WL, const float* __restrict__ Zprev,
+// FMAs and the two barriers per sample, behind which the next sample's rows are already on their way.  (Two blocks per SM at n_L
+// above 10 need more registers than there are: 88 bytes of spills, 784-1000-16 at 12000 rows 266 us instead of 260 a product.)
+template <int NLMAX, int STRIPS, bool REPORT>
+__global__ void __launch_bounds__(256, NLMAX * STRIPS <= 10 ? 2 : 1) factor_apply_fly_kernel(const float* __restrict__ WL, const float* __restrict__ Zprev,
                                                                   const float* __restrict__ U, long long rows, int nL, int n,
                                                                   float* __restrict__ Q, HalfInfo* info) {
   grid_dep_wait();
@@ -650,7 +657,7 @@ __global__ void __launch_bounds__(256, NLMAX * STRIPS <= 16 ? 2 : 1) factor_appl
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float largest = 0.f;
   __shared__ unsigned seen;
-  if (threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
+  if (REPORT && threadIdx.x == 0) seen = seen_amax(info);              // (there are barriers before it is used)
   float4 wv[STRIPS][NLMAX], z[STRIPS], x[STRIPS];
 #pragma unroll
   for (int s = 0; s < STRIPS; ++s) {
@@ -710,12 +717,12 @@ __global__ void __launch_bounds__(256, NLMAX * STRIPS <= 16 ? 2 : 1) factor_appl
           q.x = fmaf(wv[s][u].x * ds[s].x, pv, q.x); q.y = fmaf(wv[s][u].y * ds[s].y, pv, q.y);
           q.z = fmaf(wv[s][u].z * ds[s].z, pv, q.z); q.w = fmaf(wv[s][u].w * ds[s].w, pv, q.w);
         }
-        largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
+        if (REPORT) largest = max3_abs(max3_abs(largest, q.x, q.y), q.z, q.w);
         *reinterpret_cast<float4*>(Q + i * n + j) = q;
       }
     }
   }
-  report_amax(info, seen, largest);
+  if (REPORT) report_amax(info, seen, largest);
 }
 
 int launch_factor_last(const float* WL, const float* Zprev, int64_t rows, int nL, int n, float* D, cudaStream_t st) {
@@ -735,17 +742,17 @@ int launch_factor_apply(const float* D, const float* U, int64_t rows, int nL, in
   }
   const dim3 grid((unsigned)rows, (unsigned)groups);
   const long long ss = stream_stride;
-#define GN_FA_REG(NL, STR) { launch_pdl_grid(factor_apply_reg_kernel<NL, STR>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info); return 1; }
+#define GN_FA_REG(NL, STR) { launch_pdl_grid(info ? factor_apply_reg_kernel<NL, STR, true> : factor_apply_reg_kernel<NL, STR, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info); return 1; }
   if (vec && widest <= 1024 && nL <= 4)  GN_FA_REG(4, 1)
   if (vec && widest <= 1024 && nL <= 10) GN_FA_REG(10, 1)
   if (vec && widest <= 2048 && nL <= 4)  GN_FA_REG(4, 2)
   if (vec && widest <= 2048 && nL <= 10) GN_FA_REG(10, 2)
   if (vec && widest <= 1024 && nL <= 16) GN_FA_REG(16, 1)
 #undef GN_FA_REG
-  if (nL <= 4) launch_pdl_grid(factor_apply_kernel<4>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
-  else if (nL <= 10) launch_pdl_grid(factor_apply_kernel<10>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
-  else if (nL <= 16) launch_pdl_grid(factor_apply_kernel<16>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
-  else launch_pdl_grid(factor_apply_kernel<32>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  if (nL <= 4) launch_pdl_grid(info ? factor_apply_kernel<4, true> : factor_apply_kernel<4, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else if (nL <= 10) launch_pdl_grid(info ? factor_apply_kernel<10, true> : factor_apply_kernel<10, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else if (nL <= 16) launch_pdl_grid(info ? factor_apply_kernel<16, true> : factor_apply_kernel<16, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
+  else launch_pdl_grid(info ? factor_apply_kernel<32, true> : factor_apply_kernel<32, false>, dim3(grid), 256, 0, st, D, U, nL, n, groups, streams, ss, Q, info);
   return 1;
 }
 
@@ -757,7 +764,7 @@ int launch_factor_apply_last(const float* WL, const float* Zprev, const float* U
                    ((reinterpret_cast<uintptr_t>(U) & 15) == 0) && ((reinterpret_cast<uintptr_t>(Q) & 15) == 0);
   if (!vec) return 0;
   // (as many blocks as are resident: two per SM where W^L and the products with it leave the registers for that)
-#define GN_FA_FLY(NL, STR) { const long long blocks = (NL * STR <= 16 ? 2LL : 1LL) * num_sms(); const dim3 grid((unsigned)(rows < blocks ? rows : blocks), 1); launch_pdl_grid(factor_apply_fly_kernel<NL, STR>, dim3(grid), 256, 0, st, WL, Zprev, U, rows, nL, n, Q, info); return 1; }
+#define GN_FA_FLY(NL, STR) { const long long blocks = (NL * STR <= 10 ? 2LL : 1LL) * num_sms(); const dim3 grid((unsigned)(rows < blocks ? rows : blocks), 1); launch_pdl_grid(info ? factor_apply_fly_kernel<NL, STR, true> : factor_apply_fly_kernel<NL, STR, false>, dim3(grid), 256, 0, st, WL, Zprev, U, rows, nL, n, Q, info); return 1; }
   if (n <= 1024 && nL <= 4)  GN_FA_FLY(4, 1)
   if (n <= 1024 && nL <= 10) GN_FA_FLY(10, 1)
   if (n <= 2048 && nL <= 4)  GN_FA_FLY(4, 2)
