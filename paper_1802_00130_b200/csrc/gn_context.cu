@@ -822,19 +822,34 @@ bool half_convert(gn_ctx* c, const std::vector<HalfAmaxJob>& amax, const std::ve
 
 // Layers whose weights are an operand of a contraction that suits_half.
 bool half_layer(const gn_ctx* c, int m) { return c->w[m] >= 128 && c->w[m] % 4 == 0 && c->w[m - 1] % 4 == 0 && c->w_off[m] % 4 == 0; }
-// Whether a pass over `rows` rows is to work with copies.  They cost launches of their own (v, X, the output layer's delta) and
-// bytes; what they save grows with the weights.  Products, per mille of the time without copies: 784-300-300-10 (0.33e6 weights) 970 to
-// 1090 at 500 to 12000 rows, 784-500-500-10 (0.64e6) 920 to 970, 3072-1000-1000-10 (4.1e6) 850 to 950, 784-2000-2000-2000-10
-// 930 at 1000 rows and 690 at 12000.
-bool half_wanted(gn_ctx* c, int64_t rows) {
+// Whether a pass over `rows` rows is to work with copies.  They cost launches of their own (v, X, the output layer's delta), bytes
+// that grow with the weights, and the chained form of the pass; what they save grows with the rows times the weights.  Times with
+// copies over times without, network (weights), at 2000 / 4000 / 8000 / 16000 rows; theta new in every pass for f and the gradient:
+//                               full product           stored-factor product  gradient               f
+//   784-500-500-10 (0.65e6)     .97 1.12 1.05 .82      1.05 .94 .88 .83       1.03 1.14 1.05 .87     1.27 1.22 1.11 1.22
+//   784-800-800-10 (1.3e6)      .93 1.08  .97 .81      1.08 .97 .93 .90        .99 1.09 1.01 .86     1.12 1.12 1.14 1.13
+//   784-1000x3-10 (2.8e6)       .93 1.09  .85 .79      1.09 1.07 .99 .92      1.00 1.09  .84 .77     1.08 1.13 1.09 1.01
+//   3072-1000-1000-10 (4.1e6)   .99 1.08  .86 .81      1.02 .96 .87 .90        .97 1.01  .94 .89     1.13 1.10 1.13 1.11
+//   784-2000x3-10 (9.6e6)      1.02  .85  .87 .78      1.00 .95 .92 .89       1.07  .86  .80 .78     1.13  .99  .89  .83
+//   1024-4096x4-100 (55e6)      .85  .76               -                       .86  .75              1.00  .86
+// (at 1000 and 500 rows of the last: 0.94 and 1.12 for the product, 1.19 and 1.20 for f.)  But for block products, where all layers have
+// as many contractions (784-1000-16 at 12000 rows: 0.84), the first layer counts half: it has half of the others', and a copy of X to pay
+// for (288-2200-59 at 26013 rows: 1.04).
+enum HalfKind { kHalfStored, kHalfProduct, kHalfGrad, kHalfFun };   // block products through stored factors; full product, factors; ...
+bool half_pays(HalfKind kind, double rows, double weights) {
+  if (weights < (kind == kHalfStored ? 5e5 : 4e5)) return false;
+  if (kind == kHalfFun) return rows * weights >= 6.5e10;
+  return rows >= (kind == kHalfStored ? 3000.0 : 12000.0) || (rows >= 1000.0 && rows * weights >= 1.8e10);
+}
+bool half_wanted(gn_ctx* c, int64_t rows, HalfKind kind) {
   if (c->prec != GN_TF32 || c->half_mode == 0 || !c->half_usable || rows <= 128 || c->L < 2) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   // (what a caller captures is replayed after theta has changed: such a graph reads the FP32 matrices)
   if (!c->own_capture && cudaStreamIsCapturing(c->st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) return false;
   double weights = 0.0;
   for (int m = 1; m <= c->L; ++m)
-    if (half_layer(c, m)) weights += (double)c->w[m - 1] * c->w[m];
-  return weights > 0.0 && (c->half_mode == 2 || (weights >= 5e5 && rows * weights >= 1e9));
+    if (half_layer(c, m)) weights += (m == 1 && kind != kHalfStored ? 0.5 : 1.0) * c->w[m - 1] * c->w[m];
+  return weights > 0.0 && (c->half_mode == 2 || half_pays(kind, (double)rows, weights));
 }
 // A pass that works with copies, or not.  What is known at its end beyond theta and the stored activations is forgotten: a copy is
 // found by the address of its matrix, and the next pass may meet another matrix there (of the caller, or in memory that the
@@ -1272,7 +1287,7 @@ gn_status product_full_pass(gn_ctx* c, const float* v, float* out, float coef) {
   ++c->parts_epoch;
   const int L = c->L;
   const int64_t nS = c->nS;
-  HalfPass half_guard(c, half_wanted(c, nS));
+  HalfPass half_guard(c, half_wanted(c, nS, kHalfProduct));
   half_theta(c);
   half_vector(c, v);
   half_room(c, gn_ctx::kHRZ, c->RZ, L - 1, nS, c->capS);
@@ -1412,7 +1427,7 @@ gn_status ensure_factors(gn_ctx* c) {
     c->capF = nS;
   }
   c->launches += launch_factor_last(Wm(c, c->theta, L), c->Z[L - 1], nS, nL, c->w[L - 1], c->DF[L - 1], c->st);
-  HalfPass half_guard(c, L >= 3 && half_wanted(c, nS * nL));
+  HalfPass half_guard(c, L >= 3 && half_wanted(c, nS * nL, kHalfProduct));
   half_theta(c);
   // (the factors' copies are the largest: where they find no room the recurrence goes on without, and the other copies stay)
   const auto room = [&](int m) {
@@ -1452,7 +1467,7 @@ gn_status product_blockdiag_stored(gn_ctx* c, const float* v, float* out, float 
   const int L = c->L, nL = c->w[L];
   const int64_t nS = c->nS;
   const float inv = (float)(1.0 / (double)nS);
-  HalfPass half_guard(c, half_wanted(c, nS));
+  HalfPass half_guard(c, half_wanted(c, nS, kHalfStored));
   half_vector(c, v);
   constexpr int kGroup = 3;
   // The layers' chains are independent of one another, so each stage is issued for all layers together.
@@ -1582,7 +1597,7 @@ gn_status product_split(gn_ctx* c, const float* v, float* out, float coef) {
     c->capSplit = need;
   }
   const float inv = (float)(1.0 / (double)nS);
-  HalfPass half_guard(c, half_wanted(c, nS));
+  HalfPass half_guard(c, half_wanted(c, nS, kHalfStored));
   half_vector(c, v);
   std::vector<GemmArgs> batch;
   for (int m = 1; m <= L; ++m) {
@@ -1714,7 +1729,7 @@ gn_status fun_grad_pass(gn_ctx* c, float* d_grad, double* f_host) {
     const float* X0 = c->dX + r0 * c->w[0];
     c->cur_x = X0;
     ++c->parts_epoch;           // the batch buffers are rewritten
-    HalfPass half_guard(c, half_wanted(c, rows));
+    HalfPass half_guard(c, half_wanted(c, rows, d_grad ? kHalfGrad : kHalfFun));
     forward_pass(c, X0, rows, c->Zb, gn_ctx::kHZb, c->capB);
     c->launches += launch_loss_delta(c->Zb[L], c->dY + r0 * c->w[L], rows * c->w[L], d_grad ? c->Db[L] : nullptr,
                                      c->partial + b * per_batch, c->st);
@@ -2062,7 +2077,9 @@ static gn_status set_subsample_pass(gn_ctx* c, const int32_t* idx, int64_t nS, c
     GN_TRY(run_small_pass(c, kSmallForward, small, 0.f, nullptr, 0.f, nullptr, nullptr));
   } else {
     c->launches += launch_gather_rows(c->dX, c->l, c->w[0], c->idx, nS, c->Z[0], c->err_flag, c->st);
-    HalfPass half_guard(c, half_wanted(c, nS));
+    // (copies of the stored activations are there for the products)
+    const bool blocks = c->w[c->L] <= 16 || c->has_split;
+    HalfPass half_guard(c, half_wanted(c, nS, kHalfProduct) || (blocks && half_wanted(c, nS, kHalfStored)));
     forward_pass(c, c->Z[0], nS, c->Z, gn_ctx::kHZ, c->capS);
   }
   GN_TRY(check_launch(c, "set_subsample"));
