@@ -35,8 +35,8 @@ FP32_LANES_PER_SM, SMS = 128, 148
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant GEMM kernel from an ncu capture of the
 # kernel as it stands.  Multi-pass counters are only taken on the small case (|S| = 3000), so the figure belongs to
 # that workload; for every other workload `traffic` is None and the small-case figure is quoted beside it.
-TRAFFIC = {("tf32", "mnist2000_5"): {"bytes_per_launch": 145.1e6, "kernel": "gemm_tf32_2cta_kernel",
-                                     "launch": "forward R pass of a hidden layer, 3000 x 2000 x (2000 + 2000); 128 MB algorithmic",
+TRAFFIC = {("tf32", "mnist2000_5"): {"bytes_per_launch": 81.8e6, "kernel": "gemm_tf32_2cta_kernel",
+                                     "launch": "forward R pass of a hidden layer, 3000 x 2000 x (2000 + 2000) on FP16 copies; 100 MB algorithmic, part of it still in L2",
                                      "source": "profiles/gemm_tf32_2cta_mnist2000_5_ncu.md"}}
 
 
