@@ -244,7 +244,7 @@ struct ThinKParams {
 };
 
 // With a copy (COPY): the scale comes from |D| <= K max|A| max|B| / 4 (the sigmoid derivative), the runs looked at are a warp's 128
-// elements of a row and the block's rows of a column.  (A pass of its own for the largest magnitude and one for the copy
+// elements of a row (32 at least, at its end) and the block's rows of a column.  (A pass of its own for the largest magnitude and one for the copy
 // took 20 + 24 us at 12000 x 2000; written here it costs 7, and 5 for the largest magnitude of A.)
 template <int KMAX, bool COPY>
 __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p) {
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(128, 4) gemm_thin_k_kernel(const ThinKParams p
           const float y[4] = {t[0] * sc, t[1] * sc, t[2] * sc, t[3] * sc};
           const float row = max3_abs(max3_abs(0.f, y[0], y[1]), y[2], y[3]);
           const unsigned row_max = __reduce_max_sync(in, __float_as_uint(row));
-          if (in == 0xffffffffu) check.run(__uint_as_float(row_max));
+          if (__popc(in) >= 8) check.run(__uint_as_float(row_max));      // (32 elements)
           largest = max3_abs(largest, row, row);
 #pragma unroll
           for (int j = 0; j < 4; ++j) col[j] = max3_abs(col[j], y[j], y[j]);

@@ -32,8 +32,8 @@ struct HalfMat { void* p = nullptr; int64_t ld = 0; HalfInfo* info = nullptr; };
 // A run of elements of a row (32 or 128) or column (16, or more) whose largest scaled magnitude is below this (and not zero) makes
 // a copy bad: above it the rounding of a denormal, at most 2^-25, stays below the 2^-12 by which rounding to 11 bits changes the
 // run's largest element.  (Runs of 2 and 8 elements were too short: a few saturated neurons have them, and one run decides over a
-// whole matrix.  For the same reason what is left over at the end of a row or column, shorter than a run, is not judged by itself: the
-// row's or column's runs are.)
+// whole matrix.  For the same reason what a contraction leaves over at the end of a row or column, shorter than a run, is not judged
+// by itself: the row's or column's runs are.)
 constexpr float kHalfLeast = 1.220703125e-4f;   // 2^-13
 
 struct GemmArgs {

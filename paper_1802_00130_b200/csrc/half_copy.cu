@@ -72,7 +72,8 @@ __global__ void __launch_bounds__(512) half_amax_kernel(const __grid_constant__ 
 }
 
 // A block copies 128 rows x 128 columns, a warp 16 of the rows, a thread 4 of the columns (all requested before the first is
-// used).  The runs looked at for kHalfLeast are a row's 128 and a column's 16 elements.
+// used).  The runs looked at for kHalfLeast are a row's 128 and a column's 16 elements; the last of a row or column starts as far
+// back as it needs to be whole (what it has in common with the one before is written twice, the same).
 //
 // Sums of magnitudes, where they are asked for, are formed as whole numbers (a thread's part rounded up), so that the order in which
 // the blocks add theirs does not matter; whoever adds takes the sum so far to the maximum, and the last to add has the whole
@@ -97,10 +98,13 @@ __global__ void __launch_bounds__(256) half_copy_kernel(const __grid_constant__ 
   const float* const src = dep(s.src);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cell = (int)blockIdx.x - s.cell0, rc = cell / s.cells_ld;
-  const int c = (cell - rc * s.cells_ld) * COPY_CELL + 4 * lane, left = s.cols - c;
-  const long long r0 = (long long)rc * COPY_CELL + warp * COPY_ROWS;
+  const int c_own = (cell - rc * s.cells_ld) * COPY_CELL;
+  const int c0 = s.cols >= COPY_CELL && s.cols % 4 == 0 ? min(c_own, s.cols - COPY_CELL) : c_own;
+  const long long r_own = (long long)rc * COPY_CELL + warp * COPY_ROWS;
+  const long long r0 = s.rows >= COPY_ROWS && r_own < s.rows ? min(r_own, s.rows - COPY_ROWS) : r_own;
+  const int skip_c = c_own - c0, skip_r = (int)(r_own - r0);      // columns and rows that are others' as well
+  const int c = c0 + 4 * lane, left = s.cols - c;
   const int n_rows = (int)max(0ll, min((long long)COPY_ROWS, s.rows - r0));
-  const bool whole_col = n_rows == COPY_ROWS || s.rows < COPY_ROWS, whole_row = left + 4 * lane >= COPY_CELL || s.cols < COPY_CELL;
   float4 x[COPY_ROWS];
   const float* q = src + r0 * s.ld + c;
 #pragma unroll
@@ -148,24 +152,23 @@ __global__ void __launch_bounds__(256) half_copy_kernel(const __grid_constant__ 
 #pragma unroll
     for (int j = 0; j < 4; ++j) { col[j] = fmaxf(col[j], fabsf(y[j])); row = fmaxf(row, fabsf(y[j])); }
     if (s.row_sums) {
-      const unsigned part = __reduce_add_sync(0xffffffffu, __float2uint_ru((fabsf(y[0]) + fabsf(y[1]) + fabsf(y[2]) + fabsf(y[3])) * (float)(1 << kHalfNormExp)));
+      const float mine = 4 * lane < skip_c ? 0.f : fabsf(y[0]) + fabsf(y[1]) + fabsf(y[2]) + fabsf(y[3]);
+      const unsigned part = __reduce_add_sync(0xffffffffu, __float2uint_ru(mine * (float)(1 << kHalfNormExp)));
       if (lane == i) row_sum = part;
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) col_sum[j] += fabsf(y[j]);
-    const unsigned row_max = __reduce_max_sync(0xffffffffu, __float_as_uint(row));
-    if (whole_row || row_max > __float_as_uint(65504.f)) check.run(__uint_as_float(row_max));
+    for (int j = 0; j < 4; ++j) col_sum[j] += i < skip_r ? 0.f : fabsf(y[j]);
+    check.run(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(row))));
     if (i < n_rows && left > 0) {                 // (ld_out is a multiple of 8: a whole group always fits)
       const __half2 a = __floats2half2_rn(y[0], y[1]), b = __floats2half2_rn(y[2], y[3]);
       *reinterpret_cast<uint2*>(o) = make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b));
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (whole_col) check.run(col[j]);
+  for (int j = 0; j < 4; ++j) check.run(col[j]);
   if (__any_sync(0xffffffffu, check.bad()) && lane == 0) atomicOr(&s.info->bad, 1u);
   if (s.row_sums) {
-    unsigned long long sum = lane < n_rows ? atomicAdd(s.row_sums + r0 + lane, (unsigned long long)row_sum) + row_sum : 0ull;
+    unsigned long long sum = lane >= skip_r && lane < n_rows ? atomicAdd(s.row_sums + r0 + lane, (unsigned long long)row_sum) + row_sum : 0ull;
     report_sum(&s.info->row1, sum, lane);
   }
   if (s.col_sums) {
@@ -176,8 +179,8 @@ __global__ void __launch_bounds__(256) half_copy_kernel(const __grid_constant__ 
     for (int j = 0; j < 4; ++j) atomicAdd(part + 4 * lane + j, __float2uint_ru(col_sum[j] * (float)(1 << kHalfNormExp)));
     __syncthreads();
     if (threadIdx.x < COPY_CELL) {
-      const int cc = (cell - rc * s.cells_ld) * COPY_CELL + threadIdx.x;
-      unsigned long long sum = cc < s.cols ? atomicAdd(s.col_sums + cc, (unsigned long long)part[threadIdx.x]) + part[threadIdx.x] : 0ull;
+      const int cc = c0 + (int)threadIdx.x;
+      unsigned long long sum = cc >= c_own && cc < s.cols ? atomicAdd(s.col_sums + cc, (unsigned long long)part[threadIdx.x]) + part[threadIdx.x] : 0ull;
       report_sum(&s.info->col1, sum, lane);
     }
   }

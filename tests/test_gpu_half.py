@@ -94,6 +94,28 @@ def test_a_copy_that_cannot_hold_its_matrix_is_not_used(ctx, spoil, a_k, b_k):
         assert rows.all()
 
 
+def far_end_of_a_column(A):
+    A[:-(A.shape[0] % 16 or 16), 3] = 0
+    A[-(A.shape[0] % 16 or 16):, 3] *= 1e-11
+
+
+def far_end_of_a_row(A):
+    A[7, :-(A.shape[1] % 128)] = 0
+    A[7, -(A.shape[1] % 128):] *= 1e-11
+
+
+@pytest.mark.parametrize("spoil", [far_end_of_a_column, far_end_of_a_row])
+@pytest.mark.parametrize("a_k", [True, False])
+def test_runs_at_the_end_of_a_row_or_column_are_judged(ctx, spoil, a_k):
+    """The only numbers of a row or column stand at its end, in fewer elements than a run has, far below the others."""
+    A, B = operands(516, 392, 300, a_k, True, 13)
+    spoil(A)
+    got = ctx.debug_gemm(HALF, dev(A), dev(B), a_kmajor=a_k, b_kmajor=True).cpu().numpy()
+    ref = round11(A).astype(np.float64)
+    ref = (ref if a_k else ref.T) @ round11(B).astype(np.float64).T
+    assert (np.linalg.norm(got - ref, axis=1) <= 1e-5 * np.linalg.norm(ref, axis=1)).all()
+
+
 NETS = {
     "mid": lambda: wl.make("mid"),
     "wide_output": lambda: wl.make_custom([260, 392, 520, 260, 132], l=1500, nS=1100, C=15.0, seed=51, x="normal"),
